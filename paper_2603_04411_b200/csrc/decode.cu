@@ -252,109 +252,219 @@ __global__ void __launch_bounds__(1024) plan_kernel(DevView v, int layer, const 
 }
 
 // -------------------------------------------------------------- merge + V projection
-// One CTA per (query slot, KV head g): sums the splits, normalises, and projects the REP heads
-// of the group through U_V^-1[:, g*128 .. g*128+127].  512 threads: thread = (pair of output
-// columns, one eighth of the spectral index range), several rows of U_V^-1 in flight per thread.
-constexpr int MG_THREADS = 512;
-constexpr int MG_JGROUPS = MG_THREADS / 64;
+// A cluster of eight CTAs per (query slots, query heads of one KV head g): at most eight rows (slot, head).  CTA c takes
+// the spectral components [c d/8, (c+1) d/8): it sums their splits, normalises, and multiplies by its rows of
+// U_V^-1[:, g*128 .. g*128+127]; the eight partial [rows x 128] products meet through distributed shared memory, every CTA
+// adding and writing 16 of the columns.  What bounds it is latency: one CTA doing a group's whole sum and product went
+// through 256 KiB of U_V^-1 and every split by itself (29 us for one sequence of 1024 tokens with 64 splits, 23 us for 16
+// sequences of 32768 tokens; now 6 and 9).  Empty splits are not read (the V pass does not write them).
+constexpr int MG_THREADS = 256;
+constexpr int MG_CL = 8;                             // CTAs of a cluster
+constexpr int MG_ROWS = 8;
+
+__device__ __forceinline__ float ld_cluster_f32(uint32_t addr) {
+  float x;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(addr));
+  return x;
+}
 
 template <bool BF16>
 __global__ void __launch_bounds__(MG_THREADS)
 merge_kernel(DevView v, const unsigned short* __restrict__ Uinv_v, int n_splits, int hp, int ns, int n_seq, void* __restrict__ out) {
-  extern __shared__ float sAcc[];                    // [rows][d_kv] normalised spectral accumulators, then [MG_JGROUPS][rows][128]
-  __shared__ float sInvL[8];
-  // blockIdx.y = KV head g and which hp of its query heads (hp divides the group size; small batches use hp < group
-  // size so that the grid still fills the device); blockIdx.x = ns query slots that share the reads of U_V^-1 (large
-  // batches).  A row of this CTA is (slot, head): at most 8 rows.
-  const int qs0 = blockIdx.x * ns, parts = v.rep / hp, g = blockIdx.y / parts, tid = threadIdx.x;
+  __shared__ float4 s_part[MG_THREADS];              // split sums per (split group, row, four components)
+  __shared__ __align__(16) float s_acc[MG_ROWS * 128];    // [rows][d / 8] normalised
+  __shared__ float s_red[4][MG_ROWS][128];
+  __shared__ float s_out[MG_ROWS * 128];
+  __shared__ float s_invl[MG_ROWS];
+  // blockIdx.y = KV head g and which hp of its query heads; blockIdx.x / 8 = ns query slots that share the reads of U_V^-1
+  const int c = tc::cluster_cta_rank();
+  const int qs0 = (blockIdx.x / MG_CL) * ns, parts = v.rep / hp, g = blockIdx.y / parts, tid = threadIdx.x, lane = tid & 31;
   const int Hq = v.Hq, d_kv = v.d_kv;
-  const int REP = min(ns, n_seq - qs0) * hp;                    // rows
+  const int rows = min(ns, n_seq - qs0) * hp;
   const int head0 = g * v.rep + (blockIdx.y % parts) * hp;      // first query head of this CTA
-  // the first rows of U_V^-1 this thread needs do not depend on the sums below: their reads go out first
-  const int dp = tid & 63, jg = tid >> 6;
-  const int jn = d_kv / MG_JGROUPS, j0 = jg * jn;
-  const unsigned* ucol = reinterpret_cast<const unsigned*>(Uinv_v + g * HEAD_DIM) + dp;    // two 16-bit columns per load
-  unsigned u[16], un[16];
+  const int jn = d_kv / MG_CL, j0 = c * jn;                     // jn: a multiple of 16, at most 128
+  // this thread's rows of U_V^-1 do not depend on the sums: their reads go out first (pair of columns dp, a quarter of the rows)
+  const int dp = tid & 63, jg = tid >> 6, jr = jn / 4;
+  const unsigned* ucol = reinterpret_cast<const unsigned*>(Uinv_v + (size_t)(j0 + jg * jr) * d_kv + g * HEAD_DIM) + dp;
+  unsigned u[32];
 #pragma unroll
-  for (int t = 0; t < 16; ++t) u[t] = __ldg(ucol + (size_t)(j0 + t) * (d_kv / 2));
+  for (int t = 0; t < 32; ++t) u[t] = t < jr ? __ldg(ucol + (size_t)t * (d_kv / 2)) : 0u;
   // row sums over the splits: warp w takes row w, its lanes read the splits' parts together, lane 0 adds them in split order
-  if ((tid >> 5) < REP) {
-    const int r = tid >> 5, lane = tid & 31;
-    const int qs = qs0 + r / hp, head = head0 + r % hp;
+  if ((tid >> 5) < rows) {
+    const int r = tid >> 5, qs = qs0 + r / hp, head = head0 + r % hp;
     float l = 0.f;
     for (int s0 = 0; s0 < n_splits; s0 += 32) {
       const float mine = s0 + lane < n_splits ? v.part_l[((size_t)qs * n_splits + s0 + lane) * Hq + head] : 0.f;
       const int n = min(32, n_splits - s0);
       for (int s = 0; s < n; ++s) l += __shfl_sync(0xffffffffu, mine, s);
     }
-    if (lane == 0) sInvL[r] = l > 0.f ? 1.f / l : 0.f;
+    if (lane == 0) s_invl[r] = l > 0.f ? 1.f / l : 0.f;
   }
-  // split sums in split order: a thread owns four consecutive columns of one row (one 16-byte read per split) and has
-  // the reads of eight splits in flight before it adds them (a loop of dependent adds over one read at a time left
-  // this kernel waiting for memory latency)
-  for (int i0 = tid * 4; i0 < REP * d_kv; i0 += 4 * MG_THREADS) {
-    const int hh = i0 / d_kv, j = i0 - hh * d_kv;                     // d_kv is a multiple of 64: the four columns share a row
-    const float4* p = reinterpret_cast<const float4*>(
-        v.part_acc + (((size_t)(qs0 + hh / hp) * n_splits) * Hq + head0 + hh % hp) * d_kv + j);
+  // split sums: a thread owns four components of one row and every sg_n-th split, with eight reads in flight
+  const int q4 = jn / 4, slots = rows * q4, sg_n = MG_THREADS / slots, sg = tid / slots, sl = tid - sg * slots;
+  if (sg < sg_n) {
+    const int r = sl / q4, qs = qs0 + r / hp;
+    const float4* p = reinterpret_cast<const float4*>(v.part_acc + (((size_t)qs * n_splits) * Hq + head0 + r % hp) * d_kv + j0) + (sl - r * q4);
     const size_t stride = (size_t)Hq * d_kv / 4;
+    const int* cut = v.vcut + (size_t)qs * (n_splits + 1);
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int s0 = 0; s0 < n_splits; s0 += 8) {
+    for (int s0 = sg; s0 < n_splits; s0 += 8 * sg_n) {
       float4 t[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) t[u] = s0 + u < n_splits ? __ldg(p + (size_t)(s0 + u) * stride) : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int k = 0; k < 8; ++k) {
+        const int s = s0 + k * sg_n;
+        t[k] = s < n_splits && cut[s + 1] > cut[s] ? __ldg(p + (size_t)s * stride) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
 #pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (s0 + u < n_splits) { a.x += t[u].x; a.y += t[u].y; a.z += t[u].z; a.w += t[u].w; }
+      for (int k = 0; k < 8; ++k) { a.x += t[k].x; a.y += t[k].y; a.z += t[k].z; a.w += t[k].w; }
     }
-    *reinterpret_cast<float4*>(sAcc + i0) = a;
+    s_part[sg * slots + sl] = a;
   }
   __syncthreads();
-  for (int i0 = tid * 4; i0 < REP * d_kv; i0 += 4 * MG_THREADS) {       // each thread scales what it wrote
-    const float il = sInvL[i0 / d_kv];
-    float4 a = *reinterpret_cast<float4*>(sAcc + i0);
-    a.x *= il; a.y *= il; a.z *= il; a.w *= il;
-    *reinterpret_cast<float4*>(sAcc + i0) = a;
+  if (tid < slots) {
+    float4 a = s_part[tid];
+    for (int k = 1; k < sg_n; ++k) {                   // fixed order
+      const float4 b = s_part[k * slots + tid];
+      a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w;
+    }
+    const float il = s_invl[tid / q4];
+    *reinterpret_cast<float4*>(s_acc + tid * 4) = make_float4(a.x * il, a.y * il, a.z * il, a.w * il);
   }
   __syncthreads();
-  float o[8][2];
+  float o[MG_ROWS][2];
 #pragma unroll
-  for (int h = 0; h < 8; ++h) { o[h][0] = 0.f; o[h][1] = 0.f; }
-  for (int jb = 0; jb < jn; jb += 16) {                // jn is a multiple of 16 (d_kv a multiple of 128)
-    if (jb + 16 < jn) {                                // the next sixteen rows are on their way while these are used
+  for (int h = 0; h < MG_ROWS; ++h) { o[h][0] = 0.f; o[h][1] = 0.f; }
 #pragma unroll
-      for (int t = 0; t < 16; ++t) un[t] = __ldg(ucol + (size_t)(j0 + jb + 16 + t) * (d_kv / 2));
-    }
+  for (int t = 0; t < 32; t += 4) {
+    if (t >= jr) break;                                // jr is a multiple of 4
+    float u0[4], u1[4];
 #pragma unroll
-    for (int t = 0; t < 16; ++t) {
-      const float u0 = to_f32<BF16>((unsigned short)(u[t] & 0xffffu)), u1 = to_f32<BF16>((unsigned short)(u[t] >> 16));
+    for (int e = 0; e < 4; ++e) { u0[e] = to_f32<BF16>((unsigned short)(u[t + e] & 0xffffu)); u1[e] = to_f32<BF16>((unsigned short)(u[t + e] >> 16)); }
 #pragma unroll
-      for (int h = 0; h < 8; ++h)
-        if (h < REP) {
-          const float a = sAcc[h * d_kv + j0 + jb + t];
-          o[h][0] += a * u0;
-          o[h][1] += a * u1;
-        }
-    }
-#pragma unroll
-    for (int t = 0; t < 16; ++t) u[t] = un[t];
+    for (int h = 0; h < MG_ROWS; ++h)
+      if (h < rows) {
+        const float4 a = *reinterpret_cast<const float4*>(s_acc + h * jn + jg * jr + t);
+        o[h][0] += a.x * u0[0]; o[h][1] += a.x * u1[0];
+        o[h][0] += a.y * u0[1]; o[h][1] += a.y * u1[1];
+        o[h][0] += a.z * u0[2]; o[h][1] += a.z * u1[2];
+        o[h][0] += a.w * u0[3]; o[h][1] += a.w * u1[3];
+      }
   }
-  __syncthreads();
-  float* red = sAcc;                                 // reuse: [MG_JGROUPS][REP][128]
 #pragma unroll
-  for (int h = 0; h < 8; ++h)
-    if (h < REP) *reinterpret_cast<float2*>(red + (jg * REP + h) * 128 + 2 * dp) = make_float2(o[h][0], o[h][1]);
+  for (int h = 0; h < MG_ROWS; ++h)
+    if (h < rows) *reinterpret_cast<float2*>(&s_red[jg][h][2 * dp]) = make_float2(o[h][0], o[h][1]);
   __syncthreads();
-  for (int i = tid; i < REP * 128; i += MG_THREADS) {
+  for (int i = tid; i < rows * 128; i += MG_THREADS)
+    s_out[i] = ((s_red[0][i >> 7][i & 127] + s_red[1][i >> 7][i & 127]) + s_red[2][i >> 7][i & 127]) + s_red[3][i >> 7][i & 127];
+  tc::cluster_sync_all();
+  constexpr int CW = 128 / MG_CL;                      // columns this CTA writes
+  if (tid < rows * CW) {
+    const int h = tid / CW, dc = c * CW + tid % CW;
+    const uint32_t at = tc::smem_addr(s_out + h * 128 + dc);
     float val = 0.f;
 #pragma unroll
-    for (int k = 0; k < MG_JGROUPS; ++k) val += red[k * REP * 128 + i];        // fixed order
-    const int h = i >> 7, dc = i & 127;
+    for (int k = 0; k < MG_CL; ++k) val += ld_cluster_f32(tc::cluster_map(at, k));       // fixed order
     const int oslot = qs0 + h / hp;
     const size_t oi = ((size_t)(v.qmap ? v.qmap[oslot] : oslot) * Hq + head0 + h % hp) * HEAD_DIM + dc;
     if (v.out_dtype == TWKV_F32) reinterpret_cast<float*>(out)[oi] = val;
     else if (v.out_dtype == TWKV_BF16) reinterpret_cast<unsigned short*>(out)[oi] = from_f32<true>(val);
     else reinterpret_cast<unsigned short*>(out)[oi] = from_f32<false>(val);
   }
+  tc::cluster_sync_all();                              // the partners have read this CTA's part
+}
+
+// The same for large batches: 32 rows per cluster share a CTA's slice of U_V^-1, staged in shared memory; thread = (pair of
+// columns, a quarter of the rows).  With eight rows the reads of U_V^-1 (256 KiB per eight rows and KV head) bound it: 62 us
+// for 64 sequences of 8192 tokens.
+constexpr int MW_ROWS = 32;
+constexpr int MW_SMEM = 128 * 128 * 2 + 2 * MW_ROWS * 128 * 4 + MW_ROWS * 4;
+
+template <bool BF16>
+__global__ void __launch_bounds__(MG_THREADS)
+merge_wide_kernel(DevView v, const unsigned short* __restrict__ Uinv_v, int n_splits, int n_seq, void* __restrict__ out) {
+  extern __shared__ __align__(16) unsigned char mw_smem[];
+  unsigned* s_u = reinterpret_cast<unsigned*>(mw_smem);                                // [d / 8][64] pairs of columns
+  float* s_acc = reinterpret_cast<float*>(mw_smem + 128 * 128 * 2);                    // [rows][d / 8]
+  float* s_out = s_acc + MW_ROWS * 128;                                                // [rows][128]
+  float* s_invl = s_out + MW_ROWS * 128;
+  const int c = tc::cluster_cta_rank(), g = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int ns = MW_ROWS / v.rep, qs0 = (blockIdx.x / MG_CL) * ns;
+  const int Hq = v.Hq, d_kv = v.d_kv, rep = v.rep;
+  const int rows = min(ns, n_seq - qs0) * rep;
+  const int jn = d_kv / MG_CL, j0 = c * jn;
+  for (int i = tid; i < jn * 16; i += MG_THREADS) {                                    // 16-byte pieces of this CTA's rows of U_V^-1
+    const uint4 w = __ldg(reinterpret_cast<const uint4*>(Uinv_v + (size_t)(j0 + (i >> 4)) * d_kv + g * HEAD_DIM) + (i & 15));
+    reinterpret_cast<uint4*>(s_u)[i] = w;
+  }
+  for (int r = warp; r < rows; r += MG_THREADS / 32) {
+    const int qs = qs0 + r / rep, head = g * rep + r % rep;
+    float l = 0.f;
+    for (int s0 = 0; s0 < n_splits; s0 += 32) {
+      const float mine = s0 + lane < n_splits ? v.part_l[((size_t)qs * n_splits + s0 + lane) * Hq + head] : 0.f;
+      const int n = min(32, n_splits - s0);
+      for (int s = 0; s < n; ++s) l += __shfl_sync(0xffffffffu, mine, s);
+    }
+    if (lane == 0) s_invl[r] = l > 0.f ? 1.f / l : 0.f;
+  }
+  __syncthreads();
+  const int q4 = jn / 4;
+  for (int i = tid; i < rows * q4; i += MG_THREADS) {
+    const int r = i / q4, qs = qs0 + r / rep;
+    const float4* p = reinterpret_cast<const float4*>(v.part_acc + (((size_t)qs * n_splits) * Hq + g * rep + r % rep) * d_kv + j0) + (i - r * q4);
+    const size_t stride = (size_t)Hq * d_kv / 4;
+    const int* cut = v.vcut + (size_t)qs * (n_splits + 1);
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s0 = 0; s0 < n_splits; s0 += 4) {
+      float4 t[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        t[k] = s0 + k < n_splits && cut[s0 + k + 1] > cut[s0 + k] ? __ldg(p + (size_t)(s0 + k) * stride) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) { a.x += t[k].x; a.y += t[k].y; a.z += t[k].z; a.w += t[k].w; }
+    }
+    const float il = s_invl[r];
+    *reinterpret_cast<float4*>(s_acc + i * 4) = make_float4(a.x * il, a.y * il, a.z * il, a.w * il);
+  }
+  __syncthreads();
+  const int dp = tid & 63, r0 = (tid >> 6) * (MW_ROWS / 4);
+  if (r0 < rows) {
+    float o[MW_ROWS / 4][2];
+#pragma unroll
+    for (int h = 0; h < MW_ROWS / 4; ++h) { o[h][0] = 0.f; o[h][1] = 0.f; }
+    for (int t = 0; t < jn; t += 4) {
+      float u0[4], u1[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const unsigned w = s_u[(t + e) * 64 + dp];
+        u0[e] = to_f32<BF16>((unsigned short)(w & 0xffffu)); u1[e] = to_f32<BF16>((unsigned short)(w >> 16));
+      }
+#pragma unroll
+      for (int h = 0; h < MW_ROWS / 4; ++h) {          // rows past the last hold whatever is in shared memory and are not written out
+        const float4 a = *reinterpret_cast<const float4*>(s_acc + (r0 + h) * jn + t);
+        o[h][0] += a.x * u0[0]; o[h][1] += a.x * u1[0];
+        o[h][0] += a.y * u0[1]; o[h][1] += a.y * u1[1];
+        o[h][0] += a.z * u0[2]; o[h][1] += a.z * u1[2];
+        o[h][0] += a.w * u0[3]; o[h][1] += a.w * u1[3];
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < MW_ROWS / 4; ++h) *reinterpret_cast<float2*>(s_out + (r0 + h) * 128 + 2 * dp) = make_float2(o[h][0], o[h][1]);
+  }
+  tc::cluster_sync_all();
+  constexpr int CW = 128 / MG_CL;                      // columns this CTA writes
+  for (int i = tid; i < rows * CW; i += MG_THREADS) {
+    const int h = i / CW, dc = c * CW + i % CW;
+    const uint32_t at = tc::smem_addr(s_out + h * 128 + dc);
+    float val = 0.f;
+#pragma unroll
+    for (int k = 0; k < MG_CL; ++k) val += ld_cluster_f32(tc::cluster_map(at, k));       // fixed order
+    const int oslot = qs0 + h / rep;
+    const size_t oi = ((size_t)(v.qmap ? v.qmap[oslot] : oslot) * Hq + g * rep + h % rep) * HEAD_DIM + dc;
+    if (v.out_dtype == TWKV_F32) reinterpret_cast<float*>(out)[oi] = val;
+    else if (v.out_dtype == TWKV_BF16) reinterpret_cast<unsigned short*>(out)[oi] = from_f32<true>(val);
+    else reinterpret_cast<unsigned short*>(out)[oi] = from_f32<false>(val);
+  }
+  tc::cluster_sync_all();                              // the partners have read this CTA's part
 }
 
 // ------------------------------------------------------------------------- host side
@@ -380,18 +490,35 @@ static cudaError_t launch_decode_t(const DevView& v, int layer, const LayerParam
     cudaError_t e = launch_vacc_tc(v, layer, maps->blocks, maps->scores, seq_ids, n_seq, n_splits, st);
     if (e != cudaSuccess) return e;
   }
-  // query heads per merge CTA: the whole group when the batch fills the device, fewer (a divisor) for small batches;
-  // query slots per CTA: more than one (they share the reads of U_V^-1) while the grid still fills most of the device
-  int hp = v.rep;
-  while (hp % 2 == 0 && 2 * n_seq * v.Hkv * (v.rep / hp) < sm_count) hp /= 2;
-  int ns = 1;
-  while (2 * ns * hp <= 8 && 4 * (n_seq * v.Hkv * (v.rep / hp) / (2 * ns)) >= 3 * sm_count) ns *= 2;
-  const size_t mg_a = (size_t)ns * hp * v.d_kv * 4, mg_b = (size_t)MG_JGROUPS * ns * hp * 128 * 4;
-  const size_t mg_smem = mg_a > mg_b ? mg_a : mg_b;
   {
     ProfScope ps(TWKV_K_MERGE, st);
-    merge_kernel<BF16><<<dim3((n_seq + ns - 1) / ns, v.Hkv * (v.rep / hp)), MG_THREADS, mg_smem, st>>>(
-        v, reinterpret_cast<const unsigned short*>(lp.Uinv_v), n_splits, hp, ns, n_seq, out);
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(MG_THREADS);
+    cfg.stream = st;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = MG_CL; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    const unsigned short* uv = reinterpret_cast<const unsigned short*>(lp.Uinv_v);
+    const int wide = (n_seq * v.rep + MW_ROWS - 1) / MW_ROWS;
+    cudaError_t e;
+    if (MG_CL * wide * v.Hkv >= 2 * sm_count) {
+      // 32 rows per cluster while that still makes two CTAs per SM
+      cfg.gridDim = dim3(MG_CL * wide, v.Hkv);
+      cfg.dynamicSmemBytes = MW_SMEM;
+      e = cudaFuncSetAttribute(merge_wide_kernel<BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, MW_SMEM);
+      if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, merge_wide_kernel<BF16>, v, uv, n_splits, n_seq, out);
+    } else {
+      // query heads per cluster: the whole group, fewer (a divisor) while there are less than two CTAs per SM; then query
+      // slots per cluster (they share the reads of U_V^-1) while there are more
+      int hp = v.rep, ns = 1;
+      while (hp % 2 == 0 && MG_CL * n_seq * v.Hkv * (v.rep / hp) < 2 * sm_count) hp /= 2;
+      while (2 * ns * hp <= MG_ROWS && MG_CL * (n_seq * v.Hkv * (v.rep / hp) / (2 * ns)) >= 2 * sm_count) ns *= 2;
+      cfg.gridDim = dim3(MG_CL * ((n_seq + ns - 1) / ns), v.Hkv * (v.rep / hp));
+      e = cudaLaunchKernelEx(&cfg, merge_kernel<BF16>, v, uv, n_splits, hp, ns, n_seq, out);
+    }
+    if (e != cudaSuccess) return e;
   }
   count_launch(4);
   return cudaGetLastError();

@@ -366,7 +366,8 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
     float* pa = v.part_acc + pidx * Hq * d_kv;
     const int quad = warp & 3;                                  // the TMEM lanes this warp may read
     const int used_pairs = ready ? (max_cls + 1) >> 1 : 0;
-    for (int pair = (warp - 2) >> 2; pair < n_pairs; pair += 2) {
+    // (a split without tiles leaves its part unwritten: the merge kernel knows it from the cut points)
+    for (int pair = (warp - 2) >> 2; pair < n_pairs && n_mine > 0; pair += 2) {
       const int col = pair * 128 + quad * 32 + lane;            // spectral column of this thread's TMEM lane
       const bool used = pair < used_pairs;
       const uint32_t src = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(pair * N);
