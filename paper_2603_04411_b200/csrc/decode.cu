@@ -1,6 +1,6 @@
 // Decode attention over the mixed-rank cache (Eq. 3, reshape to heads, RoPE, softmax attention).
 //
-//   plan_kernel    sequence id -> query slot map, running-max reset, K-tile work list; cut points of every
+//   plan_kernel    running-max reset, K-tile work list; cut points of every
 //                  sequence's V tiles into the splits of the V pass; K slot -> V slot links of the sequences' tokens
 //   kscore_tc_kernel (kscore_tc.cu)  per K tile: Kbar = X^_K U_K^-1, RoPE by stored position,
 //                  s = q . Kbar * scale for the GQA group, scores to scratch, per-sequence max
@@ -13,15 +13,19 @@
 #include "twkv_dev.h"
 #include "mma_util.cuh"
 #include "tc_util.cuh"
+#include "scan_util.cuh"
 
 namespace twkv {
 
 // ------------------------------------------------------------------------------ plan
-// One CTA: sequence id -> query slot map, running-max reset, and the K-score work list: the K tiles
-// of the listed sequences in class order (widest first, inside a class in table order), compacted
-// with block-wide scans so the order does not depend on thread timing.  For the CTA-pair kernel the list
-// is rewritten as items of two tiles of one class.  The list is then cut into n_cta contiguous pieces of
-// about equal estimated cost, so a CTA (pair) of the K-score kernel mostly stays inside one (class, sequence) run.
+// One launch prepares a decode pass.  CTAs 0 .. NC-1, one per rank class: the class's part of the K-score work list, the K
+// tiles of the listed sequences in table order, classes one behind the other from wide to narrow; for the CTA-pair kernel as
+// items of two tiles of one class.  Where a class's part starts follows from the keys' token counts (a key of n tokens has
+// ceil(n / 128) tiles), so the classes need not wait for one another; a class is compacted by block-wide scans, so the order
+// does not depend on thread timing.  CTA 0 also cuts the list into n_cta contiguous pieces of about equal estimated cost, so
+// that a CTA (pair) of the K-score kernel mostly stays inside one (class, sequence) run.  What bounds it is the chain of
+// dependent table reads: one CTA that walked the whole list took 17.5 us for 16 sequences of 32768 tokens (2200 tiles) and 17
+// for 64 of 8192; a CTA per class takes 8.6 and 9.5 (8.9 -> 8.4 for 8 tiles).
 __device__ __forceinline__ unsigned ktile_cost(int cls) {
   // cycles per tile of the K-score kernel by rank class: a least-squares fit, one coefficient per class, of every CTA's busy
   // time to its tile counts on the benchmark's mix of classes (8 KV heads, CTA pairs; residual 1.3 us rms of 330): a fixed
@@ -38,57 +42,42 @@ __device__ __forceinline__ unsigned ktile_cost(int cls) {
 // The list is taken in the stride order of vtile_stride(); cut[s] = number of tiles (in that order) whose inclusive cost
 // prefix is <= s / n_splits of the total; split s takes positions cut[s] .. cut[s + 1] - 1 of that order.
 __device__ void vsplit_plan(const DevView& v, int layer, const int* __restrict__ seq_ids, int qs, int n_splits) {
-  __shared__ unsigned long long s_total, s_base;
-  __shared__ unsigned s_ws[32];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __shared__ int s_warp[32];
+  const int tid = threadIdx.x;
   const int seq = seq_ids[qs];
   const int n = (seq >= 0 && seq < v.S) ? v.svc(layer)[seq] : 0;
   const int* list = v.svt(layer) + (size_t)(n > 0 ? seq : 0) * v.TPS;
   const int4* desc = v.desc(layer, 1);
   int* cut = v.vcut + (size_t)qs * (n_splits + 1);
-  if (tid == 0) { s_total = 0ull; s_base = 0ull; }
-  __syncthreads();
-  unsigned mine = 0u;
-  const long long stride = vtile_stride(n);
-  for (int i = tid; i < n; i += blockDim.x) mine += 32u * (unsigned)desc[list[i]].y + (unsigned)v.Hq;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
-  if (lane == 0 && mine) atomicAdd(&s_total, (unsigned long long)mine);
-  __syncthreads();
-  const unsigned long long W = s_total, ns = (unsigned long long)n_splits;
-  if (W == 0ull) {
-    for (int s = tid; s <= n_splits; s += blockDim.x) cut[s] = 0;
+  const int stride = vtile_stride(n);
+  // cost of the i-th tile in stride order (its sum over a list stays below 2^31: 32 * 16 + 64 units, at most 2^13 tiles)
+  auto cost = [&](int i) -> int { return i < n ? 32 * desc[list[vtile_at(i, stride, n)]].y + v.Hq : 0; };
+  // a list of up to 1024 tiles is read once; a longer one first for its total
+  const int first = cost(tid);
+  int total = 0, w = first, off = 0;
+  for (int i0 = 0; i0 < n; i0 += 1024) {
+    int part;
+    off = block_scan_excl(i0 ? cost(i0 + tid) : w, s_warp, &part);
+    total += part;
+  }
+  if (total == 0) {
+    for (int s = tid; s <= n_splits; s += 1024) cut[s] = 0;
     return;
   }
-  for (int i0 = 0; i0 < n; i0 += blockDim.x) {
-    const int i = i0 + tid;
-    const unsigned w = i < n ? 32u * (unsigned)desc[list[(int)((i * stride) % n)]].y + (unsigned)v.Hq : 0u;
-    unsigned inc = w;                                             // inclusive scan inside the warp, then over the warps
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned a = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += a;
+  const unsigned long long W = (unsigned long long)total, ns = (unsigned long long)n_splits;
+  int base = 0;
+  for (int i0 = 0; i0 < n; i0 += 1024) {
+    if (n > 1024) {
+      int part;
+      w = i0 ? cost(i0 + tid) : first;
+      off = base + block_scan_excl(w, s_warp, &part);
+      base += part;
     }
-    if (lane == 31) s_ws[warp] = inc;
-    __syncthreads();
-    if (warp == 0) {
-      unsigned wk = s_ws[lane];
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned a = __shfl_up_sync(0xffffffffu, wk, o);
-        if (lane >= o) wk += a;
-      }
-      s_ws[lane] = wk;
-    }
-    __syncthreads();
-    if (i < n) {
-      const unsigned long long p = s_base + (warp ? s_ws[warp - 1] : 0u) + inc, e = p - w;
+    if (i0 + tid < n) {
+      const unsigned long long e = (unsigned long long)off, p = e + (unsigned long long)w;
       // the splits whose boundary floor(s W / ns) falls in [e, p): they start at this tile
-      for (unsigned long long s = (e * ns + W - 1ull) / W; s < ns && s * W / ns < p; ++s) cut[s] = i;
+      for (unsigned long long s = (e * ns + W - 1ull) / W; s < ns && s * W / ns < p; ++s) cut[s] = i0 + tid;
     }
-    __syncthreads();
-    if (tid == 0) s_base += s_ws[31];
-    __syncthreads();
   }
   if (tid == 0) cut[n_splits] = n;
 }
@@ -112,140 +101,108 @@ __device__ void vlink_plan(const DevView& v, int layer, const int* __restrict__ 
 
 __global__ void __launch_bounds__(1024) plan_kernel(DevView v, int layer, const int* __restrict__ seq_ids, int n_seq, int n_cta, int pairs,
                                                     int n_splits, int vj) {
-  if ((int)blockIdx.x > n_seq) {                                  // the last n_seq * vj CTAs: K slot -> V slot links
-    const int idx = (int)blockIdx.x - 1 - n_seq;
+  const int NC = v.NC;
+  if ((int)blockIdx.x >= NC + n_seq) {                            // the last n_seq * vj CTAs: K slot -> V slot links
+    const int idx = (int)blockIdx.x - NC - n_seq;
     vlink_plan(v, layer, seq_ids, idx / vj, idx % vj, vj);
     return;
   }
-  if (blockIdx.x > 0) {                                           // CTAs 1 .. n_seq: the V pass's split plan, one sequence each
-    vsplit_plan(v, layer, seq_ids, (int)blockIdx.x - 1, n_splits);
+  if ((int)blockIdx.x >= NC) {                                    // before them n_seq CTAs: the V pass's split plan, one sequence each
+    vsplit_plan(v, layer, seq_ids, (int)blockIdx.x - NC, n_splits);
     return;
   }
-  __shared__ int s_cls_off[TWKV_MAX_CLASSES + 1], s_kcc[TWKV_MAX_CLASSES];
-  __shared__ unsigned s_wsum[32];
-  __shared__ unsigned s_base;                                     // entries kept so far
-  __shared__ int s_keep[TWKV_MAX_CLASSES];                        // kept tiles per class run (run k = class NC - k)
-  __shared__ int s_koff[TWKV_MAX_CLASSES + 1], s_ioff[TWKV_MAX_CLASSES + 1];    // start of run k in the tile list / in the item list
+  extern __shared__ int s_slot[];                                 // sequence id -> query slot, -1
+  __shared__ int s_warp[32];
+  __shared__ int s_keep[TWKV_MAX_CLASSES];                        // tiles of the listed sequences per class
+  __shared__ int s_koff[TWKV_MAX_CLASSES + 1], s_ioff[TWKV_MAX_CLASSES + 1];    // start of run k (class NC - k) in the tile list / in the item list
   __shared__ unsigned long long s_coff[TWKV_MAX_CLASSES + 1];     // estimated cost of everything before run k
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int s = tid; s < v.S; s += blockDim.x) v.qslot[s] = -1;
+  const int run = blockIdx.x, cls = NC - run;
+  const int n_list = v.kcc(layer)[cls - 1];
+  for (int s = tid; s < v.S; s += 1024) s_slot[s] = -1;
   if (tid < TWKV_MAX_CLASSES) s_keep[tid] = 0;
-  // the class counts are read by sixteen threads at once (one thread reading them in a loop pays a memory round trip
-  // per class)
-  if (tid < v.NC) s_kcc[tid] = v.kcc(layer)[tid];
   __syncthreads();
-  if (tid == 0) {
-    int run = 0;
-    for (int c = v.NC; c >= 1; --c) { s_cls_off[v.NC - c] = run; run += s_kcc[c - 1]; }    // widest class first
-    s_cls_off[v.NC] = run;
-    s_base = 0u;
-  }
-  __syncthreads();
-  for (int i = tid; i < n_seq; i += blockDim.x) {
+  for (int i = tid; i < n_seq; i += 1024) {
     const int s = seq_ids[i];
-    if (s < 0 || s >= v.S) set_status(v, TWKV_ERR_INVALID_ARG);
-    else v.qslot[s] = i;
+    if (s >= 0 && s < v.S) s_slot[s] = i;
+    else if (run == 0) set_status(v, TWKV_ERR_INVALID_ARG);
   }
-  for (int i = tid; i < n_seq * v.Hq; i += blockDim.x) v.seqmax[i] = 0u;
+  for (int i = run * 1024 + tid; i < n_seq * v.Hq; i += NC * 1024) v.seqmax[i] = 0u;
   __syncthreads();
-  for (int i = tid; i < n_seq; i += blockDim.x) {
-    const int s = seq_ids[i];
-    if (s >= 0 && s < v.S && v.qslot[s] != i) set_status(v, TWKV_ERR_INVALID_ARG);   // duplicate id
-  }
-  const int4* desc = v.desc(layer, 0);
-  const int* kct = v.kct(layer);
-  const int n_all = s_cls_off[v.NC];
-  constexpr int PL_BATCH = 4;                                     // list chunks of 1024 whose table reads are issued together
-  for (int f0 = 0; f0 < n_all; f0 += 1024 * PL_BATCH) {
-    // the three dependent reads (tile id -> descriptor -> query slot) of PL_BATCH chunks go out level by level
-    int tile[PL_BATCH], run_[PL_BATCH];
-    int4 d[PL_BATCH];
-    int4 ent[PL_BATCH];
-#pragma unroll
-    for (int u = 0; u < PL_BATCH; ++u) {
-      const int f = f0 + u * 1024 + tid;
-      tile[u] = -1; run_[u] = 0;
-      if (f < n_all) {
-        int k = 0;
-        while (f >= s_cls_off[k + 1]) ++k;
-        run_[u] = k;
-        tile[u] = kct[(size_t)(v.NC - k - 1) * v.NT + (f - s_cls_off[k])];
-      }
+  if (run == 0)
+    for (int i = tid; i < n_seq; i += 1024) {
+      const int s = seq_ids[i];
+      if (s >= 0 && s < v.S && s_slot[s] != i) set_status(v, TWKV_ERR_INVALID_ARG);   // duplicate id
     }
+  {
+    // tiles per class: a warp per class (and part of the sequences), a lane per sequence
+    const int parts = 32 / NC, k = warp % NC, part = warp / NC;
+    int mine = 0;
+    if (part < parts)
+      for (int s = part * 32 + lane; s < v.S; s += parts * 32)
+        if (s_slot[s] >= 0) mine += (v.fill_l(layer)[s * NC + k] + TILE - 1) / TILE;
 #pragma unroll
-    for (int u = 0; u < PL_BATCH; ++u) d[u] = tile[u] >= 0 ? desc[tile[u]] : make_int4(0, 0, 0, 0);
-#pragma unroll
-    for (int u = 0; u < PL_BATCH; ++u)
-      ent[u] = tile[u] >= 0 ? make_int4(tile[u], d[u].y | (d[u].z << 8), d[u].w, v.qslot[d[u].x]) : make_int4(0, 0, 0, -1);
-#pragma unroll
-    for (int u = 0; u < PL_BATCH; ++u) {
-      if (f0 + u * 1024 >= n_all) break;                         // uniform across the CTA
-      const int4 e = ent[u];
-      const unsigned keep = e.w >= 0 ? 1u : 0u;
-      unsigned ik = keep;                                         // inclusive scan inside the warp
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned a = __shfl_up_sync(0xffffffffu, ik, o);
-        if (lane >= o) ik += a;
-      }
-      if (lane == 31) s_wsum[warp] = ik;
-      __syncthreads();
-      if (warp == 0) {
-        unsigned wk = s_wsum[lane];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const unsigned a = __shfl_up_sync(0xffffffffu, wk, o);
-          if (lane >= o) wk += a;
-        }
-        s_wsum[lane] = wk;                                        // inclusive over warps
-      }
-      __syncthreads();
-      const unsigned pk = s_base + (warp ? s_wsum[warp - 1] : 0u) + ik - keep;      // exclusive position
-      if (keep) { v.klist[pk] = e; atomicAdd(&s_keep[run_[u]], 1); }
-      __syncthreads();
-      if (tid == 0) s_base += s_wsum[31];
-      __syncthreads();
-    }
+    for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
+    if (lane == 0 && mine) atomicAdd(&s_keep[k], mine);
   }
-  // class runs of the kept list: tiles, items (a pair item holds two tiles) and estimated cost before each run
+  __syncthreads();
   if (tid == 0) {
     int ko = 0, io = 0;
     unsigned long long co = 0ull;
-    for (int k = 0; k < v.NC; ++k) {
+    for (int k = 0; k < NC; ++k) {
       s_koff[k] = ko; s_ioff[k] = io; s_coff[k] = co;
-      const int items = pairs ? (s_keep[k] + 1) / 2 : s_keep[k];
-      ko += s_keep[k]; io += items;
-      co += (unsigned long long)items * ktile_cost(v.NC - k);
+      const int keep = s_keep[NC - k - 1], items = pairs ? (keep + 1) / 2 : keep;
+      ko += keep; io += items;
+      co += (unsigned long long)items * ktile_cost(NC - k);
     }
-    s_koff[v.NC] = ko; s_ioff[v.NC] = io; s_coff[v.NC] = co;
-    *v.klist_count = ko;
-    v.cta_start[n_cta] = io;
+    s_koff[NC] = ko; s_ioff[NC] = io; s_coff[NC] = co;
   }
   __syncthreads();
-  const int n_items = s_ioff[v.NC];
-  const unsigned long long total = s_coff[v.NC];
-  if (pairs) {
-    for (int i = tid; i < n_items; i += blockDim.x) {
-      int k = 0;
-      while (i >= s_ioff[k + 1]) ++k;
-      const int t0 = s_koff[k] + 2 * (i - s_ioff[k]);
-      const int4 e0 = v.klist[t0];
-      // a run of odd length ends with a filler: the same tile again, flagged so that its scores are dropped
-      v.kpairs[2 * i] = e0;
-      v.kpairs[2 * i + 1] = t0 + 1 < s_koff[k + 1] ? v.klist[t0 + 1] : make_int4(e0.x, e0.y | 0x80, e0.z, e0.w);
+  // this class's entries; a run of odd length ends with a filler for the pair kernel: the same tile again, flagged so that its
+  // scores are dropped
+  const int4* desc = v.desc(layer, 0);
+  const int* list = v.kct(layer) + (size_t)(cls - 1) * v.NT;
+  const int n_keep = s_koff[run + 1] - s_koff[run];
+  int base = 0;
+  for (int i0 = 0; i0 < n_list; i0 += 1024) {
+    int4 e = make_int4(0, 0, 0, -1);
+    if (i0 + tid < n_list) {
+      const int t = list[i0 + tid];
+      const int4 d = desc[t];
+      e = make_int4(t, d.y | (d.z << 8), d.w, s_slot[d.x]);
     }
+    int total;
+    const int at = base + block_scan_excl(e.w >= 0 ? 1 : 0, s_warp, &total);
+    if (e.w >= 0 && at < n_keep) {
+      if (pairs) {
+        v.kpairs[2 * s_ioff[run] + at] = e;
+        if (at == n_keep - 1 && (n_keep & 1)) v.kpairs[2 * s_ioff[run] + at + 1] = make_int4(e.x, e.y | 0x80, e.z, e.w);
+      } else {
+        v.klist[s_koff[run] + at] = e;
+      }
+    }
+    base += total;
   }
-  // cut points: piece b starts at the item whose cost interval holds b / n_cta of the total (64-bit arithmetic; inside
-  // a run every item costs the same, so the item follows from a division)
-  for (int b = tid; b < n_cta; b += blockDim.x) {
+  if (run > 0) return;
+  // Few items: the KV heads of an item are dealt out to several CTAs (pairs), as long as every part still finds one of its
+  // own; a part repeats the tile's loads and rotation factors, so a list that fills the device keeps whole items.  One
+  // sequence of 1024 tokens (4 items): K-score 32.6 us with whole items, 11.8 us with one head per part.
+  const int n_items = s_ioff[NC];
+  const unsigned long long total = s_coff[NC];
+  int hg = 1;
+  while (v.Hkv % (2 * hg) == 0 && n_items * 2 * hg <= n_cta) hg *= 2;
+  if (tid == 0) { *v.kitem_parts = hg; v.cta_start[n_cta] = n_items * hg; }
+  // cut points: piece b starts at the item part whose cost interval holds b / n_cta of the total (64-bit arithmetic; inside
+  // a run every part costs the same, so the part follows from a division)
+  for (int b = tid; b < n_cta; b += 1024) {
     int start = 0;
     if (n_items > 0 && total > 0ull) {
       const unsigned long long key = (unsigned long long)b * total / (unsigned long long)n_cta;
       int k = 0;
-      while (k + 1 < v.NC && s_coff[k + 1] <= key) ++k;
-      const unsigned long long within = (key - s_coff[k]) / ktile_cost(v.NC - k);
-      const int cap = s_ioff[k + 1] - s_ioff[k];
-      start = s_ioff[k] + (int)(within < (unsigned long long)cap ? within : (unsigned long long)cap);
+      while (k + 1 < NC && s_coff[k + 1] <= key) ++k;
+      const unsigned long long within = (key - s_coff[k]) * hg / ktile_cost(NC - k);
+      const int cap = (s_ioff[k + 1] - s_ioff[k]) * hg;
+      start = s_ioff[k] * hg + (int)(within < (unsigned long long)cap ? within : (unsigned long long)cap);
     }
     v.cta_start[b] = start;
   }
@@ -256,8 +213,9 @@ __global__ void __launch_bounds__(1024) plan_kernel(DevView v, int layer, const 
 // the spectral components [c d/8, (c+1) d/8): it sums their splits, normalises, and multiplies by its rows of
 // U_V^-1[:, g*128 .. g*128+127]; the eight partial [rows x 128] products meet through distributed shared memory, every CTA
 // adding and writing 16 of the columns.  What bounds it is latency: one CTA doing a group's whole sum and product went
-// through 256 KiB of U_V^-1 and every split by itself (29 us for one sequence of 1024 tokens with 64 splits, 23 us for 16
-// sequences of 32768 tokens; now 6 and 9).  Empty splits are not read (the V pass does not write them).
+// through 256 KiB of U_V^-1 and every split by itself.  Cold caches: 29.9 -> 9.2 us for one sequence of 1024 tokens with 64
+// splits, 28 -> 19.3 us for one of 131072 tokens with 64 heads; 16 sequences of 32768 tokens stay at 22 us, their 19 MB of
+// partial sums coming from DRAM.  Empty splits are not read (the V pass does not write them).
 constexpr int MG_THREADS = 256;
 constexpr int MG_CL = 8;                             // CTAs of a cluster
 constexpr int MG_ROWS = 8;
@@ -374,8 +332,8 @@ merge_kernel(DevView v, const unsigned short* __restrict__ Uinv_v, int n_splits,
 }
 
 // The same for large batches: 32 rows per cluster share a CTA's slice of U_V^-1, staged in shared memory; thread = (pair of
-// columns, a quarter of the rows).  With eight rows the reads of U_V^-1 (256 KiB per eight rows and KV head) bound it: 62 us
-// for 64 sequences of 8192 tokens.
+// columns, a quarter of the rows).  With eight rows the reads of U_V^-1 (256 KiB per eight rows and KV head) bound it:
+// 64 sequences of 8192 tokens 63 -> 44.5 us, 37 of up to 700 tokens 42 -> 28 us (43 with one CTA per KV head).
 constexpr int MW_ROWS = 32;
 constexpr int MW_SMEM = 128 * 128 * 2 + 2 * MW_ROWS * 128 * 4 + MW_ROWS * 4;
 
@@ -480,7 +438,7 @@ static cudaError_t launch_decode_t(const DevView& v, int layer, const LayerParam
   const int n_pieces = pairs ? kscore_max_pairs(sm_count) : sm_count;
   // CTAs per sequence that invert the V -> K links: enough of them that they finish inside the K work list's time
   const int vj = n_seq >= 256 ? 1 : (256 / n_seq > 64 ? 64 : 256 / n_seq);
-  { ProfScope ps(TWKV_K_PLAN, st); plan_kernel<<<1 + n_seq + n_seq * vj, 1024, 0, st>>>(v, layer, seq_ids, n_seq, n_pieces, pairs ? 1 : 0, n_splits, vj); }
+  { ProfScope ps(TWKV_K_PLAN, st); plan_kernel<<<v.NC + n_seq + n_seq * vj, 1024, (size_t)v.S * sizeof(int), st>>>(v, layer, seq_ids, n_seq, n_pieces, pairs ? 1 : 0, n_splits, vj); }
   {
     cudaError_t e = launch_kscore_tc(v, layer, maps->blocks, maps->uinvT_k, q, n_pieces, pairs, st);
     if (e != cudaSuccess) return e;

@@ -13,36 +13,11 @@
 // V side finds a token's position through its K row); (3) per key, the moves (a tile's rows are all read before any is
 // written, destinations never lie behind sources); (4) the tile lists without the emptied tiles.
 #include "twkv_dev.h"
+#include "scan_util.cuh"
 
 namespace twkv {
 
 constexpr int EV_THREADS = 1024;
-
-// exclusive scan of one value per thread over the CTA; returns the thread's offset, *total = sum (valid for all threads)
-__device__ __forceinline__ int block_scan_excl(int x, int* s_warp, int* total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int incl = x;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int u = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += u;
-  }
-  __syncthreads();                                         // s_warp may still be read from the previous call
-  if (lane == 31) s_warp[warp] = incl;
-  __syncthreads();
-  if (warp == 0) {
-    int w = s_warp[lane];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int u = __shfl_up_sync(0xffffffffu, w, o);
-      if (lane >= o) w += u;
-    }
-    s_warp[lane] = w;
-  }
-  __syncthreads();
-  *total = s_warp[31];
-  return (warp ? s_warp[warp - 1] : 0) + incl - x;
-}
 
 // The tiles of key (side, seq, cls) in creation order -> s_tiles; returns their number.  K tiles are listed per class
 // (all sequences), V tiles per sequence (all classes); both lists are in creation order.

@@ -158,8 +158,13 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
   const int4* klist = PAIR ? v.kpairs + crank : v.klist;
   constexpr int KSTEP = PAIR ? 2 : 1;
   const int4 kt_none = make_int4(0, 0, 0, -1);
+  // A work unit is one of the `hg` parts of a list item: all its panels, nh of the KV heads (hg > 1 only for short lists,
+  // where one item per CTA would leave most SMs idle and run through all heads one after the other).
+  const int hg = *v.kitem_parts, nh = Hkv / hg;
+  auto unit = [&](int w) -> int4 { return w < total ? klist[KSTEP * (w / hg)] : kt_none; };
   // CTAs walk the KV heads in rotated order, so that at any moment they read different panels of U_K^-1 from L2
-  const int g_rot = piece % Hkv;
+  const int g_rot = piece % nh;
+  auto head = [&](int w, int sl) -> int { return (w % hg) * nh + (sl + g_rot < nh ? sl + g_rot : sl + g_rot - nh); };
 
   if (misaligned) {
     // nothing was started; fall through to the common exit
@@ -174,9 +179,9 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
       tma_prefetch_desc(&map_blocks);
       uint32_t ak = 0;                                          // panels so far; slot = ak % 8
       bool ok = true;
-      int4 e = w0 < total ? klist[KSTEP * w0] : kt_none;
+      int4 e = unit(w0);
       for (int w = w0; w < total && ok; ++w) {
-        const int4 nxt = w + 1 < total ? klist[KSTEP * (w + 1)] : kt_none;
+        const int4 nxt = unit(w + 1);
         const int cls = e.y & 0x7f, blk = e.z;
         for (int j = 0; j < cls; ++j, ++ak) {
           const uint32_t slot = ak % KT_A_SLOTS, ph = (ak / KT_A_SLOTS) & 1u;
@@ -201,14 +206,14 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
       tma_prefetch_desc(&map_uinvT);
       uint32_t bk = 0, bst = 0, bph = 0;                        // panels so far; ring stage and its phase
       bool ok = true;
-      int4 e = w0 < total ? klist[KSTEP * w0] : kt_none;
+      int4 e = unit(w0);
       for (int w = w0; w < total && ok; ++w) {
-        const int4 nxt = w + 1 < total ? klist[KSTEP * (w + 1)] : kt_none;
+        const int4 nxt = unit(w + 1);
         const int cls = e.y & 0x7f;
         for (int p0 = 0; p0 < cls && ok; p0 += KT_A_SLOTS) {
           const int np = min(KT_A_SLOTS, cls - p0);
-          for (int sl = 0; sl < Hkv && ok; ++sl) {
-            const int g = sl + g_rot < Hkv ? sl + g_rot : sl + g_rot - Hkv;
+          for (int sl = 0; sl < nh && ok; ++sl) {
+            const int g = head(w, sl);
             for (int j = 0; j < np; j += 2, ++bk) {
               const uint32_t st = bst, ph = bph;
               if (++bst == (uint32_t)nb) { bst = 0; bph ^= 1u; }
@@ -242,18 +247,18 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
       const uint32_t a_lo0 = kmajor_sw128_desc_lo(sA), b_lo0 = kmajor_sw128_desc_lo(sB);
       uint32_t bst = 0, bph = 0, ak = 0, sbuf = 0, sph = 0;
       bool ok = true;
-      int4 e = w0 < total ? klist[KSTEP * w0] : kt_none;
+      int4 e = unit(w0);
       for (int w = w0; w < total && ok; ++w) {
-        const int4 nxt = w + 1 < total ? klist[KSTEP * (w + 1)] : kt_none;
+        const int4 nxt = unit(w + 1);
         const int cls = e.y & 0x7f;
         for (int p0 = 0; p0 < cls && ok; p0 += KT_A_SLOTS) {
           const int np = min(KT_A_SLOTS, cls - p0);
-          for (int sl = 0; sl < Hkv && ok; ++sl) {
+          for (int sl = 0; sl < nh && ok; ++sl) {
             // the buffer is free once the score products over its previous contents have retired
             if (!(ok = mbar_wait_thin(slab_empty + 8 * sbuf, sph ^ 1u, abort_flag))) break;
             fence_after_sync();
             const uint32_t d = tmem_base + TM_SLAB + sbuf * 128;
-            const bool first = sl == 0, last = sl == Hkv - 1;
+            const bool first = sl == 0, last = sl == nh - 1;
             uint32_t an = ak;
             for (int j = 0; j < np; j += 2, an += 2) {
               const bool two = j + 1 < np;
@@ -297,13 +302,13 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
       const uint32_t q_lo0 = kmajor_sw128_desc_lo(sQ);
       uint32_t sbuf = 0, sph = 0, slot = 0, slph = 0;
       bool ok = true;
-      int4 e = w0 < total ? klist[KSTEP * w0] : kt_none;
+      int4 e = unit(w0);
       for (int w = w0; w < total && ok; ++w) {
-        const int4 nxt = w + 1 < total ? klist[KSTEP * (w + 1)] : kt_none;
+        const int4 nxt = unit(w + 1);
         const int cls = e.y & 0x7f;
         for (int p0 = 0; p0 < cls && ok; p0 += KT_A_SLOTS) {
-          for (int sl = 0; sl < Hkv; ++sl) {
-            const int g = sl + g_rot < Hkv ? sl + g_rot : sl + g_rot - Hkv;
+          for (int sl = 0; sl < nh; ++sl) {
+            const int g = head(w, sl);
             if (!(ok = mbar_wait_thin(kr_full + 8 * sbuf, sph, abort_flag))) break;
             if (!(ok = mbar_wait_thin(s_empty + 8 * slot, slph ^ 1u, abort_flag))) break;
             fence_after_sync();
@@ -380,17 +385,17 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
       fence_proxy_async_smem();
     };
     uint32_t last_slot = 0, last_slph = 0;                          // score accumulator of the slab rotated last, and its phase
-    int4 e = w0 < total ? klist[KSTEP * w0] : kt_none;
+    int4 e = unit(w0);
     int pos_cur = w0 < total ? kpos[(size_t)e.x * TILE + row] : 0;              // this row's position in the current tile
     if (w0 < total) { write_q(e.w); rope_setup(pos_cur); }
     for (int w = w0; w < total && ok; ++w) {
-      const int4 nxt = w + 1 < total ? klist[KSTEP * (w + 1)] : kt_none;
+      const int4 nxt = unit(w + 1);
       const int cls = e.y & 0x7f, qs = e.w;
       [[maybe_unused]] const int n_valid = e.y >> 8;
       const int passes = (cls + KT_A_SLOTS - 1) / KT_A_SLOTS;
       const int pos_next = nxt.w >= 0 ? kpos[(size_t)nxt.x * TILE + row] : 0;      // fetched now, used after the tile's slabs
       for (int ps = 0; ps < passes && ok; ++ps) {
-        for (int sli = 0; sli < Hkv; ++sli) {
+        for (int sli = 0; sli < nh; ++sli) {
           if (!(ok = __all_sync(0xffffffffu, mbar_wait(slab_full + 8 * sbuf, sph, abort_flag)))) break;
           fence_after_sync();
           const uint32_t sl_addr = lane_addr + TM_SLAB + sbuf * 128 + hf * 32;
@@ -448,7 +453,7 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
         }
       }
       if (!ok) break;
-      if (nxt.w >= 0) rope_setup(pos_next);
+      if (nxt.w >= 0 && nxt.x != e.x) rope_setup(pos_next);      // a further part of the same tile: the factors stay
       pos_cur = pos_next;
       if (nxt.w != qs) {
         // last tile of this query slot in the piece: the query operand may only change once every score product that
@@ -475,12 +480,12 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
     const int* kpos = v.aux(layer, 0);
     uint32_t slot = 0, slph = 0;
     bool ok = true;
-    int4 e = w0 < total ? klist[KSTEP * w0] : kt_none;
+    int4 e = unit(w0);
     int pos_cur = w0 < total ? kpos[(size_t)e.x * TILE + row] : 0;
     // the row of the score scratch this token's scores go to: its V slot (rows past the tile's last token have none)
     int vrow_cur = w0 < total && row < (e.y >> 8) ? v.kv_link[(size_t)e.x * TILE + row] : 0;
     for (int w = w0; w < total && ok; ++w) {
-      const int4 nxt = w + 1 < total ? klist[KSTEP * (w + 1)] : kt_none;
+      const int4 nxt = unit(w + 1);
       const int cls = e.y & 0x7f, n_valid = e.y >> 8, qs = e.w;
       const bool discard = (e.y & KE_DISCARD) != 0;
       const int passes = (cls + KT_A_SLOTS - 1) / KT_A_SLOTS;
@@ -493,8 +498,8 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
       const bool live = row < n_valid && pos_cur <= pos_limit;
       for (int ps = 0; ps < passes && ok; ++ps) {
         const uint32_t mode = discard ? KP_DISCARD : passes == 1 ? KP_STORE_FINAL : (ps == 0 ? KP_STORE_PART : KP_ADD_FINAL);
-        for (int sli = 0; sli < Hkv; ++sli) {
-          const int g = sli + g_rot < Hkv ? sli + g_rot : sli + g_rot - Hkv;
+        for (int sli = 0; sli < nh; ++sli) {
+          const int g = head(w, sli);
           if (!(ok = __all_sync(0xffffffffu, mbar_wait(s_full + 8 * slot, slph, abort_flag)))) break;
           fence_after_sync();
           float sv[REP];

@@ -55,7 +55,6 @@ struct DevView {
   int* key_old_last;         // [NK]  the key's newest tile before the piece
   float* scores;             // [NT*128][Hq]  row = V slot of the token (the V pass reads a tile's rows together)
   unsigned* seqmax;          // [S][Hq]  order-preserving encoding of the running max
-  int* qslot;                // [S]   sequence id -> query index of the current decode call, -1
   // chunked prefill (null for a decode call): per query slot, the row of q / out it stands for and the last position it
   // may attend to
   const int* qmap;
@@ -68,8 +67,8 @@ struct DevView {
   int4* klist;               // [NT]  K tiles of the current decode call, widest class first: (tile, class | n_valid << 8, base block, query slot)
   int4* kpairs;              // [NT + 64]  the same list as items of two tiles of one class (entries 2 i, 2 i + 1) for the CTA-pair kernel;
                              //            a class with an odd number of tiles ends with a filler entry (.y bit 7 set)
-  int* klist_count;          // [1]
-  int* cta_start;            // [MAX_PLAN_CTAS + 1]  first list entry of every K-score CTA
+  int* kitem_parts;          // [1]  parts the KV heads of a list item are dealt out in
+  int* cta_start;            // [MAX_PLAN_CTAS + 1]  first item part of every K-score CTA (pair)
   int* kv_link;              // [NT * 128]  K slot -> V slot of the same token, for the sequences of the current decode pass (rebuilt by every pass)
   int* vcut;                 // [query slots][n_splits + 1]  cut points of every sequence's V tile list into the splits of the V pass
   float* part_acc;           // [max_partials][Hq][d_kv]
@@ -127,6 +126,11 @@ __device__ inline int vtile_stride(int n) {
     while (b) { const int t = a % b; a = b; b = t; }
     if (a == 1) return s;
   }
+}
+
+// the i-th tile of that order
+__device__ inline int vtile_at(int i, int stride, int n) {
+  return n <= 65535 ? (int)(((unsigned)i * (unsigned)stride) % (unsigned)n) : (int)(((long long)i * stride) % n);
 }
 
 // Makes `dev` the current device for the scope of a host call.

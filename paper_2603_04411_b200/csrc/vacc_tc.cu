@@ -95,7 +95,7 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
   const int* cut = v.vcut + (size_t)qs * (n_splits + 1) + split;
   const int t_first = cut[0], n_mine = seq_ok ? cut[1] - t_first : 0;
   const int n_tiles = seq_ok ? v.svc(layer)[seq] : 0;
-  const long long t_stride = vtile_stride(n_tiles);
+  const int t_stride = vtile_stride(n_tiles);
   const int* list = v.svt(layer) + (size_t)(seq_ok ? seq : 0) * v.TPS;
   const int4* desc = v.desc(layer, 1);
 
@@ -162,7 +162,7 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
     const int cn = min(VT_META, n_mine - c0);
     // descriptors of this chunk of the split's tiles
     for (int i = tid; i < cn; i += VT_THREADS) {
-      const int t = list[(int)(((long long)(t_first + c0 + i) * t_stride) % n_tiles)];
+      const int t = list[vtile_at(t_first + c0 + i, t_stride, n_tiles)];
       const int4 d = desc[t];
       s_meta[i] = make_int4(t, d.y, d.z, d.w);
     }

@@ -1,0 +1,41 @@
+"""The planner of a decode pass where its split of the work changes: few tiles (the KV heads of a tile dealt out to several
+CTAs), head counts that do not divide, unlisted sequences in between, a V tile list longer than one block-wide scan."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2603_04411_b200 import workloads
+from tests.helpers import GpuCache, attn_errors, oracle_decode
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("hkv,rep,n_seq,ctx,recipe,pick", [
+    (8, 4, 1, 1, "any", [0]),                   # one tile: every head a part of its own
+    (8, 1, 1, 129, "any", [0]),
+    (8, 4, 3, 1000, "levels", [2, 0]),          # around ten items: parts of several heads; sequence 1 not listed
+    (8, 2, 9, 600, "any", list(range(9))),      # enough items that they stay whole
+    (3, 2, 2, 300, "any", [1, 0]),              # an odd number of KV heads, six classes
+    (6, 8, 2, 140, "any", [0, 1]),              # heads split in two, not in four
+    (1, 1, 1, 133000, "levels", [0]),           # more than 1024 V tiles in one sequence
+])
+def test_decode_where_the_work_split_changes(hkv, rep, n_seq, ctx, recipe, pick):
+    from paper_2603_04411_b200 import build
+    build.build()
+    from paper_2603_04411_b200 import binding as B
+    d = hkv * 128
+    li = workloads.build_layer(820 + ctx, n_seq=n_seq, ctx=ctx, n_q_heads=hkv * rep, n_kv_heads=hkv, n_calib=2 * d, outlier="none",
+                               mode="forced", rank_recipe=recipe)
+    ranks = np.minimum(li.ranks.numpy().astype(np.int64), d)
+    gc = GpuCache(B, n_layers=1, n_q_heads=hkv * rep, n_kv_heads=hkv, dtype=torch.float16, out_dtype=torch.float32, max_seqs=n_seq,
+                  max_tokens_per_seq=ctx, payload_bytes=int((-(-ranks // 64) * 128).sum()))
+    B.twkv_cache_set_layer_params(gc.h, 0, li.Uinv_k.cuda(), li.Uinv_v.cuda())
+    B.twkv_compress(gc.h, 0, li.xt_k.cuda(), li.xt_v.cuda(), li.seq_ids.cuda(), li.positions.cuda(), None,
+                    torch.from_numpy(ranks.astype(np.int16)).cuda(), B.TWKV_GATE_FORCED)
+    li.q = li.q[pick].contiguous()
+    out = torch.full((len(pick), hkv * rep, 128), float("nan"), device="cuda")
+    B.twkv_decode_attn(gc.h, 0, li.q.cuda(), torch.tensor(pick, dtype=torch.int32, device="cuda"), out)
+    assert B.twkv_cache_status(gc.h) == B.TWKV_OK
+    max_abs, rel_l2 = attn_errors(out.cpu().numpy(), oracle_decode(li, ranks, pick))
+    gc.close()
+    assert max_abs < 2e-3 and rel_l2 < 1e-3, (max_abs, rel_l2)      # the bars of every decode test
