@@ -312,10 +312,11 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
             if (!(ok = mbar_wait_thin(kr_full + 8 * sbuf, sph, abort_flag))) break;
             if (!(ok = mbar_wait_thin(s_empty + 8 * slot, slph ^ 1u, abort_flag))) break;
             fence_after_sync();
-            // the rotated keys come as a high and a low f16 part (their sum carries 21 bits): two products into the same S
+            // the rotated keys come as a high and a low f16 part (their sum carries 21 bits): two products into the same S,
+            // the low one first (the tensor core cuts its fp32 sum after every instruction: half as many cuts at full size)
             const uint32_t kr = tmem_base + TM_SLAB + sbuf * 128, sd = tmem_base + TM_S + 16 * slot;
-            mma_f16_ts_k128_cg<CG>(sd, kr, q_lo0 + g * (1024 >> 4), KT_Q_PANEL_BYTES >> 4, idesc_s, 0u);
-            mma_f16_ts_k128_cg<CG>(sd, kr + 64, q_lo0 + g * (1024 >> 4), KT_Q_PANEL_BYTES >> 4, idesc_s, 1u);
+            mma_f16_ts_k128_cg<CG>(sd, kr + 64, q_lo0 + g * (1024 >> 4), KT_Q_PANEL_BYTES >> 4, idesc_s, 0u);
+            mma_f16_ts_k128_cg<CG>(sd, kr, q_lo0 + g * (1024 >> 4), KT_Q_PANEL_BYTES >> 4, idesc_s, 1u);
             if constexpr (PAIR) { mma_commit_pair(slab_empty + 8 * sbuf); mma_commit_pair_both(s_full + 8 * slot); }
             else { mma_commit(slab_empty + 8 * sbuf); mma_commit(s_full + 8 * slot); }   // buffer reusable; scores complete
             if (++sbuf == (uint32_t)KT_SLABS) { sbuf = 0; sph ^= 1u; }

@@ -1,7 +1,7 @@
 // V-side of decode attention on the 5th-generation tensor cores.
 //
 // By linearity of Eq. 3 the weighted sum of the values is taken in spectral space: per (query slot, split, head group)
-//   acc[j][h] = sum over the split's tokens t of  X^_V[t][j] * p[t][h],   p = exp(s - max) rounded to the cache dtype,
+//   acc[j][h] = sum over the split's tokens t of  X^_V[t][j] * p[t][h],   p = exp(s - max) as two parts of the cache dtype,
 //   l[h]      = sum over t of p[t][h],
 // and merge_kernel projects acc / l through U_V^-1 once.  A V tile of rank class c is c panels [128 tokens x 64
 // columns] in HBM.  Two panels at a time form the A operand of one tcgen05.mma chain (M = 128 spectral columns, N = the
@@ -15,11 +15,11 @@
 // The probabilities are the B operand (K-major: [head][token], two 64-token halves), written by 8 warps: thread =
 // (head, 8 consecutive tokens), one 16-byte swizzled store per 8 weights.  The K-score kernel stores a token's scores at
 // its V slot, so a tile's 128 score rows lie next to each other: one TMA box [128 rows x the CTA's heads] per tile,
-// issued by the producer thread two tiles ahead into a ring of four tiles in shared memory (TS = true).  A narrow tile
+// issued by the producer thread two tiles ahead into a ring of three tiles in shared memory (TS = true).  A narrow tile
 // reads as many bytes of scores as of values, and with one tile in flight their latency bound the kernel.  Where the
 // head count is not a multiple of four (rows not 16-byte aligned: no tensor map) each warp copies the rows of its own
 // token groups with cp.async instead (TS = false).
-// bf16 weights go in as two bf16 parts (see below), two chains per pair.
+// Weights go in as two parts of the cache type (see below), two chains per pair.
 //
 // Warp roles (320 threads, one CTA per SM):
 //   warp 0      TMA producer of V panels (ring of 32-KiB pair stages; one elected lane)
@@ -41,11 +41,11 @@ constexpr uint32_t VT_PANEL_BYTES = 16384;
 constexpr uint32_t VT_STAGE_BYTES = 2 * VT_PANEL_BYTES;
 constexpr uint32_t VT_ZERO_BYTES = 2048;                       // 16 token rows of zeros: the missing partner of a lone panel
 constexpr uint32_t VT_SMEM_MAX = 232448;
-constexpr int VT_SC = 4;                                       // tiles of scores in flight
+constexpr int VT_SC = 3;                                       // tiles of scores in flight (a fourth would cost a stage of the panel ring)
 
 template <bool BF16, int N>
 struct VtCfg {
-  static constexpr int PARTS = BF16 ? 2 : 1;                   // operands per weight
+  static constexpr int PARTS = 2;                              // operands per weight (high and low part)
   static constexpr uint32_t P_HALF_BYTES = N * 128;            // [N heads][64 tokens]
   static constexpr uint32_t P_PART_BYTES = 2 * P_HALF_BYTES;
   static constexpr uint32_t P_BUF_BYTES = PARTS * P_PART_BYTES;
@@ -58,19 +58,24 @@ struct VtCfg {
   static constexpr int ITEMS = N / 16;                         // (head, 8-token group) items per probability thread and tile
 };
 
-// Two fp32 -> one packed pair in the cache dtype (a in the low half), round to nearest; r0 / r1: the rounded values.
-template <bool BF16> __device__ __forceinline__ uint32_t vt_pack2(float a, float b, float& r0, float& r1) {
-  uint32_t d;
+constexpr float VT_LOG2E = 1.44269504088896340736f;
+__device__ __forceinline__ uint64_t vt_pack(float a, float b) { uint64_t r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b)); return r; }
+__device__ __forceinline__ void vt_unpack(uint64_t v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ uint64_t vt_fma2(uint64_t a, uint64_t b, uint64_t c) { uint64_t r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
+__device__ __forceinline__ uint64_t vt_add2(uint64_t a, uint64_t b) { uint64_t r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ uint64_t vt_sub2(uint64_t a, uint64_t b) { uint64_t r; asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ float vt_ex2(float x) { float r; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
+// Two packed fp32 weights -> their high parts (mantissa cut to the type) and the rest, each as a packed pair of the cache dtype.
+template <bool BF16> __device__ __forceinline__ void vt_split(uint64_t v, uint32_t& hi, uint32_t& lo) {
+  const uint64_t h = v & (BF16 ? 0xFFFF0000FFFF0000ull : 0xFFFFE000FFFFE000ull);
+  const uint64_t l = vt_sub2(v, h);
   if constexpr (BF16) {
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(b), "f"(a));
-    r0 = __uint_as_float(d << 16);
-    r1 = __uint_as_float(d & 0xffff0000u);
+    asm("{\n\t.reg .b32 a, b;\n\tmov.b64 {a, b}, %1;\n\tprmt.b32 %0, a, b, 0x7632;\n\t}" : "=r"(hi) : "l"(h));
+    asm("{\n\t.reg .f32 a, b;\n\tmov.b64 {a, b}, %1;\n\tcvt.rn.bf16x2.f32 %0, b, a;\n\t}" : "=r"(lo) : "l"(l));
   } else {
-    asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(b), "f"(a));
-    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&d));
-    r0 = f.x; r1 = f.y;
+    asm("{\n\t.reg .f32 a, b;\n\tmov.b64 {a, b}, %1;\n\tcvt.rn.f16x2.f32 %0, b, a;\n\t}" : "=r"(hi) : "l"(h));
+    asm("{\n\t.reg .f32 a, b;\n\tmov.b64 {a, b}, %1;\n\tcvt.rn.f16x2.f32 %0, b, a;\n\t}" : "=r"(lo) : "l"(l));
   }
-  return d;
 }
 
 // Instruction descriptor: kind::f16, fp32 accumulate, A MN-major (bit 15), B K-major, M = 128.
@@ -146,16 +151,18 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
   uint32_t touched = 0;                                         // issuer: panel pairs whose accumulator holds a value
   bool ok = true;
   int max_cls = 0;                                              // probability warps: widest class seen (which accumulators to read)
-  float l_sum = 0.f;                                            // probability threads: sum of this thread's weights
+  uint64_t l_sum2 = 0;                                          // probability threads: two sums of this thread's weights
 
   // probability threads: fixed head, items = 8-token groups
   const int pt = tid - 64;                                      // 0 .. 255 for warps 2-9
   const int ph_ = pt & (N - 1);                                 // head within the CTA's group
-  float m_h = 0.f;
+  uint64_t nm2 = 0;                                             // minus the head's maximum, in powers of two
+  const uint64_t log2e2 = vt_pack(VT_LOG2E, VT_LOG2E);
   if (warp >= 2) {
     // a query that sees no token (chunked prefill, every cached position after its own) has no maximum: weights stay 0
     const float m = ph_ < nh ? dec_ordered(v.seqmax[qs * Hq + h0 + ph_]) : 0.f;
-    m_h = m == -INFINITY ? 0.f : m;
+    const float m_h = m == -INFINITY ? 0.f : m;
+    nm2 = vt_pack(-m_h * VT_LOG2E, -m_h * VT_LOG2E);
   }
 
   for (int c0 = 0; c0 < n_mine; c0 += VT_META) {
@@ -314,34 +321,32 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
         const float* srow = reinterpret_cast<const float*>(sS_ptr + (uint32_t)(k % VT_SC) * C::SC_STAGE_BYTES) + ph_;
         const int rs = TS ? NB : N;                             // floats per score row in the stage
         // a box holds whatever the scratch holds in rows past the tile's last token and has no columns past the last head
-        const bool head_ok = !TS || ph_ < nh;
+        const bool head_ok = !TS || ph_ < nh, all_valid = n_valid_i == TILE && nh == N;
 #pragma unroll
         for (int it = 0; it < ITEMS; ++it) {
           const int tg = (it * VT_PTHREADS + pt) / N;
-          uint32_t hi[4];
-          [[maybe_unused]] uint32_t lo[4];
+          // Two weights at a time, packed: exp2 of one fused multiply-add, the high part cut off (exact in the type), the low
+          // part rounded.  bf16 keeps 8 bits of a weight, f16 11: with few tokens per sequence that rounding alone reaches 1e-3
+          // and 1e-4 of the output, so the remainder goes into a second operand (16 and 22 bits in all).
+          // Measured at 64 heads bf16 over 131072 tokens 41.3 -> 39.3 us (fewer instructions, one more ring stage); f16 pays for its
+          // second chain of products: 68.1 -> 68.7 us (16 x 32768), 77.1 -> 80.6 us (64 x 8192, narrow tiles).
+          uint32_t hi[4], lo[4];
 #pragma unroll
           for (int u = 0; u < 8; u += 2) {
-            float p0 = __expf(srow[(tg * 8 + u) * rs] - m_h), p1 = __expf(srow[(tg * 8 + u + 1) * rs] - m_h);
-            if constexpr (TS) {
+            float a0, a1;
+            vt_unpack(vt_fma2(vt_pack(srow[(tg * 8 + u) * rs], srow[(tg * 8 + u + 1) * rs]), log2e2, nm2), a0, a1);
+            float p0 = vt_ex2(a0), p1 = vt_ex2(a1);
+            if (TS && !all_valid) {                             // uniform: tiles with fewer than 128 tokens, CTAs with fewer heads than N
               p0 = (head_ok && tg * 8 + u < n_valid_i) ? p0 : 0.f;
               p1 = (head_ok && tg * 8 + u + 1 < n_valid_i) ? p1 : 0.f;
             }
-            // two weights per conversion instruction (single conversions run at a quarter of the rate and bound this loop)
-            float r0, r1;
-            hi[u >> 1] = vt_pack2<BF16>(p0, p1, r0, r1);
-            l_sum += r0 + r1;
-            if constexpr (BF16) {
-              // bf16 keeps 8 bits of a weight: with few tokens per sequence that rounding alone reaches 1e-3 of the
-              // output, so the remainder goes into a second operand (16 bits in all)
-              float q0, q1;
-              lo[u >> 1] = vt_pack2<true>(p0 - r0, p1 - r1, q0, q1);
-              l_sum += q0 + q1;
-            }
+            const uint64_t p = vt_pack(p0, p1);
+            l_sum2 = vt_add2(l_sum2, p);
+            vt_split<BF16>(p, hi[u >> 1], lo[u >> 1]);
           }
           const uint32_t off = (uint32_t)(tg >> 3) * C::P_HALF_BYTES + (uint32_t)ph_ * 128u + ((((uint32_t)tg & 7u) ^ ((uint32_t)ph_ & 7u)) << 4);
           *reinterpret_cast<uint4*>(pb + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-          if constexpr (BF16) *reinterpret_cast<uint4*>(pb + C::P_PART_BYTES + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+          *reinterpret_cast<uint4*>(pb + C::P_PART_BYTES + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
         }
         fence_proxy_async_smem();
         __syncwarp();                                           // also: the stage is read before the next copies into it start
@@ -359,7 +364,11 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
   // ----------------------------------------------------------------- partial results of this split
   const size_t pidx = (size_t)qs * n_splits + split;
   if (warp >= 2) {
-    s_l[pt] = l_sum;
+    {
+      float a, b;
+      vt_unpack(l_sum2, a, b);
+      s_l[pt] = a + b;
+    }
     bool ready = ok;
     if (ready && n_mine > 0) ready = __all_sync(0xffffffffu, mbar_wait(acc_done, 0u, abort_flag));
     fence_after_sync();
