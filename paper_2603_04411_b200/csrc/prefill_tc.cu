@@ -167,3 +167,360 @@ __global__ void __launch_bounds__(1024) pf_rows_kernel(DevView v, PfCall a, int 
   }
 }
 
+// ------------------------------------------------------------------------------------------ reconstruction
+constexpr int PR_THREADS = 384;                                 // warps 0 and 1: producer and issuer, 4 to 11: epilogue
+constexpr int PR_REGS_LIGHT = 56, PR_REGS_EPI = 224;            // 384 threads of 168 registers, divided again by warpgroup
+constexpr int PR_STAGES = 3;
+constexpr uint32_t PR_A_BYTES = 16384;                          // [128 tokens][64 components]
+constexpr uint32_t PR_ATOM_BYTES = 8192;                        // [64 components][64 output dims]: one MN-major atom of U^-1
+constexpr uint32_t PR_STAGE_BYTES = PR_A_BYTES + 4 * PR_ATOM_BYTES;
+constexpr uint32_t PR_OUT_BYTES = 8192;                         // per warp: 32 half rows of 128 bytes on their way out, both parts
+constexpr int PR_ROPE_STRIDE = 33;                              // float4 per row of the small RoPE table (32 + 1 against bank conflicts)
+constexpr uint32_t PR_ROPE_BYTES = ROPE_LO * PR_ROPE_STRIDE * 16;
+constexpr uint32_t PR_SMEM = PR_STAGES * PR_STAGE_BYTES + 8 * PR_OUT_BYTES + PR_ROPE_BYTES + 8 * (2 * PR_STAGES + 4) + 16;
+// Panels summed into one accumulator; the sums of several accumulators are added in fp32 registers.  The tensor core cuts its
+// fp32 sum after every instruction (K = 16), so the error grows with the length of a chain.  K: eight panels, the length of
+// decode attention's passes, so that both round alike.  V: two panels; decode attention sums values over tokens, not over
+// components (largest difference between the two at rank 512: 2.9e-6 with eight panels, 1.9e-6 with two).
+__host__ __device__ constexpr int pr_chain(int side) { return side ? 2 : 8; }
+
+__device__ __forceinline__ uint64_t pk2(float a, float b) { uint64_t r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b)); return r; }
+__device__ __forceinline__ uint64_t pk2u(uint32_t a, uint32_t b) { uint64_t r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(a), "r"(b)); return r; }
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) { uint64_t r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) { uint64_t r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) { uint64_t r; asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) { uint64_t r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
+__device__ __forceinline__ void unpk2(uint64_t v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+// Two packed fp32 -> their high and low 16-bit parts (high: the value cut to the type's mantissa; low: the rest, rounded).
+template <bool BF16> __device__ __forceinline__ void split2(uint64_t v, uint32_t& hi, uint32_t& lo) {
+  const uint64_t h = v & (BF16 ? 0xFFFF0000FFFF0000ull : 0xFFFFE000FFFFE000ull);
+  const uint64_t l = sub2(v, h);
+  if constexpr (BF16) {
+    asm("{\n\t.reg .b32 a, b;\n\tmov.b64 {a, b}, %1;\n\tprmt.b32 %0, a, b, 0x7632;\n\t}" : "=r"(hi) : "l"(h));
+    asm("{\n\t.reg .f32 a, b;\n\tmov.b64 {a, b}, %1;\n\tcvt.rn.bf16x2.f32 %0, b, a;\n\t}" : "=r"(lo) : "l"(l));
+  } else {
+    asm("{\n\t.reg .f32 a, b;\n\tmov.b64 {a, b}, %1;\n\tcvt.rn.satfinite.f16x2.f32 %0, b, a;\n\t}" : "=r"(hi) : "l"(h));
+    asm("{\n\t.reg .f32 a, b;\n\tmov.b64 {a, b}, %1;\n\tcvt.rn.satfinite.f16x2.f32 %0, b, a;\n\t}" : "=r"(lo) : "l"(l));
+  }
+}
+// The same with the high part rounded to nearest: the low part is half as large, and so the product of two low parts, which
+// the second product of attention leaves out.
+template <bool BF16> __device__ __forceinline__ void split2_rn(uint64_t v, uint32_t& hi, uint32_t& lo) {
+  float a, b;
+  unpk2(v, a, b);
+  if constexpr (BF16) {
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(hi) : "f"(b), "f"(a));
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(b - __uint_as_float(hi & 0xffff0000u)), "f"(a - __uint_as_float(hi << 16)));
+  } else {
+    hi = pack_f16x2_sat(a, b);
+    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&hi));
+    lo = pack_f16x2_sat(a - f.x, b - f.y);
+  }
+}
+
+// One work item = (tile, slab of NS = 256 output dims, i.e. two KV heads; 128 where d_kv is not a multiple of 256).
+// [128 x NS] accumulators alternate between two TMEM buffers; state panels (K-major A) and U^-1 atoms (rows of the caller's
+// matrix as they lie: MN-major B) stream through a ring of three stages.  Eight epilogue warps (thread = one token row x
+// half of a head's dims) rotate (K), split into two parts and hand the rows out through shared memory: a row's place in the
+// segment buffer is its token's dense row, so a warp stores four whole 128-byte pieces per instruction instead of 32
+// scattered 16-byte ones.
+template <bool BF16>
+__global__ void __launch_bounds__(PR_THREADS, 1)
+pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_constant__ CUtensorMap map_uk,
+                const __grid_constant__ CUtensorMap map_uv, DevView v, PfCall a, int layer, int seg) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t s0 = smem_addr(smem_raw);
+  unsigned char* out_stage = smem_raw + PR_STAGES * PR_STAGE_BYTES;
+  float4* sRope = reinterpret_cast<float4*>(out_stage + 8 * PR_OUT_BYTES);
+  unsigned char* tail = out_stage + 8 * PR_OUT_BYTES + PR_ROPE_BYTES;
+  const uint32_t bars = smem_addr(tail);
+  const uint32_t full = bars, empty = full + 8 * PR_STAGES, acc_full = empty + 8 * PR_STAGES, acc_empty = acc_full + 16;
+  uint32_t* s_tmem_base = reinterpret_cast<uint32_t*>(tail + 8 * (2 * PR_STAGES + 4));
+  volatile int* abort_flag = reinterpret_cast<int*>(s_tmem_base + 1);
+  const bool misaligned = (s0 & 1023u) != 0;
+
+  if (tid == 0) {
+    for (int i = 0; i < PR_STAGES; ++i) { mbar_init(full + 8 * i, 1); mbar_init(empty + 8 * i, 1); }
+    for (int i = 0; i < 2; ++i) { mbar_init(acc_full + 8 * i, 1); mbar_init(acc_empty + 8 * i, 8); }
+    *abort_flag = misaligned ? 1 : 0;
+    mbar_init_fence();
+  }
+  if (warp == 1) tmem_alloc(smem_addr(s_tmem_base), 512);
+  for (int i = tid; i < ROPE_LO * 32; i += PR_THREADS) sRope[(i >> 5) * PR_ROPE_STRIDE + (i & 31)] = v.rope_lo[i];
+  fence_before_sync();
+  __syncthreads();
+  fence_after_sync();
+  const uint32_t tmem_base = *s_tmem_base;
+
+  const int NS = v.d_kv % 256 == 0 ? 256 : 128, n_slabs = v.d_kv / NS;
+  const int nk = v.ntiles(layer)[0], n_items = (nk + v.ntiles(layer)[1]) * n_slabs;
+  const int step = gridDim.x;
+  // the items of this CTA whose tile has rows in the segment; every role walks them in the same order, 32 looked up at once
+  auto entry = [&](int i, int& side, int& t) -> int4 {
+    const int e = i / n_slabs;
+    side = e >= nk;
+    t = side ? e - nk : e;
+    return side ? v.kpairs[t] : v.klist[t];
+  };
+  auto lookup = [&](int i0) -> unsigned {
+    const int i = i0 + lane * step;
+    bool mine = false;
+    if (i < n_items) {
+      int side, t;
+      const int z = entry(i, side, t).z;
+      mine = (z & 0xffff) <= seg && seg <= (z >> 16);
+    }
+    return __ballot_sync(0xffffffffu, mine);
+  };
+
+  if (misaligned) {
+    // nothing was started
+  } else if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(PR_REGS_LIGHT));
+    if (warp == 0) {
+      // ------------------------------------------------------------- TMA producer
+      uint32_t n_loaded = 0;                                    // panels so far; stage = panel % 3
+      bool ok = true;
+      if (elect_one()) { tma_prefetch_desc(&map_blocks); tma_prefetch_desc(&map_uk); tma_prefetch_desc(&map_uv); }
+      for (int i0 = blockIdx.x; i0 < n_items && ok; i0 += 32 * step) {
+        for (unsigned m = lookup(i0); m && ok; m &= m - 1) {
+          const int i = i0 + (__ffs(m) - 1) * step;
+          int side, t;
+          const int4 en = entry(i, side, t);
+          const int cls = en.x & 0xff, n0 = (i % n_slabs) * NS;
+          if (elect_one()) {
+            const CUtensorMap* mu = side ? &map_uv : &map_uk;
+            for (int p = 0; p < cls; ++p) {
+              const uint32_t n = n_loaded + p, st = n % PR_STAGES, ph = (n / PR_STAGES) & 1u;
+              if (!(ok = mbar_wait_thin(empty + 8 * st, ph ^ 1u, abort_flag))) break;
+              mbar_expect_tx(full + 8 * st, PR_A_BYTES + (uint32_t)NS * 128u);
+              const uint32_t dst = s0 + st * PR_STAGE_BYTES;
+              tma_load_2d(dst, &map_blocks, full + 8 * st, 0, (en.y + p) * TILE);
+              for (int at = 0; at < NS / 64; ++at) tma_load_2d(dst + PR_A_BYTES + at * PR_ATOM_BYTES, mu, full + 8 * st, n0 + at * 64, p * PANEL);
+            }
+          }
+          __syncwarp();
+          n_loaded += cls;
+          ok = __all_sync(0xffffffffu, ok);
+        }
+      }
+      if (!ok)                                                  // let copies in flight land before the CTA goes away
+        for (uint32_t i = 0; i < PR_STAGES && i < n_loaded; ++i) {
+          const uint32_t n = n_loaded - 1 - i;
+          mbar_wait_drain(full + 8 * (n % PR_STAGES), (n / PR_STAGES) & 1u);
+        }
+    } else if (warp == 1) {
+      // ------------------------------------------------------------- MMA issuer
+      const uint32_t idesc = idesc_f16(BF16 ? 1 : 0, 128, NS) | (1u << 16);           // B MN-major
+      uint32_t n_used = 0, ac = 0;
+      bool ok = true;
+      for (int i0 = blockIdx.x; i0 < n_items && ok; i0 += 32 * step) {
+        for (unsigned m = lookup(i0); m && ok; m &= m - 1) {
+          const int i = i0 + (__ffs(m) - 1) * step;
+          int side, t;
+          const int cls = entry(i, side, t).x & 0xff, len = pr_chain(side);
+          if (elect_one()) {
+            for (int p = 0; p < cls && ok; ++p) {
+              const uint32_t chain = ac + p / len, buf = chain & 1u;
+              if (p % len == 0) {
+                if (!(ok = mbar_wait(acc_empty + 8 * buf, ((chain >> 1) & 1u) ^ 1u, abort_flag))) break;
+                fence_after_sync();
+              }
+              const uint32_t n = n_used + p, st = n % PR_STAGES, ph = (n / PR_STAGES) & 1u;
+              if (!(ok = mbar_wait_thin(full + 8 * st, ph, abort_flag))) break;
+              fence_after_sync();
+              const uint32_t sa = s0 + st * PR_STAGE_BYTES, sb = sa + PR_A_BYTES;
+#pragma unroll
+              for (int ks = 0; ks < 4; ++ks) {
+                const uint32_t a_lo = kmajor_sw128_desc_lo(sa) + 2 * ks;
+                const uint32_t b_lo = (((sb + ks * 2048u) >> 4) & 0x3fffu) | ((PR_ATOM_BYTES >> 4) << 16);
+                mma_f16_ss(tmem_base + buf * 256, ((uint64_t)KMAJOR_SW128_DESC_HI << 32) | a_lo, ((uint64_t)KMAJOR_SW128_DESC_HI << 32) | b_lo,
+                           idesc, (p % len > 0 || ks > 0) ? 1u : 0u);
+              }
+              mma_commit(empty + 8 * st);
+              if (p % len == len - 1 || p == cls - 1) mma_commit(acc_full + 8 * buf);
+            }
+          }
+          __syncwarp();
+          n_used += cls;
+          ac += (cls + len - 1) / len;
+          ok = __all_sync(0xffffffffu, ok);
+        }
+      }
+    }
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(PR_REGS_EPI));
+    // ------------------------------------------------------------- epilogue
+    const int ew = warp - 4, quarter = warp & 3, hf = ew >> 2;
+    const int row = quarter * 32 + lane;
+    const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16);
+    unsigned char* stage = out_stage + ew * PR_OUT_BYTES;       // [high | low][32 rows][128 bytes]
+    const size_t plane = (size_t)a.seg_rows * 256;              // bytes of one part of one head
+    const int heads = NS / 128;
+    const int* kpos = v.aux(layer, 0);
+    const int seg0 = seg * a.seg_rows;
+    // rows behind a sequence's last one, up to the next multiple of 128: their weights are zero, so their values must be finite
+    for (int u = blockIdx.x; u < a.n_u; u += step) {
+      const int r0 = a.base[u] + a.rows[u], r1 = a.base[u] + (a.rows[u] + TILE - 1) / TILE * TILE;
+      if (r0 == r1 || r0 < seg0 || r0 >= seg0 + a.seg_rows) continue;
+      for (int i = tid - 128; i < (r1 - r0) * 32 * v.Hkv; i += 256) {
+        const int g = i / ((r1 - r0) * 32), rem = i - g * (r1 - r0) * 32, part = 2 + rem / ((r1 - r0) * 16), w = rem % ((r1 - r0) * 16);
+        *reinterpret_cast<uint4*>(a.seg_buf + (g * 4 + part) * plane + (size_t)(r0 - seg0) * 256 + (size_t)w * 16) = make_uint4(0u, 0u, 0u, 0u);
+      }
+    }
+    uint32_t ac = 0;
+    bool ok = true;
+    for (int i0 = blockIdx.x; i0 < n_items && ok; i0 += 32 * step) {
+      for (unsigned m = lookup(i0); m; m &= m - 1) {
+        const int i = i0 + (__ffs(m) - 1) * step;
+        int side, t;
+        const int cls = entry(i, side, t).x & 0xff, chains = (cls + pr_chain(side) - 1) / pr_chain(side);
+        const int g0 = (i % n_slabs) * heads;
+        int local = (side ? a.vrow : a.krow_out)[(size_t)t * TILE + row] - seg0;         // rows past the tile's last token hold -1
+        if (local < 0 || local >= a.seg_rows) local = -1;
+        auto stage_piece = [&](int piece, const uint32_t* hi, const uint32_t* lo) {      // 16 bytes of this thread's row, both parts
+          unsigned char* d = stage + lane * 128 + ((piece ^ (lane & 7)) << 4);
+          *reinterpret_cast<uint4*>(d) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+          *reinterpret_cast<uint4*>(d + 4096) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+        };
+        auto rows_out = [&](int g) {                             // the warp's 32 half rows: four whole 128-byte pieces per instruction
+          __syncwarp();
+          unsigned char* dst = a.seg_buf + (g * 4 + side * 2) * plane + hf * 128 + (lane & 7) * 16;
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            const int r = 4 * k + (lane >> 3);
+            const int lr = __shfl_sync(0xffffffffu, local, r);
+            const unsigned char* s = stage + r * 128 + (((lane & 7) ^ (r & 7)) << 4);
+            if (lr >= 0) {
+              *reinterpret_cast<uint4*>(dst + (size_t)lr * 256) = *reinterpret_cast<const uint4*>(s);
+              *reinterpret_cast<uint4*>(dst + plane + (size_t)lr * 256) = *reinterpret_cast<const uint4*>(s + 4096);
+            }
+          }
+          __syncwarp();
+        };
+        auto wait_chain = [&](uint32_t n) -> bool {
+          const bool got = __all_sync(0xffffffffu, mbar_wait(acc_full + 8 * (n & 1u), (n >> 1) & 1u, abort_flag));
+          fence_after_sync();
+          return got;
+        };
+        auto free_chain = [&](uint32_t n) {
+          fence_before_sync();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(acc_empty + 8 * (n & 1u));
+        };
+        if (!side) {
+          // K: this thread's half of the RoPE frequencies; dims 32 hf + 8 c .. + 7 and the eight 64 above them at a time.
+          // cos / sin of (position, frequency pair) by the angle-addition formulas from the two table rows.
+          const int pos = local >= 0 ? kpos[(size_t)t * TILE + row] : 0;
+          const float4* __restrict__ th = v.rope_hi + (size_t)((pos >> 4) & (ROPE_HI - 1)) * 32 + hf * 16;
+          const float4* tl = sRope + (pos & 15) * PR_ROPE_STRIDE + hf * 16;
+          uint64_t cs[16], sn[16];
+#pragma unroll
+          for (int b = 0; b < 16; b += 8) {
+            float4 h4[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) h4[k] = __ldg(th + b + k);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+              const float4 l4 = tl[b + k];
+              const uint64_t ch = pk2(h4[k].x, h4[k].y), sh = pk2(h4[k].z, h4[k].w), cl = pk2(l4.x, l4.y), sl = pk2(l4.z, l4.w);
+              cs[b + k] = sub2(mul2(ch, cl), mul2(sh, sl));
+              sn[b + k] = fma2(sh, cl, mul2(ch, sl));
+            }
+          }
+          ok = wait_chain(ac);
+          if (ok && chains == 2) ok = wait_chain(ac + 1);
+          if (!ok) break;
+          for (int hh = 0; hh < heads; ++hh) {
+            const uint32_t src = lane_addr + (ac & 1u) * 256 + hh * 128 + hf * 32, src2 = lane_addr + ((ac + 1) & 1u) * 256 + hh * 128 + hf * 32;
+            uint32_t x[64];                                      // 32 dims, then the 32 dims 64 above
+            tmem_ld32(src, x);
+            tmem_ld32(src + 64, x + 32);
+            tmem_ld_wait();
+            if (chains == 2) {
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                uint32_t y[16];
+                tmem_ld16(src2 + 64 * (e >> 1) + 16 * (e & 1), y);
+                tmem_ld_wait();
+#pragma unroll
+                for (int k = 0; k < 16; ++k) x[16 * e + k] = __float_as_uint(__uint_as_float(x[16 * e + k]) + __uint_as_float(y[k]));
+              }
+            }
+            if (hh == heads - 1) { free_chain(ac); if (chains == 2) free_chain(ac + 1); }
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              uint32_t hi[8], lo[8];
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+                const uint64_t L = pk2u(x[8 * c + 2 * k], x[8 * c + 2 * k + 1]), H = pk2u(x[32 + 8 * c + 2 * k], x[33 + 8 * c + 2 * k]);
+                const uint64_t rl = sub2(mul2(L, cs[4 * c + k]), mul2(H, sn[4 * c + k])), rh = fma2(L, sn[4 * c + k], mul2(H, cs[4 * c + k]));
+                split2<false>(rl, hi[k], lo[k]);
+                split2<false>(rh, hi[4 + k], lo[4 + k]);
+              }
+              if (v.debug) {                                     // TWKV_DEBUG: a rotated key beyond the f16 range was clamped
+                bool sat = false;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) sat |= (hi[k] & 0x7fffu) == 0x7bffu || ((hi[k] >> 16) & 0x7fffu) == 0x7bffu;
+                if (sat && local >= 0) set_status(v, TWKV_ERR_DEVICE_CHECK);
+              }
+              // keys are stored in the order in which decode attention contracts them (pairs of pieces 64 dims apart), so that the
+              // sums round alike
+              stage_piece(2 * c, hi, lo);
+              stage_piece(2 * c + 1, hi + 4, lo + 4);
+            }
+            rows_out(g0 + hh);
+          }
+          ac += chains;
+        } else {
+          // V: dims 64 hf .. + 63 of both heads, summed over the chains
+          uint32_t x[2][64];
+          for (int ch = 0; ch < chains; ++ch, ++ac) {
+            if (!(ok = wait_chain(ac))) break;
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh) {
+              if (hh >= heads) break;
+              const uint32_t src = lane_addr + (ac & 1u) * 256 + hh * 128 + hf * 64;
+              if (ch == 0) {
+                tmem_ld32(src, x[hh]);
+                tmem_ld32(src + 32, x[hh] + 32);
+              } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                  uint32_t y[16];
+                  tmem_ld16(src + 16 * e, y);
+                  tmem_ld_wait();
+#pragma unroll
+                  for (int k = 0; k < 16; ++k) x[hh][16 * e + k] = __float_as_uint(__uint_as_float(x[hh][16 * e + k]) + __uint_as_float(y[k]));
+                }
+              }
+            }
+            tmem_ld_wait();
+            free_chain(ac);
+          }
+          if (!ok) break;
+#pragma unroll
+          for (int hh = 0; hh < 2; ++hh) {
+            if (hh >= heads) break;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+              uint32_t hi[4], lo[4];
+#pragma unroll
+              for (int k = 0; k < 4; ++k) split2_rn<BF16>(pk2u(x[hh][8 * c + 2 * k], x[hh][8 * c + 2 * k + 1]), hi[k], lo[k]);
+              stage_piece(c, hi, lo);
+            }
+            rows_out(g0 + hh);
+          }
+        }
+      }
+    }
+    tmem_ld_wait();
+  }
+  fence_before_sync();
+  __syncthreads();
+  fence_after_sync();
+  if (warp == 1) tmem_dealloc(tmem_base, 512);
+  if (tid == 0 && *abort_flag) set_status(v, misaligned ? TWKV_ERR_DEVICE_CHECK : TWKV_ERR_TIMEOUT);
+}
+
