@@ -524,3 +524,462 @@ pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_con
   if (tid == 0 && *abort_flag) set_status(v, misaligned ? TWKV_ERR_DEVICE_CHECK : TWKV_ERR_TIMEOUT);
 }
 
+// ------------------------------------------------------------------------------------------ attention
+// One work item = (block of queries, KV head, split of the segment's rows).  A block is two tiles of 128 rows, row =
+// (query, head of the group); their queries stay in shared memory, their accumulators in TMEM:
+//   columns   0 .. 127 scores / weights of tile 0 | 128 .. 255 of tile 1 | 256 .. 383 output of tile 0 | 384 .. 511 of tile 1
+// The weights overwrite the scores they come from (of every 16 columns the first 8 become high parts, the others low parts),
+// and are the A operand of the second product from there.  Order of the products per key block j: O0 += P0 V(j), S0 = Q0
+// K(j+1)^T, O1 += P1 V(j), S1 = Q1 K(j+1)^T, so that one tile's softmax runs beside the other's products; products of one
+// thread retire in order, so S0 may overwrite P0 without a wait.
+// The running maximum a row is scaled by moves only when it would grow by more than 2^8 (f16 holds 2^15): the accumulator in
+// TMEM is rescaled rarely, and by the softmax warps themselves.
+// What bounds it: a tile's softmax plus its own products must fit beside the other tile's products (2 x 2560 tensor cycles per
+// key block); eight warps per tile, thread = half a row.
+// Warp roles (640 threads): 0 TMA producer, 1 MMA issuer, 4-11 softmax of tile 0, 12-19 softmax of tile 1.
+constexpr int PA_THREADS = 640;
+constexpr int PA_REGS_LIGHT = 64, PA_REGS_SOFTMAX = 104;        // 640 threads of 96 registers, divided again by warpgroup
+constexpr int PA_STAGES = 5;                                    // 32-KiB stages: one part (high or low) of 128 keys or values
+constexpr uint32_t PA_STAGE_BYTES = 32768, PA_PANEL_BYTES = 16384;
+constexpr uint32_t PA_Q_BYTES = 2 * 32768;
+constexpr uint32_t PA_X_BYTES = 2 * 2 * TILE * 4;               // [tile][half][row]: row maxima of a half; row sums at the end
+constexpr uint32_t PA_SMEM = PA_Q_BYTES + PA_STAGES * PA_STAGE_BYTES + PA_X_BYTES + 8 * (2 * PA_STAGES + 8) + 16;
+
+__device__ __forceinline__ float ex2(float x) { float r; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
+
+struct PfItem { int first, cnt, tiles, g, split, blk, row_lo, key0, n_blk, dup; };
+
+__device__ __forceinline__ PfItem pf_item(const DevView& v, const PfCall& a, int i, int seg) {
+  PfItem it;
+  const int per = v.Hkv * a.n_splits;
+  it.blk = a.blk0 + a.blk_n - 1 - i / per;                      // late queries (they see most) first
+  it.g = (i / a.n_splits) % v.Hkv;
+  it.split = i % a.n_splits;
+  const int2 q = a.blocks[it.blk];
+  const int4 b = a.binfo[it.blk];
+  it.first = q.x;
+  it.cnt = q.y & 0x1ff;
+  it.tiles = it.cnt * v.rep > TILE ? 2 : 1;
+  it.dup = b.z;
+  const int s0 = seg * a.seg_rows;
+  const int lo = max(b.x, s0), hi = min(b.x + b.y, s0 + a.seg_rows);
+  const int nb = hi > lo ? (hi - lo + TILE - 1) / TILE : 0;
+  const int j0 = nb * it.split / a.n_splits, j1 = nb * (it.split + 1) / a.n_splits;
+  it.row_lo = lo - s0 + j0 * TILE;                              // first row inside the segment buffer
+  it.key0 = lo - b.x + j0 * TILE;                               // the same row, counted from the sequence's first
+  it.n_blk = j1 - j0;
+  return it;
+}
+
+template <bool BF16>
+__global__ void __launch_bounds__(PA_THREADS, 1)
+pf_attn_kernel(const __grid_constant__ CUtensorMap map_seg, DevView v, PfCall a, int seg, const unsigned short* __restrict__ q) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t s0 = smem_addr(smem_raw);
+  const bool misaligned = (s0 & 1023u) != 0;
+  const uint32_t sQ = s0, sR = s0 + PA_Q_BYTES;
+  float* sX = reinterpret_cast<float*>(smem_raw + PA_Q_BYTES + PA_STAGES * PA_STAGE_BYTES);
+  unsigned char* tail = smem_raw + PA_Q_BYTES + PA_STAGES * PA_STAGE_BYTES + PA_X_BYTES;
+  const uint32_t bars = smem_addr(tail);
+  const uint32_t full = bars, empty = full + 8 * PA_STAGES, q_full = empty + 8 * PA_STAGES, s_full = q_full + 16, p_full = s_full + 16, o_done = p_full + 16;
+  uint32_t* s_tmem_base = reinterpret_cast<uint32_t*>(tail + 8 * (2 * PA_STAGES + 8));
+  volatile int* abort_flag = reinterpret_cast<int*>(s_tmem_base + 1);
+  if (tid == 0) {
+    for (int i = 0; i < PA_STAGES; ++i) { mbar_init(full + 8 * i, 1); mbar_init(empty + 8 * i, 1); }
+    for (int i = 0; i < 2; ++i) { mbar_init(q_full + 8 * i, 8); mbar_init(s_full + 8 * i, 1); mbar_init(p_full + 8 * i, 8); mbar_init(o_done + 8 * i, 1); }
+    *abort_flag = misaligned ? 1 : 0;
+    mbar_init_fence();
+  }
+  if (warp == 1) tmem_alloc(smem_addr(s_tmem_base), 512);
+  fence_before_sync();
+  __syncthreads();
+  fence_after_sync();
+  const uint32_t tmem_base = *s_tmem_base;
+  const int n_items = a.blk_n * v.Hkv * a.n_splits;
+
+  if (misaligned) {
+    // nothing was started
+  } else if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(PA_REGS_LIGHT));
+    if (warp == 0) {
+      // ------------------------------------------------------------- TMA producer: K low, K high, V high, V low of every key block
+      if (elect_one()) {
+        tma_prefetch_desc(&map_seg);
+        uint32_t st = 0, ph = 0, n_loaded = 0;
+        bool ok = true;
+        for (int i = blockIdx.x; i < n_items && ok; i += gridDim.x) {
+          const PfItem it = pf_item(v, a, i, seg);
+          for (int j = 0; j < it.n_blk && ok; ++j)
+            for (int part = 0; part < 4; ++part) {
+              if (!(ok = mbar_wait_thin(empty + 8 * st, ph ^ 1u, abort_flag))) break;
+              mbar_expect_tx(full + 8 * st, PA_STAGE_BYTES);
+              const int y = (it.g * 4 + (part < 2 ? part ^ 1 : part)) * a.seg_rows + it.row_lo + j * TILE;
+              tma_load_2d(sR + st * PA_STAGE_BYTES, &map_seg, full + 8 * st, 0, y);
+              tma_load_2d(sR + st * PA_STAGE_BYTES + PA_PANEL_BYTES, &map_seg, full + 8 * st, 64, y);
+              ++n_loaded;
+              if (++st == PA_STAGES) { st = 0; ph ^= 1u; }
+            }
+        }
+        if (!ok)                                                // let copies in flight land before the CTA goes away
+          for (uint32_t i = 0; i < PA_STAGES && i < n_loaded; ++i) {
+            const uint32_t n = n_loaded - 1 - i;
+            mbar_wait_drain(full + 8 * (n % PA_STAGES), (n / PA_STAGES) & 1u);
+          }
+      }
+      __syncwarp();
+    } else if (warp == 1) {
+      // ------------------------------------------------------------- MMA issuer (one elected lane)
+      if (elect_one()) {
+        constexpr uint32_t idesc_s = idesc_f16(0, 128, 128);                            // f16 queries and keys, both K-major
+        constexpr uint32_t idesc_o = idesc_f16(BF16 ? 1 : 0, 128, 128) | (1u << 16);    // values MN-major
+        uint32_t st = 0, ph = 0, qph[2] = {0, 0}, pph[2] = {0, 0};
+        bool ok = true;
+        // two consecutive stages (both parts of a block of keys or values)
+        auto take = [&](uint32_t (&pair)[2]) -> bool {
+          for (int k = 0; k < 2; ++k) {
+            if (!mbar_wait_thin(full + 8 * st, ph, abort_flag)) return false;
+            pair[k] = st;
+            if (++st == PA_STAGES) { st = 0; ph ^= 1u; }
+          }
+          fence_after_sync();
+          return true;
+        };
+        auto scores = [&](int h, const uint32_t (&k)[2]) {
+          const uint32_t qa = kmajor_sw128_desc_lo(sQ + h * 32768u), d = tmem_base + h * 128;
+#pragma unroll
+          for (int part = 0; part < 2; ++part)                  // the low parts first: the sum is cut after every instruction
+#pragma unroll
+            for (int pn = 0; pn < 2; ++pn)
+              mma_f16_ss_panel(d, qa + pn * (PA_PANEL_BYTES >> 4), kmajor_sw128_desc_lo(sR + k[part] * PA_STAGE_BYTES + pn * PA_PANEL_BYTES), idesc_s,
+                               part + pn > 0 ? 1u : 0u);
+          mma_commit(s_full + 8 * h);
+        };
+        auto values = [&](int h, const uint32_t (&vv)[2], bool first) {
+          const uint32_t p = tmem_base + h * 128, d = tmem_base + 256 + h * 128;
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {                         // high . high, high . low, low . high
+            const uint32_t pa = p + (c == 2 ? 8 : 0);
+            const uint32_t vb = (((sR + vv[c == 1] * PA_STAGE_BYTES) >> 4) & 0x3fffu) | ((PA_PANEL_BYTES >> 4) << 16);
+#pragma unroll
+            for (int ks = 0; ks < 8; ++ks)
+              mma_f16_ts(d, pa + 16 * ks, ((uint64_t)KMAJOR_SW128_DESC_HI << 32) | (vb + ks * 128u), idesc_o,
+                         (c > 0 || ks > 0) ? 1u : (first ? 0u : 1u));
+          }
+          mma_commit(o_done + 8 * h);
+        };
+        for (int i = blockIdx.x; i < n_items && ok; i += gridDim.x) {
+          const PfItem it = pf_item(v, a, i, seg);
+          for (int h = 0; h < it.tiles && ok; ++h) { ok = mbar_wait(q_full + 8 * h, qph[h], abort_flag); qph[h] ^= 1u; }
+          if (!ok) break;
+          fence_after_sync();
+          if (it.n_blk == 0) continue;
+          uint32_t kk[2], vv[2];
+          if (!(ok = take(kk))) break;
+          for (int h = 0; h < it.tiles; ++h) scores(h, kk);
+          mma_commit(empty + 8 * kk[0]); mma_commit(empty + 8 * kk[1]);
+          for (int j = 0; j < it.n_blk && ok; ++j) {
+            if (!(ok = take(vv))) break;
+            const bool more = j + 1 < it.n_blk;
+            for (int h = 0; h < it.tiles; ++h) {
+              if (!(ok = mbar_wait_thin(p_full + 8 * h, pph[h], abort_flag))) break;
+              pph[h] ^= 1u;
+              fence_after_sync();
+              values(h, vv, j == 0);
+              if (h == it.tiles - 1) { mma_commit(empty + 8 * vv[0]); mma_commit(empty + 8 * vv[1]); }
+              if (more) {
+                if (h == 0 && !(ok = take(kk))) break;
+                scores(h, kk);
+                if (h == it.tiles - 1) { mma_commit(empty + 8 * kk[0]); mma_commit(empty + 8 * kk[1]); }
+              }
+            }
+          }
+        }
+      }
+      __syncwarp();
+    }
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(PA_REGS_SOFTMAX));
+    // ------------------------------------------------------------- softmax
+    const int grp = (warp - 4) >> 2, h = grp >> 1, hf = grp & 1, quarter = warp & 3, row = quarter * 32 + lane;
+    const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16);
+    const uint32_t tS = lane_addr + h * 128 + hf * 64, tO = lane_addr + 256 + h * 128 + hf * 64;
+    unsigned char* sq = smem_raw + h * 32768 + hf * PA_PANEL_BYTES;
+    const int pair_bar = 1 + h * 4 + quarter;                    // the two warps that share 32 rows
+    float* xs = sX + h * 2 * TILE + row;
+    const int rep = v.rep, QT = TILE / rep;
+    // scores in powers of two; a negative scale goes into the queries, a zero one zeroes them (-inf masks need a positive factor)
+    const float scale = v.sm_scale == 0.f ? 1.f : fabsf(v.sm_scale) * 1.44269504088896340736f;
+    const unsigned flip = v.sm_scale < 0.f ? 0x80008000u : 0u, keep_q = v.sm_scale == 0.f ? 0u : 0xffffffffu;
+    uint32_t sph = 0, oph = 0;                                   // phases of s_full and of the next o_done
+    bool ok = true;
+    for (int i = blockIdx.x; i < n_items && ok; i += gridDim.x) {
+      const PfItem it = pf_item(v, a, i, seg);
+      if (h >= it.tiles) continue;
+      // this warp's half of its 32 query rows as the K-major operand, four rows per instruction
+#pragma unroll 4
+      for (int k = 0; k < 8; ++k) {
+        const int r = quarter * 32 + 4 * k + (lane >> 3), k8 = lane & 7;
+        const int ch = hf * 4 + (k8 >> 1) + 8 * (k8 & 1);        // the keys' order: pairs of pieces 64 dims apart
+        const int ql = h * QT + r / rep;
+        uint4 val = make_uint4(0u, 0u, 0u, 0u);
+        if (ql < it.cnt)
+          val = __ldg(reinterpret_cast<const uint4*>(q + ((size_t)a.qrow[it.first + ql] * v.Hq + it.g * rep + r % rep) * HEAD_DIM) + ch);
+        if constexpr (BF16) {
+          const unsigned w[4] = {val.x, val.y, val.z, val.w};
+          unsigned o[4];
+          bool over = false;
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const float lo = __uint_as_float(w[e] << 16), hi = __uint_as_float(w[e] & 0xffff0000u);
+            over |= !(fabsf(lo) <= 65504.f) || !(fabsf(hi) <= 65504.f);
+            o[e] = pack_f16x2_sat(lo, hi);
+          }
+          if (over) set_status(v, TWKV_ERR_DEVICE_CHECK);        // a bf16 query beyond the f16 range would be clamped
+          val = make_uint4(o[0], o[1], o[2], o[3]);
+        }
+        val.x = (val.x ^ flip) & keep_q; val.y = (val.y ^ flip) & keep_q; val.z = (val.z ^ flip) & keep_q; val.w = (val.w ^ flip) & keep_q;
+        *reinterpret_cast<uint4*>(sq + r * 128 + ((k8 ^ (r & 7)) << 4)) = val;
+      }
+      fence_proxy_async_smem();
+      fence_before_sync();                                       // the previous item's accumulator has been read as well
+      __syncwarp();
+      if (lane == 0) mbar_arrive(q_full + 8 * h);
+
+      const int ql = h * QT + row / rep;
+      const int vis = ql < it.cnt ? a.qvis[it.first + ql] : 0;
+      const int qpos = it.dup && ql < it.cnt ? a.qpos[it.first + ql] : -1;
+      float m = -INFINITY;
+      uint64_t l2 = 0;                                           // two partial sums of this half's weights
+      for (int j = 0; j < it.n_blk; ++j) {
+        ok = __all_sync(0xffffffffu, mbar_wait(s_full + 8 * h, sph, abort_flag));
+        sph ^= 1u;
+        fence_after_sync();
+        uint32_t x[64];
+        tmem_ld32(tS, x);
+        tmem_ld32(tS + 32, x + 32);
+        tmem_ld_wait();
+        const int left = vis - (it.key0 + j * TILE) - hf * 64;   // columns of this half that the row sees (repeated positions: that hold a token)
+        if (it.dup || __any_sync(0xffffffffu, left < 64)) {
+          unsigned see[2];                                       // one bit per column
+#pragma unroll
+          for (int e = 0; e < 2; ++e) see[e] = left >= 32 * (e + 1) ? 0xffffffffu : (left <= 32 * e ? 0u : (1u << (left - 32 * e)) - 1u);
+          if (it.dup) {
+            const int* rp = a.rowpos + (size_t)seg * a.seg_rows + it.row_lo + j * TILE + hf * 64;
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+#pragma unroll 1
+              for (int c = 0; c < 32; ++c)
+                if (32 * e + c < left && rp[32 * e + c] > qpos) see[e] &= ~(1u << c);
+          }
+#pragma unroll
+          for (int c = 0; c < 64; ++c) x[c] = (see[c >> 5] >> (c & 31)) & 1u ? x[c] : 0xff800000u;
+        }
+        float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+        for (int c = 0; c < 64; c += 8)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) mx[e] = fmaxf(mx[e], fmaxf(__uint_as_float(x[c + e]), __uint_as_float(x[c + 4 + e])));
+        float top = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+        // Both halves of a row scale by the same maximum.  The next scores arrive only when both warps have handed over these
+        // weights, so a warp never overwrites a value that its partner still reads.  A wait that ran out in either warp ends
+        // the loop in both: neither is left at a barrier.
+        xs[hf * TILE] = top;
+        if (!(ok = named_bar_and(pair_bar, 64, ok))) break;
+        top = fmaxf(top, xs[(hf ^ 1) * TILE]) * scale;
+        const bool grow = top > m + 8.f;                          // also the first finite maximum
+        if (__any_sync(0xffffffffu, grow)) {
+          const float m_new = grow ? top : m;
+          const float f = m == m_new ? 1.f : ex2(m - m_new);      // 0 when there was no maximum yet
+          m = m_new;
+          l2 = mul2(l2, pk2(f, f));
+          if (j > 0) {
+            // the previous block's product (a wait that ran out has raised the abort flag and ends the loop at the next barrier)
+            const bool got = __all_sync(0xffffffffu, mbar_wait(o_done + 8 * h, oph ^ 1u, abort_flag));
+            fence_after_sync();
+            if (got) {
+#pragma unroll 1
+              for (int c = 0; c < 8; ++c) {
+                uint32_t o[8];
+                tmem_ld8(tO + 8 * c, o);
+                tmem_ld_wait();
+#pragma unroll
+                for (int k = 0; k < 8; ++k) o[k] = __float_as_uint(__uint_as_float(o[k]) * f);
+                tmem_st8(tO + 8 * c, o);
+              }
+            }
+          }
+        }
+        const float mu = m == -INFINITY ? 0.f : m;
+        const uint64_t nm2 = pk2(-mu, -mu), sc2 = pk2(scale, scale);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          uint32_t w[16];                                        // 8 columns of high parts, 8 of low ones, over the scores they come from
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            float p0, p1;
+            unpk2(fma2(pk2u(x[16 * c + 2 * k], x[16 * c + 2 * k + 1]), sc2, nm2), p0, p1);
+            const uint64_t p = pk2(ex2(p0), ex2(p1));
+            l2 = add2(l2, p);
+            split2<BF16>(p, w[k], w[8 + k]);
+          }
+          tmem_st16(tS + 16 * c, w);
+        }
+        tmem_st_wait();
+        fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(p_full + 8 * h);
+        oph ^= 1u;
+      }
+      float l = 0.f;
+      if (it.n_blk > 0) {
+        if (!ok) break;                                          // agreed by both warps above
+        ok = __all_sync(0xffffffffu, mbar_wait(o_done + 8 * h, oph ^ 1u, abort_flag));
+        fence_after_sync();
+        float la, lb;
+        unpk2(l2, la, lb);
+        xs[hf * TILE] = la + lb;                                 // the row sum of both halves
+        if (!(ok = named_bar_and(pair_bar, 64, ok))) break;
+        l = xs[0] + xs[TILE];                                    // (read before this warp hands over the next item's queries)
+      }
+      // the item's partial result, joined with what earlier segments left; column-major, so that a warp's rows lie together
+      float* part = a.slots + ((((size_t)(it.blk - a.blk0) * v.Hkv + it.g) * a.n_splits + it.split) * 2 + h) * (130 * TILE) + row;
+      if (it.n_blk > 0) {
+        float wo = 1.f, wp = 0.f;
+        if (seg > 0) {
+          const float mp = part[128 * TILE], lp = part[129 * TILE];
+          named_bar_sync(pair_bar, 64);                          // both halves have read them
+          if (lp > 0.f) {
+            const float mm = fmaxf(m, mp);
+            wo = m == -INFINITY ? 0.f : ex2(m - mm);
+            wp = ex2(mp - mm);
+            l = l * wo + lp * wp;
+            m = mm;
+          }
+        }
+#pragma unroll 1
+        for (int c = 0; c < 4; ++c) {
+          uint32_t o[16];
+          tmem_ld16(tO + 16 * c, o);
+          tmem_ld_wait();
+          float* pc = part + (size_t)(hf * 64 + 16 * c) * TILE;
+          if (wp > 0.f) {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) pc[k * TILE] = __uint_as_float(o[k]) * wo + pc[k * TILE] * wp;
+          } else {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) pc[k * TILE] = __uint_as_float(o[k]);
+          }
+        }
+        if (hf == 0) { part[128 * TILE] = m; part[129 * TILE] = l; }
+      } else if (seg == 0 && hf == 0) {
+        part[128 * TILE] = -INFINITY; part[129 * TILE] = 0.f;
+      }
+    }
+    tmem_ld_wait();
+  }
+  fence_before_sync();
+  __syncthreads();
+  fence_after_sync();
+  if (warp == 1) tmem_dealloc(tmem_base, 512);
+  if (tid == 0 && *abort_flag) set_status(v, misaligned ? TWKV_ERR_DEVICE_CHECK : TWKV_ERR_TIMEOUT);
+}
+
+// Joins the splits of one tile of rows and writes the queries' outputs.  One CTA per (block of queries, KV head, tile, 32
+// columns); a thread owns one row of 16 of the columns, so reads are coalesced along the rows; rows leave through shared
+// memory.
+template <int OUT>
+__global__ void __launch_bounds__(256) pf_combine_kernel(DevView v, PfCall a, void* __restrict__ out) {
+  __shared__ float s[TILE][33];
+  const int c0 = (blockIdx.x & 3) * 32, h = (blockIdx.x >> 2) & 1, bg = blockIdx.x >> 3, g = bg % v.Hkv, blk = bg / v.Hkv;
+  const int2 q = a.blocks[a.blk0 + blk];
+  const int cnt = q.y & 0x1ff, rep = v.rep, QT = TILE / rep;
+  const int rows = min(TILE, (cnt - h * QT) * rep);
+  if (rows <= 0) return;
+  const int tid = threadIdx.x, row = tid & (TILE - 1), cc = (tid >> 7) * 16;
+  const size_t stride = (size_t)2 * 130 * TILE;
+  const float* part = a.slots + (((size_t)blk * v.Hkv + g) * a.n_splits * 2 + h) * (130 * TILE) + row;
+  float m = -INFINITY, l = 0.f;
+  float acc[16];
+#pragma unroll
+  for (int c = 0; c < 16; ++c) acc[c] = 0.f;
+  for (int k = 0; k < a.n_splits; ++k) {
+    const float lk = part[k * stride + 129 * TILE], mk = part[k * stride + 128 * TILE];
+    if (!(lk > 0.f)) continue;
+    float x[16];
+#pragma unroll
+    for (int c = 0; c < 16; ++c) x[c] = part[k * stride + (c0 + cc + c) * TILE];
+    const float mn = fmaxf(m, mk), wo = ex2(m - mn), wk = ex2(mk - mn);     // first split: wo = 0
+    l = l * wo + lk * wk;
+#pragma unroll
+    for (int c = 0; c < 16; ++c) acc[c] = acc[c] * wo + x[c] * wk;
+    m = mn;
+  }
+  const float inv = l > 0.f ? 1.f / l : 0.f;
+#pragma unroll
+  for (int c = 0; c < 16; ++c) s[row][cc + c] = acc[c] * inv;
+  __syncthreads();
+  for (int i = tid; i < rows * 4; i += 256) {                     // eight columns of one row
+    const int r = i >> 2, c8 = (i & 3) * 8;
+    const int ql = h * QT + r / rep;
+    const size_t o = ((size_t)a.qrow[q.x + ql] * v.Hq + g * rep + r % rep) * HEAD_DIM + c0 + c8;
+    const float* x = &s[r][c8];
+    if constexpr (OUT == TWKV_F32) {
+      float4* d = reinterpret_cast<float4*>(reinterpret_cast<float*>(out) + o);
+      d[0] = make_float4(x[0], x[1], x[2], x[3]);
+      d[1] = make_float4(x[4], x[5], x[6], x[7]);
+    } else {
+      unsigned w[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if constexpr (OUT == TWKV_BF16) asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w[k]) : "f"(x[2 * k + 1]), "f"(x[2 * k]));
+        else asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(w[k]) : "f"(x[2 * k + 1]), "f"(x[2 * k]));
+      }
+      *reinterpret_cast<uint4*>(reinterpret_cast<unsigned short*>(out) + o) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+  }
+}
+
+// ------------------------------------------------------------------------------------------ host side
+cudaError_t launch_pf_tables(const DevView& v, const PfCall& a, int layer, int sm_count, cudaStream_t st) {
+  ProfScope ps(TWKV_K_PLAN, st);
+  const int zc = (a.n_words + 8191) / 8192, qctas = (a.n_blocks + 31) / 32;
+  pf_init_kernel<<<zc < 1 ? 1 : (zc > sm_count ? sm_count : zc), 1024, 0, st>>>(v, a);
+  pf_bits_kernel<<<sm_count, 1024, 0, st>>>(v, a, layer);
+  pf_scan_kernel<<<a.n_u, 1024, 0, st>>>(v, a, layer);
+  const int qc = qctas > sm_count ? sm_count : qctas;
+  pf_rows_kernel<<<sm_count + qc, 1024, 0, st>>>(v, a, layer, qc);
+  count_launch(4);
+  return cudaGetLastError();
+}
+
+template <bool BF16>
+static cudaError_t launch_pf_segment_t(const DevView& v, const PfCall& a, const PfMaps& maps, int layer, int seg, const void* q, int sm_count, cudaStream_t st) {
+  cudaError_t e = cudaFuncSetAttribute(pf_recon_kernel<BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PR_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(pf_attn_kernel<BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PA_SMEM);
+  if (e != cudaSuccess) return e;
+  { ProfScope ps(TWKV_K_KSCORE, st); pf_recon_kernel<BF16><<<sm_count, PR_THREADS, PR_SMEM, st>>>(maps.blocks, maps.uk, maps.uv, v, a, layer, seg); }
+  const int n_items = a.blk_n * v.Hkv * a.n_splits;
+  {
+    ProfScope ps(TWKV_K_VACC, st);
+    pf_attn_kernel<BF16><<<n_items < sm_count ? n_items : sm_count, PA_THREADS, PA_SMEM, st>>>(maps.seg, v, a, seg, reinterpret_cast<const unsigned short*>(q));
+  }
+  count_launch(2);
+  return cudaGetLastError();
+}
+cudaError_t launch_pf_segment(const DevView& v, const PfCall& a, const PfMaps& maps, int layer, int seg, const void* q, int sm_count, cudaStream_t st) {
+  return v.dtype == TWKV_BF16 ? launch_pf_segment_t<true>(v, a, maps, layer, seg, q, sm_count, st)
+                              : launch_pf_segment_t<false>(v, a, maps, layer, seg, q, sm_count, st);
+}
+
+cudaError_t launch_pf_combine(const DevView& v, const PfCall& a, void* out, cudaStream_t st) {
+  ProfScope ps(TWKV_K_MERGE, st);
+  const int grid = a.blk_n * v.Hkv * 8;
+  if (v.out_dtype == TWKV_F32) pf_combine_kernel<TWKV_F32><<<grid, 256, 0, st>>>(v, a, out);
+  else if (v.out_dtype == TWKV_BF16) pf_combine_kernel<TWKV_BF16><<<grid, 256, 0, st>>>(v, a, out);
+  else pf_combine_kernel<TWKV_F16><<<grid, 256, 0, st>>>(v, a, out);
+  count_launch();
+  return cudaGetLastError();
+}
+
+}  // namespace twkv
