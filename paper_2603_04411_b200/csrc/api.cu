@@ -1,4 +1,5 @@
 // C ABI of libtwkv: cache lifetime, argument checks, piece loop, launch bookkeeping.
+#include <algorithm>
 #include <atomic>
 #include <cstdio>
 #include <cstdlib>
@@ -10,6 +11,7 @@
 
 #include "twkv_dev.h"
 #include "tc_util.cuh"
+#include "prefill.h"
 
 namespace twkv {
 
@@ -99,6 +101,9 @@ struct Layout {
 };
 
 constexpr int GATE_PIECE = 8192;       // tokens per COMPUTE-mode gate piece (logits scratch rows)
+// Queries of one sequence from which the tiled prefill kernels take over from waves of decode passes: a wave rebuilds every key
+// (and shares nothing), the tiled kernels rebuild keys and values once but store both in full width.
+constexpr int PF_MIN_WAVES = 4;
 constexpr int GATE_TC_MIN_TOKENS = 1024;   // calls at least this large run the fused tcgen05 gate kernel
 
 struct Offsets {
@@ -228,7 +233,18 @@ struct twkv_cache {
   std::vector<char> prepared_w;        // per layer: those copies and maps are current
   bool kscore_pairs = false;           // the K-score kernel runs on CTA pairs (the device can co-schedule them)
   std::vector<unsigned long long> guards;   // byte offsets (from the pool's start) of the guard words
+  // Upper bound on the tokens a layer holds: tokens handed to twkv_compress since the last reset (refused and evicted ones
+  // included).  Bounds the launches of a prefill call; void once a compress call has been captured into a graph, since
+  // replays append tokens that the host does not see.
+  std::vector<std::atomic<long long>> appended;
+  std::atomic<bool> append_captured{false};
 };
+
+static bool is_capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &s) != cudaSuccess) { cudaGetLastError(); return true; }
+  return s != cudaStreamCaptureStatusNone;
+}
 
 
 extern "C" {
@@ -301,6 +317,8 @@ twkv_status twkv_cache_reset(twkv_cache* c, void* stream) {
   if (cudaMemsetAsync(c->pool + c->off.key_last, 0xff, (size_t)c->cfg.n_layers * c->dims.NK * sizeof(int), st) != cudaSuccess)
     return TWKV_ERR_CUDA;
   if (cudaMemsetAsync(c->pool + c->off.status, 0, 8 * sizeof(int), st) != cudaSuccess) return TWKV_ERR_CUDA;
+  if (!is_capturing(st))
+    for (auto& n : c->appended) n.store(0, std::memory_order_relaxed);
   return TWKV_OK;
 }
 
@@ -341,6 +359,7 @@ twkv_status twkv_cache_create(const twkv_config* cfg, void* pool, size_t pool_by
   c->map_wT.resize(2 * (size_t)cfg->n_layers);
   c->map_wT_half.resize(2 * (size_t)cfg->n_layers);
   c->prepared_w.assign(cfg->n_layers, 0);
+  c->appended = std::vector<std::atomic<long long>>(cfg->n_layers);
   if (!make_tmap_2d(&c->map_blocks, c->view.blocks, (uint64_t)c->view.n_blocks * TILE, PANEL, PANEL * 2, TILE)) { delete c; return TWKV_ERR_CUDA; }
   if (c->cfg.n_q_heads % 4 == 0) {
     const int hq = c->cfg.n_q_heads, nb = hq < 16 ? hq : (hq <= 16 ? 16 : 32);
@@ -428,6 +447,8 @@ twkv_status twkv_compress(twkv_cache* c, int layer, const void* K, const void* V
   cudaStream_t st = (cudaStream_t)stream;
   const DevView& v = c->view;
   const size_t row = (size_t)v.d_kv * 2;
+  if (is_capturing(st)) c->append_captured.store(true, std::memory_order_relaxed);
+  c->appended[layer].fetch_add(n_tok, std::memory_order_relaxed);
   if (mode == TWKV_GATE_LOGITS) {
     if (launch_gate_rank(v, scores, levels, n_tok, st) != cudaSuccess) return TWKV_ERR_CUDA;
   } else if (mode == TWKV_GATE_COMPUTE && n_tok >= GATE_TC_MIN_TOKENS && c->sm_count <= 160) {
@@ -516,20 +537,133 @@ twkv_status twkv_decode_attn(twkv_cache* c, int layer, const void* q, const int3
   return decode_pass(c, layer, q, seq_ids, n_seq, out, num_splits, nullptr, nullptr, (cudaStream_t)stream);
 }
 
+// The tiled form of a prefill call: queries sorted by (sequence, position), dense rows of the visible tokens in segments.
+// `order`: query indices sorted that way.  Sets *done = false, with nothing launched, where the call's tables do not fit the
+// scratch regions they live in (the caller then serves the queries in waves).
+static twkv_status prefill_tiled(twkv_cache* c, int layer, const void* q, const int32_t* q_seq, const int32_t* q_pos, const std::vector<int>& order,
+                                 void* out, cudaStream_t st, bool* done) {
+  const DevView& v = c->view;
+  const int n_q = (int)order.size(), QT = TILE / v.rep, pos_end = ROPE_LO * ROPE_HI;
+  *done = false;
+  std::vector<int> host(2 * (size_t)n_q), blocks, seqs;
+  long long n_words = 0, rows_cap = 0;
+  const long long tmax_rows = (c->cfg.max_tokens_per_seq + TILE - 1) / TILE * (long long)TILE;
+  for (int lo = 0; lo < n_q;) {
+    int hi = lo;
+    while (hi < n_q && q_seq[order[hi]] == q_seq[order[lo]]) ++hi;
+    const int u = (int)seqs.size() / 3, maxq = std::min(q_pos[order[hi - 1]], pos_end - 1);
+    seqs.push_back(q_seq[order[lo]]); seqs.push_back(maxq); seqs.push_back((int)n_words);
+    n_words += (maxq + 32) >> 5;
+    rows_cap += tmax_rows;
+    for (int b = lo; b < hi; b += 2 * QT) { blocks.push_back(b); blocks.push_back(u << 9 | std::min(2 * QT, hi - b)); }
+    lo = hi;
+  }
+  for (int i = 0; i < n_q; ++i) { host[i] = order[i]; host[n_q + i] = q_pos[order[i]]; }
+  const int n_u = (int)seqs.size() / 3, n_blocks = (int)blocks.size() / 2;
+  host.insert(host.end(), blocks.begin(), blocks.end());
+  host.insert(host.end(), seqs.begin(), seqs.end());
+  // the tables made on the device share the region of the gate's fix-up list
+  const size_t fix_ints = gate_tc_fix_bytes() / sizeof(int);
+  const size_t need = 4 * (size_t)n_blocks + n_q + 3 * (size_t)n_u + 4 + (size_t)v.S + 2 * (size_t)n_words;
+  if (need > fix_ints || host.size() > 3 * (size_t)TWKV_PREFILL_MAX_QUERIES) return TWKV_OK;
+
+  PfCall a = {};
+  const int* w = v.wave_buf;
+  a.qrow = w; a.qpos = w + n_q; a.blocks = (const int2*)(w + 2 * (size_t)n_q); a.seqs = w + 2 * (size_t)n_q + blocks.size();
+  a.n_u = n_u; a.n_blocks = n_blocks; a.n_words = (int)n_words;
+  a.binfo = v.gate_fix;
+  int* p = (int*)(v.gate_fix + n_blocks);
+  a.qvis = p; p += n_q;
+  a.rows = p; a.base = p + n_u; a.dup = p + 2 * (size_t)n_u; p += 3 * (size_t)n_u;
+  a.ticket = p; p += 4;
+  a.slot = p; p += v.S;
+  a.bits = (unsigned*)p; a.pref = p + n_words;
+  a.krow = v.kv_link; a.krow_out = v.evict_map; a.vrow = v.evict_map + (size_t)v.NT * TILE;
+  a.rowpos = (int*)v.scores;
+  a.seg_buf = (unsigned char*)v.gate_scratch;
+
+  // how many rows the sequences can have: their capacity, or what the layer was ever given
+  long long rows_max = rows_cap;
+  if (!c->append_captured.load(std::memory_order_relaxed) && !is_capturing(st))
+    rows_max = std::min(rows_max, c->appended[layer].load(std::memory_order_relaxed) + (TILE - 1) * (long long)n_u);
+  if (rows_max > 32767ll * (GATE_PIECE / 2)) return TWKV_OK;         // a tile's segments are kept in two 16-bit halves
+  // Segments of 8192 rows with the partial results in the V pass's region, or of 4096 rows with them in the second half of
+  // the gate scratch (fewer heads leave the first region small); splits of a segment's rows where the blocks of queries
+  // alone leave SMs idle.  Estimated in key blocks of one CTA: its share of a segment plus 1.5 for an item's start and end.
+  const size_t slot_bytes = PF_SLOT_FLOATS * sizeof(float);
+  double best = 1e300;
+  int best_rows = 0, best_splits = 1, best_group = 1;
+  for (int half = 0; half < 2; ++half) {
+    const int seg_rows = half ? GATE_PIECE / 2 : GATE_PIECE;
+    const size_t region = half ? (size_t)GATE_PIECE * v.d_kv * sizeof(float) : (size_t)c->dims.max_partials * v.Hq * v.d_kv * sizeof(float);
+    const long long cap = (long long)(region / slot_bytes);
+    const int group = (int)std::min<long long>(n_blocks, cap / v.Hkv);
+    if (group < 1) continue;
+    const double groups = (double)((n_blocks + group - 1) / group), segs = (double)((rows_max + seg_rows - 1) / seg_rows);
+    const int seg_blocks = std::max(1, (int)((std::min<long long>(rows_max, seg_rows) + TILE - 1) / TILE));
+    for (int ns = 1; ns <= 32 && ns <= seg_blocks && (long long)group * v.Hkv * ns <= cap; ++ns) {
+      const long long rounds = ((long long)group * v.Hkv * ns + c->sm_count - 1) / c->sm_count;
+      const double cost = groups * segs * ((double)rounds * ((seg_blocks + ns - 1) / ns + 1.5) + 4.0 + seg_rows / 1024.0);
+      if (cost < best) { best = cost; best_rows = seg_rows; best_splits = ns; best_group = group; }
+    }
+  }
+  if (!best_rows) return TWKV_OK;
+  a.seg_rows = best_rows; a.n_splits = best_splits;
+  a.slots = best_rows == GATE_PIECE ? v.part_acc : (float*)(a.seg_buf + (size_t)GATE_PIECE * v.d_kv * sizeof(float));
+
+  PfMaps maps;
+  maps.blocks = c->map_blocks;
+  const uint64_t d = (uint64_t)v.d_kv;
+  if (!make_tmap_2d(&maps.uk, c->params[layer].Uinv_k, d, d, d * 2, PANEL) || !make_tmap_2d(&maps.uv, c->params[layer].Uinv_v, d, d, d * 2, PANEL) ||
+      !make_tmap_2d(&maps.seg, a.seg_buf, (uint64_t)v.Hkv * 4 * a.seg_rows, HEAD_DIM, HEAD_DIM * 2, TILE)) return TWKV_ERR_CUDA;
+  // pieces below 64 KiB: a larger copy from pageable memory would wait for the stream before it returns
+  const char* src = (const char*)host.data();
+  for (size_t at = 0, bytes = host.size() * sizeof(int); at < bytes; at += 49152)
+    if (cudaMemcpyAsync((char*)v.wave_buf + at, src + at, std::min<size_t>(49152, bytes - at), cudaMemcpyHostToDevice, st) != cudaSuccess) return TWKV_ERR_CUDA;
+  *done = true;
+  if (launch_pf_tables(v, a, layer, c->sm_count, st) != cudaSuccess) return TWKV_ERR_CUDA;
+  const int n_segs = std::max(1, (int)((rows_max + a.seg_rows - 1) / a.seg_rows));
+  for (a.blk0 = 0; a.blk0 < n_blocks; a.blk0 += best_group) {
+    a.blk_n = std::min(best_group, n_blocks - a.blk0);
+    for (int seg = 0; seg < n_segs; ++seg)
+      if (launch_pf_segment(v, a, maps, layer, seg, q, c->sm_count, st) != cudaSuccess) return TWKV_ERR_CUDA;
+    if (launch_pf_combine(v, a, out, st) != cudaSuccess) return TWKV_ERR_CUDA;
+  }
+  return TWKV_OK;
+}
+
 twkv_status twkv_prefill_attn(twkv_cache* c, int layer, const void* q, const int32_t* q_seq, const int32_t* q_pos, int n_q,
                               void* out, int num_splits, void* stream) {
   if (!c || layer < 0 || layer >= c->cfg.n_layers || n_q < 0 || num_splits < 0) return TWKV_ERR_INVALID_ARG;
   if (n_q == 0) return TWKV_OK;
   if (!q || !q_seq || !q_pos || !out || n_q > TWKV_PREFILL_MAX_QUERIES) return TWKV_ERR_INVALID_ARG;
   if (((uintptr_t)q | (uintptr_t)out) % 16) return TWKV_ERR_INVALID_ARG;
+  if (!c->params[layer].Uinv_k || !c->params[layer].Uinv_v) return TWKV_ERR_INVALID_ARG;
   const int S = c->cfg.max_seqs;
   // wave k = the k-th query of every sequence, in order of appearance; inside a wave the sequences are distinct
   std::vector<int> seen(S, 0), wave_of(n_q);
-  int n_waves = 0;
+  int n_waves = 0, n_distinct = 0;
+  bool sorted = true;
   for (int i = 0; i < n_q; ++i) {
     if (q_seq[i] < 0 || q_seq[i] >= S || q_pos[i] < 0) return TWKV_ERR_INVALID_ARG;
+    n_distinct += seen[q_seq[i]] == 0;
     wave_of[i] = seen[q_seq[i]]++;
     if (wave_of[i] + 1 > n_waves) n_waves = wave_of[i] + 1;
+    if (i && (q_seq[i] < q_seq[i - 1] || (q_seq[i] == q_seq[i - 1] && q_pos[i] < q_pos[i - 1]))) sorted = false;
+  }
+  if ((long long)n_distinct * num_splits > c->dims.max_partials) return TWKV_ERR_INVALID_ARG;
+  DeviceGuard g(c->device);
+  if (!g.ok) return TWKV_ERR_CUDA;
+  cudaStream_t st = (cudaStream_t)stream;
+  if (n_waves >= PF_MIN_WAVES) {
+    ProfBind pb(&c->prof);
+    std::vector<int> order(n_q);
+    for (int i = 0; i < n_q; ++i) order[i] = i;
+    if (!sorted)
+      std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return q_seq[x] != q_seq[y] ? q_seq[x] < q_seq[y] : q_pos[x] < q_pos[y]; });
+    bool done = false;
+    const twkv_status s = prefill_tiled(c, layer, q, q_seq, q_pos, order, out, st, &done);
+    if (done || s != TWKV_OK) return s;
   }
   std::vector<int> wave_start(n_waves + 1, 0), fill(n_waves, 0);
   for (int i = 0; i < n_q; ++i) ++wave_start[wave_of[i] + 1];
@@ -541,9 +675,6 @@ twkv_status twkv_prefill_attn(twkv_cache* c, int layer, const void* q, const int
     host[TWKV_PREFILL_MAX_QUERIES + at] = i;
     host[2 * TWKV_PREFILL_MAX_QUERIES + at] = q_pos[i];
   }
-  DeviceGuard g(c->device);
-  if (!g.ok) return TWKV_ERR_CUDA;
-  cudaStream_t st = (cudaStream_t)stream;
   // the copy is staged from pageable memory before the call returns, so `host` may go out of scope afterwards
   if (cudaMemcpyAsync(c->view.wave_buf, host.data(), host.size() * sizeof(int), cudaMemcpyHostToDevice, st) != cudaSuccess) return TWKV_ERR_CUDA;
   for (int w = 0; w < n_waves; ++w) {
