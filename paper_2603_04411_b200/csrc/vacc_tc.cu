@@ -8,7 +8,7 @@
 // CTA's heads padded to 16 / 32, K = 16 tokens per instruction, 8 instructions per tile): a panel as TMA lands it
 // (rows of 128 bytes, 128-byte swizzle) is exactly the MN-major operand layout, the second panel of the pair being the
 // second 64-column atom along M (leading byte offset = one panel).  The fp32 accumulator of panel pair i is N columns of
-// TMEM at column i * N and stays there for the whole kernel; no accumulator lives in registers and the panels are read
+// TMEM (two parts each) at column 2 i N and stays there for the whole kernel; no accumulator lives in registers and the panels are read
 // from shared memory by the tensor core only.  A class with an odd number of panels ends with a lone panel; its chain
 // points the second atom at a small zero block instead (the leading byte offset is free per instruction), so the pair's
 // upper accumulator half adds zeros.
@@ -19,7 +19,8 @@
 // reads as many bytes of scores as of values, and with one tile in flight their latency bound the kernel.  Where the
 // head count is not a multiple of four (rows not 16-byte aligned: no tensor map) each warp copies the rows of its own
 // token groups with cp.async instead (TS = false).
-// Weights go in as two parts of the cache type (see below), two chains per pair.
+// Weights go in as two parts of the cache type (see below): 2 N rows of one B operand, so that a panel is read once for both;
+// the two halves of the accumulator are added at the end.
 //
 // Warp roles (320 threads, one CTA per SM):
 //   warp 0      TMA producer of V panels (ring of 32-KiB pair stages; one elected lane)
@@ -46,9 +47,10 @@ constexpr int VT_SC = 3;                                       // tiles of score
 template <bool BF16, int N>
 struct VtCfg {
   static constexpr int PARTS = 2;                              // operands per weight (high and low part)
-  static constexpr uint32_t P_HALF_BYTES = N * 128;            // [N heads][64 tokens]
-  static constexpr uint32_t P_PART_BYTES = 2 * P_HALF_BYTES;
-  static constexpr uint32_t P_BUF_BYTES = PARTS * P_PART_BYTES;
+  static constexpr int NB = PARTS * N;                         // rows of the B operand: the N heads' high parts, then their low parts
+  static constexpr uint32_t P_PART_BYTES = N * 128;            // [N heads][64 tokens]
+  static constexpr uint32_t P_HALF_BYTES = PARTS * P_PART_BYTES;
+  static constexpr uint32_t P_BUF_BYTES = 2 * P_HALF_BYTES;
   static constexpr uint32_t TAIL_BYTES = VT_META * 16 + VT_PTHREADS * 4 + 256;      // descriptors, row sums, barriers
   static constexpr uint32_t SC_STAGE_BYTES = 128 * N * 4;      // [128 tokens][N heads] fp32
   static constexpr uint32_t FIXED_BYTES = VT_ZERO_BYTES + 2 * P_BUF_BYTES + VT_SC * SC_STAGE_BYTES + TAIL_BYTES + 1024;   // + alignment slack
@@ -86,7 +88,7 @@ __global__ void __launch_bounds__(VT_THREADS, 1)
 vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_constant__ CUtensorMap map_scores, DevView v, int layer,
                const int* __restrict__ seq_ids, int n_splits) {
   using C = VtCfg<BF16, N>;
-  constexpr int S = C::STAGES, PARTS = C::PARTS, ITEMS = C::ITEMS;
+  constexpr int S = C::STAGES, ITEMS = C::ITEMS;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int Hq = v.Hq, d_kv = v.d_kv;
@@ -125,7 +127,7 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
 
   const int n_pairs = (v.NC + 1) >> 1;
   uint32_t tmem_cols = 32;
-  while (tmem_cols < (uint32_t)(n_pairs * N)) tmem_cols <<= 1;
+  while (tmem_cols < (uint32_t)(n_pairs * C::NB)) tmem_cols <<= 1;
 
   if (tid == 0) {
     for (int i = 0; i < S; ++i) { mbar_init(full + 8 * i, 1); mbar_init(empty + 8 * i, 1); }
@@ -221,7 +223,7 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
     } else if (warp == 1) {
       // ------------------------------------------------------------- MMA issuer
       if (elect_one()) {
-        constexpr uint32_t idesc = vt_idesc(BF16 ? 1 : 0, N);
+        constexpr uint32_t idesc = vt_idesc(BF16 ? 1 : 0, C::NB);
         for (int i = 0; i < cn && ok; ++i) {
           const int k = c0 + i;
           const int cls = s_meta[i].y;
@@ -233,21 +235,17 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
             fence_after_sync();
             const uint32_t a0 = sRing + st * VT_STAGE_BYTES;
             const bool two = j + 1 < cls;
-            const uint32_t pair = (uint32_t)j >> 1, d_tmem = tmem_base + pair * N;
+            const uint32_t pair = (uint32_t)j >> 1, d_tmem = tmem_base + pair * C::NB;
             uint32_t acc = (touched >> pair) & 1u;
 #pragma unroll
-            for (int part = 0; part < PARTS; ++part) {
-#pragma unroll
-              for (int ks = 0; ks < 8; ++ks) {
-                const uint32_t a_addr = a0 + ks * 2048u;                                   // 16 token rows per instruction
-                const uint32_t lbo = two ? VT_PANEL_BYTES : sZero - a_addr;               // where the second 64 columns are
-                const uint32_t a_lo = ((a_addr >> 4) & 0x3fffu) | ((lbo >> 4) << 16);
-                const uint32_t b_addr = pb + part * C::P_PART_BYTES + (ks >> 2) * C::P_HALF_BYTES + (ks & 3) * 32u;
-                const uint32_t b_lo = kmajor_sw128_desc_lo(b_addr);
-                const uint64_t ad = ((uint64_t)KMAJOR_SW128_DESC_HI << 32) | a_lo, bd = ((uint64_t)KMAJOR_SW128_DESC_HI << 32) | b_lo;
-                mma_f16_ss(d_tmem, ad, bd, idesc, acc);
-                acc = 1u;
-              }
+            for (int ks = 0; ks < 8; ++ks) {
+              const uint32_t a_addr = a0 + ks * 2048u;                                     // 16 token rows per instruction
+              const uint32_t lbo = two ? VT_PANEL_BYTES : sZero - a_addr;                 // where the second 64 columns are
+              const uint32_t a_lo = ((a_addr >> 4) & 0x3fffu) | ((lbo >> 4) << 16);
+              const uint32_t b_lo = kmajor_sw128_desc_lo(pb + (ks >> 2) * C::P_HALF_BYTES + (ks & 3) * 32u);
+              const uint64_t ad = ((uint64_t)KMAJOR_SW128_DESC_HI << 32) | a_lo, bd = ((uint64_t)KMAJOR_SW128_DESC_HI << 32) | b_lo;
+              mma_f16_ss(d_tmem, ad, bd, idesc, acc);
+              acc = 1u;
             }
             touched |= 1u << pair;
             mma_commit(empty + 8 * st);
@@ -328,8 +326,8 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
           // Two weights at a time, packed: exp2 of one fused multiply-add, the high part cut off (exact in the type), the low
           // part rounded.  bf16 keeps 8 bits of a weight, f16 11: with few tokens per sequence that rounding alone reaches 1e-3
           // and 1e-4 of the output, so the remainder goes into a second operand (16 and 22 bits in all).
-          // Measured at 64 heads bf16 over 131072 tokens 41.3 -> 39.3 us (fewer instructions, one more ring stage); f16 pays for its
-          // second chain of products: 68.1 -> 68.7 us (16 x 32768), 77.1 -> 80.6 us (64 x 8192, narrow tiles).
+          // Measured with both parts in one B operand: 64 heads bf16 over 131072 tokens 33.4 us (41.3 with two chains of products and
+          // rounded parts), f16 16 x 32768 66.1 us and 64 x 8192 78 us (68.1 and 77.1 with one f16 part).
           uint32_t hi[4], lo[4];
 #pragma unroll
           for (int u = 0; u < 8; u += 2) {
@@ -379,13 +377,17 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
     for (int pair = (warp - 2) >> 2; pair < n_pairs && n_mine > 0; pair += 2) {
       const int col = pair * 128 + quad * 32 + lane;            // spectral column of this thread's TMEM lane
       const bool used = pair < used_pairs;
-      const uint32_t src = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(pair * N);
+      const uint32_t src = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(pair * C::NB);
 #pragma unroll 1
       for (int n0 = 0; n0 < N; n0 += 16) {                      // sixteen heads at a time
         float val[16];
         if (used) {
+          float low[16];
           tmem_ld16(src + n0, reinterpret_cast<uint32_t*>(val));
+          tmem_ld16(src + N + n0, reinterpret_cast<uint32_t*>(low));
           tmem_ld_wait();
+#pragma unroll
+          for (int n = 0; n < 16; ++n) val[n] += low[n];
         } else {
 #pragma unroll
           for (int n = 0; n < 16; ++n) val[n] = 0.f;
