@@ -101,9 +101,11 @@ struct Layout {
 };
 
 constexpr int GATE_PIECE = 8192;       // tokens per COMPUTE-mode gate piece (logits scratch rows)
-// Queries of one sequence from which the tiled prefill kernels take over from waves of decode passes: a wave rebuilds every key
-// (and shares nothing), the tiled kernels rebuild keys and values once but store both in full width.
-constexpr int PF_MIN_WAVES = 4;
+// Whether the tiled prefill kernels serve a call that would take n_waves decode passes over `rows` tokens.  A wave rebuilds every
+// key (and shares nothing), the tiled kernels rebuild keys and values once but store both in full width.  Microseconds measured
+// with one sequence (8 KV heads, ranks around 256): 1, 2, 3 waves 65, 112, 163 over 1024 tokens, 90, 164, 239 over 32768; tiled,
+// 4 to 8 queries, 80 over 1024, 184 over 8192, 408 over 32768.
+static bool prefill_tiled_pays(int n_waves, double rows) { return n_waves >= 2 && n_waves * (50.0 + rows / 1000.0) >= 75.0 + rows / 100.0; }
 constexpr int GATE_TC_MIN_TOKENS = 1024;   // calls at least this large run the fused tcgen05 gate kernel
 
 struct Offsets {
@@ -538,23 +540,21 @@ twkv_status twkv_decode_attn(twkv_cache* c, int layer, const void* q, const int3
 }
 
 // The tiled form of a prefill call: queries sorted by (sequence, position), dense rows of the visible tokens in segments.
-// `order`: query indices sorted that way.  Sets *done = false, with nothing launched, where the call's tables do not fit the
+// `order`: query indices sorted that way; rows_max: upper bound on the rows.  Sets *done = false, with nothing launched, where the call's tables do not fit the
 // scratch regions they live in (the caller then serves the queries in waves).
 static twkv_status prefill_tiled(twkv_cache* c, int layer, const void* q, const int32_t* q_seq, const int32_t* q_pos, const std::vector<int>& order,
-                                 void* out, cudaStream_t st, bool* done) {
+                                 long long rows_max, void* out, cudaStream_t st, bool* done) {
   const DevView& v = c->view;
   const int n_q = (int)order.size(), QT = TILE / v.rep, pos_end = ROPE_LO * ROPE_HI;
   *done = false;
   std::vector<int> host(2 * (size_t)n_q), blocks, seqs;
-  long long n_words = 0, rows_cap = 0;
-  const long long tmax_rows = (c->cfg.max_tokens_per_seq + TILE - 1) / TILE * (long long)TILE;
+  long long n_words = 0;
   for (int lo = 0; lo < n_q;) {
     int hi = lo;
     while (hi < n_q && q_seq[order[hi]] == q_seq[order[lo]]) ++hi;
     const int u = (int)seqs.size() / 3, maxq = std::min(q_pos[order[hi - 1]], pos_end - 1);
     seqs.push_back(q_seq[order[lo]]); seqs.push_back(maxq); seqs.push_back((int)n_words);
     n_words += (maxq + 32) >> 5;
-    rows_cap += tmax_rows;
     for (int b = lo; b < hi; b += 2 * QT) { blocks.push_back(b); blocks.push_back(u << 9 | std::min(2 * QT, hi - b)); }
     lo = hi;
   }
@@ -582,10 +582,6 @@ static twkv_status prefill_tiled(twkv_cache* c, int layer, const void* q, const 
   a.rowpos = (int*)v.scores;
   a.seg_buf = (unsigned char*)v.gate_scratch;
 
-  // how many rows the sequences can have: their capacity, or what the layer was ever given
-  long long rows_max = rows_cap;
-  if (!c->append_captured.load(std::memory_order_relaxed) && !is_capturing(st))
-    rows_max = std::min(rows_max, c->appended[layer].load(std::memory_order_relaxed) + (TILE - 1) * (long long)n_u);
   if (rows_max > 32767ll * (GATE_PIECE / 2)) return TWKV_OK;         // a tile's segments are kept in two 16-bit halves
   // Segments of 8192 rows with the partial results in the V pass's region, or of 4096 rows with them in the second half of
   // the gate scratch (fewer heads leave the first region small); splits of a segment's rows where the blocks of queries
@@ -655,14 +651,19 @@ twkv_status twkv_prefill_attn(twkv_cache* c, int layer, const void* q, const int
   DeviceGuard g(c->device);
   if (!g.ok) return TWKV_ERR_CUDA;
   cudaStream_t st = (cudaStream_t)stream;
-  if (n_waves >= PF_MIN_WAVES) {
+  // how many rows (tokens, a sequence's rounded up to whole tiles) the sequences can have: their capacity, or what the layer was
+  // ever given
+  long long rows_max = n_distinct * ((c->cfg.max_tokens_per_seq + TILE - 1) / TILE * (long long)TILE);
+  if (!c->append_captured.load(std::memory_order_relaxed) && !is_capturing(st))
+    rows_max = std::min(rows_max, c->appended[layer].load(std::memory_order_relaxed) + (TILE - 1) * (long long)n_distinct);
+  if (prefill_tiled_pays(n_waves, (double)rows_max)) {
     ProfBind pb(&c->prof);
     std::vector<int> order(n_q);
     for (int i = 0; i < n_q; ++i) order[i] = i;
     if (!sorted)
       std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return q_seq[x] != q_seq[y] ? q_seq[x] < q_seq[y] : q_pos[x] < q_pos[y]; });
     bool done = false;
-    const twkv_status s = prefill_tiled(c, layer, q, q_seq, q_pos, order, out, st, &done);
+    const twkv_status s = prefill_tiled(c, layer, q, q_seq, q_pos, order, rows_max, out, st, &done);
     if (done || s != TWKV_OK) return s;
   }
   std::vector<int> wave_start(n_waves + 1, 0), fill(n_waves, 0);
