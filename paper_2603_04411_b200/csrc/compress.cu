@@ -6,6 +6,7 @@
 // Slot assignment is a function of the token order only (no atomics decide placement), so the
 // packed bytes and tables are reproducible.
 #include "twkv_dev.h"
+#include "scan_util.cuh"
 
 namespace twkv {
 
@@ -145,7 +146,7 @@ __device__ __forceinline__ int ceil_div(int a, int b) { return (a + b - 1) / b; 
 __global__ void __launch_bounds__(1024) alloc_kernel(DevView v0, int layer, int n_pieces, const int* __restrict__ seq_ids,
                                                      const int* __restrict__ positions, const unsigned short* __restrict__ levels,
                                                      int count_tok) {
-  __shared__ int s_scan[3][1024];
+  __shared__ int s_warp[32];
   __shared__ int s_fail;
   const int tid = threadIdx.x;
   const int NK = v0.NK;
@@ -188,16 +189,8 @@ __global__ void __launch_bounds__(1024) alloc_kernel(DevView v0, int layer, int 
       if (k < half) sum_tk += nnew; else sum_tv += nnew;
       sum_b += nnew * (k % v.NC + 1);
     }
-    s_scan[0][tid] = sum_tk; s_scan[1][tid] = sum_tv; s_scan[2][tid] = sum_b;
-    __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {                 // inclusive Hillis-Steele scan
-      int a = 0, b = 0, c = 0;
-      if (tid >= o) { a = s_scan[0][tid - o]; b = s_scan[1][tid - o]; c = s_scan[2][tid - o]; }
-      __syncthreads();
-      s_scan[0][tid] += a; s_scan[1][tid] += b; s_scan[2][tid] += c;
-      __syncthreads();
-    }
-    const int tot_tk = s_scan[0][1023], tot_tv = s_scan[1][1023], tot_b = s_scan[2][1023];
+    int tot_tk, tot_tv, tot_b;
+    int off_tk = block_scan_excl(sum_tk, s_warp, &tot_tk), off_tv = block_scan_excl(sum_tv, s_warp, &tot_tv), off_b = block_scan_excl(sum_b, s_warp, &tot_b);
     const int next_block = v.status[1];
     const int ntk = ntiles[0], ntv = ntiles[1];
     // capacity: tokens per sequence
@@ -220,7 +213,6 @@ __global__ void __launch_bounds__(1024) alloc_kernel(DevView v0, int layer, int 
       continue;
     }
     // commit
-    int off_tk = s_scan[0][tid] - sum_tk, off_tv = s_scan[1][tid] - sum_tv, off_b = s_scan[2][tid] - sum_b;
     for (int k = k0; k < k1; ++k) {
       const int cnt = v.key_cnt[k], old = v.key_old_fill[k];
       const int side = k >= half ? 1 : 0;
