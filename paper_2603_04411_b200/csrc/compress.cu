@@ -17,8 +17,10 @@ namespace twkv {
 //   r = #{i : m_i > tau} = d - #{n : c_n <= tau} (Eq. 8).
 // The comparison c_n <= tau is done as S_n <= tau * S_d on the unnormalised sums.
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) gate_rank_kernel(const float* __restrict__ logits, unsigned short* __restrict__ levels,
-                                                        int n_rows, int d, float tau, int* status) {
+__global__ void __launch_bounds__(256) gate_rank_kernel(const float* logits, unsigned short* levels, int n_rows, int d, float tau,
+                                                        int* status) {
+  chain_start();
+  chain_wait();
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (warp >= n_rows) return;
@@ -70,9 +72,10 @@ cudaError_t launch_gate_rank(const DevView& v, const float* logits, unsigned sho
   const int rows = n_tok * 2;
   if (rows == 0) return cudaSuccess;
   const int blocks = (rows + 7) / 8;
-  { ProfScope ps(TWKV_K_GATE_RANK, st); gate_rank_kernel<<<blocks, 256, 0, st>>>(logits, levels, rows, v.d_kv, v.tau, v.status); }
+  cudaError_t e;
+  { ProfScope ps(TWKV_K_GATE_RANK, st); e = launch_chained(gate_rank_kernel, dim3(blocks), dim3(256), dim3(1), 0, st, logits, levels, rows, v.d_kv, v.tau, v.status); }
   count_launch();
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // ------------------------------------------------------------------------------------------
@@ -111,6 +114,8 @@ __global__ void __launch_bounds__(CHUNK_TOKENS) hist_kernel(DevView v0, const in
 // Warp per key: the key's per-chunk counts (contiguous, [key][chunk]) become exclusive bases, their sum the key's count.
 // grid: one warp per (piece, key); total_chunks counts the chunks of all pieces of the launch group
 __global__ void __launch_bounds__(256) scan_kernel(DevView v0, int n_pieces, int total_chunks) {
+  chain_start();
+  chain_wait();
   const int widx = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (widx >= v0.NK * n_pieces) return;
   const int piece = widx / v0.NK, key = widx - piece * v0.NK;
@@ -143,9 +148,10 @@ __device__ __forceinline__ int ceil_div(int a, int b) { return (a + b - 1) / b; 
 // token) is refused whole and the later pieces carry on from the unchanged tables.
 // A call of at most one chunk (the decode-time append) skips the histogram and scan launches: `count_tok` > 0 makes
 // this kernel count the call's tokens per key itself (one piece, one chunk, so every per-chunk base is 0).
-__global__ void __launch_bounds__(1024) alloc_kernel(DevView v0, int layer, int n_pieces, const int* __restrict__ seq_ids,
-                                                     const int* __restrict__ positions, const unsigned short* __restrict__ levels,
-                                                     int count_tok) {
+__global__ void __launch_bounds__(1024) alloc_kernel(DevView v0, int layer, int n_pieces, const int* seq_ids, const int* positions,
+                                                     const unsigned short* levels, int count_tok) {
+  chain_start();
+  chain_wait();
   __shared__ int s_warp[32];
   __shared__ int s_fail;
   const int tid = threadIdx.x;
@@ -307,9 +313,10 @@ struct Place { int base, slot_cls_r; };   // slot | cls << 8 | r << 16
 // each (part 0 writes the tables): what bounds a small call is the round trips that one CTA's 128 threads need for a chunk's
 // up to 512 KiB.  1024 tokens 36.0 -> 9.3 us, 9 x 1777 ragged 28.0 -> 14.2, an append of 64 tokens 18.5 -> 11.4; 524288 tokens
 // (one part each) 214.6 before and after.
-__global__ void __launch_bounds__(CHUNK_TOKENS, 7) pack_kernel(DevView v0, int layer, const void* __restrict__ K, const void* __restrict__ V,
-                                                            const int* __restrict__ seq_ids, const int* __restrict__ positions,
-                                                            const unsigned short* __restrict__ levels, int n_tok, int parts) {
+__global__ void __launch_bounds__(CHUNK_TOKENS, 7) pack_kernel(DevView v0, int layer, const void* K, const void* V, const int* seq_ids, const int* positions,
+                                                            const unsigned short* levels, int n_tok, int parts) {
+  chain_start();
+  chain_wait();
   const int n_chunks = (n_tok + CHUNK_TOKENS - 1) / CHUNK_TOKENS;
   const int bid = blockIdx.x / parts, part = blockIdx.x - bid * parts;      // of a token CTA
   const int tail = (int)blockIdx.x - n_chunks * parts;                        // >= 0: a tail CTA
@@ -456,8 +463,8 @@ __global__ void __launch_bounds__(CHUNK_TOKENS, 7) pack_kernel(DevView v0, int l
         const int slot = p.slot_cls_r & 0xff, rr = p.slot_cls_r >> 16;
         keep[u] = rr - j * 8;
         if (keep[u] > 0)
-          val[u] = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const unsigned char*>(side ? V : K) +
-                                                        (size_t)(bid * CHUNK_TOKENS + t) * row_bytes) + j);
+          val[u] = reinterpret_cast<const uint4*>(reinterpret_cast<const unsigned char*>(side ? V : K) +
+                                                  (size_t)(bid * CHUNK_TOKENS + t) * row_bytes)[j];
         dst[u] = v.blocks + (size_t)(p.base + (j >> 3)) * BLOCK_BYTES + slot * (PANEL * 2) + (j & 7) * 16;
       }
     }
@@ -487,6 +494,7 @@ cudaError_t launch_compress_pieces(const DevView& v, int layer, const void* K, c
   const int n_chunks = (n_tok + CHUNK_TOKENS - 1) / CHUNK_TOKENS;
   const int n_pieces = (n_chunks + PIECE_CHUNKS - 1) / PIECE_CHUNKS;
   // CTAs per chunk: enough that a small call fills the device once (7 CTAs per SM), never more than a chunk has rounds of loads
+  cudaError_t e = cudaSuccess;
   int parts = 1, sms = 148;
   {
     int dev = 0;
@@ -497,23 +505,36 @@ cudaError_t launch_compress_pieces(const DevView& v, int layer, const void* K, c
   // scan_kernel reads the counts four at a time; a launch group of several pieces clears its tables whole
   if (n_chunks == 1) {
     // decode-time append: the allocator counts the tokens itself, two launches in all
-    { ProfScope ps(TWKV_K_ALLOC, st); alloc_kernel<<<1, 1024, 0, st>>>(v, layer, 1, seq_ids, positions, levels, n_tok); }
-    { ProfScope ps(TWKV_K_PACK, st); pack_kernel<<<parts + v.NK, CHUNK_TOKENS, 0, st>>>(v, layer, K, V, seq_ids, positions, levels, n_tok, parts); }
+    { ProfScope ps(TWKV_K_ALLOC, st); e = launch_chained(alloc_kernel, dim3(1), dim3(1024), dim3(1), 0, st, v, layer, 1, seq_ids, positions, levels, n_tok); }
+    if (e != cudaSuccess) return e;
+    {
+      ProfScope ps(TWKV_K_PACK, st);
+      e = launch_chained(pack_kernel, dim3(parts + v.NK), dim3(CHUNK_TOKENS), dim3(1), 0, st, v, layer, K, V, seq_ids, positions, levels, n_tok, parts);
+    }
+    if (e != cudaSuccess) return e;
     count_launch(2);
     return cudaGetLastError();
   }
   const int n_cols = n_pieces > 1 ? PIECE_CHUNKS : (n_chunks + 3) & ~3;
-  cudaError_t e = cudaMemset2DAsync(v.hist, (size_t)PIECE_CHUNKS * sizeof(int), 0, (size_t)n_cols * sizeof(int), (size_t)v.NK * n_pieces, st);
+  e = cudaMemset2DAsync(v.hist, (size_t)PIECE_CHUNKS * sizeof(int), 0, (size_t)n_cols * sizeof(int), (size_t)v.NK * n_pieces, st);
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(v.pflags, 0, (size_t)v.batch * 2 * sizeof(int), st);
   if (e != cudaSuccess) return e;
   { ProfScope ps(TWKV_K_HIST, st); hist_kernel<<<n_chunks, CHUNK_TOKENS, 0, st>>>(v, seq_ids, positions, levels, n_tok); }
   {
     ProfScope ps(TWKV_K_ALLOC, st);
-    scan_kernel<<<(v.NK * n_pieces + 7) / 8, 256, 0, st>>>(v, n_pieces, n_chunks);
-    alloc_kernel<<<1, 1024, 0, st>>>(v, layer, n_pieces, nullptr, nullptr, nullptr, 0);
+    e = launch_chained(scan_kernel, dim3((v.NK * n_pieces + 7) / 8), dim3(256), dim3(1), 0, st, v, n_pieces, n_chunks);
+    if (e == cudaSuccess)
+      e = launch_chained(alloc_kernel, dim3(1), dim3(1024), dim3(1), 0, st, v, layer, n_pieces, (const int*)nullptr, (const int*)nullptr,
+                         (const unsigned short*)nullptr, 0);
+    if (e != cudaSuccess) return e;
   }
-  { ProfScope ps(TWKV_K_PACK, st); pack_kernel<<<n_chunks * parts + v.NK * n_pieces, CHUNK_TOKENS, 0, st>>>(v, layer, K, V, seq_ids, positions, levels, n_tok, parts); }
+  {
+    ProfScope ps(TWKV_K_PACK, st);
+    e = launch_chained(pack_kernel, dim3(n_chunks * parts + v.NK * n_pieces), dim3(CHUNK_TOKENS), dim3(1), 0, st, v, layer, K, V, seq_ids, positions,
+                       levels, n_tok, parts);
+    if (e != cudaSuccess) return e;
+  }
   count_launch(4);
   return cudaGetLastError();
 }

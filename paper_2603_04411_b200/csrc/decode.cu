@@ -41,7 +41,7 @@ __device__ __forceinline__ unsigned ktile_cost(int cls) {
 // classes 1 to 16 dealt out by count alone left the slowest CTA with half as much again as the mean.
 // The list is taken in the stride order of vtile_stride(); cut[s] = number of tiles (in that order) whose inclusive cost
 // prefix is <= s / n_splits of the total; split s takes positions cut[s] .. cut[s + 1] - 1 of that order.
-__device__ void vsplit_plan(const DevView& v, int layer, const int* __restrict__ seq_ids, int qs, int n_splits) {
+__device__ void vsplit_plan(const DevView& v, int layer, const int* seq_ids, int qs, int n_splits) {
   __shared__ int s_warp[32];
   const int tid = threadIdx.x;
   const int seq = seq_ids[qs];
@@ -85,7 +85,7 @@ __device__ void vsplit_plan(const DevView& v, int layer, const int* __restrict__
 // K slot -> V slot of every token of one sequence (the V slots carry the opposite link): the K-score kernel stores a
 // token's scores at its V slot, so that the V pass finds a tile's score rows next to each other.  CTA j of the vj CTAs of
 // a sequence takes the V tiles j * 8 .. j * 8 + 7, then vj * 8 further on, eight tiles (1024 slots) at a time.
-__device__ void vlink_plan(const DevView& v, int layer, const int* __restrict__ seq_ids, int qs, int j, int vj) {
+__device__ void vlink_plan(const DevView& v, int layer, const int* seq_ids, int qs, int j, int vj) {
   const int seq = seq_ids[qs];
   if (seq < 0 || seq >= v.S) return;
   const int n = v.svc(layer)[seq];
@@ -99,8 +99,10 @@ __device__ void vlink_plan(const DevView& v, int layer, const int* __restrict__ 
   }
 }
 
-__global__ void __launch_bounds__(1024) plan_kernel(DevView v, int layer, const int* __restrict__ seq_ids, int n_seq, int n_cta, int pairs,
+__global__ void __launch_bounds__(1024) plan_kernel(DevView v, int layer, const int* seq_ids, int n_seq, int n_cta, int pairs,
                                                     int n_splits, int vj) {
+  chain_start();
+  chain_wait();
   const int NC = v.NC;
   if ((int)blockIdx.x >= NC + n_seq) {                            // the last n_seq * vj CTAs: K slot -> V slot links
     const int idx = (int)blockIdx.x - NC - n_seq;
@@ -228,12 +230,14 @@ __device__ __forceinline__ float ld_cluster_f32(uint32_t addr) {
 
 template <bool BF16>
 __global__ void __launch_bounds__(MG_THREADS)
-merge_kernel(DevView v, const unsigned short* __restrict__ Uinv_v, int n_splits, int hp, int ns, int n_seq, void* __restrict__ out) {
+merge_kernel(DevView v, const unsigned short* Uinv_v, int n_splits, int hp, int ns, int n_seq, void* out) {
   __shared__ float4 s_part[MG_THREADS];              // split sums per (split group, row, four components)
   __shared__ __align__(16) float s_acc[MG_ROWS * 128];    // [rows][d / 8] normalised
   __shared__ float s_red[4][MG_ROWS][128];
   __shared__ float s_out[MG_ROWS * 128];
   __shared__ float s_invl[MG_ROWS];
+  chain_start();
+  chain_wait();
   // blockIdx.y = KV head g and which hp of its query heads; blockIdx.x / 8 = ns query slots that share the reads of U_V^-1
   const int c = tc::cluster_cta_rank();
   const int qs0 = (blockIdx.x / MG_CL) * ns, parts = v.rep / hp, g = blockIdx.y / parts, tid = threadIdx.x, lane = tid & 31;
@@ -246,7 +250,7 @@ merge_kernel(DevView v, const unsigned short* __restrict__ Uinv_v, int n_splits,
   const unsigned* ucol = reinterpret_cast<const unsigned*>(Uinv_v + (size_t)(j0 + jg * jr) * d_kv + g * HEAD_DIM) + dp;
   unsigned u[32];
 #pragma unroll
-  for (int t = 0; t < 32; ++t) u[t] = t < jr ? __ldg(ucol + (size_t)t * (d_kv / 2)) : 0u;
+  for (int t = 0; t < 32; ++t) u[t] = t < jr ? ucol[(size_t)t * (d_kv / 2)] : 0u;
   // row sums over the splits: warp w takes row w, its lanes read the splits' parts together, lane 0 adds them in split order
   if ((tid >> 5) < rows) {
     const int r = tid >> 5, qs = qs0 + r / hp, head = head0 + r % hp;
@@ -271,7 +275,7 @@ merge_kernel(DevView v, const unsigned short* __restrict__ Uinv_v, int n_splits,
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
         const int s = s0 + k * sg_n;
-        t[k] = s < n_splits && cut[s + 1] > cut[s] ? __ldg(p + (size_t)s * stride) : make_float4(0.f, 0.f, 0.f, 0.f);
+        t[k] = s < n_splits && cut[s + 1] > cut[s] ? p[(size_t)s * stride] : make_float4(0.f, 0.f, 0.f, 0.f);
       }
 #pragma unroll
       for (int k = 0; k < 8; ++k) { a.x += t[k].x; a.y += t[k].y; a.z += t[k].z; a.w += t[k].w; }
@@ -339,19 +343,21 @@ constexpr int MW_SMEM = 128 * 128 * 2 + 2 * MW_ROWS * 128 * 4 + MW_ROWS * 4;
 
 template <bool BF16>
 __global__ void __launch_bounds__(MG_THREADS)
-merge_wide_kernel(DevView v, const unsigned short* __restrict__ Uinv_v, int n_splits, int n_seq, void* __restrict__ out) {
+merge_wide_kernel(DevView v, const unsigned short* Uinv_v, int n_splits, int n_seq, void* out) {
   extern __shared__ __align__(16) unsigned char mw_smem[];
   unsigned* s_u = reinterpret_cast<unsigned*>(mw_smem);                                // [d / 8][64] pairs of columns
   float* s_acc = reinterpret_cast<float*>(mw_smem + 128 * 128 * 2);                    // [rows][d / 8]
   float* s_out = s_acc + MW_ROWS * 128;                                                // [rows][128]
   float* s_invl = s_out + MW_ROWS * 128;
+  chain_start();
+  chain_wait();
   const int c = tc::cluster_cta_rank(), g = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int ns = MW_ROWS / v.rep, qs0 = (blockIdx.x / MG_CL) * ns;
   const int Hq = v.Hq, d_kv = v.d_kv, rep = v.rep;
   const int rows = min(ns, n_seq - qs0) * rep;
   const int jn = d_kv / MG_CL, j0 = c * jn;
   for (int i = tid; i < jn * 16; i += MG_THREADS) {                                    // 16-byte pieces of this CTA's rows of U_V^-1
-    const uint4 w = __ldg(reinterpret_cast<const uint4*>(Uinv_v + (size_t)(j0 + (i >> 4)) * d_kv + g * HEAD_DIM) + (i & 15));
+    const uint4 w = reinterpret_cast<const uint4*>(Uinv_v + (size_t)(j0 + (i >> 4)) * d_kv + g * HEAD_DIM)[i & 15];
     reinterpret_cast<uint4*>(s_u)[i] = w;
   }
   for (int r = warp; r < rows; r += MG_THREADS / 32) {
@@ -376,7 +382,7 @@ merge_wide_kernel(DevView v, const unsigned short* __restrict__ Uinv_v, int n_sp
       float4 t[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k)
-        t[k] = s0 + k < n_splits && cut[s0 + k + 1] > cut[s0 + k] ? __ldg(p + (size_t)(s0 + k) * stride) : make_float4(0.f, 0.f, 0.f, 0.f);
+        t[k] = s0 + k < n_splits && cut[s0 + k + 1] > cut[s0 + k] ? p[(size_t)(s0 + k) * stride] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int k = 0; k < 4; ++k) { a.x += t[k].x; a.y += t[k].y; a.z += t[k].z; a.w += t[k].w; }
     }
@@ -438,7 +444,12 @@ static cudaError_t launch_decode_t(const DevView& v, int layer, const LayerParam
   const int n_pieces = pairs ? kscore_max_pairs(sm_count) : sm_count;
   // CTAs per sequence that invert the V -> K links: enough of them that they finish inside the K work list's time
   const int vj = n_seq >= 256 ? 1 : (256 / n_seq > 64 ? 64 : 256 / n_seq);
-  { ProfScope ps(TWKV_K_PLAN, st); plan_kernel<<<v.NC + n_seq + n_seq * vj, 1024, (size_t)v.S * sizeof(int), st>>>(v, layer, seq_ids, n_seq, n_pieces, pairs ? 1 : 0, n_splits, vj); }
+  {
+    ProfScope ps(TWKV_K_PLAN, st);
+    cudaError_t e = launch_chained(plan_kernel, dim3(v.NC + n_seq + n_seq * vj), dim3(1024), dim3(1), (size_t)v.S * sizeof(int), st, v, layer, seq_ids,
+                                   n_seq, n_pieces, pairs ? 1 : 0, n_splits, vj);
+    if (e != cudaSuccess) return e;
+  }
   {
     cudaError_t e = launch_kscore_tc(v, layer, maps->blocks, maps->uinvT_k, q, n_pieces, pairs, st);
     if (e != cudaSuccess) return e;
@@ -450,31 +461,21 @@ static cudaError_t launch_decode_t(const DevView& v, int layer, const LayerParam
   }
   {
     ProfScope ps(TWKV_K_MERGE, st);
-    cudaLaunchConfig_t cfg = {};
-    cfg.blockDim = dim3(MG_THREADS);
-    cfg.stream = st;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = MG_CL; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
     const unsigned short* uv = reinterpret_cast<const unsigned short*>(lp.Uinv_v);
     const int wide = (n_seq * v.rep + MW_ROWS - 1) / MW_ROWS;
     cudaError_t e;
     if (MG_CL * wide * v.Hkv >= 2 * sm_count) {
       // 32 rows per cluster while that still makes two CTAs per SM
-      cfg.gridDim = dim3(MG_CL * wide, v.Hkv);
-      cfg.dynamicSmemBytes = MW_SMEM;
       e = cudaFuncSetAttribute(merge_wide_kernel<BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, MW_SMEM);
-      if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, merge_wide_kernel<BF16>, v, uv, n_splits, n_seq, out);
+      if (e == cudaSuccess) e = launch_chained(merge_wide_kernel<BF16>, dim3(MG_CL * wide, v.Hkv), dim3(MG_THREADS), dim3(MG_CL), MW_SMEM, st, v, uv, n_splits, n_seq, out);
     } else {
       // query heads per cluster: the whole group, fewer (a divisor) while there are less than two CTAs per SM; then query
       // slots per cluster (they share the reads of U_V^-1) while there are more
       int hp = v.rep, ns = 1;
       while (hp % 2 == 0 && MG_CL * n_seq * v.Hkv * (v.rep / hp) < 2 * sm_count) hp /= 2;
       while (2 * ns * hp <= MG_ROWS && MG_CL * (n_seq * v.Hkv * (v.rep / hp) / (2 * ns)) >= 2 * sm_count) ns *= 2;
-      cfg.gridDim = dim3(MG_CL * ((n_seq + ns - 1) / ns), v.Hkv * (v.rep / hp));
-      e = cudaLaunchKernelEx(&cfg, merge_kernel<BF16>, v, uv, n_splits, hp, ns, n_seq, out);
+      e = launch_chained(merge_kernel<BF16>, dim3(MG_CL * ((n_seq + ns - 1) / ns), v.Hkv * (v.rep / hp)), dim3(MG_THREADS), dim3(MG_CL), 0, st, v, uv,
+                         n_splits, hp, ns, n_seq, out);
     }
     if (e != cudaSuccess) return e;
   }

@@ -15,9 +15,10 @@ constexpr int GG_THREADS = 256;
 
 template <bool BF16>
 __global__ void __launch_bounds__(GG_THREADS, 1)
-gate_gemm_kernel(const unsigned short* __restrict__ Xk, const unsigned short* __restrict__ Xv,
-                 const unsigned short* __restrict__ Wk, const unsigned short* __restrict__ Wv,
-                 const float* __restrict__ bk, const float* __restrict__ bv, int n_tok, int d, int ks_n, float* __restrict__ Z) {
+gate_gemm_kernel(const unsigned short* Xk, const unsigned short* Xv, const unsigned short* Wk, const unsigned short* Wv, const float* bk,
+                 const float* bv, int n_tok, int d, int ks_n, float* Z) {
+  chain_start();
+  chain_wait();
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned char* sA = smem;
   unsigned char* sB = smem + GG_STAGES * 16384;
@@ -123,20 +124,11 @@ cudaError_t launch_gate_logits(const DevView& v, const LayerParams& lp, const vo
   while (ks > 1 && ((v.d_kv / 64) % ks || tiles * ks > 296)) ks /= 2;
   ProfScope ps(TWKV_K_GATE_GEMM, st);
   auto X = [](const void* p) { return reinterpret_cast<const unsigned short*>(p); };
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((n_tok + 127) / 128, v.d_kv / 128, 2 * ks);
-  cfg.blockDim = dim3(GG_THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = 1; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = ks;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
   auto kernel = v.dtype == TWKV_BF16 ? gate_gemm_kernel<true> : gate_gemm_kernel<false>;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess)
-    e = cudaLaunchKernelEx(&cfg, kernel, X(K), X(V), X(lp.W_k), X(lp.W_v), lp.b_k, lp.b_v, n_tok, v.d_kv, ks, logits);
+    e = launch_chained(kernel, dim3((n_tok + 127) / 128, v.d_kv / 128, 2 * ks), dim3(GG_THREADS), dim3(1, 1, ks), smem, st, X(K), X(V), X(lp.W_k),
+                       X(lp.W_v), lp.b_k, lp.b_v, n_tok, v.d_kv, ks, logits);
   if (e != cudaSuccess) return e;
   count_launch();
   return cudaGetLastError();

@@ -97,7 +97,8 @@ constexpr int KE_DISCARD = 0x80;                               // list entry, .y
 template <bool BF16, int REP, bool PAIR, bool DBG>
 __global__ void __launch_bounds__(KT_THREADS, 1)
 kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_constant__ CUtensorMap map_uinvT,
-                 DevView v, int layer, const unsigned short* __restrict__ q, int nb) {
+                 DevView v, int layer, const unsigned short* q, int nb) {
+  chain_start();
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   constexpr int CG = PAIR ? 2 : 1;
   // a ring stage of U_K^-1 holds two consecutive panels of one KV head (their halves in a pair CTA): one barrier wait
@@ -142,6 +143,7 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
   }
   for (int i = tid; i < 2 * (int)KT_Q_PANEL_BYTES / 16; i += KT_THREADS)        // padding rows of the query operand stay zero
     reinterpret_cast<uint4*>(sQ_ptr)[i] = make_uint4(0u, 0u, 0u, 0u);
+  chain_wait();
   for (int i = tid; i < ROPE_LO * 32; i += KT_THREADS) sRope[(i >> 5) * KT_ROPE_STRIDE + (i & 31)] = v.rope_lo[i];
   fence_proxy_async_smem();
   fence_before_sync();
@@ -645,23 +647,14 @@ static cudaError_t launch_kscore_tc_t(const DevView& v, int layer, const CUtenso
   const int nb = PAIR ? KT_NB_PAIR : KT_NB_SINGLE;
   const size_t smem = kscore_tc_smem_bytes(nb, PAIR ? PANEL_BYTES : 2 * PANEL_BYTES);
   const unsigned short* qq = reinterpret_cast<const unsigned short*>(q);
-  cudaLaunchConfig_t cfg = {};
-  cfg.blockDim = dim3(KT_THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cfg.gridDim = dim3(PAIR ? 2 * n_pieces : n_pieces);
-  cudaLaunchAttribute pair_attr;
-  pair_attr.id = cudaLaunchAttributeClusterDimension;
-  pair_attr.val.clusterDim.x = 2; pair_attr.val.clusterDim.y = 1; pair_attr.val.clusterDim.z = 1;
-  cfg.attrs = PAIR ? &pair_attr : nullptr;
-  cfg.numAttrs = PAIR ? 1 : 0;
   ProfScope ps(TWKV_K_KSCORE, st);
   cudaError_t e = cudaSuccess;
 #define TWKV_KT(REP)                                                                                                  \
   {                                                                                                                   \
     e = cudaFuncSetAttribute(kscore_tc_kernel<BF16, REP, PAIR, DBG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
     if (e != cudaSuccess) return e;                                                                                   \
-    e = cudaLaunchKernelEx(&cfg, kscore_tc_kernel<BF16, REP, PAIR, DBG>, map_blocks, map_uinvT, v, layer, qq, nb);        \
+    e = launch_chained(kscore_tc_kernel<BF16, REP, PAIR, DBG>, dim3(PAIR ? 2 * n_pieces : n_pieces), dim3(KT_THREADS),   \
+                       dim3(PAIR ? 2 : 1), smem, st, map_blocks, map_uinvT, v, layer, qq, nb);                         \
   }
   switch (v.rep) {
     case 1: TWKV_KT(1) break;

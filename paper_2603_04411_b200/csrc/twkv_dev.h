@@ -146,6 +146,29 @@ struct DeviceGuard {
   int target = -1;
 };
 
+// Programmatic dependent launch: the small kernels of an append or a decode pass follow one another, and each would wait for the
+// last CTA of the one before to leave before its own launch and set-up begin.  A kernel launched with launch_chained() may start
+// while the kernel before it still runs: it calls chain_start() first (the next kernel may be launched once all of its CTAs
+// have) and chain_wait() before it reads or writes any memory another kernel touches; chain_wait() returns when the kernel
+// before has completed.  Every CTA of a chained kernel waits, so that completion passes down the chain.  Such a kernel reads
+// nothing through the read-only path that an earlier kernel may have written (no __restrict__, no __ldg): those loads could
+// be moved before the wait.
+__device__ __forceinline__ void chain_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, dim3 cluster, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster.x; attr[1].val.clusterDim.y = cluster.y; attr[1].val.clusterDim.z = cluster.z;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster.x * cluster.y * cluster.z > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // launch bookkeeping (host)
 void count_launch(int n = 1);
 // optional per-kernel event timing of the cache whose API call is running on this thread

@@ -86,7 +86,8 @@ __host__ __device__ constexpr uint32_t vt_idesc(int fmt, int n) { return idesc_f
 template <bool BF16, int N, bool TS>
 __global__ void __launch_bounds__(VT_THREADS, 1)
 vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_constant__ CUtensorMap map_scores, DevView v, int layer,
-               const int* __restrict__ seq_ids, int n_splits) {
+               const int* seq_ids, int n_splits) {
+  chain_start();
   using C = VtCfg<BF16, N>;
   constexpr int S = C::STAGES, ITEMS = C::ITEMS;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -95,18 +96,7 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
   const int qs = blockIdx.x / n_splits, split = blockIdx.x - qs * n_splits;
   const int h0 = blockIdx.y * N, nh = min(N, Hq - h0);
   const int NB = min(N, Hq);                                    // heads per score row in shared memory (TS: the box's width)
-  const int seq = seq_ids[qs];
-  const bool seq_ok = seq >= 0 && seq < v.S;
-  // this split's range of the sequence's V tile list in stride order, cut by plan_kernel to equal cost; an id outside
-  // the cache has no tiles and contributes nothing: zero partials
-  const int* cut = v.vcut + (size_t)qs * (n_splits + 1) + split;
-  const int t_first = cut[0], n_mine = seq_ok ? cut[1] - t_first : 0;
-  const int n_tiles = seq_ok ? v.svc(layer)[seq] : 0;
-  const int t_stride = vtile_stride(n_tiles);
-  const int* list = v.svt(layer) + (size_t)(seq_ok ? seq : 0) * v.TPS;
-  const int4* desc = v.desc(layer, 1);
-
-  // shared memory: ring | zero block | probabilities [2 buffers][PARTS][2 halves][N][128 B] | score ring | descriptors | row sums | barriers
+  // shared memory: ring | zero block | probabilities [2 buffers][2 halves][2 N][128 B] | score ring | descriptors | row sums | barriers
   const uint32_t s0 = smem_addr(smem_raw);
   const uint32_t pad = (1024u - (s0 & 1023u)) & 1023u;          // operand tiles need 1024-byte alignment for the swizzle
   unsigned char* base_ptr = smem_raw + pad;
@@ -145,6 +135,18 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
   __syncthreads();
   fence_after_sync();
   const uint32_t tmem_base = *s_tmem_base;
+
+  chain_wait();
+  const int seq = seq_ids[qs];
+  const bool seq_ok = seq >= 0 && seq < v.S;
+  // this split's range of the sequence's V tile list in stride order, cut by plan_kernel to equal cost; an id outside
+  // the cache has no tiles and contributes nothing: zero partials
+  const int* cut = v.vcut + (size_t)qs * (n_splits + 1) + split;
+  const int t_first = cut[0], n_mine = seq_ok ? cut[1] - t_first : 0;
+  const int n_tiles = seq_ok ? v.svc(layer)[seq] : 0;
+  const int t_stride = vtile_stride(n_tiles);
+  const int* list = v.svt(layer) + (size_t)(seq_ok ? seq : 0) * v.TPS;
+  const int4* desc = v.desc(layer, 1);
 
   // role state that survives the descriptor chunks
   uint32_t st = 0, st_ph = 0;                                   // producer / issuer: ring stage and its phase
@@ -423,8 +425,8 @@ static cudaError_t launch_vacc_tc_n(const DevView& v, int layer, const CUtensorM
   cudaError_t e = cudaFuncSetAttribute(vacc_tc_kernel<BF16, N, TS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM_BYTES);
   if (e != cudaSuccess) return e;
   const dim3 grid(n_seq * n_splits, (v.Hq + N - 1) / N);
-  vacc_tc_kernel<BF16, N, TS><<<grid, VT_THREADS, C::SMEM_BYTES, st>>>(map_blocks, map_scores, v, layer, seq_ids, n_splits);
-  return cudaGetLastError();
+  e = launch_chained(vacc_tc_kernel<BF16, N, TS>, grid, dim3(VT_THREADS), dim3(1), C::SMEM_BYTES, st, map_blocks, map_scores, v, layer, seq_ids, n_splits);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // map_scores: the score scratch as a tensor map (boxes of 128 rows x min(N, Hq) heads), or null: rows copied with cp.async.
