@@ -162,11 +162,13 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
   const int4 kt_none = make_int4(0, 0, 0, -1);
   // A work unit is one of the `hg` parts of a list item: all its panels, nh of the KV heads (hg > 1 only for short lists,
   // where one item per CTA would leave most SMs idle and run through all heads one after the other).
-  const int hg = *v.kitem_parts, nh = Hkv / hg;
-  auto unit = [&](int w) -> int4 { return w < total ? klist[KSTEP * (w / hg)] : kt_none; };
+  // (hg is a power of two; the single-thread roles pay for every instruction of theirs, so no divisions here)
+  const int hs = __ffs(*v.kitem_parts) - 1, nh = Hkv >> hs;
+  auto unit = [&](int w) -> int4 { return w < total ? klist[KSTEP * (w >> hs)] : kt_none; };
   // CTAs walk the KV heads in rotated order, so that at any moment they read different panels of U_K^-1 from L2
   const int g_rot = piece % nh;
-  auto head = [&](int w, int sl) -> int { return (w % hg) * nh + (sl + g_rot < nh ? sl + g_rot : sl + g_rot - nh); };
+  auto first_head = [&](int w) -> int { return (w & ((1 << hs) - 1)) * nh; };
+  auto head = [&](int g0, int sl) -> int { return g0 + (sl + g_rot < nh ? sl + g_rot : sl + g_rot - nh); };
 
   if (misaligned) {
     // nothing was started; fall through to the common exit
@@ -212,10 +214,11 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
       for (int w = w0; w < total && ok; ++w) {
         const int4 nxt = unit(w + 1);
         const int cls = e.y & 0x7f;
+        const int g0 = first_head(w);
         for (int p0 = 0; p0 < cls && ok; p0 += KT_A_SLOTS) {
           const int np = min(KT_A_SLOTS, cls - p0);
           for (int sl = 0; sl < nh && ok; ++sl) {
-            const int g = head(w, sl);
+            const int g = head(g0, sl);
             for (int j = 0; j < np; j += 2, ++bk) {
               const uint32_t st = bst, ph = bph;
               if (++bst == (uint32_t)nb) { bst = 0; bph ^= 1u; }
@@ -308,9 +311,10 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
       for (int w = w0; w < total && ok; ++w) {
         const int4 nxt = unit(w + 1);
         const int cls = e.y & 0x7f;
+        const int g0 = first_head(w);
         for (int p0 = 0; p0 < cls && ok; p0 += KT_A_SLOTS) {
           for (int sl = 0; sl < nh; ++sl) {
-            const int g = head(w, sl);
+            const int g = head(g0, sl);
             if (!(ok = mbar_wait_thin(kr_full + 8 * sbuf, sph, abort_flag))) break;
             if (!(ok = mbar_wait_thin(s_empty + 8 * slot, slph ^ 1u, abort_flag))) break;
             fence_after_sync();
@@ -490,6 +494,7 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
     for (int w = w0; w < total && ok; ++w) {
       const int4 nxt = unit(w + 1);
       const int cls = e.y & 0x7f, n_valid = e.y >> 8, qs = e.w;
+      const int g0 = first_head(w);
       const bool discard = (e.y & KE_DISCARD) != 0;
       const int passes = (cls + KT_A_SLOTS - 1) / KT_A_SLOTS;
       const int pos_next = nxt.w >= 0 ? kpos[(size_t)nxt.x * TILE + row] : 0;
@@ -502,7 +507,7 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
       for (int ps = 0; ps < passes && ok; ++ps) {
         const uint32_t mode = discard ? KP_DISCARD : passes == 1 ? KP_STORE_FINAL : (ps == 0 ? KP_STORE_PART : KP_ADD_FINAL);
         for (int sli = 0; sli < nh; ++sli) {
-          const int g = head(w, sli);
+          const int g = head(g0, sli);
           if (!(ok = __all_sync(0xffffffffu, mbar_wait(s_full + 8 * slot, slph, abort_flag)))) break;
           fence_after_sync();
           float sv[REP];
