@@ -61,13 +61,12 @@ __device__ __forceinline__ float2 unpack_f16x2(uint32_t v) {
   return r;
 }
 
-// One row decided again in fp32 by a whole warp (Eq. 5, 6, 8 for the 32 logits of the block in which the cumulative
-// sum crosses tau): every logit is a dot product over d spread across the lanes (coalesced reads of the transposed
-// weights, butterfly sum), the terms exp(z - M) continue the cumulative sum from `base`, the block summaries before
-// the crossing block having been taken in fp32 already.
-__device__ __forceinline__ void gate_redo_row(const GateRaw& raw, int bf16, int d, const float* __restrict__ bias_k,
-                                              const float* __restrict__ bias_v, int side, int row, int b_s, float base, float thr,
-                                              float M, unsigned short* __restrict__ levels, int lane) {
+// One row decided again in fp32 (Eq. 5, 6, 8 for the 32 logits of the block in which the cumulative sum crosses tau), in two
+// steps for a whole warp each.  gate_redo_logits: logits j0 .. j1-1 of the block (multiples of four), each a dot product over d
+// spread across the lanes (coalesced reads of the transposed weights, butterfly sum); lane j ends with logit j, without the
+// bias.  gate_redo_finish: the terms exp(z - M) continue the cumulative sum from `base`, the block summaries before the
+// crossing block having been taken in fp32 already.
+__device__ __forceinline__ float gate_redo_logits(const GateRaw& raw, int bf16, int d, int side, int row, int b_s, int first, int j1, int lane) {
   const int n16 = d >> 3;                                      // 16-byte pieces per row; lane takes pieces lane, lane + 32, ...
   auto widen = [&](const uint4 q, float* f) {
     const uint32_t w4[4] = {q.x, q.y, q.z, q.w};
@@ -86,7 +85,7 @@ __device__ __forceinline__ void gate_redo_row(const GateRaw& raw, int bf16, int 
   const unsigned short* wbase = (side ? raw.wvT : raw.wkT) + (size_t)(b_s * 32) * d;
   float z = 0.f;
 #pragma unroll 1
-  for (int j0 = 0; j0 < 32; j0 += 4) {
+  for (int j0 = first; j0 < j1; j0 += 4) {
     uint4 wq[4][4];
 #pragma unroll
     for (int jj = 0; jj < 4; ++jj) {
@@ -109,6 +108,10 @@ __device__ __forceinline__ void gate_redo_row(const GateRaw& raw, int bf16, int 
       if (lane == j0 + jj) z = acc;
     }
   }
+  return z;
+}
+__device__ __forceinline__ void gate_redo_finish(float z, int d, const float* __restrict__ bias_k, const float* __restrict__ bias_v, int side,
+                                                 int row, int b_s, float base, float thr, float M, unsigned short* __restrict__ levels, int lane) {
   const float* bias = side ? bias_v : bias_k;
   if (bias) z += __ldg(bias + b_s * 32 + lane);
   float incl = __expf(z - M);
@@ -125,19 +128,33 @@ __device__ __forceinline__ void gate_redo_row(const GateRaw& raw, int bf16, int 
   }
 }
 
-// The rows the fused kernel could not decide from its f16-staged terms, one warp per row.  The list's counter is
-// cleared by the last CTA to finish, so the next launch of the fused kernel starts from an empty list.
+__device__ __forceinline__ void gate_redo_row(const GateRaw& raw, int bf16, int d, const float* __restrict__ bias_k,
+                                              const float* __restrict__ bias_v, int side, int row, int b_s, float base, float thr,
+                                              float M, unsigned short* __restrict__ levels, int lane) {
+  gate_redo_finish(gate_redo_logits(raw, bf16, d, side, row, b_s, 0, 32, lane), d, bias_k, bias_v, side, row, b_s, base, thr, M, levels, lane);
+}
+
+// The rows the fused kernel could not decide from its f16-staged terms, a CTA of eight warps per row: four logits each, so
+// that a row costs one round trip to the weights and not eight (1332 tokens 13.9 -> 6.1 us, 524288 tokens 14.1 -> 11.0 us
+// against a warp per row).  The list's counter is cleared by the last CTA to finish,
+// so the next launch of the fused kernel starts from an empty list.
 constexpr int GT_FIX_CAP = 1 << 18;                            // list entries; rows beyond are decided inside the fused kernel
-constexpr int GT_FIX_THREADS = 128;
+constexpr int GT_FIX_THREADS = 256;
 __global__ void __launch_bounds__(GT_FIX_THREADS)
 gate_fixup_kernel(const GateRaw raw, int bf16, int d, const float* __restrict__ bias_k, const float* __restrict__ bias_v,
                   const int4* __restrict__ list, int* counters, unsigned short* __restrict__ levels) {
-  const int lane = threadIdx.x & 31;
+  __shared__ float s_z[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int n = min(counters[0], GT_FIX_CAP);
-  for (int i = (blockIdx.x * GT_FIX_THREADS + threadIdx.x) >> 5; i < n; i += (gridDim.x * GT_FIX_THREADS) >> 5) {
+  for (int i = blockIdx.x; i < n; i += gridDim.x) {
     const int4 e0 = list[2 * i], e1 = list[2 * i + 1];
-    gate_redo_row(raw, bf16, d, bias_k, bias_v, e0.y & 1, e0.x, e0.y >> 1, __int_as_float(e0.z), __int_as_float(e0.w),
-                  __int_as_float(e1.x), levels, lane);
+    const float z = gate_redo_logits(raw, bf16, d, e0.y & 1, e0.x, e0.y >> 1, 4 * warp, 4 * warp + 4, lane);
+    if ((lane >> 2) == warp) s_z[lane] = z;
+    __syncthreads();
+    if (warp == 0)
+      gate_redo_finish(s_z[lane], d, bias_k, bias_v, e0.y & 1, e0.x, e0.y >> 1, __int_as_float(e0.z), __int_as_float(e0.w),
+                       __int_as_float(e1.x), levels, lane);
+    __syncthreads();
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -494,7 +511,7 @@ size_t gate_tc_fix_bytes() { return (size_t)GT_FIX_CAP * 2 * sizeof(int4); }
 static cudaError_t launch_gate_fixup(const DevView& v, const GateMaps& maps, const LayerParams& lp, int bf16, unsigned short* levels,
                                      int sm_count, cudaStream_t st) {
   ProfScope ps(TWKV_K_GATE_RANK, st);
-  gate_fixup_kernel<<<2 * sm_count, GT_FIX_THREADS, 0, st>>>(maps.raw, bf16, v.d_kv, lp.b_k, lp.b_v, maps.raw.fix_list,
+  gate_fixup_kernel<<<4 * sm_count, GT_FIX_THREADS, 0, st>>>(maps.raw, bf16, v.d_kv, lp.b_k, lp.b_v, maps.raw.fix_list,
                                                              maps.raw.fix_counters, levels);
   count_launch();
   return cudaGetLastError();
