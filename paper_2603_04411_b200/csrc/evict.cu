@@ -43,7 +43,9 @@ __device__ int collect_key_tiles(const DevView& v, int layer, int side, int seq,
   return base;
 }
 
-__global__ void __launch_bounds__(EV_THREADS) evict_bitmap_kernel(DevView v, int layer, int seq, const int* __restrict__ keep, int n_keep) {
+__global__ void __launch_bounds__(EV_THREADS) evict_bitmap_kernel(DevView v, int layer, int seq, const int* keep, int n_keep) {
+  chain_start();
+  chain_wait();
   unsigned* bm = v.evict_bitmap;
   for (int i = threadIdx.x; i < (ROPE_LO * ROPE_HI) / 32; i += EV_THREADS) bm[i] = 0u;
   __syncthreads();
@@ -56,6 +58,8 @@ __global__ void __launch_bounds__(EV_THREADS) evict_bitmap_kernel(DevView v, int
 
 // grid (NC, 2): one CTA per key of the sequence.  evict_map[side][tile * 128 + slot] = new global slot, or -1.
 __global__ void __launch_bounds__(EV_THREADS) evict_plan_kernel(DevView v, int layer, int seq) {
+  chain_start();
+  chain_wait();
   extern __shared__ int s_tiles[];
   __shared__ int s_warp[32];
   const int cls = blockIdx.x + 1, side = blockIdx.y, tid = threadIdx.x;
@@ -105,6 +109,8 @@ __global__ void __launch_bounds__(EV_THREADS) evict_plan_kernel(DevView v, int l
 // tokens of all classes 41.4 -> 16.9 us against one CTA per key that took its tiles and panels one by one.
 constexpr int EV_BATCH = 4;
 __global__ void __launch_bounds__(EV_THREADS) evict_move_kernel(DevView v, int layer, int seq) {
+  chain_start();
+  chain_wait();
   extern __shared__ int s_tiles[];
   __shared__ int s_warp[32];
   const int cls = blockIdx.x + 1, side = blockIdx.y, panel = blockIdx.z, tid = threadIdx.x;
@@ -164,6 +170,8 @@ __global__ void __launch_bounds__(EV_THREADS) evict_move_kernel(DevView v, int l
 
 // grid NC + 1: the K tile list of every class, and the sequence's V tile list, without the emptied tiles of `seq`
 __global__ void __launch_bounds__(EV_THREADS) evict_lists_kernel(DevView v, int layer, int seq) {
+  chain_start();
+  chain_wait();
   __shared__ int s_warp[32];
   const bool vlist = (int)blockIdx.x == v.NC;
   const int side = vlist ? 1 : 0;
@@ -197,10 +205,12 @@ cudaError_t launch_evict(const DevView& v, int layer, int seq, const int* keep_p
     if (e != cudaSuccess) return e;
   }
   ProfScope ps(TWKV_K_OTHER, st);
-  evict_bitmap_kernel<<<1, EV_THREADS, 0, st>>>(v, layer, seq, keep_positions, n_keep);
-  evict_plan_kernel<<<dim3(v.NC, 2), EV_THREADS, smem, st>>>(v, layer, seq);
-  evict_move_kernel<<<dim3(v.NC, 2, v.NC), EV_THREADS, smem, st>>>(v, layer, seq);
-  evict_lists_kernel<<<v.NC + 1, EV_THREADS, 0, st>>>(v, layer, seq);
+  const dim3 b(EV_THREADS), one(1);
+  cudaError_t e = launch_chained(evict_bitmap_kernel, one, b, one, 0, st, v, layer, seq, keep_positions, n_keep);
+  if (e == cudaSuccess) e = launch_chained(evict_plan_kernel, dim3(v.NC, 2), b, one, smem, st, v, layer, seq);
+  if (e == cudaSuccess) e = launch_chained(evict_move_kernel, dim3(v.NC, 2, v.NC), b, one, smem, st, v, layer, seq);
+  if (e == cudaSuccess) e = launch_chained(evict_lists_kernel, dim3(v.NC + 1), b, one, 0, st, v, layer, seq);
+  if (e != cudaSuccess) return e;
   count_launch(4);
   return cudaGetLastError();
 }

@@ -28,6 +28,8 @@ using namespace tc;
 // ------------------------------------------------------------------------------------------ tables
 // Zeroes the position bitmaps and maps sequence ids to the call's sequence slots.
 __global__ void __launch_bounds__(1024) pf_init_kernel(DevView v, PfCall a) {
+  chain_start();
+  chain_wait();
   for (int i = blockIdx.x * 1024 + threadIdx.x; i < a.n_words; i += gridDim.x * 1024) a.bits[i] = 0u;
   if (blockIdx.x > 0) return;
   for (int s = threadIdx.x; s < v.S; s += 1024) a.slot[s] = -1;
@@ -38,6 +40,8 @@ __global__ void __launch_bounds__(1024) pf_init_kernel(DevView v, PfCall a) {
 
 // Sets the bit of every visible token's position; a position met twice marks its sequence.
 __global__ void __launch_bounds__(1024) pf_bits_kernel(DevView v, PfCall a, int layer) {
+  chain_start();
+  chain_wait();
   const int sub = threadIdx.x >> 7, slot = threadIdx.x & (TILE - 1);
   const int n = v.ntiles(layer)[0];
   const int4* desc = v.desc(layer, 0);
@@ -56,6 +60,8 @@ __global__ void __launch_bounds__(1024) pf_bits_kernel(DevView v, PfCall a, int 
 // One CTA per sequence: exclusive prefix of the bitmap's word counts and the number of rows; the last CTA to finish lays
 // the sequences out one behind the other.
 __global__ void __launch_bounds__(1024) pf_scan_kernel(DevView v, PfCall a, int layer) {
+  chain_start();
+  chain_wait();
   __shared__ int s_warp[32];
   __shared__ int s_last;
   const int u = blockIdx.x, tid = threadIdx.x;
@@ -111,6 +117,8 @@ __device__ __forceinline__ int pf_rank(const PfCall& a, int off, int pos) {     
 // Dense row of every K and V slot, position of every row, the segments a tile touches; per query and per block of queries
 // what it may see.  The last `qctas` CTAs take the queries.
 __global__ void __launch_bounds__(1024) pf_rows_kernel(DevView v, PfCall a, int layer, int qctas) {
+  chain_start();
+  chain_wait();
   const int tctas = (int)gridDim.x - qctas;
   if ((int)blockIdx.x >= tctas) {
     for (int b = ((int)blockIdx.x - tctas) * 32 + (threadIdx.x >> 5); b < a.n_blocks; b += qctas * 32) {       // a warp per block
@@ -228,6 +236,7 @@ template <bool BF16>
 __global__ void __launch_bounds__(PR_THREADS, 1)
 pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_constant__ CUtensorMap map_uk,
                 const __grid_constant__ CUtensorMap map_uv, DevView v, PfCall a, int layer, int seg) {
+  chain_start();
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t s0 = smem_addr(smem_raw);
@@ -247,6 +256,7 @@ pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_con
     mbar_init_fence();
   }
   if (warp == 1) tmem_alloc(smem_addr(s_tmem_base), 512);
+  chain_wait();
   for (int i = tid; i < ROPE_LO * 32; i += PR_THREADS) sRope[(i >> 5) * PR_ROPE_STRIDE + (i & 31)] = v.rope_lo[i];
   fence_before_sync();
   __syncthreads();
@@ -573,7 +583,8 @@ __device__ __forceinline__ PfItem pf_item(const DevView& v, const PfCall& a, int
 
 template <bool BF16>
 __global__ void __launch_bounds__(PA_THREADS, 1)
-pf_attn_kernel(const __grid_constant__ CUtensorMap map_seg, DevView v, PfCall a, int seg, const unsigned short* __restrict__ q) {
+pf_attn_kernel(const __grid_constant__ CUtensorMap map_seg, DevView v, PfCall a, int seg, const unsigned short* q) {
+  chain_start();
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t s0 = smem_addr(smem_raw);
@@ -597,6 +608,7 @@ pf_attn_kernel(const __grid_constant__ CUtensorMap map_seg, DevView v, PfCall a,
   fence_after_sync();
   const uint32_t tmem_base = *s_tmem_base;
   const int n_items = a.blk_n * v.Hkv * a.n_splits;
+  chain_wait();
 
   if (misaligned) {
     // nothing was started
@@ -724,7 +736,7 @@ pf_attn_kernel(const __grid_constant__ CUtensorMap map_seg, DevView v, PfCall a,
         const int ql = h * QT + r / rep;
         uint4 val = make_uint4(0u, 0u, 0u, 0u);
         if (ql < it.cnt)
-          val = __ldg(reinterpret_cast<const uint4*>(q + ((size_t)a.qrow[it.first + ql] * v.Hq + it.g * rep + r % rep) * HEAD_DIM) + ch);
+          val = reinterpret_cast<const uint4*>(q + ((size_t)a.qrow[it.first + ql] * v.Hq + it.g * rep + r % rep) * HEAD_DIM)[ch];
         if constexpr (BF16) {
           const unsigned w[4] = {val.x, val.y, val.z, val.w};
           unsigned o[4];
@@ -889,8 +901,10 @@ pf_attn_kernel(const __grid_constant__ CUtensorMap map_seg, DevView v, PfCall a,
 // columns); a thread owns one row of 16 of the columns, so reads are coalesced along the rows; rows leave through shared
 // memory.
 template <int OUT>
-__global__ void __launch_bounds__(256) pf_combine_kernel(DevView v, PfCall a, void* __restrict__ out) {
+__global__ void __launch_bounds__(256) pf_combine_kernel(DevView v, PfCall a, void* out) {
   __shared__ float s[TILE][33];
+  chain_start();
+  chain_wait();
   const int c0 = (blockIdx.x & 3) * 32, h = (blockIdx.x >> 2) & 1, bg = blockIdx.x >> 3, g = bg % v.Hkv, blk = bg / v.Hkv;
   const int2 q = a.blocks[a.blk0 + blk];
   const int cnt = q.y & 0x1ff, rep = v.rep, QT = TILE / rep;
@@ -944,11 +958,13 @@ __global__ void __launch_bounds__(256) pf_combine_kernel(DevView v, PfCall a, vo
 cudaError_t launch_pf_tables(const DevView& v, const PfCall& a, int layer, int sm_count, cudaStream_t st) {
   ProfScope ps(TWKV_K_PLAN, st);
   const int zc = (a.n_words + 8191) / 8192, qctas = (a.n_blocks + 31) / 32;
-  pf_init_kernel<<<zc < 1 ? 1 : (zc > sm_count ? sm_count : zc), 1024, 0, st>>>(v, a);
-  pf_bits_kernel<<<sm_count, 1024, 0, st>>>(v, a, layer);
-  pf_scan_kernel<<<a.n_u, 1024, 0, st>>>(v, a, layer);
   const int qc = qctas > sm_count ? sm_count : qctas;
-  pf_rows_kernel<<<sm_count + qc, 1024, 0, st>>>(v, a, layer, qc);
+  const dim3 b(1024), one(1);
+  cudaError_t e = launch_chained(pf_init_kernel, dim3(zc < 1 ? 1 : (zc > sm_count ? sm_count : zc)), b, one, 0, st, v, a);
+  if (e == cudaSuccess) e = launch_chained(pf_bits_kernel, dim3(sm_count), b, one, 0, st, v, a, layer);
+  if (e == cudaSuccess) e = launch_chained(pf_scan_kernel, dim3(a.n_u), b, one, 0, st, v, a, layer);
+  if (e == cudaSuccess) e = launch_chained(pf_rows_kernel, dim3(sm_count + qc), b, one, 0, st, v, a, layer, qc);
+  if (e != cudaSuccess) return e;
   count_launch(4);
   return cudaGetLastError();
 }
@@ -958,11 +974,17 @@ static cudaError_t launch_pf_segment_t(const DevView& v, const PfCall& a, const 
   cudaError_t e = cudaFuncSetAttribute(pf_recon_kernel<BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PR_SMEM);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(pf_attn_kernel<BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PA_SMEM);
   if (e != cudaSuccess) return e;
-  { ProfScope ps(TWKV_K_KSCORE, st); pf_recon_kernel<BF16><<<sm_count, PR_THREADS, PR_SMEM, st>>>(maps.blocks, maps.uk, maps.uv, v, a, layer, seg); }
+  {
+    ProfScope ps(TWKV_K_KSCORE, st);
+    e = launch_chained(pf_recon_kernel<BF16>, dim3(sm_count), dim3(PR_THREADS), dim3(1), PR_SMEM, st, maps.blocks, maps.uk, maps.uv, v, a, layer, seg);
+    if (e != cudaSuccess) return e;
+  }
   const int n_items = a.blk_n * v.Hkv * a.n_splits;
   {
     ProfScope ps(TWKV_K_VACC, st);
-    pf_attn_kernel<BF16><<<n_items < sm_count ? n_items : sm_count, PA_THREADS, PA_SMEM, st>>>(maps.seg, v, a, seg, reinterpret_cast<const unsigned short*>(q));
+    e = launch_chained(pf_attn_kernel<BF16>, dim3(n_items < sm_count ? n_items : sm_count), dim3(PA_THREADS), dim3(1), PA_SMEM, st, maps.seg, v, a, seg,
+                       reinterpret_cast<const unsigned short*>(q));
+    if (e != cudaSuccess) return e;
   }
   count_launch(2);
   return cudaGetLastError();
@@ -975,9 +997,9 @@ cudaError_t launch_pf_segment(const DevView& v, const PfCall& a, const PfMaps& m
 cudaError_t launch_pf_combine(const DevView& v, const PfCall& a, void* out, cudaStream_t st) {
   ProfScope ps(TWKV_K_MERGE, st);
   const int grid = a.blk_n * v.Hkv * 8;
-  if (v.out_dtype == TWKV_F32) pf_combine_kernel<TWKV_F32><<<grid, 256, 0, st>>>(v, a, out);
-  else if (v.out_dtype == TWKV_BF16) pf_combine_kernel<TWKV_BF16><<<grid, 256, 0, st>>>(v, a, out);
-  else pf_combine_kernel<TWKV_F16><<<grid, 256, 0, st>>>(v, a, out);
+  auto kernel = v.out_dtype == TWKV_F32 ? pf_combine_kernel<TWKV_F32> : v.out_dtype == TWKV_BF16 ? pf_combine_kernel<TWKV_BF16> : pf_combine_kernel<TWKV_F16>;
+  const cudaError_t e = launch_chained(kernel, dim3(grid), dim3(256), dim3(1), 0, st, v, a, out);
+  if (e != cudaSuccess) return e;
   count_launch();
   return cudaGetLastError();
 }
