@@ -183,9 +183,9 @@ twkv_status twkv_decode_attn(twkv_cache* cache, int layer, const void* q, const 
  *   q_seq    [n_q] int32, HOST memory: sequence id of every query (any order, repeats allowed)
  *   q_pos    [n_q] int32, HOST memory: RoPE position of every query (>= 0)
  *   n_q      at most TWKV_PREFILL_MAX_QUERIES
- * The queries are served in waves of at most one query per sequence (the k-th query of every sequence together);
- * each wave is one pass of the decode kernels with the causal limit applied to the scores.  The host arrays are
- * read before the call returns.  Errors as for twkv_decode_attn; an id or position out of range returns
+ * Keys and values of the visible tokens are rebuilt once per call and shared by its queries; calls of few queries per
+ * sequence run as passes of the decode kernels instead, one query per sequence at a time (num_splits applies to those).
+ * The host arrays are read before the call returns.  Errors as for twkv_decode_attn; an id or position out of range returns
  * TWKV_ERR_INVALID_ARG before anything is launched.
  */
 twkv_status twkv_prefill_attn(twkv_cache* cache, int layer, const void* q, const int32_t* q_seq /*host*/,
