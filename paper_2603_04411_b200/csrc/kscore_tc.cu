@@ -62,11 +62,6 @@ __device__ __forceinline__ uint64_t f2_pack_bits(uint32_t a, uint32_t b) { uint6
 __device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) { uint64_t r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 __device__ __forceinline__ uint64_t f2_sub(uint64_t a, uint64_t b) { uint64_t r; asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 __device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) { uint64_t r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
-__device__ __forceinline__ uint32_t f2_to_f16x2_sat(uint64_t v) {       // (lo lane -> bits 0..15), saturating
-  uint32_t d;
-  asm("{\n\t.reg .f32 a, b;\n\tmov.b64 {a, b}, %1;\n\tcvt.rn.satfinite.f16x2.f32 %0, b, a;\n\t}" : "=r"(d) : "l"(v));
-  return d;
-}
 __device__ __forceinline__ unsigned warp_max_u32(unsigned x) {
   unsigned r;
   asm volatile("redux.sync.max.u32 %0, %1, 0xffffffff;" : "=r"(r) : "r"(x));
@@ -420,8 +415,8 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
               tmem_ld8(sl_addr + 8 * (c + 1), nx);
               tmem_ld8(sl_addr + 64 + 8 * (c + 1), nx + 8);
             }
-            // a rotated value leaves as two f16: the value with its low 13 mantissa bits cleared (exact in f16) and the
-            // rest (rounded to f16: 2^-21 of the value instead of the 2^-11 of one f16), so that the score error stays
+            // a rotated value leaves as two f16: the nearest one and the
+            // rest (rounded to f16: 2^-22 of the value instead of the 2^-11 of one f16), so that the score error stays
             // far below the bar even where a few key channels carry most of the magnitude
             uint32_t oh[8], ol[8];
 #pragma unroll
@@ -430,11 +425,8 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
               const uint64_t L = f2_pack_bits(cur[2 * u], cur[2 * u + 1]), H = f2_pack_bits(cur[8 + 2 * u], cur[8 + 2 * u + 1]);
               const uint64_t a = f2_sub(f2_mul(L, cs2[t]), f2_mul(H, sn2[t]));           // lo cos - hi sin
               const uint64_t b = f2_fma(L, sn2[t], f2_mul(H, cs2[t]));                   // hi cos + lo sin
-              const uint64_t ah = a & 0xFFFFE000FFFFE000ull, bh = b & 0xFFFFE000FFFFE000ull;
-              oh[u] = f2_to_f16x2_sat(ah);
-              oh[4 + u] = f2_to_f16x2_sat(bh);
-              ol[u] = f2_to_f16x2_sat(f2_sub(a, ah));
-              ol[4 + u] = f2_to_f16x2_sat(f2_sub(b, bh));
+              split_pair_16<false>(a, oh[u], ol[u]);
+              split_pair_16<false>(b, oh[4 + u], ol[4 + u]);
             }
             if constexpr (DBG) {
               // TWKV_DEBUG: a rotated key beyond the f16 range was clamped by the conversion above (its high part reads

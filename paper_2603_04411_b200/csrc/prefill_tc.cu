@@ -199,33 +199,6 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) { uint64_t r; a
 __device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) { uint64_t r; asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) { uint64_t r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
 __device__ __forceinline__ void unpk2(uint64_t v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
-// Two packed fp32 -> their high and low 16-bit parts (high: the value cut to the type's mantissa; low: the rest, rounded).
-template <bool BF16> __device__ __forceinline__ void split2(uint64_t v, uint32_t& hi, uint32_t& lo) {
-  const uint64_t h = v & (BF16 ? 0xFFFF0000FFFF0000ull : 0xFFFFE000FFFFE000ull);
-  const uint64_t l = sub2(v, h);
-  if constexpr (BF16) {
-    asm("{\n\t.reg .b32 a, b;\n\tmov.b64 {a, b}, %1;\n\tprmt.b32 %0, a, b, 0x7632;\n\t}" : "=r"(hi) : "l"(h));
-    asm("{\n\t.reg .f32 a, b;\n\tmov.b64 {a, b}, %1;\n\tcvt.rn.bf16x2.f32 %0, b, a;\n\t}" : "=r"(lo) : "l"(l));
-  } else {
-    asm("{\n\t.reg .f32 a, b;\n\tmov.b64 {a, b}, %1;\n\tcvt.rn.satfinite.f16x2.f32 %0, b, a;\n\t}" : "=r"(hi) : "l"(h));
-    asm("{\n\t.reg .f32 a, b;\n\tmov.b64 {a, b}, %1;\n\tcvt.rn.satfinite.f16x2.f32 %0, b, a;\n\t}" : "=r"(lo) : "l"(l));
-  }
-}
-// The same with the high part rounded to nearest: the low part is half as large, and so the product of two low parts, which
-// the second product of attention leaves out.
-template <bool BF16> __device__ __forceinline__ void split2_rn(uint64_t v, uint32_t& hi, uint32_t& lo) {
-  float a, b;
-  unpk2(v, a, b);
-  if constexpr (BF16) {
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(hi) : "f"(b), "f"(a));
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(b - __uint_as_float(hi & 0xffff0000u)), "f"(a - __uint_as_float(hi << 16)));
-  } else {
-    hi = pack_f16x2_sat(a, b);
-    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&hi));
-    lo = pack_f16x2_sat(a - f.x, b - f.y);
-  }
-}
-
 // One work item = (tile, slab of NS = 256 output dims, i.e. two KV heads; 128 where d_kv is not a multiple of 256).
 // [128 x NS] accumulators alternate between two TMEM buffers; state panels (K-major A) and U^-1 atoms (rows of the caller's
 // matrix as they lie: MN-major B) stream through a ring of three stages.  Eight epilogue warps (thread = one token row x
@@ -466,8 +439,8 @@ pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_con
               for (int k = 0; k < 4; ++k) {
                 const uint64_t L = pk2u(x[8 * c + 2 * k], x[8 * c + 2 * k + 1]), H = pk2u(x[32 + 8 * c + 2 * k], x[33 + 8 * c + 2 * k]);
                 const uint64_t rl = sub2(mul2(L, cs[4 * c + k]), mul2(H, sn[4 * c + k])), rh = fma2(L, sn[4 * c + k], mul2(H, cs[4 * c + k]));
-                split2<false>(rl, hi[k], lo[k]);
-                split2<false>(rh, hi[4 + k], lo[4 + k]);
+                split_pair_16<false>(rl, hi[k], lo[k]);
+                split_pair_16<false>(rh, hi[4 + k], lo[4 + k]);
               }
               if (v.debug) {                                     // TWKV_DEBUG: a rotated key beyond the f16 range was clamped
                 bool sat = false;
@@ -517,7 +490,7 @@ pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_con
             for (int c = 0; c < 8; ++c) {
               uint32_t hi[4], lo[4];
 #pragma unroll
-              for (int k = 0; k < 4; ++k) split2_rn<BF16>(pk2u(x[hh][8 * c + 2 * k], x[hh][8 * c + 2 * k + 1]), hi[k], lo[k]);
+              for (int k = 0; k < 4; ++k) split_pair_16<BF16>(pk2u(x[hh][8 * c + 2 * k], x[hh][8 * c + 2 * k + 1]), hi[k], lo[k]);
               stage_piece(c, hi, lo);
             }
             rows_out(g0 + hh);
@@ -833,7 +806,7 @@ pf_attn_kernel(const __grid_constant__ CUtensorMap map_seg, DevView v, PfCall a,
             unpk2(fma2(pk2u(x[16 * c + 2 * k], x[16 * c + 2 * k + 1]), sc2, nm2), p0, p1);
             const uint64_t p = pk2(ex2(p0), ex2(p1));
             l2 = add2(l2, p);
-            split2<BF16>(p, w[k], w[8 + k]);
+            split_pair_16<BF16>(p, w[k], w[8 + k]);
           }
           tmem_st16(tS + 16 * c, w);
         }

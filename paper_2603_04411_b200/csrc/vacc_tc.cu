@@ -65,21 +65,7 @@ __device__ __forceinline__ uint64_t vt_pack(float a, float b) { uint64_t r; asm(
 __device__ __forceinline__ void vt_unpack(uint64_t v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
 __device__ __forceinline__ uint64_t vt_fma2(uint64_t a, uint64_t b, uint64_t c) { uint64_t r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
 __device__ __forceinline__ uint64_t vt_add2(uint64_t a, uint64_t b) { uint64_t r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
-__device__ __forceinline__ uint64_t vt_sub2(uint64_t a, uint64_t b) { uint64_t r; asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 __device__ __forceinline__ float vt_ex2(float x) { float r; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
-// Two packed fp32 weights -> their high parts (mantissa cut to the type) and the rest, each as a packed pair of the cache dtype.
-template <bool BF16> __device__ __forceinline__ void vt_split(uint64_t v, uint32_t& hi, uint32_t& lo) {
-  const uint64_t h = v & (BF16 ? 0xFFFF0000FFFF0000ull : 0xFFFFE000FFFFE000ull);
-  const uint64_t l = vt_sub2(v, h);
-  if constexpr (BF16) {
-    asm("{\n\t.reg .b32 a, b;\n\tmov.b64 {a, b}, %1;\n\tprmt.b32 %0, a, b, 0x7632;\n\t}" : "=r"(hi) : "l"(h));
-    asm("{\n\t.reg .f32 a, b;\n\tmov.b64 {a, b}, %1;\n\tcvt.rn.bf16x2.f32 %0, b, a;\n\t}" : "=r"(lo) : "l"(l));
-  } else {
-    asm("{\n\t.reg .f32 a, b;\n\tmov.b64 {a, b}, %1;\n\tcvt.rn.f16x2.f32 %0, b, a;\n\t}" : "=r"(hi) : "l"(h));
-    asm("{\n\t.reg .f32 a, b;\n\tmov.b64 {a, b}, %1;\n\tcvt.rn.f16x2.f32 %0, b, a;\n\t}" : "=r"(lo) : "l"(l));
-  }
-}
-
 // Instruction descriptor: kind::f16, fp32 accumulate, A MN-major (bit 15), B K-major, M = 128.
 __host__ __device__ constexpr uint32_t vt_idesc(int fmt, int n) { return idesc_f16(fmt, 128, n) | (1u << 15); }
 
@@ -325,8 +311,7 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
 #pragma unroll
         for (int it = 0; it < ITEMS; ++it) {
           const int tg = (it * VT_PTHREADS + pt) / N;
-          // Two weights at a time, packed: exp2 of one fused multiply-add, the high part cut off (exact in the type), the low
-          // part rounded.  bf16 keeps 8 bits of a weight, f16 11: with few tokens per sequence that rounding alone reaches 1e-3
+          // Two weights at a time, packed: exp2 of one fused multiply-add, then the nearest value of the type and the rest.  bf16 keeps 8 bits of a weight, f16 11: with few tokens per sequence that rounding alone reaches 1e-3
           // and 1e-4 of the output, so the remainder goes into a second operand (16 and 22 bits in all).
           // Measured with both parts in one B operand: 64 heads bf16 over 131072 tokens 33.4 us (41.3 with two chains of products and
           // rounded parts), f16 16 x 32768 66.1 us and 64 x 8192 78 us (68.1 and 77.1 with one f16 part).
@@ -342,7 +327,7 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
             }
             const uint64_t p = vt_pack(p0, p1);
             l_sum2 = vt_add2(l_sum2, p);
-            vt_split<BF16>(p, hi[u >> 1], lo[u >> 1]);
+            split_pair_16<BF16>(p, hi[u >> 1], lo[u >> 1]);
           }
           const uint32_t off = (uint32_t)(tg >> 3) * C::P_HALF_BYTES + (uint32_t)ph_ * 128u + ((((uint32_t)tg & 7u) ^ ((uint32_t)ph_ & 7u)) << 4);
           *reinterpret_cast<uint4*>(pb + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
