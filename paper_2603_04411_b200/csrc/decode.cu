@@ -26,15 +26,13 @@ namespace twkv {
 // that a CTA (pair) of the K-score kernel mostly stays inside one (class, sequence) run.  What bounds it is the chain of
 // dependent table reads: one CTA that walked the whole list took 17.5 us for 16 sequences of 32768 tokens (2200 tiles) and 17
 // for 64 of 8192; a CTA per class takes 8.6 and 9.5 (8.9 -> 8.4 for 8 tiles).
-__device__ __forceinline__ unsigned ktile_cost(int cls) {
-  // cycles per tile of the K-score kernel by rank class: a least-squares fit, one coefficient per class, of every CTA's busy
-  // time to its tile counts on the benchmark's mix of classes (8 KV heads, CTA pairs; residual 1.3 us rms of 330): a fixed
-  // part (rotation factors, the per-slab epilogue and score products) plus a per-panel part, an odd panel count costing a
-  // little more than the even one above it saves; classes above 8 run as two passes.  Only the ratios matter.
-  constexpr unsigned kCost[TWKV_MAX_CLASSES] = {14300u, 16600u, 18600u, 19500u, 22100u, 23000u, 25400u, 26200u,
-                                                38800u, 38700u, 42000u, 42800u, 45600u, 45800u, 49300u, 50700u};
-  return kCost[min(max(cls, 1), TWKV_MAX_CLASSES) - 1];
-}
+// cycles per tile of the K-score kernel by rank class: a least-squares fit, one coefficient per class, of every CTA's busy
+// time to its tile counts on the benchmark's mix of classes (8 KV heads, CTA pairs; residual 1.3 us rms of 330): a fixed
+// part (rotation factors, the per-slab epilogue and score products) plus a per-panel part, an odd panel count costing a
+// little more than the even one above it saves; classes above 8 run as two passes.  Only the ratios matter.
+__constant__ unsigned kTileCost[TWKV_MAX_CLASSES] = {14300u, 16600u, 18600u, 19500u, 22100u, 23000u, 25400u, 26200u,
+                                                   38800u, 38700u, 42000u, 42800u, 45600u, 45800u, 49300u, 50700u};
+__device__ __forceinline__ unsigned ktile_cost(int cls) { return kTileCost[min(max(cls, 1), TWKV_MAX_CLASSES) - 1]; }
 
 // Cut points of one sequence's V tile list into n_splits contiguous ranges of about equal cost (a tile costs its
 // panels plus its score rows, counted in 512-byte units): the V pass is bound by the bytes a CTA reads, and tiles of
@@ -118,6 +116,7 @@ __global__ void __launch_bounds__(1024) plan_kernel(DevView v, int layer, const 
   __shared__ int s_keep[TWKV_MAX_CLASSES];                        // tiles of the listed sequences per class
   __shared__ int s_koff[TWKV_MAX_CLASSES + 1], s_ioff[TWKV_MAX_CLASSES + 1];    // start of run k (class NC - k) in the tile list / in the item list
   __shared__ unsigned long long s_coff[TWKV_MAX_CLASSES + 1];     // estimated cost of everything before run k
+  __shared__ int s_hg;                                            // parts per item
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int run = blockIdx.x, cls = NC - run;
   const int n_list = v.kcc(layer)[cls - 1];
@@ -158,6 +157,23 @@ __global__ void __launch_bounds__(1024) plan_kernel(DevView v, int layer, const 
       co += (unsigned long long)items * ktile_cost(NC - k);
     }
     s_koff[NC] = ko; s_ioff[NC] = io; s_coff[NC] = co;
+    // The KV heads of an item may be dealt out to several CTAs (pairs): finer work for lists that leave some idle or that a few
+    // wide tiles decide.  A part repeats the tile's loads and rotation factors.  Least estimate of the slowest piece, in cycles:
+    // the widest part where every part has a CTA to itself, else the mean piece plus most of the widest part (numbers fitted to
+    // the lists below).  Whole items against this rule: 1 x 8192 62 -> 54 us, 4 x 1000 66 -> 57, 16 x 500 102
+    // -> 92, 8 x 8192 121 -> 114; 64 x 2000 and 16 x 32768 keep whole items.
+    constexpr float PART_COST = 2600.f;
+    int widest = 0;
+    while (widest < NC && s_ioff[widest + 1] == s_ioff[widest]) ++widest;
+    const float wide_cost = widest < NC ? (float)ktile_cost(NC - widest) : 0.f, per_cta = 1.f / (float)n_cta;
+    float best = 3.4e38f;
+    s_hg = 1;
+    float part = 1.f;
+    for (int h = 1; v.Hkv % h == 0; h *= 2, part *= 0.5f) {
+      const float est = io * h <= n_cta ? wide_cost * part
+                                        : ((float)co + (float)io * (float)(h - 1) * PART_COST) * per_cta + 0.7f * wide_cost * part;
+      if (est < best) { best = est; s_hg = h; }
+    }
   }
   __syncthreads();
   // this class's entries; a run of odd length ends with a filler for the pair kernel: the same tile again, flagged so that its
@@ -186,13 +202,9 @@ __global__ void __launch_bounds__(1024) plan_kernel(DevView v, int layer, const 
     base += total;
   }
   if (run > 0) return;
-  // Few items: the KV heads of an item are dealt out to several CTAs (pairs), as long as every part still finds one of its
-  // own; a part repeats the tile's loads and rotation factors, so a list that fills the device keeps whole items.  One
-  // sequence of 1024 tokens (4 items): K-score 32.6 us with whole items, 11.8 us with one head per part.
-  const int n_items = s_ioff[NC];
+  // (the parts the KV heads of an item are dealt out in: chosen above)
+  const int n_items = s_ioff[NC], hg = s_hg;
   const unsigned long long total = s_coff[NC];
-  int hg = 1;
-  while (v.Hkv % (2 * hg) == 0 && n_items * 2 * hg <= n_cta) hg *= 2;
   if (tid == 0) { *v.kitem_parts = hg; v.cta_start[n_cta] = n_items * hg; }
   // cut points: piece b starts at the item part whose cost interval holds b / n_cta of the total (64-bit arithmetic; inside
   // a run every part costs the same, so the part follows from a division)
