@@ -625,11 +625,12 @@ static twkv_status prefill_tiled(twkv_cache* c, int layer, const void* q, const 
   *done = true;
   if (launch_pf_tables(v, a, layer, c->sm_count, st) != cudaSuccess) return TWKV_ERR_CUDA;
   const int n_segs = std::max(1, (int)((rows_max + a.seg_rows - 1) / a.seg_rows));
+  const bool whole = n_segs == 1 && a.n_splits == 1;
   for (a.blk0 = 0; a.blk0 < n_blocks; a.blk0 += best_group) {
     a.blk_n = std::min(best_group, n_blocks - a.blk0);
     for (int seg = 0; seg < n_segs; ++seg)
-      if (launch_pf_segment(v, a, maps, layer, seg, q, c->sm_count, st) != cudaSuccess) return TWKV_ERR_CUDA;
-    if (launch_pf_combine(v, a, out, st) != cudaSuccess) return TWKV_ERR_CUDA;
+      if (launch_pf_segment(v, a, maps, layer, seg, q, whole ? out : nullptr, c->sm_count, st) != cudaSuccess) return TWKV_ERR_CUDA;
+    if (!whole && launch_pf_combine(v, a, out, st) != cudaSuccess) return TWKV_ERR_CUDA;
   }
   return TWKV_OK;
 }

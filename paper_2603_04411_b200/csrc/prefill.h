@@ -32,8 +32,9 @@ struct PfCall {
 };
 struct PfMaps { CUtensorMap blocks, uk, uv, seg; };
 
+// out: not null where one split of one segment is a query's whole result: the attention kernel then writes the outputs itself
 cudaError_t launch_pf_tables(const DevView& v, const PfCall& a, int layer, int sm_count, cudaStream_t st);
-cudaError_t launch_pf_segment(const DevView& v, const PfCall& a, const PfMaps& maps, int layer, int seg, const void* q, int sm_count, cudaStream_t st);
+cudaError_t launch_pf_segment(const DevView& v, const PfCall& a, const PfMaps& maps, int layer, int seg, const void* q, void* out, int sm_count, cudaStream_t st);
 cudaError_t launch_pf_combine(const DevView& v, const PfCall& a, void* out, cudaStream_t st);
 
 }  // namespace twkv

@@ -554,9 +554,28 @@ __device__ __forceinline__ PfItem pf_item(const DevView& v, const PfCall& a, int
   return it;
 }
 
+// Sixteen consecutive outputs (element offset o) in the output type.
+__device__ __forceinline__ void pf_store16(void* out, int out_dtype, size_t o, const float* x) {
+  if (out_dtype == TWKV_F32) {
+    float4* d = reinterpret_cast<float4*>(reinterpret_cast<float*>(out) + o);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) d[k] = make_float4(x[4 * k], x[4 * k + 1], x[4 * k + 2], x[4 * k + 3]);
+  } else {
+    unsigned w[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      if (out_dtype == TWKV_BF16) asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w[k]) : "f"(x[2 * k + 1]), "f"(x[2 * k]));
+      else asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(w[k]) : "f"(x[2 * k + 1]), "f"(x[2 * k]));
+    }
+    uint4* d = reinterpret_cast<uint4*>(reinterpret_cast<unsigned short*>(out) + o);
+    d[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    d[1] = make_uint4(w[4], w[5], w[6], w[7]);
+  }
+}
+
 template <bool BF16>
 __global__ void __launch_bounds__(PA_THREADS, 1)
-pf_attn_kernel(const __grid_constant__ CUtensorMap map_seg, DevView v, PfCall a, int seg, const unsigned short* q) {
+pf_attn_kernel(const __grid_constant__ CUtensorMap map_seg, DevView v, PfCall a, int seg, const unsigned short* q, void* out) {
   chain_start();
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -827,6 +846,27 @@ pf_attn_kernel(const __grid_constant__ CUtensorMap map_seg, DevView v, PfCall a,
         if (!(ok = named_bar_and(pair_bar, 64, ok))) break;
         l = xs[0] + xs[TILE];                                    // (read before this warp hands over the next item's queries)
       }
+      if (out) {
+        // one split of one segment: this is the whole result.  A thread writes its row's 64 columns itself (4096-token prompt in four
+        // calls 783 -> 751 us, five short prompts 204 -> 189 against partial results and the combine kernel).
+        const float inv = l > 0.f ? 1.f / l : 0.f;
+        const bool mine = ql < it.cnt;
+        const size_t o0 = mine ? ((size_t)a.qrow[it.first + ql] * v.Hq + it.g * rep + row % rep) * HEAD_DIM + hf * 64 : 0;
+#pragma unroll 1
+        for (int c = 0; c < 4; ++c) {
+          float x[16];
+#pragma unroll
+          for (int k = 0; k < 16; ++k) x[k] = 0.f;
+          if (it.n_blk > 0) {                                    // (the same for the whole warp, as the load demands)
+            tmem_ld16(tO + 16 * c, reinterpret_cast<uint32_t*>(x));
+            tmem_ld_wait();
+#pragma unroll
+            for (int k = 0; k < 16; ++k) x[k] *= inv;
+          }
+          if (mine) pf_store16(out, v.out_dtype, o0 + 16 * c, x);
+        }
+        continue;
+      }
       // the item's partial result, joined with what earlier segments left; column-major, so that a warp's rows lie together
       float* part = a.slots + ((((size_t)(it.blk - a.blk0) * v.Hkv + it.g) * a.n_splits + it.split) * 2 + h) * (130 * TILE) + row;
       if (it.n_blk > 0) {
@@ -943,7 +983,7 @@ cudaError_t launch_pf_tables(const DevView& v, const PfCall& a, int layer, int s
 }
 
 template <bool BF16>
-static cudaError_t launch_pf_segment_t(const DevView& v, const PfCall& a, const PfMaps& maps, int layer, int seg, const void* q, int sm_count, cudaStream_t st) {
+static cudaError_t launch_pf_segment_t(const DevView& v, const PfCall& a, const PfMaps& maps, int layer, int seg, const void* q, void* out, int sm_count, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(pf_recon_kernel<BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PR_SMEM);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(pf_attn_kernel<BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PA_SMEM);
   if (e != cudaSuccess) return e;
@@ -956,15 +996,15 @@ static cudaError_t launch_pf_segment_t(const DevView& v, const PfCall& a, const 
   {
     ProfScope ps(TWKV_K_VACC, st);
     e = launch_chained(pf_attn_kernel<BF16>, dim3(n_items < sm_count ? n_items : sm_count), dim3(PA_THREADS), dim3(1), PA_SMEM, st, maps.seg, v, a, seg,
-                       reinterpret_cast<const unsigned short*>(q));
+                       reinterpret_cast<const unsigned short*>(q), out);
     if (e != cudaSuccess) return e;
   }
   count_launch(2);
   return cudaGetLastError();
 }
-cudaError_t launch_pf_segment(const DevView& v, const PfCall& a, const PfMaps& maps, int layer, int seg, const void* q, int sm_count, cudaStream_t st) {
-  return v.dtype == TWKV_BF16 ? launch_pf_segment_t<true>(v, a, maps, layer, seg, q, sm_count, st)
-                              : launch_pf_segment_t<false>(v, a, maps, layer, seg, q, sm_count, st);
+cudaError_t launch_pf_segment(const DevView& v, const PfCall& a, const PfMaps& maps, int layer, int seg, const void* q, void* out, int sm_count, cudaStream_t st) {
+  return v.dtype == TWKV_BF16 ? launch_pf_segment_t<true>(v, a, maps, layer, seg, q, out, sm_count, st)
+                              : launch_pf_segment_t<false>(v, a, maps, layer, seg, q, out, sm_count, st);
 }
 
 cudaError_t launch_pf_combine(const DevView& v, const PfCall& a, void* out, cudaStream_t st) {

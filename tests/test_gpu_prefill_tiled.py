@@ -16,7 +16,8 @@ pytestmark = pytest.mark.gpu
     (1, 8, torch.float16, 1, 200, 1100, 1),      # more blocks of queries than the partial results have room for
     (3, 1, torch.bfloat16, 2, 300, 150, 1),      # 384 channels: one head per reconstruction slab, six classes
     (2, 2, torch.float16, 3, 260, 65, 2),        # every position held by two tokens
-    (8, 4, torch.float16, 2, 129, 4, 1),         # the fewest queries that leave the waves
+    (8, 4, torch.float16, 2, 129, 4, 1),         # few queries: several splits
+    (2, 4, torch.bfloat16, 1, 100, 50, 1),       # one split of one segment is the whole result
 ])
 def test_tiled_prefill_where_the_work_split_changes(B, hkv, rep, dtype, n_seq, ctx, n_q, repeat):
     d = hkv * 128
