@@ -106,7 +106,12 @@ constexpr int GATE_PIECE = 8192;       // tokens per COMPUTE-mode gate piece (lo
 // with one sequence (8 KV heads, ranks around 256): 1, 2, 3 waves 65, 112, 163 over 1024 tokens, 90, 164, 239 over 32768; tiled,
 // 4 to 8 queries, 80 over 1024, 184 over 8192, 408 over 32768.
 static bool prefill_tiled_pays(int n_waves, double rows) { return n_waves >= 2 && n_waves * (50.0 + rows / 1000.0) >= 75.0 + rows / 100.0; }
-constexpr int GATE_TC_MIN_TOKENS = 1024;   // calls at least this large run the fused tcgen05 gate kernel
+// COMPUTE-mode calls of this many tokens form the logits with gate_logits_tc_kernel; smaller ones, bound by launches and the
+// weights' way in, with the warp-MMA kernel; larger ones run the fused tcgen05 gate kernel, whose logits stay on the SM.
+// A whole compress call in us, warp-MMA / spread / fused (d_kv 1024): 128 tokens 39.2 / 32.8 / -, 1000 67.7 / 46.2 / -,
+// 2048 81.3 / 54.3 / 61.8, 3072 104 / 60.6 / 63.1, 4096 131 / 72.0 / 66.3; d_kv 512: 100 tokens 28.7 / 28.7 / -, 1000 47.7 / 38.2 / -,
+// 3072 61.6 / 46.0 / 52.3, 6000 80.3 / 57.7 / 51.4; d_kv 384: 3072 tokens - / 44.1 / 47.4, 4096 - / 51.4 / 47.4.
+constexpr int GATE_LOGITS_TC_MIN = 128, GATE_LOGITS_TC_MAX = 3072;
 
 struct Offsets {
   size_t status, pflags, rope_lo, rope_hi, n_tiles, tile_desc, tile_aux, tile_rank, fill, key_last, kclass_count,
@@ -453,8 +458,12 @@ twkv_status twkv_compress(twkv_cache* c, int layer, const void* K, const void* V
   c->appended[layer].fetch_add(n_tok, std::memory_order_relaxed);
   if (mode == TWKV_GATE_LOGITS) {
     if (launch_gate_rank(v, scores, levels, n_tok, st) != cudaSuccess) return TWKV_ERR_CUDA;
-  } else if (mode == TWKV_GATE_COMPUTE && n_tok >= GATE_TC_MIN_TOKENS && c->sm_count <= 160) {
-    // fused tcgen05 kernel: logits and ranks in one launch, the logits never leave the CTA's staging block
+  } else if (mode == TWKV_GATE_COMPUTE && n_tok >= GATE_LOGITS_TC_MIN && c->sm_count <= 160 &&
+             (n_tok > GATE_LOGITS_TC_MAX || c->prepared_w[layer] || !is_capturing(st))) {
+    // up to GATE_LOGITS_TC_MAX tokens: tcgen05 logits spread over all SMs, then the rank kernel (a call that is captured before the
+    // weights were laid out reads them as they are, below); above: fused tcgen05 kernel, logits and ranks in one launch, the logits
+    // never leave the CTA's staging block
+    const bool spread = n_tok <= GATE_LOGITS_TC_MAX;
     const int d = c->dims.d_kv;
     if (!c->prepared_w[layer]) {
       // first COMPUTE call after the parameters were (re)set: K-major copies of W_k, W_v for the tensor cores
@@ -469,14 +478,17 @@ twkv_status twkv_compress(twkv_cache* c, int layer, const void* K, const void* V
     }
     const bool pairs = d % 256 == 0 && gate_tc_max_pairs(c->sm_count) > 0;
     GateMaps maps;
-    maps.wk = (pairs ? c->map_wT_half : c->map_wT)[2 * (size_t)layer];
-    maps.wv = (pairs ? c->map_wT_half : c->map_wT)[2 * (size_t)layer + 1];
+    maps.wk = (pairs || spread ? c->map_wT_half : c->map_wT)[2 * (size_t)layer];
+    maps.wv = (pairs || spread ? c->map_wT_half : c->map_wT)[2 * (size_t)layer + 1];
     if (!make_tmap_2d(&maps.xk, K, (uint64_t)n_tok, d, (uint64_t)d * 2, TILE) ||
         !make_tmap_2d(&maps.xv, V, (uint64_t)n_tok, d, (uint64_t)d * 2, TILE)) return TWKV_ERR_CUDA;
     const unsigned char* wT = c->pool + c->off.prep_wT + (size_t)layer * 2 * d * d * 2;
     maps.raw = GateRaw{(const unsigned short*)K, (const unsigned short*)V, (const unsigned short*)wT,
                        (const unsigned short*)(wT + (size_t)d * d * 2), v.gate_fix, v.status + 2};
-    if (launch_gate_ranks_tc(v, maps, c->params[layer], n_tok, levels, c->sm_count, pairs, st) != cudaSuccess) return TWKV_ERR_CUDA;
+    if (spread) {
+      if (launch_gate_logits_tc(v, maps, c->params[layer], n_tok, c->sm_count, st) != cudaSuccess) return TWKV_ERR_CUDA;
+      if (launch_gate_rank(v, v.gate_scratch, levels, n_tok, st) != cudaSuccess) return TWKV_ERR_CUDA;
+    } else if (launch_gate_ranks_tc(v, maps, c->params[layer], n_tok, levels, c->sm_count, pairs, st) != cudaSuccess) return TWKV_ERR_CUDA;
   } else if (mode == TWKV_GATE_COMPUTE) {
     for (int lo = 0; lo < n_tok; lo += GATE_PIECE) {
       const int n = n_tok - lo < GATE_PIECE ? n_tok - lo : GATE_PIECE;

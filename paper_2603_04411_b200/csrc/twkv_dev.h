@@ -191,6 +191,7 @@ cudaError_t launch_decode(const DevView& v, int layer, const LayerParams& lp, co
 struct GateMaps;   // tensor maps of the fused gate kernel (api.cu)
 cudaError_t launch_gate_ranks_tc(const DevView& v, const GateMaps& maps, const LayerParams& lp, int n_tok, unsigned short* levels,
                                  int sm_count, bool pairs, cudaStream_t st);
+cudaError_t launch_gate_logits_tc(const DevView& v, const GateMaps& maps, const LayerParams& lp, int n_tok, int sm_count, cudaStream_t st);
 int gate_tc_max_pairs(int sm_count);
 size_t gate_tc_stage_bytes(int n_cta, int d);
 size_t gate_tc_fix_bytes();
