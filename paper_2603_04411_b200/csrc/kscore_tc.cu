@@ -33,7 +33,7 @@
 // All waits are bounded (tc_util.cuh); a wait that runs out ends the kernel with TWKV_ERR_TIMEOUT.
 //
 // Precision: X^_K, U_K^-1 keep the cache dtype with fp32 accumulation; queries enter the score product as
-// f16 (a bf16 query must be finite in f16), rotated keys as the sum of two f16 (21 significant bits; they
+// f16 (a bf16 query must be finite in f16), rotated keys as the sum of two f16 (22 significant bits; they
 // saturate at +-65504).
 #include "twkv_dev.h"
 #include "tc_util.cuh"
@@ -313,7 +313,7 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
             if (!(ok = mbar_wait_thin(kr_full + 8 * sbuf, sph, abort_flag))) break;
             if (!(ok = mbar_wait_thin(s_empty + 8 * slot, slph ^ 1u, abort_flag))) break;
             fence_after_sync();
-            // the rotated keys come as a high and a low f16 part (their sum carries 21 bits): two products into the same S,
+            // the rotated keys come as a high and a low f16 part (their sum carries 22 bits): two products into the same S,
             // the low one first (the tensor core cuts its fp32 sum after every instruction: half as many cuts at full size)
             const uint32_t kr = tmem_base + TM_SLAB + sbuf * 128, sd = tmem_base + TM_S + 16 * slot;
             mma_f16_ts_k128_cg<CG>(sd, kr + 64, q_lo0 + g * (1024 >> 4), KT_Q_PANEL_BYTES >> 4, idesc_s, 0u);

@@ -11,7 +11,7 @@
 //   row; per query the number of rows it may see.  Should two visible tokens of a sequence share a position, the rows of that
 //   sequence follow the K tiles instead and the causal mask compares positions.
 //
-// Precision: as in decode attention, keys are carried as two f16 (21 bits), queries as f16, softmax weights as two parts of
+// Precision: as in decode attention, keys are carried as two f16 (22 bits), queries as f16, softmax weights as two parts of
 // the cache type; values are two parts of the cache type as well (22 bits for f16, 16 for bf16), so that the result is the
 // spectral-space one to rounding.  The products high.high, high.low and low.high of weights and values are formed.
 //
