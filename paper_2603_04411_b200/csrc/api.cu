@@ -541,6 +541,7 @@ static twkv_status decode_pass(twkv_cache* c, int layer, const void* q, const in
   maps.blocks = c->map_blocks;
   maps.scores = c->scores_tma ? &c->map_scores : nullptr;
   maps.uinvT_k = c->map_uinvT[layer];
+  maps.uinv_k = c->pool + c->off.prep_uinvT + (size_t)layer * c->dims.d_kv * c->dims.d_kv * 2;
   DevView v = c->view;
   v.qmap = qmap; v.qpos = qpos;
   if (launch_decode(v, layer, c->params[layer], q, seq_ids, n_seq, out, num_splits, c->sm_count, &maps, c->kscore_pairs,

@@ -18,6 +18,13 @@ __global__ void __launch_bounds__(GG_THREADS, 1)
 gate_gemm_kernel(const unsigned short* Xk, const unsigned short* Xv, const unsigned short* Wk, const unsigned short* Wv, const float* bk,
                  const float* bv, int n_tok, int d, int ks_n, float* Z) {
   chain_start();
+  {
+    const size_t bytes = (size_t)d * d * 2;
+    const unsigned t = ((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * GG_THREADS + threadIdx.x;
+    const unsigned n = gridDim.x * gridDim.y * gridDim.z * GG_THREADS;
+    l2_prefetch(Wk, bytes, t, n);
+    l2_prefetch(Wv, bytes, t, n);
+  }
   chain_wait();
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned char* sA = smem;

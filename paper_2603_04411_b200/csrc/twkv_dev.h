@@ -155,6 +155,12 @@ struct DeviceGuard {
 // be moved before the wait.
 __device__ __forceinline__ void chain_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Asks for this thread's share of `bytes` bytes at `p` in L2, without waiting: before chain_wait(), so that matrices no kernel of the
+// chain writes (or whose copies are finished by an earlier one) come in while the kernel before still runs.
+__device__ __forceinline__ void l2_prefetch(const void* p, size_t bytes, unsigned thread, unsigned n_threads) {
+  for (size_t at = (size_t)thread * 128; at < bytes; at += (size_t)n_threads * 128)
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(p) + at));
+}
 template <class... P, class... A>
 cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, dim3 cluster, size_t smem, cudaStream_t st, A&&... args) {
   cudaLaunchConfig_t cfg = {};
