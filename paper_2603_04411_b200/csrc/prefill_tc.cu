@@ -674,10 +674,10 @@ pf_attn_kernel(const __grid_constant__ CUtensorMap map_seg, DevView v, PfCall a,
         };
         for (int i = blockIdx.x; i < n_items && ok; i += gridDim.x) {
           const PfItem it = pf_item(v, a, i, seg);
+          if (it.n_blk == 0) continue;                           // no hand-over of queries either, as in the softmax warps
           for (int h = 0; h < it.tiles && ok; ++h) { ok = mbar_wait(q_full + 8 * h, qph[h], abort_flag); qph[h] ^= 1u; }
           if (!ok) break;
           fence_after_sync();
-          if (it.n_blk == 0) continue;
           uint32_t kk[2], vv[2];
           if (!(ok = take(kk))) break;
           for (int h = 0; h < it.tiles; ++h) scores(h, kk);
@@ -720,35 +720,40 @@ pf_attn_kernel(const __grid_constant__ CUtensorMap map_seg, DevView v, PfCall a,
     for (int i = blockIdx.x; i < n_items && ok; i += gridDim.x) {
       const PfItem it = pf_item(v, a, i, seg);
       if (h >= it.tiles) continue;
-      // this warp's half of its 32 query rows as the K-major operand, four rows per instruction
+      // An item without key blocks hands nothing over: nothing would hold these warps back, and two items ahead of the other tile
+      // they would complete a phase of q_full that the issuer (which waits for the tiles in turn) has not seen.  With keys, o_done
+      // keeps them within one item.
+      if (it.n_blk > 0) {
+        // this warp's half of its 32 query rows as the K-major operand, four rows per instruction
 #pragma unroll 4
-      for (int k = 0; k < 8; ++k) {
-        const int r = quarter * 32 + 4 * k + (lane >> 3), k8 = lane & 7;
-        const int ch = hf * 4 + (k8 >> 1) + 8 * (k8 & 1);        // the keys' order: pairs of pieces 64 dims apart
-        const int ql = h * QT + r / rep;
-        uint4 val = make_uint4(0u, 0u, 0u, 0u);
-        if (ql < it.cnt)
-          val = reinterpret_cast<const uint4*>(q + ((size_t)a.qrow[it.first + ql] * v.Hq + it.g * rep + r % rep) * HEAD_DIM)[ch];
-        if constexpr (BF16) {
-          const unsigned w[4] = {val.x, val.y, val.z, val.w};
-          unsigned o[4];
-          bool over = false;
+        for (int k = 0; k < 8; ++k) {
+          const int r = quarter * 32 + 4 * k + (lane >> 3), k8 = lane & 7;
+          const int ch = hf * 4 + (k8 >> 1) + 8 * (k8 & 1);        // the keys' order: pairs of pieces 64 dims apart
+          const int ql = h * QT + r / rep;
+          uint4 val = make_uint4(0u, 0u, 0u, 0u);
+          if (ql < it.cnt)
+            val = reinterpret_cast<const uint4*>(q + ((size_t)a.qrow[it.first + ql] * v.Hq + it.g * rep + r % rep) * HEAD_DIM)[ch];
+          if constexpr (BF16) {
+            const unsigned w[4] = {val.x, val.y, val.z, val.w};
+            unsigned o[4];
+            bool over = false;
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float lo = __uint_as_float(w[e] << 16), hi = __uint_as_float(w[e] & 0xffff0000u);
-            over |= !(fabsf(lo) <= 65504.f) || !(fabsf(hi) <= 65504.f);
-            o[e] = pack_f16x2_sat(lo, hi);
+            for (int e = 0; e < 4; ++e) {
+              const float lo = __uint_as_float(w[e] << 16), hi = __uint_as_float(w[e] & 0xffff0000u);
+              over |= !(fabsf(lo) <= 65504.f) || !(fabsf(hi) <= 65504.f);
+              o[e] = pack_f16x2_sat(lo, hi);
+            }
+            if (over) set_status(v, TWKV_ERR_DEVICE_CHECK);        // a bf16 query beyond the f16 range would be clamped
+            val = make_uint4(o[0], o[1], o[2], o[3]);
           }
-          if (over) set_status(v, TWKV_ERR_DEVICE_CHECK);        // a bf16 query beyond the f16 range would be clamped
-          val = make_uint4(o[0], o[1], o[2], o[3]);
+          val.x = (val.x ^ flip) & keep_q; val.y = (val.y ^ flip) & keep_q; val.z = (val.z ^ flip) & keep_q; val.w = (val.w ^ flip) & keep_q;
+          *reinterpret_cast<uint4*>(sq + r * 128 + ((k8 ^ (r & 7)) << 4)) = val;
         }
-        val.x = (val.x ^ flip) & keep_q; val.y = (val.y ^ flip) & keep_q; val.z = (val.z ^ flip) & keep_q; val.w = (val.w ^ flip) & keep_q;
-        *reinterpret_cast<uint4*>(sq + r * 128 + ((k8 ^ (r & 7)) << 4)) = val;
+        fence_proxy_async_smem();
+        fence_before_sync();                                       // the previous item's accumulator has been read as well
+        __syncwarp();
+        if (lane == 0) mbar_arrive(q_full + 8 * h);
       }
-      fence_proxy_async_smem();
-      fence_before_sync();                                       // the previous item's accumulator has been read as well
-      __syncwarp();
-      if (lane == 0) mbar_arrive(q_full + 8 * h);
 
       const int ql = h * QT + row / rep;
       const int vis = ql < it.cnt ? a.qvis[it.first + ql] : 0;

@@ -6,7 +6,8 @@ import pytest
 import torch
 
 from paper_2603_04411_b200 import workloads
-from tests.test_gpu_prefill import MAX_ABS, REL_L2, B, _case
+from tests.helpers import GpuCache, attn_errors
+from tests.test_gpu_prefill import MAX_ABS, REL_L2, B, _case, _oracle_prefill
 
 pytestmark = pytest.mark.gpu
 
@@ -32,3 +33,41 @@ def test_tiled_prefill_where_the_work_split_changes(B, hkv, rep, dtype, n_seq, c
     q = torch.randn(n_seq * n_q, hkv * rep, 128, generator=torch.Generator().manual_seed(ctx)).to(dtype)
     (max_abs, rel_l2), _, _ = _case(B, li, ranks, q, q_seq, q_pos)
     assert max_abs < MAX_ABS and rel_l2 < REL_L2, (max_abs, rel_l2)
+
+
+def _filled(B, li, ranks, *, out_dtype=torch.float32, **cfg):
+    """A cache with the layer's tokens, one compress call."""
+    n_seq = int(li.seq_ids.max()) + 1
+    sizes = dict(max_seqs=n_seq, max_tokens_per_seq=int(np.bincount(li.seq_ids.numpy()).max()))
+    gc = GpuCache(B, n_layers=1, n_q_heads=li.n_q_heads, n_kv_heads=li.n_kv_heads, dtype=li.dtype, out_dtype=out_dtype,
+                  payload_bytes=int((-(-ranks // 64) * 128).sum()), **{**sizes, **cfg})
+    B.twkv_cache_set_layer_params(gc.h, 0, li.Uinv_k.cuda(), li.Uinv_v.cuda())
+    B.twkv_compress(gc.h, 0, li.xt_k.cuda(), li.xt_v.cuda(), li.seq_ids.cuda(), li.positions.cuda(), None,
+                    torch.from_numpy(ranks.astype(np.int16)).cuda(), B.TWKV_GATE_FORCED)
+    return gc
+
+
+def _prefill(B, gc, q, q_seq, q_pos, num_splits=0):
+    out = torch.full((len(q_seq), q.shape[1], 128), float("nan"), dtype={0: torch.float16, 1: torch.bfloat16, 2: torch.float32}[gc.cfg.out_dtype],
+                     device="cuda")
+    B.twkv_prefill_attn(gc.h, 0, q.cuda(), q_seq, q_pos, out, num_splits)
+    assert B.twkv_cache_status(gc.h) == B.TWKV_OK
+    return out.float().cpu().numpy()
+
+
+def test_tiled_prefill_with_many_items_that_have_no_keys(B):
+    # four sequences over two segments, four items per CTA: in the second segment three sequences out of four have no rows, so
+    # the CTAs meet such items one after the other, between items with keys
+    n_seq, ctx, n_q, hq = 4, 2100, 600, 64
+    li = workloads.build_layer(861, n_seq=n_seq, ctx=ctx, n_q_heads=hq, outlier="pct:1", mode="forced", level_probs=(0.05, 0.15, 0.4, 0.4))
+    ranks = li.ranks.numpy().astype(np.int64)
+    q_seq = np.repeat(np.arange(n_seq), n_q)
+    q_pos = np.tile(np.arange(ctx - n_q, ctx), n_seq)
+    q = torch.randn(n_seq * n_q, hq, 128, generator=torch.Generator().manual_seed(3)).to(torch.float16)
+    gc = _filled(B, li, ranks)
+    got = _prefill(B, gc, q, q_seq, q_pos)
+    assert np.all(np.isfinite(got))
+    pick = np.random.default_rng(4).choice(n_seq * n_q, 40, replace=False)
+    max_abs, rel_l2 = attn_errors(got[pick], _oracle_prefill(li, ranks, q[pick], q_seq[pick], q_pos[pick]))
+    assert max_abs < MAX_ABS and rel_l2 < REL_L2, (max_abs, rel_l2)
+    gc.close()
