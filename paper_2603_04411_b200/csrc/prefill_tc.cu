@@ -854,7 +854,7 @@ pf_attn_kernel(const __grid_constant__ CUtensorMap map_seg, DevView v, PfCall a,
       if (out) {
         // one split of one segment: this is the whole result.  A thread writes its row's 64 columns itself (4096-token prompt in four
         // calls 783 -> 751 us, five short prompts 204 -> 189 against partial results and the combine kernel).
-        const float inv = l > 0.f ? 1.f / l : 0.f;
+        const float inv = l == 0.f ? 0.f : 1.f / l;              // 0: no token seen; a NaN stays one
         const bool mine = ql < it.cnt;
         const size_t o0 = mine ? ((size_t)a.qrow[it.first + ql] * v.Hq + it.g * rep + row % rep) * HEAD_DIM + hf * 64 : 0;
 #pragma unroll 1
@@ -879,7 +879,7 @@ pf_attn_kernel(const __grid_constant__ CUtensorMap map_seg, DevView v, PfCall a,
         if (seg > 0) {
           const float mp = part[128 * TILE], lp = part[129 * TILE];
           named_bar_sync(pair_bar, 64);                          // both halves have read them
-          if (lp > 0.f) {
+          if (lp != 0.f) {                                       // (also a NaN, which the result must show)
             const float mm = fmaxf(m, mp);
             wo = m == -INFINITY ? 0.f : ex2(m - mm);
             wp = ex2(mp - mm);
@@ -937,7 +937,7 @@ __global__ void __launch_bounds__(256) pf_combine_kernel(DevView v, PfCall a, vo
   for (int c = 0; c < 16; ++c) acc[c] = 0.f;
   for (int k = 0; k < a.n_splits; ++k) {
     const float lk = part[k * stride + 129 * TILE], mk = part[k * stride + 128 * TILE];
-    if (!(lk > 0.f)) continue;
+    if (lk == 0.f) continue;                                      // nothing seen; a NaN goes into the sum
     float x[16];
 #pragma unroll
     for (int c = 0; c < 16; ++c) x[c] = part[k * stride + (c0 + cc + c) * TILE];
@@ -947,7 +947,7 @@ __global__ void __launch_bounds__(256) pf_combine_kernel(DevView v, PfCall a, vo
     for (int c = 0; c < 16; ++c) acc[c] = acc[c] * wo + x[c] * wk;
     m = mn;
   }
-  const float inv = l > 0.f ? 1.f / l : 0.f;
+  const float inv = l == 0.f ? 0.f : 1.f / l;
 #pragma unroll
   for (int c = 0; c < 16; ++c) s[row][cc + c] = acc[c] * inv;
   __syncthreads();

@@ -71,3 +71,28 @@ def test_tiled_prefill_with_many_items_that_have_no_keys(B):
     max_abs, rel_l2 = attn_errors(got[pick], _oracle_prefill(li, ranks, q[pick], q_seq[pick], q_pos[pick]))
     assert max_abs < MAX_ABS and rel_l2 < REL_L2, (max_abs, rel_l2)
     gc.close()
+
+
+@pytest.mark.parametrize("hkv,rep,ctx,n_q", [
+    (8, 4, 1000, 8),                             # several splits of one segment
+    (1, 8, 9000, 33),                            # several segments, then the join of their results
+    (2, 4, 100, 50),                             # one split of one segment is the whole result
+])
+def test_tiled_prefill_shows_a_key_that_is_not_a_number(B, hkv, rep, ctx, n_q):
+    # a NaN in one token's key: the queries that see the token get NaN, the others what they would get without it
+    bad = ctx // 3
+    li = workloads.build_layer(870 + ctx, n_seq=1, ctx=ctx, n_q_heads=hkv * rep, n_kv_heads=hkv, n_calib=256 * hkv, mode="forced", rank_recipe="any")
+    ranks = li.ranks.numpy().astype(np.int64)
+    q_pos = np.sort(np.random.default_rng(1).integers(0, ctx, n_q))
+    q_pos[0], q_pos[1], q_pos[-1] = bad - 1, bad, ctx - 1
+    q_seq = np.zeros(n_q, np.int64)
+    q = torch.randn(n_q, hkv * rep, 128, generator=torch.Generator().manual_seed(2)).to(torch.float16)
+    want = _oracle_prefill(li, ranks, q, q_seq, q_pos)
+    li.xt_k[(li.positions == bad).nonzero()[0], 0] = float("nan")
+    gc = _filled(B, li, ranks)
+    got = _prefill(B, gc, q, q_seq, q_pos)
+    gc.close()
+    sees = q_pos >= bad
+    assert np.all(np.isnan(got[sees]))
+    max_abs, rel_l2 = attn_errors(got[~sees], want[~sees])
+    assert max_abs < MAX_ABS and rel_l2 < REL_L2, (max_abs, rel_l2)
