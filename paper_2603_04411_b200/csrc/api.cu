@@ -600,6 +600,8 @@ static twkv_status prefill_tiled(twkv_cache* c, int layer, const void* q, const 
   a.krow = v.kv_link; a.krow_out = v.evict_map; a.vrow = v.evict_map + (size_t)v.NT * TILE;
   a.rowpos = (int*)v.scores;
   a.seg_buf = (unsigned char*)v.gate_scratch;
+  a.vexp = (signed char*)v.hist;                                    // 8448 bytes per KV head of at least 16384
+  a.vflag = (int*)(a.vexp + (size_t)GATE_PIECE * v.Hkv);
 
   if (rows_max > 32767ll * (GATE_PIECE / 2)) return TWKV_OK;         // a tile's segments are kept in two 16-bit halves
   // Segments of 8192 rows with the partial results in the V pass's region, or of 4096 rows with them in the second half of

@@ -28,6 +28,10 @@ struct PfCall {
   int *krow_out, *vrow; // [NT * 128] dense row of every K / V slot, -1 = not visible
   int* rowpos;          // [rows] position of a dense row
   unsigned char* seg_buf;   // [Hkv][4 parts][seg_rows][128] 16-bit
+  // the power of two a row's value was divided by before it was split, per KV head; segment + 1 of the last segment
+  // in which a block of 128 rows held one other than 0
+  signed char* vexp;    // [Hkv][seg_rows]
+  int* vflag;           // [seg_rows / 128][Hkv]
   float* slots;         // [blk_n * Hkv * n_splits][PF_SLOT_FLOATS]
 };
 struct PfMaps { CUtensorMap blocks, uk, uv, seg; };

@@ -11,12 +11,17 @@
 //   row; per query the number of rows it may see.  Should two visible tokens of a sequence share a position, the rows of that
 //   sequence follow the K tiles instead and the causal mask compares positions.
 //
-// Precision: as in decode attention, keys are carried as two f16 (22 bits), queries as f16, softmax weights as two parts of
-// the cache type; values are two parts of the cache type as well (22 bits for f16, 16 for bf16), so that the result is the
-// spectral-space one to rounding.  The products high.high, high.low and low.high of weights and values are formed.
+// Precision: as in decode attention, keys are carried as two f16 (22 bits) and queries as f16; softmax weights and values are two
+// f16 as well, whatever the cache type, so that the result is the spectral-space one to rounding.  The products high.high,
+// high.low and low.high of weights and values are formed.
+// A rebuilt value may lie outside f16 although the stored 16-bit components do not.  A row (token, KV head) whose largest value is
+// beyond 65504, or so small that the low parts would lose bits, is divided by a power of two before the split, and its softmax
+// weights carry that power; blocks of keys without such a row (nearly all, for values around 1) run as if there were none.
 //
 // Cost per 128 x 128 tile of (query row, token): 2 + 3 tensor-core units of 2 x 128^3 flop; the softmax of one tile runs
 // beside the products of the other.
+#include <type_traits>
+
 #include "twkv_dev.h"
 #include "tc_util.cuh"
 #include "scan_util.cuh"
@@ -35,6 +40,7 @@ __global__ void __launch_bounds__(1024) pf_init_kernel(DevView v, PfCall a) {
   for (int s = threadIdx.x; s < v.S; s += 1024) a.slot[s] = -1;
   __syncthreads();
   for (int u = threadIdx.x; u < a.n_u; u += 1024) { a.slot[a.seqs[3 * u]] = u; a.dup[u] = 0; }
+  for (int i = threadIdx.x; i < a.seg_rows / TILE * v.Hkv; i += 1024) a.vflag[i] = 0;
   if (threadIdx.x == 0) *a.ticket = 0;
 }
 
@@ -186,6 +192,11 @@ constexpr uint32_t PR_OUT_BYTES = 8192;                         // per warp: 32 
 constexpr int PR_ROPE_STRIDE = 33;                              // float4 per row of the small RoPE table (32 + 1 against bank conflicts)
 constexpr uint32_t PR_ROPE_BYTES = ROPE_LO * PR_ROPE_STRIDE * 16;
 constexpr uint32_t PR_SMEM = PR_STAGES * PR_STAGE_BYTES + 8 * PR_OUT_BYTES + PR_ROPE_BYTES + 8 * (2 * PR_STAGES + 4) + 16;
+// A row whose largest value lies outside these is scaled: a small one to [2^-3, 2^-2), a large one to [2^14, 2^15).  A part is exact
+// to 2^-25: values at the lower line keep 20 bits, scaled ones 22; scaled further up, their weights (which shrink by as much) would
+// lose bits beside those of rows that are not scaled.
+constexpr float PR_V_MIN = 0x1p-5f, PR_V_MAX = 65504.f;
+constexpr int PR_EXP_MIN = -90, PR_EXP_MAX = 113;               // 2^-e times a sum of weights stays an fp32 number
 // Panels summed into one accumulator; the sums of several accumulators are added in fp32 registers.  The tensor core cuts its
 // fp32 sum after every instruction (K = 16), so the error grows with the length of a chain.  K: eight panels, the length of
 // decode attention's passes, so that both round alike.  V: two panels; decode attention sums values over tokens, not over
@@ -198,6 +209,11 @@ __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) { uint64_t r; a
 __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) { uint64_t r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 __device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) { uint64_t r; asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) { uint64_t r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
+__device__ __forceinline__ float max_abs3(float a, uint32_t b, uint32_t c) {      // the largest magnitude
+  float r;
+  asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "r"(b), "r"(c));
+  return r;
+}
 __device__ __forceinline__ void unpk2(uint64_t v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
 // One work item = (tile, slab of NS = 256 output dims, i.e. two KV heads; 128 where d_kv is not a multiple of 256).
 // [128 x NS] accumulators alternate between two TMEM buffers; state panels (K-major A) and U^-1 atoms (rows of the caller's
@@ -367,9 +383,9 @@ pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_con
           *reinterpret_cast<uint4*>(d) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
           *reinterpret_cast<uint4*>(d + 4096) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
         };
-        auto rows_out = [&](int g) {                             // the warp's 32 half rows: four whole 128-byte pieces per instruction
+        auto rows_out = [&](int g, int half) {                   // the warp's 32 half rows: four whole 128-byte pieces per instruction
           __syncwarp();
-          unsigned char* dst = a.seg_buf + (g * 4 + side * 2) * plane + hf * 128 + (lane & 7) * 16;
+          unsigned char* dst = a.seg_buf + (g * 4 + side * 2) * plane + half * 128 + (lane & 7) * 16;
 #pragma unroll
           for (int k = 0; k < 8; ++k) {
             const int r = 4 * k + (lane >> 3);
@@ -453,21 +469,22 @@ pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_con
               stage_piece(2 * c, hi, lo);
               stage_piece(2 * c + 1, hi + 4, lo + 4);
             }
-            rows_out(g0 + hh);
+            rows_out(g0 + hh, hf);
           }
           ac += chains;
         } else {
-          // V: dims 64 hf .. + 63 of both heads, summed over the chains
+          // V, summed over the chains.  A thread takes its row of head hf whole, both halves, so that it sees the row's largest value by
+          // itself (finding it at a barrier of two half rows cost 7 % of the kernel); with one head per slab the two sets of warps take
+          // turns, tile by tile.
           uint32_t x[2][64];
           for (int ch = 0; ch < chains; ++ch, ++ac) {
             if (!(ok = wait_chain(ac))) break;
 #pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-              if (hh >= heads) break;
-              const uint32_t src = lane_addr + (ac & 1u) * 256 + hh * 128 + hf * 64;
+            for (int p = 0; p < 2; ++p) {
+              const uint32_t src = lane_addr + (ac & 1u) * 256 + (heads == 2 ? hf * 128 : 0) + p * 64;
               if (ch == 0) {
-                tmem_ld32(src, x[hh]);
-                tmem_ld32(src + 32, x[hh] + 32);
+                tmem_ld32(src, x[p]);
+                tmem_ld32(src + 32, x[p] + 32);
               } else {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
@@ -475,7 +492,7 @@ pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_con
                   tmem_ld16(src + 16 * e, y);
                   tmem_ld_wait();
 #pragma unroll
-                  for (int k = 0; k < 16; ++k) x[hh][16 * e + k] = __float_as_uint(__uint_as_float(x[hh][16 * e + k]) + __uint_as_float(y[k]));
+                  for (int k = 0; k < 16; ++k) x[p][16 * e + k] = __float_as_uint(__uint_as_float(x[p][16 * e + k]) + __uint_as_float(y[k]));
                 }
               }
             }
@@ -483,17 +500,34 @@ pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_con
             free_chain(ac);
           }
           if (!ok) break;
+          float mx[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-          for (int hh = 0; hh < 2; ++hh) {
-            if (hh >= heads) break;
+          for (int k = 0; k < 128; k += 2) mx[(k >> 1) & 3] = max_abs3(mx[(k >> 1) & 3], x[k >> 6][k & 63], x[k >> 6][(k & 63) + 1]);
+          const float top = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+          int e = 0;                                             // (an infinite row is left as it is)
+          if ((top > PR_V_MAX && top < INFINITY) || (top < PR_V_MIN && top > 0.f))
+            e = max((int)(__float_as_uint(top) >> 23) - 127 + (top < 1.f ? 3 : -14), PR_EXP_MIN);
+          const int g = heads == 2 ? g0 + hf : g0;
+          if (heads == 1 && (t & 1) != hf) local = -1;           // (leaving the branch here instead cost 12 % of the kernel in spills)
+          if (local >= 0) {
+            a.vexp[(size_t)g * a.seg_rows + local] = (signed char)e;
+            if (e != 0) a.vflag[(local / TILE) * v.Hkv + g] = seg + 1;
+          }
+          if (__any_sync(0xffffffffu, e != 0)) {
+            const float f = __uint_as_float((uint32_t)(127 - e) << 23);
+#pragma unroll
+            for (int k = 0; k < 128; ++k) x[k >> 6][k & 63] = __float_as_uint(__uint_as_float(x[k >> 6][k & 63]) * f);
+          }
+#pragma unroll
+          for (int p = 0; p < 2; ++p) {
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
               uint32_t hi[4], lo[4];
 #pragma unroll
-              for (int k = 0; k < 4; ++k) split_pair_16<BF16>(pk2u(x[hh][8 * c + 2 * k], x[hh][8 * c + 2 * k + 1]), hi[k], lo[k]);
+              for (int k = 0; k < 4; ++k) split_pair_16<false, false>(pk2u(x[p][8 * c + 2 * k], x[p][8 * c + 2 * k + 1]), hi[k], lo[k]);
               stage_piece(c, hi, lo);
             }
-            rows_out(g0 + hh);
+            rows_out(g, p);
           }
         }
       }
@@ -636,7 +670,7 @@ pf_attn_kernel(const __grid_constant__ CUtensorMap map_seg, DevView v, PfCall a,
       // ------------------------------------------------------------- MMA issuer (one elected lane)
       if (elect_one()) {
         constexpr uint32_t idesc_s = idesc_f16(0, 128, 128);                            // f16 queries and keys, both K-major
-        constexpr uint32_t idesc_o = idesc_f16(BF16 ? 1 : 0, 128, 128) | (1u << 16);    // values MN-major
+        constexpr uint32_t idesc_o = idesc_f16(0, 128, 128) | (1u << 16);               // values MN-major
         uint32_t st = 0, ph = 0, qph[2] = {0, 0}, pph[2] = {0, 0};
         bool ok = true;
         // two consecutive stages (both parts of a block of keys or values)
@@ -761,6 +795,7 @@ pf_attn_kernel(const __grid_constant__ CUtensorMap map_seg, DevView v, PfCall a,
       float m = -INFINITY;
       uint64_t l2 = 0;                                           // two partial sums of this half's weights
       for (int j = 0; j < it.n_blk; ++j) {
+        const int flag = a.vflag[((it.row_lo >> 7) + j) * v.Hkv + it.g];         // (on its way while the scores are waited for)
         ok = __all_sync(0xffffffffu, mbar_wait(s_full + 8 * h, sph, abort_flag));
         sph ^= 1u;
         fence_after_sync();
@@ -783,6 +818,22 @@ pf_attn_kernel(const __grid_constant__ CUtensorMap map_seg, DevView v, PfCall a,
           }
 #pragma unroll
           for (int c = 0; c < 64; ++c) x[c] = (see[c >> 5] >> (c & 31)) & 1u ? x[c] : 0xff800000u;
+        }
+        // Scaled rows: a score takes its row's power of two along, so that maximum and weights are those of weight x value; the
+        // sum of the weights leaves it out again.
+        const bool scaled = flag == seg + 1;
+        auto exps = [&](int c) -> int4 {                          // of columns 16 c .. 16 c + 15
+          return reinterpret_cast<const int4*>(a.vexp + (size_t)it.g * a.seg_rows + it.row_lo + j * TILE + hf * 64)[c];
+        };
+        if (scaled) {
+          const float inv_scale = fminf(1.f / scale, 1e30f);
+#pragma unroll
+          for (int c = 0; c < 64; c += 16) {
+            const int4 w = exps(c >> 4);
+            const int e4[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+            for (int k = 0; k < 16; ++k) x[c + k] = __float_as_uint(__uint_as_float(x[c + k]) + (float)(signed char)(e4[k >> 2] >> (8 * (k & 3))) * inv_scale);
+          }
         }
         float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
@@ -821,19 +872,35 @@ pf_attn_kernel(const __grid_constant__ CUtensorMap map_seg, DevView v, PfCall a,
         }
         const float mu = m == -INFINITY ? 0.f : m;
         const uint64_t nm2 = pk2(-mu, -mu), sc2 = pk2(scale, scale);
+        auto weights = [&](auto with_exps) {
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          uint32_t w[16];                                        // 8 columns of high parts, 8 of low ones, over the scores they come from
+          for (int c = 0; c < 4; ++c) {
+            uint32_t w[16];                                      // 8 columns of high parts, 8 of low ones, over the scores they come from
+            int4 ex = make_int4(0, 0, 0, 0);
+            if constexpr (with_exps.value) ex = exps(c);
+            const int e4[4] = {ex.x, ex.y, ex.z, ex.w};
 #pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            float p0, p1;
-            unpk2(fma2(pk2u(x[16 * c + 2 * k], x[16 * c + 2 * k + 1]), sc2, nm2), p0, p1);
-            const uint64_t p = pk2(ex2(p0), ex2(p1));
-            l2 = add2(l2, p);
-            split_pair_16<BF16>(p, w[k], w[8 + k]);
+            for (int k = 0; k < 8; ++k) {
+              float p0, p1;
+              unpk2(fma2(pk2u(x[16 * c + 2 * k], x[16 * c + 2 * k + 1]), sc2, nm2), p0, p1);
+              const uint64_t p = pk2(ex2(p0), ex2(p1));
+              if constexpr (with_exps.value) {
+                float f[2];
+#pragma unroll
+                for (int b = 0; b < 2; ++b) {                     // (bytes of rows that hold no token may be anything: their weight is 0)
+                  const int e = min(max((int)(signed char)(e4[k >> 1] >> (16 * (k & 1) + 8 * b)), PR_EXP_MIN), PR_EXP_MAX);
+                  f[b] = __uint_as_float((uint32_t)(127 - e) << 23);
+                }
+                l2 = fma2(p, pk2(f[0], f[1]), l2);
+              } else {
+                l2 = add2(l2, p);
+              }
+              split_pair_16<false>(p, w[k], w[8 + k]);
+            }
+            tmem_st16(tS + 16 * c, w);
           }
-          tmem_st16(tS + 16 * c, w);
-        }
+        };
+        if (scaled) weights(std::true_type{}); else weights(std::false_type{});
         tmem_st_wait();
         fence_before_sync();
         __syncwarp();

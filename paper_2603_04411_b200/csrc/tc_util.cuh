@@ -272,8 +272,13 @@ __device__ __forceinline__ uint32_t pack_f16x2_sat(float lo, float hi) {
 // The differences are mixed-precision operations on the packed result: nothing is masked or converted back, two instructions
 // per value instead of three (K-score kernel, whose rotating warps are bound by the instructions they issue: 385 -> 367 us
 // for 16 x 32768 against a high part cut by a mask).
-template <bool BF16> __device__ __forceinline__ void split_pair_16(uint64_t v, uint32_t& hi, uint32_t& lo) {
-  if constexpr (BF16) {
+// f16 saturates unless SAT is false (an infinite value then leaves as an infinity and a NaN).
+template <bool BF16, bool SAT = true> __device__ __forceinline__ void split_pair_16(uint64_t v, uint32_t& hi, uint32_t& lo) {
+  if constexpr (!BF16 && !SAT) {
+    asm("{\n\t.reg .f32 a, b, c, d;\n\t.reg .b16 p, q, m;\n\tmov.b64 {a, b}, %2;\n\tcvt.rn.f16x2.f32 %0, b, a;\n\t"
+        "mov.b32 {p, q}, %0;\n\tmov.b16 m, 0xBC00;\n\tfma.rn.f32.f16 c, p, m, a;\n\tfma.rn.f32.f16 d, q, m, b;\n\t"
+        "cvt.rn.f16x2.f32 %1, d, c;\n\t}" : "=&r"(hi), "=r"(lo) : "l"(v));
+  } else if constexpr (BF16) {
     asm("{\n\t.reg .f32 a, b, c, d;\n\t.reg .b16 p, q, m;\n\tmov.b64 {a, b}, %2;\n\tcvt.rn.bf16x2.f32 %0, b, a;\n\t"
         "mov.b32 {p, q}, %0;\n\tmov.b16 m, 0xBF80;\n\tfma.rn.f32.bf16 c, p, m, a;\n\tfma.rn.f32.bf16 d, q, m, b;\n\t"
         "cvt.rn.bf16x2.f32 %1, d, c;\n\t}" : "=&r"(hi), "=r"(lo) : "l"(v));

@@ -96,3 +96,41 @@ def test_tiled_prefill_shows_a_key_that_is_not_a_number(B, hkv, rep, ctx, n_q):
     assert np.all(np.isnan(got[sees]))
     max_abs, rel_l2 = attn_errors(got[~sees], want[~sees])
     assert max_abs < MAX_ABS and rel_l2 < REL_L2, (max_abs, rel_l2)
+
+
+@pytest.mark.parametrize("hkv,rep,dtype,ctx,n_q,x_scale,u_scale,every", [
+    (8, 4, torch.float16, 500, 150, 2.0 ** -13, 1.0, 1),       # values around 1e-4: one f16 low part would keep 12 bits of them
+    (8, 4, torch.float16, 500, 8, 2.0 ** 11, 64.0, 37),        # one token in 37 with values around 1e5, beyond f16; several splits
+    (3, 2, torch.float16, 300, 100, 2.0 ** 11, 64.0, 2),       # one head per slab
+    (1, 8, torch.float16, 9000, 33, 2.0 ** -10, 1.0, 3),       # several segments, large and small values mixed
+    (2, 4, torch.bfloat16, 200, 50, 2.0 ** 40, 1.0, 2),        # bf16 states far beyond f16
+])
+def test_tiled_prefill_values_of_any_size(B, hkv, rep, dtype, ctx, n_q, x_scale, u_scale, every):
+    # Rebuilt values are carried as two f16; their size must not cost precision.  fp32 output, so that nothing hides it: keys and
+    # weights of 22 bits with scores of a few tens (2^-21 x 20) and the fp32 sums stay below 2e-5, values clamped or without a low
+    # part give 1e-4 and more.
+    li = workloads.build_layer(880 + ctx, n_seq=1, ctx=ctx, n_q_heads=hkv * rep, n_kv_heads=hkv, n_calib=256 * hkv, dtype=dtype, mode="forced",
+                               rank_recipe="any")
+    li.xt_v[::every] = (li.xt_v[::every].float() * x_scale).to(dtype)
+    li.Uinv_v = (li.Uinv_v.float() * u_scale).to(dtype)
+    ranks = li.ranks.numpy().astype(np.int64)
+    q_pos = np.sort(np.random.default_rng(1).integers(0, ctx, n_q))
+    q_seq = np.zeros(n_q, np.int64)
+    q = torch.randn(n_q, hkv * rep, 128, generator=torch.Generator().manual_seed(2)).to(dtype)
+    gc = _filled(B, li, ranks)
+    got = _prefill(B, gc, q, q_seq, q_pos)
+    gc.close()
+    _, rel_l2 = attn_errors(got, _oracle_prefill(li, ranks, q, q_seq, q_pos))
+    assert rel_l2 < 2e-5, rel_l2
+
+
+def test_tiled_prefill_shows_an_infinite_value(B):
+    li = workloads.build_layer(885, n_seq=1, ctx=300, n_q_heads=32, mode="forced", rank_recipe="any")
+    ranks = li.ranks.numpy().astype(np.int64)
+    li.xt_v[(li.positions == 200).nonzero()[0], 0] = float("inf")
+    gc = _filled(B, li, ranks)
+    q_pos = np.arange(100, 300)
+    got = _prefill(B, gc, torch.ones(200, 32, 128, dtype=torch.float16), np.zeros(200, np.int64), q_pos)
+    gc.close()
+    assert not np.isfinite(got[q_pos >= 200]).any()
+    assert np.isfinite(got[q_pos < 128]).all()                 # (a block of keys that the token is not in)
