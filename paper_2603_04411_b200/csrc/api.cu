@@ -235,6 +235,8 @@ struct twkv_cache {
   bool scores_tma = false;             // the head count allows that map (rows must start on 16-byte boundaries)
   std::vector<CUtensorMap> map_uinvT;  // per layer, over the transposed copy of U_K^-1 inside the pool
   std::vector<char> prepared;          // per layer: transposed copy and its map are current
+  std::vector<CUtensorMap> map_w;      // per layer x side, over the caller's gate weights (boxes of 64 rows)
+  std::vector<char> mapped_w;          // per layer: those maps are current
   std::vector<CUtensorMap> map_wT;     // per layer x side, over the transposed copies of the gate weights (box = one slab)
   std::vector<CUtensorMap> map_wT_half; // the same with 128-row boxes, for the CTA-pair kernel
   std::vector<char> prepared_w;        // per layer: those copies and maps are current
@@ -363,6 +365,8 @@ twkv_status twkv_cache_create(const twkv_config* cfg, void* pool, size_t pool_by
   }
   c->map_uinvT.resize(cfg->n_layers);
   c->prepared.assign(cfg->n_layers, 0);
+  c->map_w.resize(2 * (size_t)cfg->n_layers);
+  c->mapped_w.assign(cfg->n_layers, 0);
   c->map_wT.resize(2 * (size_t)cfg->n_layers);
   c->map_wT_half.resize(2 * (size_t)cfg->n_layers);
   c->prepared_w.assign(cfg->n_layers, 0);
@@ -435,6 +439,7 @@ twkv_status twkv_cache_set_layer_params(twkv_cache* c, int layer, const twkv_lay
   c->params[layer] = LayerParams{p->Uinv_k, p->Uinv_v, p->W_k, p->W_v, p->b_k, p->b_v};
   c->prepared[layer] = 0;
   c->prepared_w[layer] = 0;
+  c->mapped_w[layer] = 0;
   return TWKV_OK;
 }
 
@@ -458,12 +463,22 @@ twkv_status twkv_compress(twkv_cache* c, int layer, const void* K, const void* V
   c->appended[layer].fetch_add(n_tok, std::memory_order_relaxed);
   if (mode == TWKV_GATE_LOGITS) {
     if (launch_gate_rank(v, scores, levels, n_tok, st) != cudaSuccess) return TWKV_ERR_CUDA;
-  } else if (mode == TWKV_GATE_COMPUTE && n_tok >= GATE_LOGITS_TC_MIN && c->sm_count <= 160 &&
-             (n_tok > GATE_LOGITS_TC_MAX || c->prepared_w[layer] || !is_capturing(st))) {
-    // up to GATE_LOGITS_TC_MAX tokens: tcgen05 logits spread over all SMs, then the rank kernel (a call that is captured before the
-    // weights were laid out reads them as they are, below); above: fused tcgen05 kernel, logits and ranks in one launch, the logits
-    // never leave the CTA's staging block
-    const bool spread = n_tok <= GATE_LOGITS_TC_MAX;
+  } else if (mode == TWKV_GATE_COMPUTE && n_tok >= GATE_LOGITS_TC_MIN && n_tok <= GATE_LOGITS_TC_MAX) {
+    // tcgen05 logits spread over all SMs, then the rank kernel; the weights are read as they lie
+    const uint64_t d = (uint64_t)c->dims.d_kv;
+    const LayerParams& lp = c->params[layer];
+    CUtensorMap* mw = &c->map_w[2 * (size_t)layer];
+    if (!c->mapped_w[layer]) {
+      if (!make_tmap_2d(mw, lp.W_k, d, d, d * 2, PANEL) || !make_tmap_2d(mw + 1, lp.W_v, d, d, d * 2, PANEL)) return TWKV_ERR_CUDA;
+      c->mapped_w[layer] = 1;
+    }
+    GateMaps maps;
+    maps.wk = mw[0]; maps.wv = mw[1];
+    if (!make_tmap_2d(&maps.xk, K, (uint64_t)n_tok, d, d * 2, TILE) || !make_tmap_2d(&maps.xv, V, (uint64_t)n_tok, d, d * 2, TILE)) return TWKV_ERR_CUDA;
+    if (launch_gate_logits_tc(v, maps, lp, n_tok, c->sm_count, st) != cudaSuccess) return TWKV_ERR_CUDA;
+    if (launch_gate_rank(v, v.gate_scratch, levels, n_tok, st) != cudaSuccess) return TWKV_ERR_CUDA;
+  } else if (mode == TWKV_GATE_COMPUTE && n_tok > GATE_LOGITS_TC_MAX && c->sm_count <= 160) {
+    // fused tcgen05 kernel: logits and ranks in one launch, the logits never leave the CTA's staging block
     const int d = c->dims.d_kv;
     if (!c->prepared_w[layer]) {
       // first COMPUTE call after the parameters were (re)set: K-major copies of W_k, W_v for the tensor cores
@@ -478,17 +493,14 @@ twkv_status twkv_compress(twkv_cache* c, int layer, const void* K, const void* V
     }
     const bool pairs = d % 256 == 0 && gate_tc_max_pairs(c->sm_count) > 0;
     GateMaps maps;
-    maps.wk = (pairs || spread ? c->map_wT_half : c->map_wT)[2 * (size_t)layer];
-    maps.wv = (pairs || spread ? c->map_wT_half : c->map_wT)[2 * (size_t)layer + 1];
+    maps.wk = (pairs ? c->map_wT_half : c->map_wT)[2 * (size_t)layer];
+    maps.wv = (pairs ? c->map_wT_half : c->map_wT)[2 * (size_t)layer + 1];
     if (!make_tmap_2d(&maps.xk, K, (uint64_t)n_tok, d, (uint64_t)d * 2, TILE) ||
         !make_tmap_2d(&maps.xv, V, (uint64_t)n_tok, d, (uint64_t)d * 2, TILE)) return TWKV_ERR_CUDA;
     const unsigned char* wT = c->pool + c->off.prep_wT + (size_t)layer * 2 * d * d * 2;
     maps.raw = GateRaw{(const unsigned short*)K, (const unsigned short*)V, (const unsigned short*)wT,
                        (const unsigned short*)(wT + (size_t)d * d * 2), v.gate_fix, v.status + 2};
-    if (spread) {
-      if (launch_gate_logits_tc(v, maps, c->params[layer], n_tok, c->sm_count, st) != cudaSuccess) return TWKV_ERR_CUDA;
-      if (launch_gate_rank(v, v.gate_scratch, levels, n_tok, st) != cudaSuccess) return TWKV_ERR_CUDA;
-    } else if (launch_gate_ranks_tc(v, maps, c->params[layer], n_tok, levels, c->sm_count, pairs, st) != cudaSuccess) return TWKV_ERR_CUDA;
+    if (launch_gate_ranks_tc(v, maps, c->params[layer], n_tok, levels, c->sm_count, pairs, st) != cudaSuccess) return TWKV_ERR_CUDA;
   } else if (mode == TWKV_GATE_COMPUTE) {
     for (int lo = 0; lo < n_tok; lo += GATE_PIECE) {
       const int n = n_tok - lo < GATE_PIECE ? n_tok - lo : GATE_PIECE;

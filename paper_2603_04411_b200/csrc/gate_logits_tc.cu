@@ -5,8 +5,9 @@
 // tiles; the warp-MMA kernel of the small calls is bound by its own issue from a few hundred tokens on.  With an output tile of
 // 128 x 128 per item 1024 tokens of d_kv 1024 fill 128 SMs, and the logits' way through L2 (8 KB per token, both sides) costs less
 // than the idle SMs did: a compress call of 1024 tokens takes 46.3 us (warp-MMA 67.6, fused 61.8).  A short call is bound by its
-// chain of launches and the latency of one item (16 K panels through the ring).  The main loop is the ring of tc_util.cuh (M 128,
-// N 128, K 16); the weights are the transposed copies the fused kernel reads.
+// chain of launches and the latency of one item (16 K panels through the ring).  A ring stage is one K = 64 panel of the states
+// (K-major) and of the weights, whose rows are read as the caller's matrix has them (MN-major: two atoms of [64 rows][64 columns]),
+// so that the logits are those of the weights at the time of the call and a first call needs no copies of them.
 // Warp roles (320 threads): 0 TMA producer, 1 MMA issuer, 2-9 epilogue (thread = one token row x half of the columns).
 // All waits are bounded (tc_util.cuh); a wait that runs out ends the kernel with TWKV_ERR_TIMEOUT.
 #include "twkv_dev.h"
@@ -17,7 +18,7 @@ using namespace tc;
 
 constexpr int GL_THREADS = 320;
 constexpr int GL_STAGES = 6;
-constexpr uint32_t GL_PANEL_BYTES = 16384, GL_STAGE_BYTES = 2 * GL_PANEL_BYTES;
+constexpr uint32_t GL_PANEL_BYTES = 16384, GL_ATOM_BYTES = GL_PANEL_BYTES / 2, GL_STAGE_BYTES = 2 * GL_PANEL_BYTES;
 constexpr uint32_t GL_SMEM = GL_STAGES * GL_STAGE_BYTES + 8 * (2 * GL_STAGES + 4) + 16;
 
 __global__ void __launch_bounds__(GL_THREADS, 1)
@@ -50,25 +51,58 @@ gate_logits_tc_kernel(const __grid_constant__ CUtensorMap map_xk, const __grid_c
 
   // item -> (token tile, side, slab): slab fastest, then side, so that neighbouring CTAs read the same tokens
   const int per_tile = 2 * n_slabs, n_items = per_tile * ((n_tok + TILE - 1) / TILE), it0 = blockIdx.x, itstep = gridDim.x;
-  const uint32_t n_acc = it0 < n_items ? (uint32_t)((n_items - it0 + itstep - 1) / itstep) : 0u;
 
   if (misaligned) {
     // nothing was started
   } else if (warp == 0) {
-    if (elect_one())
-      ring_gemm_produce<1>(n_acc, KP, GL_STAGES, sA, GL_STAGE_BYTES, GL_PANEL_BYTES, GL_STAGE_BYTES, full, empty, 0u, abort_flag,
-                           [&](uint32_t a, const CUtensorMap*& mx, const CUtensorMap*& mw, int& m0, int& n0) {
-                             const int it = it0 + (int)a * itstep, rem = it % per_tile;
-                             mx = rem >= n_slabs ? &map_xv : &map_xk;
-                             mw = rem >= n_slabs ? &map_wv : &map_wk;
-                             m0 = (it / per_tile) * TILE;
-                             n0 = (rem % n_slabs) * 128;
-                           });
+    if (elect_one()) {
+      uint32_t st = 0, ph = 0, n_loaded = 0;
+      bool ok = true;
+      for (int it = it0; it < n_items && ok; it += itstep) {
+        const int rem = it % per_tile, m0 = (it / per_tile) * TILE, n0 = (rem % n_slabs) * 128;
+        const CUtensorMap *mx = rem >= n_slabs ? &map_xv : &map_xk, *mw = rem >= n_slabs ? &map_wv : &map_wk;
+        for (int p = 0; p < KP; ++p, ++n_loaded) {
+          if (!(ok = mbar_wait_thin(empty + 8 * st, ph ^ 1u, abort_flag))) break;
+          const uint32_t dst = sA + st * GL_STAGE_BYTES;
+          mbar_expect_tx(full + 8 * st, GL_STAGE_BYTES);
+          tma_load_2d(dst, mx, full + 8 * st, p * PANEL, m0);
+          tma_load_2d(dst + GL_PANEL_BYTES, mw, full + 8 * st, n0, p * PANEL);
+          tma_load_2d(dst + GL_PANEL_BYTES + GL_ATOM_BYTES, mw, full + 8 * st, n0 + 64, p * PANEL);
+          if (++st == GL_STAGES) { st = 0; ph ^= 1u; }
+        }
+      }
+      if (!ok)                                                  // let copies in flight land before the CTA goes away
+        for (uint32_t i = 0; i < GL_STAGES && i < n_loaded; ++i) {
+          const uint32_t n = n_loaded - 1 - i;
+          mbar_wait_drain(full + 8 * (n % GL_STAGES), (n / GL_STAGES) & 1u);
+        }
+    }
     __syncwarp();
   } else if (warp == 1) {
-    if (elect_one())
-      ring_gemm_issue<1>(n_acc, KP, GL_STAGES, sA, GL_STAGE_BYTES, GL_PANEL_BYTES, idesc_f16(bf16 ? 1 : 0, 128, 128), tmem_base, full, empty,
-                         acc_full, acc_empty, abort_flag);
+    if (elect_one()) {
+      const uint32_t idesc = idesc_f16(bf16 ? 1 : 0, 128, 128) | (1u << 16);            // B MN-major
+      uint32_t st = 0, ph = 0, ac = 0;
+      bool ok = true;
+      for (int it = it0; it < n_items && ok; it += itstep, ++ac) {
+        const uint32_t buf = ac & 1u;
+        if (!(ok = mbar_wait(acc_empty + 8 * buf, ((ac >> 1) & 1u) ^ 1u, abort_flag))) break;
+        fence_after_sync();
+        for (int p = 0; p < KP; ++p) {
+          if (!(ok = mbar_wait(full + 8 * st, ph, abort_flag))) break;
+          fence_after_sync();
+          const uint32_t a_lo = kmajor_sw128_desc_lo(sA + st * GL_STAGE_BYTES), sb = sA + st * GL_STAGE_BYTES + GL_PANEL_BYTES;
+#pragma unroll
+          for (int ks = 0; ks < 4; ++ks) {
+            const uint32_t b_lo = (((sb + ks * 2048u) >> 4) & 0x3fffu) | ((GL_ATOM_BYTES >> 4) << 16);
+            mma_f16_ss(tmem_base + buf * 256, ((uint64_t)KMAJOR_SW128_DESC_HI << 32) | (a_lo + 2 * ks), ((uint64_t)KMAJOR_SW128_DESC_HI << 32) | b_lo,
+                       idesc, (p > 0 || ks > 0) ? 1u : 0u);
+          }
+          mma_commit(empty + 8 * st);
+          if (++st == GL_STAGES) { st = 0; ph ^= 1u; }
+        }
+        if (ok) mma_commit(acc_full + 8 * buf);
+      }
+    }
     __syncwarp();
   } else {
     const int quarter = warp & 3, half = (warp - 2) >> 2, row = quarter * 32 + lane;
@@ -106,7 +140,7 @@ gate_logits_tc_kernel(const __grid_constant__ CUtensorMap map_xk, const __grid_c
   if (tid == 0 && *abort_flag) atomicCAS(status, 0, misaligned ? TWKV_ERR_DEVICE_CHECK : TWKV_ERR_TIMEOUT);
 }
 
-// maps: states with boxes of 128 tokens, transposed weights with boxes of 128 rows.
+// maps: states with boxes of 128 tokens, weights as the caller has them with boxes of 64 rows.
 cudaError_t launch_gate_logits_tc(const DevView& v, const GateMaps& maps, const LayerParams& lp, int n_tok, int sm_count, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(gate_logits_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GL_SMEM);
   if (e != cudaSuccess) return e;
