@@ -489,7 +489,7 @@ twkv_status twkv_compress(twkv_cache* c, int layer, const void* K, const void* V
         if (!make_tmap_2d(&c->map_wT[2 * (size_t)layer + side], dst, d, d, (uint64_t)d * 2, ns) ||
             !make_tmap_2d(&c->map_wT_half[2 * (size_t)layer + side], dst, d, d, (uint64_t)d * 2, TILE)) return TWKV_ERR_CUDA;
       }
-      c->prepared_w[layer] = 1;
+      c->prepared_w[layer] = !is_capturing(st);            // a captured copy exists only once its graph runs, and then before its readers
     }
     const bool pairs = d % 256 == 0 && gate_tc_max_pairs(c->sm_count) > 0;
     GateMaps maps;
@@ -547,7 +547,7 @@ static twkv_status decode_pass(twkv_cache* c, int layer, const void* q, const in
     // box = a whole panel for the single-CTA kernel, the CTA's half of its rows for the pair kernel
     if (!make_tmap_2d(&c->map_uinvT[layer], dst, (uint64_t)c->dims.NC * c->dims.d_kv, PANEL, PANEL * 2,
                       c->kscore_pairs ? HEAD_DIM / 2 : HEAD_DIM)) return TWKV_ERR_CUDA;
-    c->prepared[layer] = 1;
+    c->prepared[layer] = !is_capturing((cudaStream_t)stream);      // (as for the gate weights)
   }
   TcMaps maps;
   maps.blocks = c->map_blocks;
