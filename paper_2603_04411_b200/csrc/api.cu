@@ -525,15 +525,14 @@ static twkv_status decode_pass(twkv_cache* c, int layer, const void* q, const in
   if (n_seq > c->cfg.max_seqs) return TWKV_ERR_INVALID_ARG;
   if (!c->params[layer].Uinv_k || !c->params[layer].Uinv_v) return TWKV_ERR_INVALID_ARG;
   const int head_groups = (c->cfg.n_q_heads + 31) / 32;
+  int min_splits = 0;
   if (num_splits == 0) {
     num_splits = c->sm_count / (n_seq * head_groups);
-    if (num_splits < 1) num_splits = 1;
-    // every split writes, and the merge reads, 4 n_q_heads d_kv bytes: twelve splits are enough for a short sequence, then one per
-    // 512 tokens (4 sequences of 1000 tokens: 37 splits 73.5 us, 12 splits 69.9, 4 splits 73.8; 4 of 8192: 37 splits 96.3, 16
-    // splits 95.6; one of 4096: 12 splits 55.4, 16 to 64 53.4; one of 131072 wants 64)
-    long long tokens = c->cfg.max_tokens_per_seq;
-    if (!c->append_captured.load(std::memory_order_relaxed)) tokens = std::min(tokens, c->appended[layer].load(std::memory_order_relaxed) / n_seq);
-    num_splits = (int)std::min<long long>(num_splits, std::max<long long>(n_seq > 1 ? 12 : 16, tokens / 512));
+    // every split writes, and the merge reads, 4 n_q_heads d_kv bytes: the plan uses min_splits of them for a short sequence, then one
+    // per DECODE_SPLIT_TOKENS of its tokens (4 sequences of 1000 tokens: 37 splits 73.5 us, 12 splits 69.9, 4 splits 73.8; 4 of 8192:
+    // 37 splits 96.3, 16 splits 95.6; one of 4096: 12 splits 55.4, 16 to 64 53.4; one of 131072 wants 64)
+    min_splits = n_seq > 1 ? 12 : 16;
+    num_splits = std::max(1, std::min(num_splits, std::max(min_splits, c->cfg.max_tokens_per_seq / DECODE_SPLIT_TOKENS)));
     if (num_splits > 64) num_splits = 64;
   }
   if ((long long)n_seq * num_splits > c->dims.max_partials) return TWKV_ERR_INVALID_ARG;
@@ -556,7 +555,7 @@ static twkv_status decode_pass(twkv_cache* c, int layer, const void* q, const in
   maps.uinv_k = c->pool + c->off.prep_uinvT + (size_t)layer * c->dims.d_kv * c->dims.d_kv * 2;
   DevView v = c->view;
   v.qmap = qmap; v.qpos = qpos;
-  if (launch_decode(v, layer, c->params[layer], q, seq_ids, n_seq, out, num_splits, c->sm_count, &maps, c->kscore_pairs,
+  if (launch_decode(v, layer, c->params[layer], q, seq_ids, n_seq, out, num_splits, min_splits, c->sm_count, &maps, c->kscore_pairs,
                     (cudaStream_t)stream) != cudaSuccess) return TWKV_ERR_CUDA;
   return TWKV_OK;
 }

@@ -39,7 +39,10 @@ __device__ __forceinline__ unsigned ktile_cost(int cls) { return kTileCost[min(m
 // classes 1 to 16 dealt out by count alone left the slowest CTA with half as much again as the mean.
 // The list is taken in the stride order of vtile_stride(); cut[s] = number of tiles (in that order) whose inclusive cost
 // prefix is <= s / n_splits of the total; split s takes positions cut[s] .. cut[s + 1] - 1 of that order.
-__device__ void vsplit_plan(const DevView& v, int layer, const int* seq_ids, int qs, int n_splits) {
+// min_splits > 0: the caller left the number open.  A sequence then uses that many, or one per DECODE_SPLIT_TOKENS of its tokens; the
+// rest stay empty.  Decided here, from what the cache holds when the call runs, and not on the host, a replayed call splits as an
+// eager one does.
+__device__ void vsplit_plan(const DevView& v, int layer, const int* seq_ids, int qs, int n_splits, int min_splits) {
   __shared__ int s_warp[32];
   const int tid = threadIdx.x;
   const int seq = seq_ids[qs];
@@ -62,7 +65,8 @@ __device__ void vsplit_plan(const DevView& v, int layer, const int* seq_ids, int
     for (int s = tid; s <= n_splits; s += 1024) cut[s] = 0;
     return;
   }
-  const unsigned long long W = (unsigned long long)total, ns = (unsigned long long)n_splits;
+  const int used = min_splits > 0 ? min(n_splits, max(min_splits, v.stok(layer)[seq] / DECODE_SPLIT_TOKENS)) : n_splits;
+  const unsigned long long W = (unsigned long long)total, ns = (unsigned long long)used;
   int base = 0;
   for (int i0 = 0; i0 < n; i0 += 1024) {
     if (n > 1024) {
@@ -77,7 +81,7 @@ __device__ void vsplit_plan(const DevView& v, int layer, const int* seq_ids, int
       for (unsigned long long s = (e * ns + W - 1ull) / W; s < ns && s * W / ns < p; ++s) cut[s] = i0 + tid;
     }
   }
-  if (tid == 0) cut[n_splits] = n;
+  if (used + tid <= n_splits) cut[used + tid] = n;               // (the library's own choice is at most 64)
 }
 
 // K slot -> V slot of every token of one sequence (the V slots carry the opposite link): the K-score kernel stores a
@@ -98,7 +102,7 @@ __device__ void vlink_plan(const DevView& v, int layer, const int* seq_ids, int 
 }
 
 __global__ void __launch_bounds__(1024) plan_kernel(DevView v, int layer, const int* seq_ids, int n_seq, int n_cta, int pairs,
-                                                    int n_splits, int vj, const void* uinv_k, const void* uinv_v) {
+                                                    int n_splits, int min_splits, int vj, const void* uinv_k, const void* uinv_v) {
   chain_start();
   {
     const size_t bytes = (size_t)v.d_kv * v.d_kv * 2;             // the bases, which the K pass and the merge read (32 layers in turn find them
@@ -115,7 +119,7 @@ __global__ void __launch_bounds__(1024) plan_kernel(DevView v, int layer, const 
     return;
   }
   if ((int)blockIdx.x >= NC) {                                    // before them n_seq CTAs: the V pass's split plan, one sequence each
-    vsplit_plan(v, layer, seq_ids, (int)blockIdx.x - NC, n_splits);
+    vsplit_plan(v, layer, seq_ids, (int)blockIdx.x - NC, n_splits, min_splits);
     return;
   }
   extern __shared__ int s_slot[];                                 // sequence id -> query slot, -1
@@ -458,7 +462,8 @@ cudaError_t launch_vacc_tc(const DevView& v, int layer, const CUtensorMap& map_b
 
 template <bool BF16>
 static cudaError_t launch_decode_t(const DevView& v, int layer, const LayerParams& lp, const void* q, const int* seq_ids,
-                                   int n_seq, void* out, int n_splits, int sm_count, const TcMaps* maps, bool pairs, cudaStream_t st) {
+                                   int n_seq, void* out, int n_splits, int min_splits, int sm_count, const TcMaps* maps, bool pairs,
+                                   cudaStream_t st) {
   // the K-score kernel's work is cut into one piece per persistent CTA, or per CTA pair
   const int n_pieces = pairs ? kscore_max_pairs(sm_count) : sm_count;
   // CTAs per sequence that invert the V -> K links: enough of them that they finish inside the K work list's time
@@ -466,7 +471,7 @@ static cudaError_t launch_decode_t(const DevView& v, int layer, const LayerParam
   {
     ProfScope ps(TWKV_K_PLAN, st);
     cudaError_t e = launch_chained(plan_kernel, dim3(v.NC + n_seq + n_seq * vj), dim3(1024), dim3(1), (size_t)v.S * sizeof(int), st, v, layer, seq_ids,
-                                   n_seq, n_pieces, pairs ? 1 : 0, n_splits, vj, maps->uinv_k, lp.Uinv_v);
+                                   n_seq, n_pieces, pairs ? 1 : 0, n_splits, min_splits, vj, maps->uinv_k, lp.Uinv_v);
     if (e != cudaSuccess) return e;
   }
   {
@@ -503,10 +508,10 @@ static cudaError_t launch_decode_t(const DevView& v, int layer, const LayerParam
 }
 
 cudaError_t launch_decode(const DevView& v, int layer, const LayerParams& lp, const void* q, const int* seq_ids,
-                          int n_seq, void* out, int num_splits, int sm_count, const TcMaps* maps, bool pairs, cudaStream_t st) {
+                          int n_seq, void* out, int num_splits, int min_splits, int sm_count, const TcMaps* maps, bool pairs, cudaStream_t st) {
   if (n_seq <= 0) return cudaSuccess;
-  return v.dtype == TWKV_BF16 ? launch_decode_t<true>(v, layer, lp, q, seq_ids, n_seq, out, num_splits, sm_count, maps, pairs, st)
-                              : launch_decode_t<false>(v, layer, lp, q, seq_ids, n_seq, out, num_splits, sm_count, maps, pairs, st);
+  return v.dtype == TWKV_BF16 ? launch_decode_t<true>(v, layer, lp, q, seq_ids, n_seq, out, num_splits, min_splits, sm_count, maps, pairs, st)
+                              : launch_decode_t<false>(v, layer, lp, q, seq_ids, n_seq, out, num_splits, min_splits, sm_count, maps, pairs, st);
 }
 
 }  // namespace twkv

@@ -18,6 +18,7 @@ constexpr int ROPE_LO = 16;                 // pos = hi * 16 + lo
 constexpr int ROPE_HI = 32768;              // positions up to 16 * 32768 - 1
 constexpr int MAX_PARTIALS_EXTRA = 320;     // V-side partial slots beyond max_seqs
 constexpr int MAX_PLAN_CTAS = 1024;         // upper bound on the K-score kernel's grid
+constexpr int DECODE_SPLIT_TOKENS = 512;    // tokens a V split is worth where the library chooses the number of splits
 constexpr unsigned long long TWKV_GUARD_WORD = 0x7477b2006b765f67ull;   // written behind every region of the pool
 
 // Device view of a cache: plain pointers into the caller's pool.  Passed to kernels by value.
@@ -193,7 +194,7 @@ cudaError_t launch_compress_pieces(const DevView& v, int layer, const void* K, c
                                   const int* positions, int n_tok, const unsigned short* levels, cudaStream_t st);
 struct TcMaps;   // tensor maps of the K-score kernel (api.cu)
 cudaError_t launch_decode(const DevView& v, int layer, const LayerParams& lp, const void* q, const int* seq_ids,
-                          int n_seq, void* out, int num_splits, int sm_count, const TcMaps* maps, bool pairs, cudaStream_t st);
+                          int n_seq, void* out, int num_splits, int min_splits, int sm_count, const TcMaps* maps, bool pairs, cudaStream_t st);
 struct GateMaps;   // tensor maps of the fused gate kernel (api.cu)
 cudaError_t launch_gate_ranks_tc(const DevView& v, const GateMaps& maps, const LayerParams& lp, int n_tok, unsigned short* levels,
                                  int sm_count, bool pairs, cudaStream_t st);

@@ -66,3 +66,58 @@ def test_a_captured_first_call_that_never_runs(B):
     graph.replay()
     check()
     gc.close()
+
+
+def _long_layer(ctx):
+    li = workloads.build_layer(942, n_seq=1, ctx=ctx, n_q_heads=8, n_kv_heads=1, n_calib=256, outlier="none", mode="forced", rank_recipe="any")
+    ranks = li.ranks.numpy().astype(np.int64)
+    gc = GpuCache(B=_binding(), n_layers=1, n_q_heads=8, n_kv_heads=1, dtype=torch.float16, out_dtype=torch.float32, max_seqs=1,
+                  max_tokens_per_seq=ctx, payload_bytes=int((-(-ranks // 64) * 128).sum()))
+    gc.B.twkv_cache_set_layer_params(gc.h, 0, li.Uinv_k.cuda(), li.Uinv_v.cuda())
+    dev = [t.cuda() for t in (li.xt_k, li.xt_v, li.seq_ids, li.positions)] + [torch.from_numpy(ranks.astype(np.int16)).cuda()]
+
+    def append(lo, hi, seq=None):
+        gc.B.twkv_compress(gc.h, 0, dev[0][lo:hi], dev[1][lo:hi], dev[2][lo:hi] if seq is None else seq, dev[3][lo:hi], None, dev[4][lo:hi],
+                           gc.B.TWKV_GATE_FORCED)
+    return gc, li, ranks, append
+
+
+def _binding():
+    from paper_2603_04411_b200 import binding
+    return binding
+
+
+def test_a_decode_call_captured_on_an_empty_cache_splits_as_an_eager_one(B):
+    # the usual warm-up: the step is captured before there are tokens, its replays meet a long context
+    gc, li, ranks, append = _long_layer(16384)
+    q, sid = li.q.cuda(), torch.zeros(1, dtype=torch.int32, device="cuda")
+    out = [torch.zeros(1, 8, 128, device="cuda") for _ in range(2)]
+    B.twkv_decode_attn(gc.h, 0, q, sid, out[0])
+    graph = _capture(lambda: B.twkv_decode_attn(gc.h, 0, q, sid, out[0]))
+    for lo, hi in ((0, 300), (300, 16384)):
+        append(lo, hi)
+        graph.replay()
+        B.twkv_decode_attn(gc.h, 0, q, sid, out[1])
+        torch.testing.assert_close(out[0], out[1], rtol=0, atol=0)
+    max_abs, rel_l2 = attn_errors(out[0].cpu().numpy(), oracle_decode(li, ranks, [0]))
+    assert max_abs < MAX_ABS and rel_l2 < REL_L2, (max_abs, rel_l2)
+    assert B.twkv_cache_status(gc.h) == B.TWKV_OK
+    gc.close()
+
+
+def test_decode_depends_on_the_tokens_in_the_cache_alone(B):
+    # calls that were refused leave no trace in the rounding of later ones
+    gc, li, ranks, append = _long_layer(16384)
+    q, sid = li.q.cuda(), torch.zeros(1, dtype=torch.int32, device="cuda")
+    out = [torch.zeros(1, 8, 128, device="cuda") for _ in range(2)]
+    for k in range(2):
+        B.twkv_cache_reset(gc.h)
+        if k:
+            for _ in range(4):
+                append(0, 8192, torch.full((8192,), 7, dtype=torch.int32, device="cuda"))     # no such sequence
+            assert B.twkv_cache_status(gc.h) == B.TWKV_ERR_INVALID_ARG
+        append(0, 8192)
+        B.twkv_decode_attn(gc.h, 0, q, sid, out[k])
+    assert B.twkv_cache_status(gc.h) == B.TWKV_OK
+    torch.testing.assert_close(out[1], out[0], rtol=0, atol=0)
+    gc.close()
