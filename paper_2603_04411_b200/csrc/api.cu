@@ -243,8 +243,8 @@ struct twkv_cache {
   bool kscore_pairs = false;           // the K-score kernel runs on CTA pairs (the device can co-schedule them)
   std::vector<unsigned long long> guards;   // byte offsets (from the pool's start) of the guard words
   // Upper bound on the tokens a layer holds: tokens handed to twkv_compress since the last reset (refused and evicted ones
-  // included).  Bounds the launches of a prefill call; void once a compress call has been captured into a graph, since
-  // replays append tokens that the host does not see.
+  // included).  Spares a prefill call launches that would find nothing to do; void once a compress call has been captured into a
+  // graph, since replays append tokens that the host does not see.
   std::vector<std::atomic<long long>> appended;
   std::atomic<bool> append_captured{false};
 };
@@ -570,10 +570,11 @@ twkv_status twkv_decode_attn(twkv_cache* c, int layer, const void* q, const int3
 }
 
 // The tiled form of a prefill call: queries sorted by (sequence, position), dense rows of the visible tokens in segments.
-// `order`: query indices sorted that way; rows_max: upper bound on the rows.  Sets *done = false, with nothing launched, where the call's tables do not fit the
-// scratch regions they live in (the caller then serves the queries in waves).
+// `order`: query indices sorted that way; rows_max: upper bound on the rows where no two tokens of a sequence share a position;
+// rows_all: the bound where they do.  Sets *done = false, with nothing launched, where the call's tables do not fit the scratch
+// regions they live in (the caller then serves the queries in waves).
 static twkv_status prefill_tiled(twkv_cache* c, int layer, const void* q, const int32_t* q_seq, const int32_t* q_pos, const std::vector<int>& order,
-                                 long long rows_max, void* out, cudaStream_t st, bool* done) {
+                                 long long rows_max, long long rows_all, void* out, cudaStream_t st, bool* done) {
   const DevView& v = c->view;
   const int n_q = (int)order.size(), QT = TILE / v.rep, pos_end = ROPE_LO * ROPE_HI;
   *done = false;
@@ -605,7 +606,7 @@ static twkv_status prefill_tiled(twkv_cache* c, int layer, const void* q, const 
   int* p = (int*)(v.gate_fix + n_blocks);
   a.qvis = p; p += n_q;
   a.rows = p; a.base = p + n_u; a.dup = p + 2 * (size_t)n_u; p += 3 * (size_t)n_u;
-  a.ticket = p; p += 4;
+  a.ticket = p; a.total = p + 1; p += 4;
   a.slot = p; p += v.S;
   a.bits = (unsigned*)p; a.pref = p + n_words;
   a.krow = v.kv_link; a.krow_out = v.evict_map; a.vrow = v.evict_map + (size_t)v.NT * TILE;
@@ -614,7 +615,7 @@ static twkv_status prefill_tiled(twkv_cache* c, int layer, const void* q, const 
   a.vexp = (signed char*)v.hist;                                    // 8448 bytes per KV head of at least 16384
   a.vflag = (int*)(a.vexp + (size_t)GATE_PIECE * v.Hkv);
 
-  if (rows_max > 32767ll * (GATE_PIECE / 2)) return TWKV_OK;         // a tile's segments are kept in two 16-bit halves
+  if (rows_all > 32767ll * (GATE_PIECE / 2)) return TWKV_OK;         // a tile's segments are kept in two 16-bit halves
   // Segments of 8192 rows with the partial results in the V pass's region, or of 4096 rows with them in the second half of
   // the gate scratch (fewer heads leave the first region small); splits of a segment's rows where the blocks of queries
   // alone leave SMs idle.  Estimated in key blocks of one CTA: its share of a segment plus 1.5 for an item's start and end.
@@ -631,7 +632,7 @@ static twkv_status prefill_tiled(twkv_cache* c, int layer, const void* q, const 
     const int seg_blocks = std::max(1, (int)((std::min<long long>(rows_max, seg_rows) + TILE - 1) / TILE));
     for (int ns = 1; ns <= 32 && ns <= seg_blocks && (long long)group * v.Hkv * ns <= cap; ++ns) {
       const long long rounds = ((long long)group * v.Hkv * ns + c->sm_count - 1) / c->sm_count;
-      const double cost = groups * segs * ((double)rounds * ((seg_blocks + ns - 1) / ns + 1.5) + 4.0 + seg_rows / 1024.0);
+      const double cost = groups * segs * ((double)rounds * ((seg_blocks + ns - 1) / ns + 1.5) + 4.0 + std::min<long long>(rows_max, seg_rows) / 1024.0);
       if (cost < best) { best = cost; best_rows = seg_rows; best_splits = ns; best_group = group; }
     }
   }
@@ -650,13 +651,13 @@ static twkv_status prefill_tiled(twkv_cache* c, int layer, const void* q, const 
     if (cudaMemcpyAsync((char*)v.wave_buf + at, src + at, std::min<size_t>(49152, bytes - at), cudaMemcpyHostToDevice, st) != cudaSuccess) return TWKV_ERR_CUDA;
   *done = true;
   if (launch_pf_tables(v, a, layer, c->sm_count, st) != cudaSuccess) return TWKV_ERR_CUDA;
-  const int n_segs = std::max(1, (int)((rows_max + a.seg_rows - 1) / a.seg_rows));
-  const bool whole = n_segs == 1 && a.n_splits == 1;
+  // the segments past the call's last row are launched for repeated positions alone: their kernels look at the number of rows and leave
+  const int n_segs = std::max(1, (int)((rows_all + a.seg_rows - 1) / a.seg_rows));
   for (a.blk0 = 0; a.blk0 < n_blocks; a.blk0 += best_group) {
     a.blk_n = std::min(best_group, n_blocks - a.blk0);
     for (int seg = 0; seg < n_segs; ++seg)
-      if (launch_pf_segment(v, a, maps, layer, seg, q, whole ? out : nullptr, c->sm_count, st) != cudaSuccess) return TWKV_ERR_CUDA;
-    if (!whole && launch_pf_combine(v, a, out, st) != cudaSuccess) return TWKV_ERR_CUDA;
+      if (launch_pf_segment(v, a, maps, layer, seg, q, out, c->sm_count, st) != cudaSuccess) return TWKV_ERR_CUDA;
+    if ((n_segs > 1 || a.n_splits > 1) && launch_pf_combine(v, a, out, st) != cudaSuccess) return TWKV_ERR_CUDA;
   }
   return TWKV_OK;
 }
@@ -684,11 +685,16 @@ twkv_status twkv_prefill_attn(twkv_cache* c, int layer, const void* q, const int
   DeviceGuard g(c->device);
   if (!g.ok) return TWKV_ERR_CUDA;
   cudaStream_t st = (cudaStream_t)stream;
-  // how many rows (tokens, a sequence's rounded up to whole tiles) the sequences can have: their capacity, or what the layer was
-  // ever given
-  long long rows_max = n_distinct * ((c->cfg.max_tokens_per_seq + TILE - 1) / TILE * (long long)TILE);
+  // How many rows (visible tokens, a sequence's rounded up to whole tiles) the call can have: one per position up to its largest query's.
+  // More only where tokens share a position: then up to the sequences' capacity, or what the layer was ever given.
+  auto rows_of = [](long long tokens) { return (tokens + TILE - 1) / TILE * TILE; };
+  std::vector<int> last(S, -1);
+  for (int i = 0; i < n_q; ++i) last[q_seq[i]] = std::max(last[q_seq[i]], q_pos[i]);
+  long long rows_max = 0, rows_all = n_distinct * rows_of(c->cfg.max_tokens_per_seq);
+  for (int s = 0; s < S; ++s)
+    if (last[s] >= 0) rows_max += rows_of(std::min<long long>(c->cfg.max_tokens_per_seq, last[s] + 1ll));
   if (!c->append_captured.load(std::memory_order_relaxed) && !is_capturing(st))
-    rows_max = std::min(rows_max, c->appended[layer].load(std::memory_order_relaxed) + (TILE - 1) * (long long)n_distinct);
+    rows_all = std::min(rows_all, c->appended[layer].load(std::memory_order_relaxed) + (TILE - 1) * (long long)n_distinct);
   if (prefill_tiled_pays(n_waves, (double)rows_max)) {
     ProfBind pb(&c->prof);
     std::vector<int> order(n_q);
@@ -696,7 +702,7 @@ twkv_status twkv_prefill_attn(twkv_cache* c, int layer, const void* q, const int
     if (!sorted)
       std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return q_seq[x] != q_seq[y] ? q_seq[x] < q_seq[y] : q_pos[x] < q_pos[y]; });
     bool done = false;
-    const twkv_status s = prefill_tiled(c, layer, q, q_seq, q_pos, order, rows_max, out, st, &done);
+    const twkv_status s = prefill_tiled(c, layer, q, q_seq, q_pos, order, rows_max, std::max(rows_max, rows_all), out, st, &done);
     if (done || s != TWKV_OK) return s;
   }
   std::vector<int> wave_start(n_waves + 1, 0), fill(n_waves, 0);

@@ -21,7 +21,7 @@ struct PfCall {
   unsigned* bits;       // [n_words] bitmaps of the visible positions
   int* pref;            // [n_words] set bits before the word, inside the sequence
   int *rows, *base, *dup;   // [n_u] rows of a sequence, its first dense row, whether a position repeats
-  int* ticket;
+  int *ticket, *total;      // [1] rows of the call, every sequence's rounded up to whole tiles
   int* qvis;            // [n] rows of its sequence a query may see
   int4* binfo;          // [n_blocks] first dense row of the sequence, most rows a query of the block sees, repeated positions
   int* krow;            // [NT * 128] K-tile-order rows of sequences with a repeated position
@@ -36,7 +36,8 @@ struct PfCall {
 };
 struct PfMaps { CUtensorMap blocks, uk, uv, seg; };
 
-// out: not null where one split of one segment is a query's whole result: the attention kernel then writes the outputs itself
+// out: where one split of one segment is a query's whole result, the attention kernel writes the outputs itself and the combine
+// kernel, launched for what may turn out otherwise, leaves
 cudaError_t launch_pf_tables(const DevView& v, const PfCall& a, int layer, int sm_count, cudaStream_t st);
 cudaError_t launch_pf_segment(const DevView& v, const PfCall& a, const PfMaps& maps, int layer, int seg, const void* q, void* out, int sm_count, cudaStream_t st);
 cudaError_t launch_pf_combine(const DevView& v, const PfCall& a, void* out, cudaStream_t st);

@@ -113,7 +113,13 @@ __global__ void __launch_bounds__(1024) pf_scan_kernel(DevView v, PfCall a, int 
     if (i < a.n_u) a.base[i] = run + e;
     run += total;
   }
+  if (tid == 0) *a.total = run;
 }
+
+// Segments past the last row have been launched as well (their set-up ran beside the kernel before).
+__device__ __forceinline__ bool pf_idle(const PfCall& a, int seg) { return seg > 0 && (long long)seg * a.seg_rows >= *a.total; }
+// Whether the attention kernel's result for a query is whole: one split of the only segment with rows.
+__device__ __forceinline__ bool pf_whole(const PfCall& a) { return a.n_splits == 1 && *a.total <= a.seg_rows; }
 
 __device__ __forceinline__ int pf_rank(const PfCall& a, int off, int pos) {      // visible tokens before position pos
   const int w = off + (pos >> 5);
@@ -246,7 +252,8 @@ pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_con
   }
   if (warp == 1) tmem_alloc(smem_addr(s_tmem_base), 512);
   chain_wait();
-  for (int i = tid; i < ROPE_LO * 32; i += PR_THREADS) sRope[(i >> 5) * PR_ROPE_STRIDE + (i & 31)] = v.rope_lo[i];
+  const bool idle = pf_idle(a, seg);
+  for (int i = tid; i < ROPE_LO * 32 && !idle; i += PR_THREADS) sRope[(i >> 5) * PR_ROPE_STRIDE + (i & 31)] = v.rope_lo[i];
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
@@ -273,7 +280,7 @@ pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_con
     return __ballot_sync(0xffffffffu, mine);
   };
 
-  if (misaligned) {
+  if (misaligned || idle) {
     // nothing was started
   } else if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(PR_REGS_LIGHT));
@@ -635,8 +642,9 @@ pf_attn_kernel(const __grid_constant__ CUtensorMap map_seg, DevView v, PfCall a,
   const uint32_t tmem_base = *s_tmem_base;
   const int n_items = a.blk_n * v.Hkv * a.n_splits;
   chain_wait();
+  const bool whole = pf_whole(a), idle = pf_idle(a, seg);
 
-  if (misaligned) {
+  if (misaligned || idle) {
     // nothing was started
   } else if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(PA_REGS_LIGHT));
@@ -918,8 +926,8 @@ pf_attn_kernel(const __grid_constant__ CUtensorMap map_seg, DevView v, PfCall a,
         if (!(ok = named_bar_and(pair_bar, 64, ok))) break;
         l = xs[0] + xs[TILE];                                    // (read before this warp hands over the next item's queries)
       }
-      if (out) {
-        // one split of one segment: this is the whole result.  A thread writes its row's 64 columns itself (4096-token prompt in four
+      if (whole) {
+        // This is the whole result.  A thread writes its row's 64 columns itself (4096-token prompt in four
         // calls 783 -> 751 us, five short prompts 204 -> 189 against partial results and the combine kernel).
         const float inv = l == 0.f ? 0.f : 1.f / l;              // 0: no token seen; a NaN stays one
         const bool mine = ql < it.cnt;
@@ -990,6 +998,7 @@ __global__ void __launch_bounds__(256) pf_combine_kernel(DevView v, PfCall a, vo
   __shared__ float s[TILE][33];
   chain_start();
   chain_wait();
+  if (pf_whole(a)) return;
   const int c0 = (blockIdx.x & 3) * 32, h = (blockIdx.x >> 2) & 1, bg = blockIdx.x >> 3, g = bg % v.Hkv, blk = bg / v.Hkv;
   const int2 q = a.blocks[a.blk0 + blk];
   const int cnt = q.y & 0x1ff, rep = v.rep, QT = TILE / rep;

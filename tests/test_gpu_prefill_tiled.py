@@ -38,9 +38,8 @@ def test_tiled_prefill_where_the_work_split_changes(B, hkv, rep, dtype, n_seq, c
 def _filled(B, li, ranks, *, out_dtype=torch.float32, **cfg):
     """A cache with the layer's tokens, one compress call."""
     n_seq = int(li.seq_ids.max()) + 1
-    sizes = dict(max_seqs=n_seq, max_tokens_per_seq=int(np.bincount(li.seq_ids.numpy()).max()))
-    gc = GpuCache(B, n_layers=1, n_q_heads=li.n_q_heads, n_kv_heads=li.n_kv_heads, dtype=li.dtype, out_dtype=out_dtype,
-                  payload_bytes=int((-(-ranks // 64) * 128).sum()), **{**sizes, **cfg})
+    sizes = dict(max_seqs=n_seq, max_tokens_per_seq=int(np.bincount(li.seq_ids.numpy()).max()), payload_bytes=int((-(-ranks // 64) * 128).sum()))
+    gc = GpuCache(B, n_layers=1, n_q_heads=li.n_q_heads, n_kv_heads=li.n_kv_heads, dtype=li.dtype, out_dtype=out_dtype, **{**sizes, **cfg})
     B.twkv_cache_set_layer_params(gc.h, 0, li.Uinv_k.cuda(), li.Uinv_v.cuda())
     B.twkv_compress(gc.h, 0, li.xt_k.cuda(), li.xt_v.cuda(), li.seq_ids.cuda(), li.positions.cuda(), None,
                     torch.from_numpy(ranks.astype(np.int16)).cuda(), B.TWKV_GATE_FORCED)
@@ -134,3 +133,46 @@ def test_tiled_prefill_shows_an_infinite_value(B):
     gc.close()
     assert not np.isfinite(got[q_pos >= 200]).any()
     assert np.isfinite(got[q_pos < 128]).all()                 # (a block of keys that the token is not in)
+
+
+@pytest.mark.parametrize("n_q", [6, 300])
+def test_tiled_prefill_does_not_depend_on_the_room_in_the_cache(B, n_q):
+    # the same chunk in a cache that just holds its sequence, and in one with room for 131072 tokens a sequence and other sequences
+    # resident: the same form, splits and bits
+    ctx, other = 1000, 30000
+    li = workloads.build_layer(891, n_seq=1, ctx=ctx, n_q_heads=32, outlier="pct:1", mode="forced", rank_recipe="any")
+    ranks = li.ranks.numpy().astype(np.int64)
+    q_pos = np.arange(ctx - n_q, ctx)
+    q = torch.randn(n_q, 32, 128, generator=torch.Generator().manual_seed(5)).to(torch.float16)
+    gc = _filled(B, li, ranks)
+    fitted = _prefill(B, gc, q, np.zeros(n_q, np.int64), q_pos)
+    gc.close()
+    max_abs, rel_l2 = attn_errors(fitted, _oracle_prefill(li, ranks, q, np.zeros(n_q, np.int64), q_pos))
+    assert max_abs < MAX_ABS and rel_l2 < REL_L2, (max_abs, rel_l2)
+    li.seq_ids = li.seq_ids + 1
+    gc = _filled(B, li, ranks, max_seqs=3, max_tokens_per_seq=131072, payload_bytes=2 * other * 256 + ctx * 4096)
+    x = torch.randn(other, 1024, device="cuda").to(torch.float16)
+    seq, pos = torch.arange(other, device="cuda", dtype=torch.int32) % 2 * 2, torch.arange(other, device="cuda", dtype=torch.int32) // 2
+    B.twkv_compress(gc.h, 0, x, x, seq, pos, None, torch.full((other, 2), 64, dtype=torch.int16, device="cuda"), B.TWKV_GATE_FORCED)
+    roomy = _prefill(B, gc, q, np.ones(n_q, np.int64), q_pos)
+    assert B.twkv_cache_check(gc.h) == (B.TWKV_OK, 0)
+    gc.close()
+    np.testing.assert_array_equal(roomy, fitted)
+
+
+@pytest.mark.parametrize("n_q,repeat", [(33, 64), (200, 30)])
+def test_tiled_prefill_of_more_tokens_than_positions(B, n_q, repeat):
+    # positions shared by so many tokens that the rows go on past the segments that the positions alone would need
+    ctx = 9000
+    li = workloads.build_layer(895, n_seq=1, ctx=ctx, n_q_heads=8, n_kv_heads=1, n_calib=256, mode="forced", rank_recipe="any", shuffle_positions=True)
+    li.positions = li.positions // repeat
+    ranks = li.ranks.numpy().astype(np.int64)
+    q_pos = np.random.default_rng(6).integers(0, ctx // repeat, n_q)
+    q_pos[0] = ctx // repeat
+    q_seq = np.zeros(n_q, np.int64)
+    q = torch.randn(n_q, 8, 128, generator=torch.Generator().manual_seed(6)).to(torch.float16)
+    gc = _filled(B, li, ranks, max_tokens_per_seq=50000)
+    got = _prefill(B, gc, q, q_seq, q_pos)
+    gc.close()
+    max_abs, rel_l2 = attn_errors(got, _oracle_prefill(li, ranks, q, q_seq, q_pos))
+    assert max_abs < MAX_ABS and rel_l2 < REL_L2, (max_abs, rel_l2)
