@@ -255,6 +255,34 @@ static bool is_capturing(cudaStream_t st) {
   return s != cudaStreamCaptureStatusNone;
 }
 
+// A call's tables, made on the host, into the pool; they may go away once the call returns.  A copy from pageable memory is staged
+// before it returns, below 64 KiB without waiting for the stream; a graph would read the memory at every replay instead, so a captured
+// call carries the values in kernel parameters.
+struct PutInts { int* dst; int n; int data[960]; };
+__global__ void put_ints_kernel(const __grid_constant__ PutInts p) {
+  for (int i = threadIdx.x; i < p.n; i += blockDim.x) p.dst[i] = p.data[i];
+}
+static cudaError_t upload_ints(int* dst, const std::vector<int>& src, cudaStream_t st) {
+  const bool captured = is_capturing(st);
+  const size_t step = captured ? sizeof(PutInts::data) / sizeof(int) : 49152 / sizeof(int);
+  for (size_t at = 0; at < src.size(); at += step) {
+    const size_t n = std::min(step, src.size() - at);
+    cudaError_t e;
+    if (captured) {
+      PutInts p;
+      p.dst = dst + at; p.n = (int)n;
+      memcpy(p.data, src.data() + at, n * sizeof(int));
+      put_ints_kernel<<<1, 256, 0, st>>>(p);
+      count_launch();
+      e = cudaGetLastError();
+    } else {
+      e = cudaMemcpyAsync(dst + at, src.data() + at, n * sizeof(int), cudaMemcpyHostToDevice, st);
+    }
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 
 extern "C" {
 
@@ -645,10 +673,7 @@ static twkv_status prefill_tiled(twkv_cache* c, int layer, const void* q, const 
   const uint64_t d = (uint64_t)v.d_kv;
   if (!make_tmap_2d(&maps.uk, c->params[layer].Uinv_k, d, d, d * 2, PANEL) || !make_tmap_2d(&maps.uv, c->params[layer].Uinv_v, d, d, d * 2, PANEL) ||
       !make_tmap_2d(&maps.seg, a.seg_buf, (uint64_t)v.Hkv * 4 * a.seg_rows, HEAD_DIM, HEAD_DIM * 2, TILE)) return TWKV_ERR_CUDA;
-  // pieces below 64 KiB: a larger copy from pageable memory would wait for the stream before it returns
-  const char* src = (const char*)host.data();
-  for (size_t at = 0, bytes = host.size() * sizeof(int); at < bytes; at += 49152)
-    if (cudaMemcpyAsync((char*)v.wave_buf + at, src + at, std::min<size_t>(49152, bytes - at), cudaMemcpyHostToDevice, st) != cudaSuccess) return TWKV_ERR_CUDA;
+  if (upload_ints(v.wave_buf, host, st) != cudaSuccess) return TWKV_ERR_CUDA;
   *done = true;
   if (launch_pf_tables(v, a, layer, c->sm_count, st) != cudaSuccess) return TWKV_ERR_CUDA;
   // the segments past the call's last row are launched for repeated positions alone: their kernels look at the number of rows and leave
@@ -708,19 +733,18 @@ twkv_status twkv_prefill_attn(twkv_cache* c, int layer, const void* q, const int
   std::vector<int> wave_start(n_waves + 1, 0), fill(n_waves, 0);
   for (int i = 0; i < n_q; ++i) ++wave_start[wave_of[i] + 1];
   for (int w = 0; w < n_waves; ++w) wave_start[w + 1] += wave_start[w];
-  std::vector<int> host(3 * (size_t)TWKV_PREFILL_MAX_QUERIES);
+  std::vector<int> host(3 * (size_t)n_q);
   for (int i = 0; i < n_q; ++i) {
     const int at = wave_start[wave_of[i]] + fill[wave_of[i]]++;
     host[at] = q_seq[i];
-    host[TWKV_PREFILL_MAX_QUERIES + at] = i;
-    host[2 * TWKV_PREFILL_MAX_QUERIES + at] = q_pos[i];
+    host[n_q + at] = i;
+    host[2 * (size_t)n_q + at] = q_pos[i];
   }
-  // the copy is staged from pageable memory before the call returns, so `host` may go out of scope afterwards
-  if (cudaMemcpyAsync(c->view.wave_buf, host.data(), host.size() * sizeof(int), cudaMemcpyHostToDevice, st) != cudaSuccess) return TWKV_ERR_CUDA;
+  int* w0 = c->view.wave_buf;
+  if (upload_ints(w0, host, st) != cudaSuccess) return TWKV_ERR_CUDA;
   for (int w = 0; w < n_waves; ++w) {
     const int off = wave_start[w], n = wave_start[w + 1] - off;
-    twkv_status s = decode_pass(c, layer, q, c->view.wave_buf + off, n, out, num_splits, c->view.wave_buf + TWKV_PREFILL_MAX_QUERIES + off,
-                                c->view.wave_buf + 2 * TWKV_PREFILL_MAX_QUERIES + off, st);
+    twkv_status s = decode_pass(c, layer, q, w0 + off, n, out, num_splits, w0 + n_q + off, w0 + 2 * (size_t)n_q + off, st);
     if (s != TWKV_OK) return s;
   }
   return TWKV_OK;

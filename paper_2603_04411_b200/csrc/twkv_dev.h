@@ -64,7 +64,8 @@ struct DevView {
   unsigned* evict_bitmap;    // one bit per position: the positions that stay
   int* evict_map;            // [2][NT * 128]  new global slot of every K / V slot of the sequence, -1 = dropped
   int* evict_fill;           // [2][NC]  survivors per key
-  int* wave_buf;             // [3][TWKV_PREFILL_MAX_QUERIES]: sequence, row and position of a prefill call's queries, wave by wave
+  int* wave_buf;             // [3 * TWKV_PREFILL_MAX_QUERIES]  the host's tables of a prefill call; in waves: sequence, row and position of
+                             // the queries, wave by wave
   int4* klist;               // [NT]  K tiles of the current decode call, widest class first: (tile, class | n_valid << 8, base block, query slot)
   int4* kpairs;              // [NT + 64]  the same list as items of two tiles of one class (entries 2 i, 2 i + 1) for the CTA-pair kernel;
                              //            a class with an odd number of tiles ends with a filler entry (.y bit 7 set)

@@ -121,3 +121,34 @@ def test_decode_depends_on_the_tokens_in_the_cache_alone(B):
     assert B.twkv_cache_status(gc.h) == B.TWKV_OK
     torch.testing.assert_close(out[1], out[0], rtol=0, atol=0)
     gc.close()
+
+
+@pytest.mark.parametrize("n_q", [300, 2])        # the tiled form; two decode passes
+def test_a_captured_prefill_call_replays_after_its_lists_are_gone(B, n_q):
+    # captured with the first tokens in the cache; the host's lists are overwritten and further tokens appended (by a graph as well)
+    ctx = 9000
+    gc, li, ranks, append = _long_layer(ctx)
+    dn = "f16"
+    q = torch.randn(n_q, 8, 128, generator=torch.Generator().manual_seed(8)).to(torch.float16)
+    q_dev, out = q.cuda(), [torch.zeros(n_q, 8, 128, device="cuda") for _ in range(2)]
+    seq, pos = np.zeros(n_q, np.int32), np.arange(ctx - n_q, ctx, dtype=np.int32)
+    append(0, 200)
+    B.twkv_prefill_attn(gc.h, 0, q_dev, seq, pos, out[1])                  # the layer's one-time set-up
+    lists = seq.copy(), pos.copy()
+    graph = _capture(lambda: B.twkv_prefill_attn(gc.h, 0, q_dev, *lists, out[0]))
+    more = _capture(lambda: append(200, 8500))
+    lists[0][:], lists[1][:] = -5, 1 << 30
+    scribble = [np.full(3 * n_q, -7, np.int32) for _ in range(200)]         # where the call's own tables may have been
+    more.replay()
+    append(8500, ctx)
+    graph.replay()
+    B.twkv_prefill_attn(gc.h, 0, q_dev, seq, pos, out[1])
+    torch.testing.assert_close(out[0], out[1], rtol=0, atol=0)
+    pick = np.arange(0, n_q, max(1, n_q // 10))
+    U = [oracle.widen16(bits16(u), dn) for u in (li.Uinv_k, li.Uinv_v)]
+    want = oracle.prefill_attn(oracle.widen16(bits16(li.xt_k), dn), oracle.widen16(bits16(li.xt_v), dn), ranks[:, 0], ranks[:, 1],
+                               li.positions.numpy(), *U, oracle.widen16(bits16(q[pick]), dn), pos[pick], 1, 500000.0, 128 ** -0.5)
+    max_abs, rel_l2 = attn_errors(out[0].cpu().numpy()[pick], want)
+    assert max_abs < MAX_ABS and rel_l2 < REL_L2, (max_abs, rel_l2)
+    assert B.twkv_cache_status(gc.h) == B.TWKV_OK and len(scribble) == 200
+    gc.close()
