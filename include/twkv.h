@@ -185,8 +185,8 @@ twkv_status twkv_decode_attn(twkv_cache* cache, int layer, const void* q, const 
  *   n_q      at most TWKV_PREFILL_MAX_QUERIES
  * Keys and values of the visible tokens are rebuilt once per call and shared by its queries; calls of few queries per
  * sequence run as passes of the decode kernels instead, one query per sequence at a time (num_splits applies to those).
- * The host arrays are read before the call returns; a call captured into a graph replays with what they held then.  Errors as for twkv_decode_attn; an id or position out of range returns
- * TWKV_ERR_INVALID_ARG before anything is launched.
+ * The host arrays are read before the call returns; a call captured into a graph replays with what they held then.
+ * Errors as for twkv_decode_attn; an id or position out of range returns TWKV_ERR_INVALID_ARG before anything is launched.
  */
 twkv_status twkv_prefill_attn(twkv_cache* cache, int layer, const void* q, const int32_t* q_seq /*host*/,
                               const int32_t* q_pos /*host*/, int n_q, void* out, int num_splits, void* stream);

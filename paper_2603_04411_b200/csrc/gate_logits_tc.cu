@@ -20,6 +20,7 @@ constexpr int GL_THREADS = 320;
 constexpr int GL_STAGES = 6;
 constexpr uint32_t GL_PANEL_BYTES = 16384, GL_ATOM_BYTES = GL_PANEL_BYTES / 2, GL_STAGE_BYTES = 2 * GL_PANEL_BYTES;
 constexpr uint32_t GL_SMEM = GL_STAGES * GL_STAGE_BYTES + 8 * (2 * GL_STAGES + 4) + 16;
+static_assert(GL_SMEM > CHAIN_TMEM_SMEM, "no other CTA with tensor memory beside this one");
 
 __global__ void __launch_bounds__(GL_THREADS, 1)
 gate_logits_tc_kernel(const __grid_constant__ CUtensorMap map_xk, const __grid_constant__ CUtensorMap map_xv,

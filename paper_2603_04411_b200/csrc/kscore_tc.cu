@@ -610,11 +610,13 @@ cudaError_t launch_transpose16(const void* in, void* out, int n, cudaStream_t st
   return cudaGetLastError();
 }
 
-size_t kscore_tc_smem_bytes(int nb, size_t stage_bytes) {
+constexpr size_t kscore_tc_smem_bytes(int nb, size_t stage_bytes) {
   return (size_t)KT_A_SLOTS * PANEL_BYTES + (size_t)nb * stage_bytes + 2 * KT_Q_PANEL_BYTES + KT_ROPE_STAGE_BYTES + 8 * (KT_N_BARS + 2 * nb) +
          2 * sizeof(int);
 }
 constexpr int KT_NB_SINGLE = 2, KT_NB_PAIR = 4;                // ring stages of two U_K^-1 panels (32 KiB) / two half panels (16 KiB)
+static_assert(kscore_tc_smem_bytes(KT_NB_SINGLE, 2 * PANEL_BYTES) > CHAIN_TMEM_SMEM && kscore_tc_smem_bytes(KT_NB_PAIR, PANEL_BYTES) > CHAIN_TMEM_SMEM,
+              "no other CTA with tensor memory beside this one");
 
 // CTA pairs of the pair kernel that can be resident at once on the current device (0: it cannot run).
 static int kscore_query_pairs(int sm_count) {

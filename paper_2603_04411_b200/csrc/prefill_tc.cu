@@ -198,6 +198,7 @@ constexpr uint32_t PR_OUT_BYTES = 8192;                         // per warp: 32 
 constexpr int PR_ROPE_STRIDE = 33;                              // float4 per row of the small RoPE table (32 + 1 against bank conflicts)
 constexpr uint32_t PR_ROPE_BYTES = ROPE_LO * PR_ROPE_STRIDE * 16;
 constexpr uint32_t PR_SMEM = PR_STAGES * PR_STAGE_BYTES + 8 * PR_OUT_BYTES + PR_ROPE_BYTES + 8 * (2 * PR_STAGES + 4) + 16;
+static_assert(PR_SMEM > CHAIN_TMEM_SMEM, "no other CTA with tensor memory beside this one");
 // A row whose largest value lies outside these is scaled: a small one to [2^-3, 2^-2), a large one to [2^14, 2^15).  A part is exact
 // to 2^-25: values at the lower line keep 20 bits, scaled ones 22; scaled further up, their weights (which shrink by as much) would
 // lose bits beside those of rows that are not scaled.
@@ -568,6 +569,7 @@ constexpr uint32_t PA_STAGE_BYTES = 32768, PA_PANEL_BYTES = 16384;
 constexpr uint32_t PA_Q_BYTES = 2 * 32768;
 constexpr uint32_t PA_X_BYTES = 2 * 2 * TILE * 4;               // [tile][half][row]: row maxima of a half; row sums at the end
 constexpr uint32_t PA_SMEM = PA_Q_BYTES + PA_STAGES * PA_STAGE_BYTES + PA_X_BYTES + 8 * (2 * PA_STAGES + 8) + 16;
+static_assert(PA_SMEM > CHAIN_TMEM_SMEM, "no other CTA with tensor memory beside this one");
 
 __device__ __forceinline__ float ex2(float x) { float r; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
 

@@ -155,6 +155,10 @@ struct DeviceGuard {
 // before has completed.  Every CTA of a chained kernel waits, so that completion passes down the chain.  Such a kernel reads
 // nothing through the read-only path that an earlier kernel may have written (no __restrict__, no __ldg): those loads could
 // be moved before the wait.
+// A chained kernel that allocates tensor memory must not share an SM with the next one of the chain: that one could take the columns
+// first and wait for the kernel that needs them.  Each of them asks for more than half of an SM's shared memory (CHAIN_TMEM_SMEM,
+// asserted beside its size), so that no two fit.
+constexpr unsigned CHAIN_TMEM_SMEM = 228 * 1024 / 2;
 __device__ __forceinline__ void chain_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Asks for this thread's share of `bytes` bytes at `p` in L2, without waiting: before chain_wait(), so that matrices no kernel of the

@@ -407,6 +407,7 @@ static cudaError_t launch_vacc_tc_n(const DevView& v, int layer, const CUtensorM
                                     const int* seq_ids, int n_seq, int n_splits, cudaStream_t st) {
   using C = VtCfg<BF16, N>;
   static_assert(C::STAGES >= 3, "the ring needs a few stages");
+  static_assert(C::SMEM_BYTES > CHAIN_TMEM_SMEM, "no other CTA with tensor memory beside this one");
   cudaError_t e = cudaFuncSetAttribute(vacc_tc_kernel<BF16, N, TS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM_BYTES);
   if (e != cudaSuccess) return e;
   const dim3 grid(n_seq * n_splits, (v.Hq + N - 1) / N);
