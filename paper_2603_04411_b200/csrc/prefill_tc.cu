@@ -12,8 +12,8 @@
 //   sequence follow the K tiles instead and the causal mask compares positions.
 //
 // Precision: as in decode attention, keys are carried as two f16 (22 bits) and queries as f16; softmax weights and values are two
-// f16 as well, whatever the cache type, so that the result is the spectral-space one to rounding.  The products high.high,
-// high.low and low.high of weights and values are formed.
+// f16 as well, whatever the cache type, so that the result is the spectral-space one to rounding.  The products high.low,
+// low.high and high.high of weights and values are formed.
 // A rebuilt value may lie outside f16 although the stored 16-bit components do not.  A row (token, KV head) whose largest value is
 // beyond 65504, or so small that the low parts would lose bits, is divided by a power of two before the split, and its softmax
 // weights carry that power; blocks of keys without such a row (nearly all, for values around 1) run as if there were none.
@@ -706,9 +706,9 @@ pf_attn_kernel(const __grid_constant__ CUtensorMap map_seg, DevView v, PfCall a,
         auto values = [&](int h, const uint32_t (&vv)[2], bool first) {
           const uint32_t p = tmem_base + h * 128, d = tmem_base + 256 + h * 128;
 #pragma unroll
-          for (int c = 0; c < 3; ++c) {                         // high . high, high . low, low . high
-            const uint32_t pa = p + (c == 2 ? 8 : 0);
-            const uint32_t vb = (((sR + vv[c == 1] * PA_STAGE_BYTES) >> 4) & 0x3fffu) | ((PA_PANEL_BYTES >> 4) << 16);
+          for (int c = 0; c < 3; ++c) {                         // high . low, low . high, high . high: the small ones first, as for the scores
+            const uint32_t pa = p + (c == 1 ? 8 : 0);
+            const uint32_t vb = (((sR + vv[c == 0] * PA_STAGE_BYTES) >> 4) & 0x3fffu) | ((PA_PANEL_BYTES >> 4) << 16);
 #pragma unroll
             for (int ks = 0; ks < 8; ++ks)
               mma_f16_ts(d, pa + 16 * ks, ((uint64_t)KMAJOR_SW128_DESC_HI << 32) | (vb + ks * 128u), idesc_o,
