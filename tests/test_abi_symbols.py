@@ -70,3 +70,22 @@ def test_projector_argument_checks_need_no_device():
     assert B.lib.twkv_projector_create(1024, B.TWKV_F16, one, one, one, 1024, None, ctypes.byref(h)) == B.TWKV_ERR_CAPACITY
     assert B.lib.twkv_project(None, one, one, one, one, 4, None) == B.TWKV_ERR_INVALID_ARG
     assert h.value is None
+
+
+def test_lists_of_integers_are_taken_as_int_takes_them(libpath):
+    # the query lists of twkv_prefill_attn: every element is int() of it in 32 bits, whatever holds it; what int() refuses is refused
+    import numpy as np
+    import torch
+    from paper_2603_04411_b200.binding import _host_int32
+    for x in ([], [3, 1, 2], (5,), range(4), iter([7, 8]), [True, 2.9, np.int64(4), torch.tensor(6)], np.arange(3), np.arange(6)[::2],
+              np.array([1.5, -2.5]), np.array([2 ** 32 + 5, -1], np.int64), np.array([2 ** 63 + 9], np.uint64), [2 ** 40 + 3],
+              np.array([258], ">i4"), torch.arange(4), torch.arange(4, dtype=torch.uint8), torch.tensor([1.9, 2.1]), torch.tensor([True]),
+              torch.tensor([2.0], dtype=torch.bfloat16), np.array([[4], [5]])):
+        x = list(x) if not isinstance(x, (np.ndarray, torch.Tensor)) else x
+        got = _host_int32(x)
+        assert got.dtype == np.int32 and got.flags.c_contiguous
+        assert got.tolist() == [ctypes.c_int32(int(v)).value for v in x]
+    for bad in ([float("nan")], np.array([1.0, np.inf]), np.zeros((2, 3), np.int32), torch.zeros(2, 3, dtype=torch.int32), [None], torch.tensor(3),
+                torch.tensor([1j])):
+        with pytest.raises((TypeError, ValueError, OverflowError, RuntimeError)):
+            _host_int32(bad)
