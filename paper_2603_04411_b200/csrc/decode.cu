@@ -503,7 +503,7 @@ static cudaError_t launch_decode_t(const DevView& v, int layer, const LayerParam
     }
     if (e != cudaSuccess) return e;
   }
-  count_launch(4);
+  count_launch(3);                                     // the K-score launch counts itself
   return cudaGetLastError();
 }
 

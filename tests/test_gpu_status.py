@@ -186,3 +186,16 @@ def test_decode_call_replays_from_a_cuda_graph():
         torch.testing.assert_close(out, eager, rtol=0, atol=0)
     assert B.twkv_cache_status(gc.h) == B.TWKV_OK
     gc.close()
+
+
+def test_a_decode_call_counts_its_kernels_once():
+    from paper_2603_04411_b200 import build
+    build.build()
+    from paper_2603_04411_b200 import binding as B
+    gc, li = _filled_cache(B)
+    _decode(B, gc, li)                                                      # the first call also lays out the basis
+    before = B.twkv_launch_count()
+    _decode(B, gc, li)
+    assert B.twkv_launch_count() - before == 4                              # plan, K scores, V sums, merge
+    assert B.twkv_cache_status(gc.h) == B.TWKV_OK
+    gc.close()
