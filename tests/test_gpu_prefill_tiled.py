@@ -1,12 +1,14 @@
 """The tiled form of chunked-prefill attention where its work split changes, against the CPU oracle: several segments of rows,
-several groups of query blocks, an odd number of KV heads, repeated positions, a block of one tile beside a block of two.
-Bars as for every attention test (max-abs 2e-3, relative L2 1e-3)."""
+several groups of query blocks, an odd number of KV heads, repeated positions, a block of one tile beside a block of two; values of
+any size, output types, score scales; and the calls that run as decode passes instead.
+Bars as for every attention test (max-abs 2e-3, relative L2 1e-3) where no other is stated."""
 import numpy as np
 import pytest
 import torch
 
+import oracle
 from paper_2603_04411_b200 import workloads
-from tests.helpers import GpuCache, attn_errors
+from tests.helpers import GpuCache, attn_errors, bits16
 from tests.test_gpu_prefill import MAX_ABS, REL_L2, B, _case, _oracle_prefill
 
 pytestmark = pytest.mark.gpu
@@ -35,11 +37,15 @@ def test_tiled_prefill_where_the_work_split_changes(B, hkv, rep, dtype, n_seq, c
     assert max_abs < MAX_ABS and rel_l2 < REL_L2, (max_abs, rel_l2)
 
 
-def _filled(B, li, ranks, *, out_dtype=torch.float32, **cfg):
+def _filled(B, li, ranks, *, out_dtype=torch.float32, sm_scale=None, **cfg):
     """A cache with the layer's tokens, one compress call."""
     n_seq = int(li.seq_ids.max()) + 1
     sizes = dict(max_seqs=n_seq, max_tokens_per_seq=int(np.bincount(li.seq_ids.numpy()).max()), payload_bytes=int((-(-ranks // 64) * 128).sum()))
     gc = GpuCache(B, n_layers=1, n_q_heads=li.n_q_heads, n_kv_heads=li.n_kv_heads, dtype=li.dtype, out_dtype=out_dtype, **{**sizes, **cfg})
+    if sm_scale is not None:
+        gc.close()
+        gc.cfg.sm_scale = sm_scale
+        gc.h = B.twkv_cache_create(gc.cfg, gc.pool)
     B.twkv_cache_set_layer_params(gc.h, 0, li.Uinv_k.cuda(), li.Uinv_v.cuda())
     B.twkv_compress(gc.h, 0, li.xt_k.cuda(), li.xt_v.cuda(), li.seq_ids.cuda(), li.positions.cuda(), None,
                     torch.from_numpy(ranks.astype(np.int16)).cuda(), B.TWKV_GATE_FORCED)
@@ -197,3 +203,107 @@ def test_tiled_prefill_is_as_exact_as_decode(B):
         gc.close()
     tiled, decode = np.mean(err, axis=0)
     assert tiled < 1.15 * decode, (tiled, decode)
+
+
+@pytest.mark.parametrize("n_q", [60, 8])         # one split: written by the attention kernel; several: by the kernel that joins them
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
+def test_tiled_prefill_output_types(B, dtype, n_q):
+    # a 16-bit output is the fp32 one rounded to nearest even, bit for bit
+    ctx = 100 if n_q == 60 else 700
+    li = workloads.build_layer(897, n_seq=1, ctx=ctx, n_q_heads=12, n_kv_heads=3, n_calib=768, dtype=dtype, mode="forced", rank_recipe="any")
+    ranks = li.ranks.numpy().astype(np.int64)
+    q_pos, q_seq = np.arange(ctx - n_q, ctx), np.zeros(n_q, np.int64)
+    q = torch.randn(n_q, 12, 128, generator=torch.Generator().manual_seed(7)).to(dtype)
+    got = {}
+    for od in (torch.float32, torch.float16, torch.bfloat16):
+        gc = _filled(B, li, ranks, out_dtype=od)
+        got[od] = torch.from_numpy(_prefill(B, gc, q, q_seq, q_pos))
+        gc.close()
+    max_abs, rel_l2 = attn_errors(got[torch.float32].numpy(), _oracle_prefill(li, ranks, q, q_seq, q_pos))
+    assert max_abs < MAX_ABS and rel_l2 < REL_L2, (max_abs, rel_l2)
+    for od in (torch.float16, torch.bfloat16):
+        torch.testing.assert_close(got[od], got[torch.float32].to(od).float(), rtol=0, atol=0)
+
+
+@pytest.mark.parametrize("sm_scale", [-0.11, 0.0, 0.5])
+def test_tiled_prefill_score_scales(B, sm_scale):
+    li = workloads.build_layer(898, n_seq=2, ctx=150, n_q_heads=8, n_kv_heads=2, n_calib=512, mode="forced", rank_recipe="any")
+    ranks = li.ranks.numpy().astype(np.int64)
+    q_seq, q_pos = np.repeat([0, 1], 40), np.tile(np.arange(110, 150), 2)
+    q = torch.randn(80, 8, 128, generator=torch.Generator().manual_seed(8)).to(torch.float16)
+    gc = _filled(B, li, ranks, sm_scale=sm_scale)
+    got = _prefill(B, gc, q, q_seq, q_pos)
+    gc.close()
+    scale = float(np.float32(sm_scale))
+    w = lambda t: oracle.widen16(bits16(t), "f16")
+    want = np.zeros((80, 8, 128))
+    for s in (0, 1):
+        idx, rows = np.nonzero(li.seq_ids.numpy() == s)[0], q_seq == s
+        want[rows] = oracle.prefill_attn(w(li.xt_k)[idx], w(li.xt_v)[idx], ranks[idx, 0], ranks[idx, 1], li.positions.numpy()[idx], w(li.Uinv_k),
+                                         w(li.Uinv_v), w(q)[rows], q_pos[rows], 2, 500000.0, scale)
+    max_abs, rel_l2 = attn_errors(got, want)
+    assert max_abs < MAX_ABS and rel_l2 < REL_L2, (max_abs, rel_l2)
+
+
+@pytest.mark.parametrize("scale,code", [(1.0, 0), (3000.0, 5)])
+def test_tiled_prefill_reports_clamped_keys_when_asked(B, monkeypatch, scale, code):
+    # a cache created with TWKV_DEBUG=1 reports rotated keys beyond the f16 range (here up to around 1e5), and only those
+    monkeypatch.setenv("TWKV_DEBUG", "1")
+    li = workloads.build_layer(899, n_seq=1, ctx=200, n_q_heads=8, n_kv_heads=2, n_calib=512, mode="forced", outlier="none", rank_recipe="any")
+    li.xt_k = (li.xt_k.float() * scale).to(torch.float16)
+    li.Uinv_k = (li.Uinv_k.float() * min(scale, 10.0)).to(torch.float16)
+    ranks = li.ranks.numpy().astype(np.int64)
+    gc = _filled(B, li, ranks)
+    out = torch.empty(50, 8, 128, device="cuda")
+    B.twkv_prefill_attn(gc.h, 0, torch.ones(50, 8, 128, dtype=torch.float16, device="cuda"), np.zeros(50, np.int64), np.arange(150, 200), out)
+    assert B.twkv_cache_status(gc.h) == code
+    gc.close()
+
+
+@pytest.mark.parametrize("counts,num_splits", [
+    ((3, 1), 0),                                 # three passes, the later ones for one sequence alone
+    ((2, 3), 5),                                 # three passes, the splits given by the caller
+    ((4, 4), 0),                                 # one query more: the tiled form
+])
+def test_prefill_on_both_sides_of_the_rule(B, counts, num_splits):
+    # few queries per sequence over 2 x 6000 tokens: passes of the decode kernels, one after the other over the same scratch
+    ctx, n_q = 6000, sum(counts)
+    li = workloads.build_layer(865, n_seq=2, ctx=ctx, n_q_heads=8, n_kv_heads=1, n_calib=256, outlier="pct:1", mode="forced", rank_recipe="any",
+                               shuffle_positions=True)
+    ranks = li.ranks.numpy().astype(np.int64)
+    rng = np.random.default_rng(n_q)
+    perm = rng.permutation(n_q)
+    q_seq, q_pos = np.repeat([0, 1], counts)[perm], rng.integers(0, ctx, n_q)
+    q_pos[[list(q_seq).index(0), list(q_seq).index(1)]] = ctx - 1
+    q = torch.randn(n_q, 8, 128, generator=torch.Generator().manual_seed(9)).to(torch.float16)
+    gc = _filled(B, li, ranks)
+    launches = B.twkv_launch_count()
+    got = _prefill(B, gc, q, q_seq, q_pos, num_splits)
+    launches = B.twkv_launch_count() - launches
+    assert (launches == 4 * max(counts) + 1) == (max(counts) == 3), launches       # four kernels a pass, and the first one's set-up
+    assert B.twkv_cache_check(gc.h) == (B.TWKV_OK, 0)
+    max_abs, rel_l2 = attn_errors(got, _oracle_prefill(li, ranks, q, q_seq, q_pos))
+    assert max_abs < MAX_ABS and rel_l2 < REL_L2, (max_abs, rel_l2)
+    if num_splits:
+        with pytest.raises(B.TwkvError) as err:                                     # more splits than the partial results have room for
+            B.twkv_prefill_attn(gc.h, 0, q.cuda(), q_seq, q_pos, torch.empty(n_q, 8, 128, device="cuda"), 1000)
+        assert err.value.code == B.TWKV_ERR_INVALID_ARG
+    gc.close()
+
+
+def test_prefill_whose_tables_do_not_fit_runs_in_passes(B):
+    # 65 sequences asked for at the last position there is: their bitmaps would need more than the region they live in
+    n_seq, ctx, n_q = 65, 100, 8
+    li = workloads.build_layer(866, n_seq=n_seq, ctx=ctx, n_q_heads=8, n_kv_heads=1, n_calib=256, mode="forced", rank_recipe="any")
+    ranks = li.ranks.numpy().astype(np.int64)
+    q_seq = np.tile(np.arange(n_seq), n_q)
+    q_pos = np.full(n_seq * n_q, 524287)
+    q_pos[:n_seq] = 40
+    q = torch.randn(n_seq * n_q, 8, 128, generator=torch.Generator().manual_seed(9)).to(torch.float16)
+    gc = _filled(B, li, ranks)
+    launches = B.twkv_launch_count()
+    got = _prefill(B, gc, q, q_seq, q_pos)
+    assert B.twkv_launch_count() - launches == 4 * n_q + 1
+    gc.close()
+    max_abs, rel_l2 = attn_errors(got, _oracle_prefill(li, ranks, q, q_seq, q_pos))
+    assert max_abs < MAX_ABS and rel_l2 < REL_L2, (max_abs, rel_l2)
