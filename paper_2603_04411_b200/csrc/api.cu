@@ -101,17 +101,14 @@ struct Layout {
 };
 
 constexpr int GATE_PIECE = 8192;       // tokens per COMPUTE-mode gate piece (logits scratch rows)
-// Whether the tiled prefill kernels serve a call that would take n_waves decode passes over `rows` tokens.  A wave rebuilds every
-// key (and shares nothing), the tiled kernels rebuild keys and values once but store both in full width.  Microseconds measured
-// with one sequence (8 KV heads, ranks around 256): 1, 2, 3 waves 65, 112, 163 over 1024 tokens, 90, 164, 239 over 32768; tiled,
-// 4 to 8 queries, 80 over 1024, 184 over 8192, 408 over 32768.
-static bool prefill_tiled_pays(int n_waves, double rows) { return n_waves >= 2 && n_waves * (50.0 + rows / 1000.0) >= 75.0 + rows / 100.0; }
 // COMPUTE-mode calls of this many tokens form the logits with gate_logits_tc_kernel; smaller ones, bound by launches and the
 // weights' way in, with the warp-MMA kernel; larger ones run the fused tcgen05 gate kernel, whose logits stay on the SM.
 // A whole compress call in us, warp-MMA / spread / fused (d_kv 1024): 128 tokens 39.2 / 32.8 / -, 1000 67.7 / 46.2 / -,
 // 2048 81.3 / 54.3 / 61.8, 3072 104 / 60.6 / 63.1, 4096 131 / 72.0 / 66.3; d_kv 512: 100 tokens 28.7 / 28.7 / -, 1000 47.7 / 38.2 / -,
 // 3072 61.6 / 46.0 / 52.3, 6000 80.3 / 57.7 / 51.4; d_kv 384: 3072 tokens - / 44.1 / 47.4, 4096 - / 51.4 / 47.4.
 constexpr int GATE_LOGITS_TC_MIN = 128, GATE_LOGITS_TC_MAX = 3072;
+
+constexpr long long PF_MAX_WORDS = 900000;   // bitmap words of a tiled prefill: two ints each beside the other tables in the region of the gate's fix-up list
 
 struct Offsets {
   size_t status, pflags, rope_lo, rope_hi, n_tiles, tile_desc, tile_aux, tile_rank, fill, key_last, kclass_count,
@@ -597,76 +594,109 @@ twkv_status twkv_decode_attn(twkv_cache* c, int layer, const void* q, const int3
   return decode_pass(c, layer, q, seq_ids, n_seq, out, num_splits, nullptr, nullptr, (cudaStream_t)stream);
 }
 
-// The tiled form of a prefill call: queries sorted by (sequence, position), dense rows of the visible tokens in segments.
-// `order`: query indices sorted that way; rows_max: upper bound on the rows where no two tokens of a sequence share a position;
-// rows_all: the bound where they do.  Sets *done = false, with nothing launched, where the call's tables do not fit the scratch
-// regions they live in (the caller then serves the queries in waves).
-static twkv_status prefill_tiled(twkv_cache* c, int layer, const void* q, const int32_t* q_seq, const int32_t* q_pos, const std::vector<int>& order,
-                                 long long rows_max, long long rows_all, void* out, cudaStream_t st, bool* done) {
+// One tiled prefill: queries lo .. hi-1 of a call's queries sorted by (sequence, position), whole sequences; dense rows of the visible
+// tokens in segments.
+struct PfPlan {
+  int lo, hi, n_u, n_blocks;
+  long long n_words;
+  int seg_rows, n_segs, n_splits, group;
+  double us;                            // estimated time
+};
+
+// rows_max: bound on the rows where no two tokens of a sequence share a position; rows_all: the bound where they do; seq_rows: every
+// sequence's part of rows_max, in order.
+static PfPlan plan_tiled(const twkv_cache* c, const int32_t* q_seq, const int32_t* q_pos, const std::vector<int>& order, int lo, int hi,
+                         const long long* seq_rows, long long rows_max, long long rows_all) {
   const DevView& v = c->view;
-  const int n_q = (int)order.size(), QT = TILE / v.rep, pos_end = ROPE_LO * ROPE_HI;
-  *done = false;
+  const int QT = TILE / v.rep;
+  PfPlan pl = {lo, hi, 0, 0, 0, 0, 0, 1, 1, 1e300};
+  std::vector<int> first;               // first block of every sequence
+  bool two_tiles = false;
+  for (int i = lo; i < hi;) {
+    int e = i;
+    while (e < hi && q_seq[order[e]] == q_seq[order[i]]) ++e;
+    first.push_back(pl.n_blocks);
+    pl.n_blocks += (e - i + 2 * QT - 1) / (2 * QT);
+    pl.n_words += (std::min(q_pos[order[e - 1]], ROPE_LO * ROPE_HI - 1) + 32) >> 5;
+    two_tiles |= e - i > QT;
+    ++pl.n_u;
+    i = e;
+  }
+  first.push_back(pl.n_blocks);
+  // what does not fit the scratch regions is left to the waves; a tile's segments are kept in two 16-bit halves
+  const size_t n_q = (size_t)(hi - lo), tables = 4 * (size_t)pl.n_blocks + n_q + 3 * (size_t)pl.n_u + 4 + (size_t)v.S + 2 * (size_t)pl.n_words;
+  if (tables > gate_tc_fix_bytes() / sizeof(int) || 2 * n_q + 2 * (size_t)pl.n_blocks + 3 * (size_t)pl.n_u > 3 * (size_t)TWKV_PREFILL_MAX_QUERIES ||
+      rows_all > 32767ll * (GATE_PIECE / 2)) return pl;
+  // Segments of 8192 rows with the partial results in the V pass's region, or of 4096 rows with them in the second half of
+  // the gate scratch (fewer heads leave the first region small); splits of a segment's rows where the blocks of queries
+  // alone leave SMs idle.  Estimated in key blocks of one CTA (4.5 us with two tiles of queries, 0.65 of that with one): the slowest
+  // item or the mean of a CTA's, 1.5 for an item's start and end, and the segment's reconstruction; besides, tables, joins, and the
+  // launches that only repeated positions need.
+  const size_t slot_bytes = PF_SLOT_FLOATS * sizeof(float);
+  const double kb = two_tiles ? 1.0 : 0.65, heads = 0.4 + 0.075 * v.Hkv;
+  for (int half = 0; half < 2; ++half) {
+    const int seg_rows = half ? GATE_PIECE / 2 : GATE_PIECE;
+    const size_t region = half ? (size_t)GATE_PIECE * v.d_kv * sizeof(float) : (size_t)c->dims.max_partials * v.Hq * v.d_kv * sizeof(float);
+    const long long cap = (long long)(region / slot_bytes);
+    const int group = (int)std::min<long long>(pl.n_blocks, cap / v.Hkv);
+    if (group < 1) continue;
+    const double groups = (double)((pl.n_blocks + group - 1) / group), segs = (double)((rows_max + seg_rows - 1) / seg_rows);
+    long long sum = 0, most = 1;        // key blocks of a segment that the blocks of queries go through
+    for (int u = 0; u < pl.n_u; ++u) {
+      const long long n = std::min<long long>(seq_rows[u], seg_rows) / TILE;
+      sum += n * (first[u + 1] - first[u]);
+      most = std::max(most, n);
+    }
+    for (int ns = 1; ns <= 32 && ns <= most && (long long)group * v.Hkv * ns <= cap; ++ns) {
+      const long long rounds = ((long long)group * v.Hkv * ns + c->sm_count - 1) / c->sm_count;
+      const double item = std::max((double)((most + ns - 1) / ns), (double)rounds * sum / ((double)pl.n_blocks * ns));
+      const double cost = groups * segs * (kb * item + 1.5 * rounds + heads * (4.0 + std::min<long long>(rows_max, seg_rows) / 1024.0));
+      const int n_segs = std::max(1, (int)((rows_all + seg_rows - 1) / seg_rows));
+      const double us = 20.0 + 4.5 * cost + (n_segs > 1 || ns > 1 ? 4.0 * groups : 0.0) + 3.4 * groups * (n_segs - segs);
+      if (us < pl.us) { pl.us = us; pl.seg_rows = seg_rows; pl.n_segs = n_segs; pl.n_splits = ns; pl.group = group; }
+    }
+  }
+  return pl;
+}
+
+static twkv_status run_tiled(twkv_cache* c, int layer, const void* q, const int32_t* q_seq, const int32_t* q_pos, const std::vector<int>& order,
+                             const PfPlan& pl, void* out, cudaStream_t st) {
+  const DevView& v = c->view;
+  const int n_q = pl.hi - pl.lo, QT = TILE / v.rep, pos_end = ROPE_LO * ROPE_HI, n_blocks = pl.n_blocks;
+  const int* ord = order.data() + pl.lo;
   std::vector<int> host(2 * (size_t)n_q), blocks, seqs;
-  long long n_words = 0;
-  for (int lo = 0; lo < n_q;) {
+  for (int lo = 0, n_words = 0; lo < n_q;) {
     int hi = lo;
-    while (hi < n_q && q_seq[order[hi]] == q_seq[order[lo]]) ++hi;
-    const int u = (int)seqs.size() / 3, maxq = std::min(q_pos[order[hi - 1]], pos_end - 1);
-    seqs.push_back(q_seq[order[lo]]); seqs.push_back(maxq); seqs.push_back((int)n_words);
+    while (hi < n_q && q_seq[ord[hi]] == q_seq[ord[lo]]) ++hi;
+    const int u = (int)seqs.size() / 3, maxq = std::min(q_pos[ord[hi - 1]], pos_end - 1);
+    seqs.push_back(q_seq[ord[lo]]); seqs.push_back(maxq); seqs.push_back(n_words);
     n_words += (maxq + 32) >> 5;
     for (int b = lo; b < hi; b += 2 * QT) { blocks.push_back(b); blocks.push_back(u << 9 | std::min(2 * QT, hi - b)); }
     lo = hi;
   }
-  for (int i = 0; i < n_q; ++i) { host[i] = order[i]; host[n_q + i] = q_pos[order[i]]; }
-  const int n_u = (int)seqs.size() / 3, n_blocks = (int)blocks.size() / 2;
+  for (int i = 0; i < n_q; ++i) { host[i] = ord[i]; host[n_q + i] = q_pos[ord[i]]; }
   host.insert(host.end(), blocks.begin(), blocks.end());
   host.insert(host.end(), seqs.begin(), seqs.end());
-  // the tables made on the device share the region of the gate's fix-up list
-  const size_t fix_ints = gate_tc_fix_bytes() / sizeof(int);
-  const size_t need = 4 * (size_t)n_blocks + n_q + 3 * (size_t)n_u + 4 + (size_t)v.S + 2 * (size_t)n_words;
-  if (need > fix_ints || host.size() > 3 * (size_t)TWKV_PREFILL_MAX_QUERIES) return TWKV_OK;
 
   PfCall a = {};
   const int* w = v.wave_buf;
   a.qrow = w; a.qpos = w + n_q; a.blocks = (const int2*)(w + 2 * (size_t)n_q); a.seqs = w + 2 * (size_t)n_q + blocks.size();
-  a.n_u = n_u; a.n_blocks = n_blocks; a.n_words = (int)n_words;
+  a.n_u = pl.n_u; a.n_blocks = n_blocks; a.n_words = (int)pl.n_words;
+  // the tables made on the device share the region of the gate's fix-up list
   a.binfo = v.gate_fix;
   int* p = (int*)(v.gate_fix + n_blocks);
   a.qvis = p; p += n_q;
-  a.rows = p; a.base = p + n_u; a.dup = p + 2 * (size_t)n_u; p += 3 * (size_t)n_u;
+  a.rows = p; a.base = p + a.n_u; a.dup = p + 2 * (size_t)a.n_u; p += 3 * (size_t)a.n_u;
   a.ticket = p; a.total = p + 1; p += 4;
   a.slot = p; p += v.S;
-  a.bits = (unsigned*)p; a.pref = p + n_words;
+  a.bits = (unsigned*)p; a.pref = p + pl.n_words;
   a.krow = v.kv_link; a.krow_out = v.evict_map; a.vrow = v.evict_map + (size_t)v.NT * TILE;
   a.rowpos = (int*)v.scores;
   a.seg_buf = (unsigned char*)v.gate_scratch;
   a.vexp = (signed char*)v.hist;                                    // 8448 bytes per KV head of at least 16384
   a.vflag = (int*)(a.vexp + (size_t)GATE_PIECE * v.Hkv);
-
-  if (rows_all > 32767ll * (GATE_PIECE / 2)) return TWKV_OK;         // a tile's segments are kept in two 16-bit halves
-  // Segments of 8192 rows with the partial results in the V pass's region, or of 4096 rows with them in the second half of
-  // the gate scratch (fewer heads leave the first region small); splits of a segment's rows where the blocks of queries
-  // alone leave SMs idle.  Estimated in key blocks of one CTA: its share of a segment plus 1.5 for an item's start and end.
-  const size_t slot_bytes = PF_SLOT_FLOATS * sizeof(float);
-  double best = 1e300;
-  int best_rows = 0, best_splits = 1, best_group = 1;
-  for (int half = 0; half < 2; ++half) {
-    const int seg_rows = half ? GATE_PIECE / 2 : GATE_PIECE;
-    const size_t region = half ? (size_t)GATE_PIECE * v.d_kv * sizeof(float) : (size_t)c->dims.max_partials * v.Hq * v.d_kv * sizeof(float);
-    const long long cap = (long long)(region / slot_bytes);
-    const int group = (int)std::min<long long>(n_blocks, cap / v.Hkv);
-    if (group < 1) continue;
-    const double groups = (double)((n_blocks + group - 1) / group), segs = (double)((rows_max + seg_rows - 1) / seg_rows);
-    const int seg_blocks = std::max(1, (int)((std::min<long long>(rows_max, seg_rows) + TILE - 1) / TILE));
-    for (int ns = 1; ns <= 32 && ns <= seg_blocks && (long long)group * v.Hkv * ns <= cap; ++ns) {
-      const long long rounds = ((long long)group * v.Hkv * ns + c->sm_count - 1) / c->sm_count;
-      const double cost = groups * segs * ((double)rounds * ((seg_blocks + ns - 1) / ns + 1.5) + 4.0 + std::min<long long>(rows_max, seg_rows) / 1024.0);
-      if (cost < best) { best = cost; best_rows = seg_rows; best_splits = ns; best_group = group; }
-    }
-  }
-  if (!best_rows) return TWKV_OK;
-  a.seg_rows = best_rows; a.n_splits = best_splits;
-  a.slots = best_rows == GATE_PIECE ? v.part_acc : (float*)(a.seg_buf + (size_t)GATE_PIECE * v.d_kv * sizeof(float));
+  a.seg_rows = pl.seg_rows; a.n_splits = pl.n_splits;
+  a.slots = pl.seg_rows == GATE_PIECE ? v.part_acc : (float*)(a.seg_buf + (size_t)GATE_PIECE * v.d_kv * sizeof(float));
 
   PfMaps maps;
   maps.blocks = c->map_blocks;
@@ -674,15 +704,13 @@ static twkv_status prefill_tiled(twkv_cache* c, int layer, const void* q, const 
   if (!make_tmap_2d(&maps.uk, c->params[layer].Uinv_k, d, d, d * 2, PANEL) || !make_tmap_2d(&maps.uv, c->params[layer].Uinv_v, d, d, d * 2, PANEL) ||
       !make_tmap_2d(&maps.seg, a.seg_buf, (uint64_t)v.Hkv * 4 * a.seg_rows, HEAD_DIM, HEAD_DIM * 2, TILE)) return TWKV_ERR_CUDA;
   if (upload_ints(v.wave_buf, host, st) != cudaSuccess) return TWKV_ERR_CUDA;
-  *done = true;
   if (launch_pf_tables(v, a, layer, c->sm_count, st) != cudaSuccess) return TWKV_ERR_CUDA;
   // the segments past the call's last row are launched for repeated positions alone: their kernels look at the number of rows and leave
-  const int n_segs = std::max(1, (int)((rows_all + a.seg_rows - 1) / a.seg_rows));
-  for (a.blk0 = 0; a.blk0 < n_blocks; a.blk0 += best_group) {
-    a.blk_n = std::min(best_group, n_blocks - a.blk0);
-    for (int seg = 0; seg < n_segs; ++seg)
+  for (a.blk0 = 0; a.blk0 < n_blocks; a.blk0 += pl.group) {
+    a.blk_n = std::min(pl.group, n_blocks - a.blk0);
+    for (int seg = 0; seg < pl.n_segs; ++seg)
       if (launch_pf_segment(v, a, maps, layer, seg, q, out, c->sm_count, st) != cudaSuccess) return TWKV_ERR_CUDA;
-    if ((n_segs > 1 || a.n_splits > 1) && launch_pf_combine(v, a, out, st) != cudaSuccess) return TWKV_ERR_CUDA;
+    if ((pl.n_segs > 1 || a.n_splits > 1) && launch_pf_combine(v, a, out, st) != cudaSuccess) return TWKV_ERR_CUDA;
   }
   return TWKV_OK;
 }
@@ -710,25 +738,56 @@ twkv_status twkv_prefill_attn(twkv_cache* c, int layer, const void* q, const int
   DeviceGuard g(c->device);
   if (!g.ok) return TWKV_ERR_CUDA;
   cudaStream_t st = (cudaStream_t)stream;
-  // How many rows (visible tokens, a sequence's rounded up to whole tiles) the call can have: one per position up to its largest query's.
-  // More only where tokens share a position: then up to the sequences' capacity, or what the layer was ever given.
-  auto rows_of = [](long long tokens) { return (tokens + TILE - 1) / TILE * TILE; };
-  std::vector<int> last(S, -1);
-  for (int i = 0; i < n_q; ++i) last[q_seq[i]] = std::max(last[q_seq[i]], q_pos[i]);
-  long long rows_max = 0, rows_all = n_distinct * rows_of(c->cfg.max_tokens_per_seq);
-  for (int s = 0; s < S; ++s)
-    if (last[s] >= 0) rows_max += rows_of(std::min<long long>(c->cfg.max_tokens_per_seq, last[s] + 1ll));
-  if (!c->append_captured.load(std::memory_order_relaxed) && !is_capturing(st))
-    rows_all = std::min(rows_all, c->appended[layer].load(std::memory_order_relaxed) + (TILE - 1) * (long long)n_distinct);
-  if (prefill_tiled_pays(n_waves, (double)rows_max)) {
-    ProfBind pb(&c->prof);
+  // A wave rebuilds every key (and shares nothing), the tiled kernels rebuild keys and values once for all queries but store both in
+  // full width, which few queries per sequence over a long context do not earn back.  Both forms are estimated, in microseconds; a
+  // wave as 38 + 0.6 per sequence + 0.9 per 1000 tokens (8 KV heads; keys and ranks both grow with their number).  Measured, tiled /
+  // waves: 16 sequences of 8192 tokens, 8 queries each 1599 / 1245, 12 queries 1601 / 1868; 64 of 8192, 12 queries 7000 / 6004, 16
+  // queries 7001 / 8373; 64 of 1000, 4 queries 764 / 552, 8 queries 778 / 1096; one of 32768, 4 queries 315 / 275, 6 queries
+  // 319 / 411; one of 2000, 2 queries 75 / 83; 4 KV heads, 16 of 8192, 12 queries 1285 / 1019, 24 queries 1302 / 2036.
+  if (n_waves >= 2) {
     std::vector<int> order(n_q);
     for (int i = 0; i < n_q; ++i) order[i] = i;
     if (!sorted)
       std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return q_seq[x] != q_seq[y] ? q_seq[x] < q_seq[y] : q_pos[x] < q_pos[y]; });
-    bool done = false;
-    const twkv_status s = prefill_tiled(c, layer, q, q_seq, q_pos, order, rows_max, std::max(rows_max, rows_all), out, st, &done);
-    if (done || s != TWKV_OK) return s;
+    // Rows (visible tokens, rounded up to whole tiles) of a sequence: one per position up to its largest query's.  More only where
+    // tokens share a position: then up to its capacity, or what the layer was ever given.
+    auto rows_of = [](long long tokens) { return (tokens + TILE - 1) / TILE * TILE; };
+    const long long tmax = c->cfg.max_tokens_per_seq;
+    const int v_heads = c->cfg.n_kv_heads;
+    long long given = 1ll << 60;
+    if (!c->append_captured.load(std::memory_order_relaxed) && !is_capturing(st)) given = c->appended[layer].load(std::memory_order_relaxed);
+    // Sequences that fit a segment together share a run of the tiled kernels; a longer one has a run of its own, so that all blocks of
+    // queries have work in every segment.
+    std::vector<PfPlan> plans;
+    std::vector<long long> rows;
+    double tiled = 0.0, waves = 38.0 * n_waves;
+    const double wave_row = 0.9e-3 * v_heads * v_heads / 64.0;
+    long long sum = 0, words = 0;
+    int lo = 0;
+    auto close = [&](int hi) {
+      const long long n = (long long)rows.size();
+      plans.push_back(plan_tiled(c, q_seq, q_pos, order, lo, hi, rows.data(), sum, std::max(sum, std::min(n * rows_of(tmax), given + n * (TILE - 1)))));
+      tiled += plans.back().us + (lo > 0 ? 8.0 : 0.0);           // (a run behind another waits for its lists)
+      rows.clear(); sum = words = 0; lo = hi;
+    };
+    for (int i = 0; i < n_q;) {
+      int e = i;
+      while (e < n_q && q_seq[order[e]] == q_seq[order[i]]) ++e;
+      const long long last = std::min(q_pos[order[e - 1]], ROPE_LO * ROPE_HI - 1), r = rows_of(std::min(tmax, last + 1));
+      if (!rows.empty() && (sum + r > GATE_PIECE || words + last / 32 > PF_MAX_WORDS)) close(i);
+      rows.push_back(r); sum += r; words += last / 32 + 1;
+      waves += (e - i) * (0.6 + wave_row * (double)r);
+      i = e;
+    }
+    close(n_q);
+    if (tiled < waves) {
+      ProfBind pb(&c->prof);
+      for (const PfPlan& pl : plans) {
+        const twkv_status s = run_tiled(c, layer, q, q_seq, q_pos, order, pl, out, st);
+        if (s != TWKV_OK) return s;
+      }
+      return TWKV_OK;
+    }
   }
   std::vector<int> wave_start(n_waves + 1, 0), fill(n_waves, 0);
   for (int i = 0; i < n_q; ++i) ++wave_start[wave_of[i] + 1];

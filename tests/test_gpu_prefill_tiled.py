@@ -291,19 +291,60 @@ def test_prefill_on_both_sides_of_the_rule(B, counts, num_splits):
     gc.close()
 
 
-def test_prefill_whose_tables_do_not_fit_runs_in_passes(B):
-    # 65 sequences asked for at the last position there is: their bitmaps would need more than the region they live in
+def test_prefill_of_many_sequences_at_the_last_positions(B):
+    # 65 sequences asked for at the last position there is: their bitmaps fill the region they live in, so the call takes several runs
     n_seq, ctx, n_q = 65, 100, 8
     li = workloads.build_layer(866, n_seq=n_seq, ctx=ctx, n_q_heads=8, n_kv_heads=1, n_calib=256, mode="forced", rank_recipe="any")
     ranks = li.ranks.numpy().astype(np.int64)
     q_seq = np.tile(np.arange(n_seq), n_q)
     q_pos = np.full(n_seq * n_q, 524287)
-    q_pos[:n_seq] = 40
+    q_pos[:n_seq], q_pos[n_seq] = 40, 2 ** 31 - 1
+    q = torch.randn(n_seq * n_q, 8, 128, generator=torch.Generator().manual_seed(9)).to(torch.float16)
+    gc = _filled(B, li, ranks)
+    got = _prefill(B, gc, q, q_seq, q_pos)
+    gc.close()
+    max_abs, rel_l2 = attn_errors(got, _oracle_prefill(li, ranks, q, q_seq, q_pos))
+    assert max_abs < MAX_ABS and rel_l2 < REL_L2, (max_abs, rel_l2)
+
+
+@pytest.mark.parametrize("lengths,n_q", [
+    ((9000, 300, 5000, 2000, 4000), 40),         # one alone over two segments, then runs of three and one
+    ((130, 70, 9), 3),                           # all in one run
+])
+def test_prefill_of_sequences_of_different_lengths(B, lengths, n_q):
+    # sequences that fit a segment together share a run of the tiled kernels, longer ones have one of their own
+    n_seq, ctx = len(lengths), max(lengths)
+    li = workloads.build_layer(867, n_seq=n_seq, ctx=ctx, n_q_heads=8, n_kv_heads=1, n_calib=256, mode="forced", rank_recipe="any")
+    stay = li.positions < torch.tensor(lengths, dtype=torch.int32)[li.seq_ids.long()]
+    for name in ["xt_k", "xt_v", "seq_ids", "positions", "ranks"]:
+        setattr(li, name, getattr(li, name)[stay].contiguous())
+    ranks = li.ranks.numpy().astype(np.int64)
+    rng = np.random.default_rng(10)
+    perm = rng.permutation(n_seq * n_q)
+    q_seq = np.repeat(np.arange(n_seq), n_q)[perm]
+    q_pos = np.concatenate([np.sort(rng.integers(0, n, n_q)) for n in lengths])[perm]
+    q = torch.randn(n_seq * n_q, 8, 128, generator=torch.Generator().manual_seed(9)).to(torch.float16)
+    gc = _filled(B, li, ranks)
+    got = _prefill(B, gc, q, q_seq, q_pos)
+    assert B.twkv_cache_check(gc.h) == (B.TWKV_OK, 0)
+    gc.close()
+    max_abs, rel_l2 = attn_errors(got, _oracle_prefill(li, ranks, q, q_seq, q_pos))
+    assert max_abs < MAX_ABS and rel_l2 < REL_L2, (max_abs, rel_l2)
+
+
+def test_prefill_of_few_queries_over_many_long_sequences_runs_in_passes(B):
+    # eight queries each over sixteen sequences that fill a segment of their own: a run of the tiled kernels per sequence would take
+    # three times the passes' time
+    n_seq, ctx, n_q = 16, 8192, 8
+    li = workloads.build_layer(868, n_seq=n_seq, ctx=ctx, n_q_heads=8, n_kv_heads=1, n_calib=256, mode="forced", rank_recipe="any")
+    ranks = li.ranks.numpy().astype(np.int64)
+    q_seq, q_pos = np.repeat(np.arange(n_seq), n_q), np.tile(np.arange(ctx - n_q, ctx), n_seq)
     q = torch.randn(n_seq * n_q, 8, 128, generator=torch.Generator().manual_seed(9)).to(torch.float16)
     gc = _filled(B, li, ranks)
     launches = B.twkv_launch_count()
     got = _prefill(B, gc, q, q_seq, q_pos)
     assert B.twkv_launch_count() - launches == 4 * n_q + 1
     gc.close()
-    max_abs, rel_l2 = attn_errors(got, _oracle_prefill(li, ranks, q, q_seq, q_pos))
+    pick = np.arange(0, n_seq * n_q, 13)
+    max_abs, rel_l2 = attn_errors(got[pick], _oracle_prefill(li, ranks, q[pick], q_seq[pick], q_pos[pick]))
     assert max_abs < MAX_ABS and rel_l2 < REL_L2, (max_abs, rel_l2)
