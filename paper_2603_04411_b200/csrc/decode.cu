@@ -488,8 +488,11 @@ static cudaError_t launch_decode_t(const DevView& v, int layer, const LayerParam
     const unsigned short* uv = reinterpret_cast<const unsigned short*>(lp.Uinv_v);
     const int wide = (n_seq * v.rep + MW_ROWS - 1) / MW_ROWS;
     cudaError_t e;
-    if (MG_CL * wide * v.Hkv >= 2 * sm_count) {
-      // 32 rows per cluster while that still makes two CTAs per SM
+    if (4 * MG_CL * wide * v.Hkv >= sm_count * (v.Hkv < 4 ? v.Hkv : 4)) {
+      // 32 rows per cluster while that still makes a CTA per SM; with few KV heads a CTA's slice of U_V^-1 is small and it is the number
+      // of clusters that costs.  The merge in us, eight / 32 rows: 32 heads on 8 KV heads, 16 sequences 23.0 / 27.1, 32 sequences
+      // 35.7 / 24.7; 64 on 8, 8 sequences 23.0 / 25.3, 16 sequences 37.2 / 25.1; 16 on 4, 24 sequences a step of 44.4 / 47.9,
+      // 64 sequences 29.2 / 17.9; 8 on 1, 64 sequences 16.5 / 12.7; 4 on 1, 64 sequences 14.8 / 12.3.
       e = cudaFuncSetAttribute(merge_wide_kernel<BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, MW_SMEM);
       if (e == cudaSuccess) e = launch_chained(merge_wide_kernel<BF16>, dim3(MG_CL * wide, v.Hkv), dim3(MG_THREADS), dim3(MG_CL), MW_SMEM, st, v, uv, n_splits, n_seq, out);
     } else {

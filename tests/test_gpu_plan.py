@@ -39,3 +39,14 @@ def test_decode_where_the_work_split_changes(hkv, rep, n_seq, ctx, recipe, pick)
     max_abs, rel_l2 = attn_errors(out.cpu().numpy(), oracle_decode(li, ranks, pick))
     gc.close()
     assert max_abs < 2e-3 and rel_l2 < 1e-3, (max_abs, rel_l2)      # the bars of every decode test
+
+
+@pytest.mark.parametrize("hkv,rep,n_seq,ctx", [
+    (8, 8, 13, 40),             # 64 query heads: the last cluster of the wide merge holds two sequences of four
+    (1, 8, 33, 40),             # one KV head: wide from a few clusters on, one sequence in the last
+    (1, 4, 35, 30),
+    (4, 4, 47, 20),
+    (8, 4, 23, 30),             # just below: eight rows per cluster
+])
+def test_merge_of_medium_batches(hkv, rep, n_seq, ctx):
+    test_decode_where_the_work_split_changes(hkv, rep, n_seq, ctx, "any", list(range(n_seq)))
