@@ -101,8 +101,8 @@ struct Layout {
 };
 
 constexpr int GATE_PIECE = 8192;       // tokens per COMPUTE-mode gate piece (logits scratch rows)
-// COMPUTE-mode calls of this many tokens form the logits with gate_logits_tc_kernel; smaller ones, bound by launches and the
-// weights' way in, with the warp-MMA kernel; larger ones run the fused tcgen05 gate kernel, whose logits stay on the SM.
+// Gate logits of this many tokens are formed by gate_logits_tc_kernel; of fewer, bound by launches and the weights' way in, by the
+// warp-MMA kernel.  COMPUTE-mode calls of more than the maximum run the fused tcgen05 gate kernel, whose logits stay on the SM.
 // A whole compress call in us, warp-MMA / spread / fused (d_kv 1024): 128 tokens 39.2 / 32.8 / -, 1000 67.7 / 46.2 / -,
 // 2048 81.3 / 54.3 / 61.8, 3072 104 / 60.6 / 63.1, 4096 131 / 72.0 / 66.3; d_kv 512: 100 tokens 28.7 / 28.7 / -, 1000 47.7 / 38.2 / -,
 // 3072 61.6 / 46.0 / 52.3, 6000 80.3 / 57.7 / 51.4; d_kv 384: 3072 tokens - / 44.1 / 47.4, 4096 - / 51.4 / 47.4.
@@ -468,6 +468,24 @@ twkv_status twkv_cache_set_layer_params(twkv_cache* c, int layer, const twkv_lay
   return TWKV_OK;
 }
 
+// Gate logits of up to GATE_PIECE tokens into the gate scratch: tcgen05 kernel over all SMs, or (few tokens) the warp-MMA kernel.  Both
+// read the weights as they lie.
+static twkv_status gate_logits(twkv_cache* c, int layer, const void* K, const void* V, int n_tok, cudaStream_t st) {
+  const DevView& v = c->view;
+  const LayerParams& lp = c->params[layer];
+  if (n_tok < GATE_LOGITS_TC_MIN) return launch_gate_logits(v, lp, K, V, n_tok, v.gate_scratch, st) == cudaSuccess ? TWKV_OK : TWKV_ERR_CUDA;
+  const uint64_t d = (uint64_t)v.d_kv;
+  CUtensorMap* mw = &c->map_w[2 * (size_t)layer];
+  if (!c->mapped_w[layer]) {
+    if (!make_tmap_2d(mw, lp.W_k, d, d, d * 2, PANEL) || !make_tmap_2d(mw + 1, lp.W_v, d, d, d * 2, PANEL)) return TWKV_ERR_CUDA;
+    c->mapped_w[layer] = 1;
+  }
+  GateMaps maps;
+  maps.wk = mw[0]; maps.wv = mw[1];
+  if (!make_tmap_2d(&maps.xk, K, (uint64_t)n_tok, d, d * 2, TILE) || !make_tmap_2d(&maps.xv, V, (uint64_t)n_tok, d, d * 2, TILE)) return TWKV_ERR_CUDA;
+  return launch_gate_logits_tc(v, maps, lp, n_tok, c->sm_count, st) == cudaSuccess ? TWKV_OK : TWKV_ERR_CUDA;
+}
+
 twkv_status twkv_compress(twkv_cache* c, int layer, const void* K, const void* V, const int32_t* seq_ids,
                           const int32_t* positions, int n_tok, const float* scores, uint16_t* levels,
                           twkv_gate_mode mode, void* stream) {
@@ -488,20 +506,6 @@ twkv_status twkv_compress(twkv_cache* c, int layer, const void* K, const void* V
   c->appended[layer].fetch_add(n_tok, std::memory_order_relaxed);
   if (mode == TWKV_GATE_LOGITS) {
     if (launch_gate_rank(v, scores, levels, n_tok, st) != cudaSuccess) return TWKV_ERR_CUDA;
-  } else if (mode == TWKV_GATE_COMPUTE && n_tok >= GATE_LOGITS_TC_MIN && n_tok <= GATE_LOGITS_TC_MAX) {
-    // tcgen05 logits spread over all SMs, then the rank kernel; the weights are read as they lie
-    const uint64_t d = (uint64_t)c->dims.d_kv;
-    const LayerParams& lp = c->params[layer];
-    CUtensorMap* mw = &c->map_w[2 * (size_t)layer];
-    if (!c->mapped_w[layer]) {
-      if (!make_tmap_2d(mw, lp.W_k, d, d, d * 2, PANEL) || !make_tmap_2d(mw + 1, lp.W_v, d, d, d * 2, PANEL)) return TWKV_ERR_CUDA;
-      c->mapped_w[layer] = 1;
-    }
-    GateMaps maps;
-    maps.wk = mw[0]; maps.wv = mw[1];
-    if (!make_tmap_2d(&maps.xk, K, (uint64_t)n_tok, d, d * 2, TILE) || !make_tmap_2d(&maps.xv, V, (uint64_t)n_tok, d, d * 2, TILE)) return TWKV_ERR_CUDA;
-    if (launch_gate_logits_tc(v, maps, lp, n_tok, c->sm_count, st) != cudaSuccess) return TWKV_ERR_CUDA;
-    if (launch_gate_rank(v, v.gate_scratch, levels, n_tok, st) != cudaSuccess) return TWKV_ERR_CUDA;
   } else if (mode == TWKV_GATE_COMPUTE && n_tok > GATE_LOGITS_TC_MAX && c->sm_count <= 160) {
     // fused tcgen05 kernel: logits and ranks in one launch, the logits never leave the CTA's staging block
     const int d = c->dims.d_kv;
@@ -529,8 +533,8 @@ twkv_status twkv_compress(twkv_cache* c, int layer, const void* K, const void* V
   } else if (mode == TWKV_GATE_COMPUTE) {
     for (int lo = 0; lo < n_tok; lo += GATE_PIECE) {
       const int n = n_tok - lo < GATE_PIECE ? n_tok - lo : GATE_PIECE;
-      if (launch_gate_logits(v, c->params[layer], (const unsigned char*)K + lo * row, (const unsigned char*)V + lo * row, n,
-                             v.gate_scratch, st) != cudaSuccess) return TWKV_ERR_CUDA;
+      const twkv_status s = gate_logits(c, layer, (const unsigned char*)K + lo * row, (const unsigned char*)V + lo * row, n, st);
+      if (s != TWKV_OK) return s;
       if (launch_gate_rank(v, v.gate_scratch, levels + 2 * (size_t)lo, n, st) != cudaSuccess) return TWKV_ERR_CUDA;
     }
   }
@@ -880,7 +884,8 @@ twkv_status twkv_gate_soft(twkv_cache* c, int layer, const void* K, const void* 
     const int n = n_tok - lo < GATE_PIECE ? n_tok - lo : GATE_PIECE;
     const unsigned char* kp = (const unsigned char*)K + lo * row;
     const unsigned char* vp = (const unsigned char*)V + lo * row;
-    if (launch_gate_logits(v, c->params[layer], kp, vp, n, v.gate_scratch, st) != cudaSuccess) return TWKV_ERR_CUDA;
+    const twkv_status s = gate_logits(c, layer, kp, vp, n, st);
+    if (s != TWKV_OK) return s;
     if (launch_gate_soft(v, v.gate_scratch, kp, vp, m_k ? m_k + lo * d : nullptr, m_v ? m_v + lo * d : nullptr,
                          xh_k ? xh_k + lo * d : nullptr, xh_v ? xh_v + lo * d : nullptr, retain ? retain + 2 * (size_t)lo : nullptr, n,
                          st) != cudaSuccess) return TWKV_ERR_CUDA;

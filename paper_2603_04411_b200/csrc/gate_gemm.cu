@@ -7,9 +7,9 @@
 
 namespace twkv {
 
-// Small calls leave most SMs idle with one CTA per output tile (16 CTAs up to 128 tokens), each walking all of d_kv with a
-// memory round trip per step; then a cluster of `ks` CTAs shares a tile, a part of d_kv each, and adds the partial tiles through
-// distributed shared memory in fixed order (4 tokens: 20.3 -> 12.3 us with cold weights).
+// For calls of fewer than 128 tokens (the append of a decode step): one CTA per output tile would leave most SMs idle (16 CTAs), each
+// walking all of d_kv with a memory round trip per step, so a cluster of `ks` CTAs shares a tile, a part of d_kv each, and adds the
+// partial tiles through distributed shared memory in fixed order (4 tokens: 20.3 -> 12.3 us with cold weights).
 constexpr int GG_STAGES = 3;
 constexpr int GG_THREADS = 256;
 
@@ -126,9 +126,8 @@ cudaError_t launch_gate_logits(const DevView& v, const LayerParams& lp, const vo
                                float* logits, cudaStream_t st) {
   if (n_tok <= 0) return cudaSuccess;
   const size_t smem = 2 * GG_STAGES * 16384;
-  const int tiles = (n_tok + 127) / 128 * (v.d_kv / 128) * 2;
-  int ks = 8;                                                     // CTAs per tile: while that stays within two CTAs per SM of a 148-SM part
-  while (ks > 1 && ((v.d_kv / 64) % ks || tiles * ks > 296)) ks /= 2;
+  int ks = 8;                                                     // CTAs per tile; d_kv / 64 may be an odd number
+  while ((v.d_kv / 64) % ks) ks /= 2;
   ProfScope ps(TWKV_K_GATE_GEMM, st);
   auto X = [](const void* p) { return reinterpret_cast<const unsigned short*>(p); };
   auto kernel = v.dtype == TWKV_BF16 ? gate_gemm_kernel<true> : gate_gemm_kernel<false>;

@@ -1,5 +1,5 @@
-// Gate logits of Eq. 5 for calls of middle size: Z = X~ W + b on the 5th-generation tensor cores, fp32 logits to the gate
-// scratch, from where the rank kernel of the small calls takes them.
+// Gate logits of Eq. 5 for calls of middle size, and for the soft gate from 128 tokens on: Z = X~ W + b on the 5th-generation tensor
+// cores, fp32 logits to the gate scratch, from where the rank kernel of the small calls or the soft gate's kernel takes them.
 //
 // The fused gate kernel keeps a token's whole row of logits on one CTA pair and leaves most SMs idle in a call of a few token
 // tiles; the warp-MMA kernel of the small calls is bound by its own issue from a few hundred tokens on.  With an output tile of
