@@ -603,7 +603,7 @@ twkv_status twkv_decode_attn(twkv_cache* c, int layer, const void* q, const int3
 struct PfPlan {
   int lo, hi, n_u, n_blocks;
   long long n_words;
-  int seg_rows, n_segs, n_splits, group;
+  int seg_rows, n_segs, seg_rest, n_splits, group;       // seg_rest: segments without those that only repeated positions could reach
   double us;                            // estimated time
 };
 
@@ -613,7 +613,7 @@ static PfPlan plan_tiled(const twkv_cache* c, const int32_t* q_seq, const int32_
                          const long long* seq_rows, long long rows_max, long long rows_all) {
   const DevView& v = c->view;
   const int QT = TILE / v.rep;
-  PfPlan pl = {lo, hi, 0, 0, 0, 0, 0, 1, 1, 1e300};
+  PfPlan pl = {lo, hi, 0, 0, 0, 0, 0, 0, 1, 1, 1e300};
   std::vector<int> first;               // first block of every sequence
   bool two_tiles = false;
   for (int i = lo; i < hi;) {
@@ -657,7 +657,7 @@ static PfPlan plan_tiled(const twkv_cache* c, const int32_t* q_seq, const int32_
       const double cost = groups * segs * (kb * item + 1.5 * rounds + heads * (4.0 + std::min<long long>(rows_max, seg_rows) / 1024.0));
       const int n_segs = std::max(1, (int)((rows_all + seg_rows - 1) / seg_rows));
       const double us = 20.0 + 4.5 * cost + (n_segs > 1 || ns > 1 ? 4.0 * groups : 0.0) + 3.4 * groups * (n_segs - segs);
-      if (us < pl.us) { pl.us = us; pl.seg_rows = seg_rows; pl.n_segs = n_segs; pl.n_splits = ns; pl.group = group; }
+      if (us < pl.us) { pl.us = us; pl.seg_rows = seg_rows; pl.n_segs = n_segs; pl.seg_rest = (int)segs; pl.n_splits = ns; pl.group = group; }
     }
   }
   return pl;
@@ -691,15 +691,16 @@ static twkv_status run_tiled(twkv_cache* c, int layer, const void* q, const int3
   int* p = (int*)(v.gate_fix + n_blocks);
   a.qvis = p; p += n_q;
   a.rows = p; a.base = p + a.n_u; a.dup = p + 2 * (size_t)a.n_u; p += 3 * (size_t)a.n_u;
-  a.ticket = p; a.total = p + 1; p += 4;
+  a.ticket = p; a.total = p + 1; a.vscale = (float*)(p + 2); p += 4;
   a.slot = p; p += v.S;
   a.bits = (unsigned*)p; a.pref = p + pl.n_words;
   a.krow = v.kv_link; a.krow_out = v.evict_map; a.vrow = v.evict_map + (size_t)v.NT * TILE;
   a.rowpos = (int*)v.scores;
+  a.uv = (const unsigned short*)c->params[layer].Uinv_v;
   a.seg_buf = (unsigned char*)v.gate_scratch;
   a.vexp = (signed char*)v.hist;                                    // 8448 bytes per KV head of at least 16384
   a.vflag = (int*)(a.vexp + (size_t)GATE_PIECE * v.Hkv);
-  a.seg_rows = pl.seg_rows; a.n_splits = pl.n_splits;
+  a.seg_rows = pl.seg_rows; a.n_splits = pl.n_splits; a.seg_rest = pl.seg_rest;
   a.slots = pl.seg_rows == GATE_PIECE ? v.part_acc : (float*)(a.seg_buf + (size_t)GATE_PIECE * v.d_kv * sizeof(float));
 
   PfMaps maps;

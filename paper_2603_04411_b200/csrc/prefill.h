@@ -5,6 +5,7 @@
 
 namespace twkv {
 
+constexpr int PF_SCALE_MIN = -60;                // of the exponent of the call's values
 constexpr int PF_SLOT_FLOATS = 2 * 130 * TILE;    // partial result of (block of queries, KV head, split): [2 tiles][128 output columns, maximum, sum][128 rows]
 
 struct PfCall {
@@ -16,6 +17,7 @@ struct PfCall {
   int n_u, n_blocks, n_words;
   int blk0, blk_n;      // the group of blocks handled now
   int n_splits, seg_rows;
+  int seg_rest;         // segments that the positions alone can need; further ones are for repeated positions
   // made on the device
   int* slot;            // [max_seqs] sequence id -> sequence slot of the call, -1
   unsigned* bits;       // [n_words] bitmaps of the visible positions
@@ -28,7 +30,9 @@ struct PfCall {
   int *krow_out, *vrow; // [NT * 128] dense row of every K / V slot, -1 = not visible
   int* rowpos;          // [rows] position of a dense row
   unsigned char* seg_buf;   // [Hkv][4 parts][seg_rows][128] 16-bit
-  // the power of two a row's value was divided by before it was split, per KV head; segment + 1 of the last segment
+  const unsigned short* uv; // U_V^-1 of the layer
+  float* vscale;        // [2] the power of two the call's values are multiplied by before they are split, and its inverse
+  // the power of two a row's value was divided by besides, per KV head; segment + 1 of the last segment
   // in which a block of 128 rows held one other than 0
   signed char* vexp;    // [Hkv][seg_rows]
   int* vflag;           // [seg_rows / 128][Hkv]

@@ -14,9 +14,10 @@
 // Precision: as in decode attention, keys are carried as two f16 (22 bits) and queries as f16; softmax weights and values are two
 // f16 as well, whatever the cache type, so that the result is the spectral-space one to rounding.  The products high.low,
 // low.high and high.high of weights and values are formed.
-// A rebuilt value may lie outside f16 although the stored 16-bit components do not.  A row (token, KV head) whose largest value is
-// beyond 65504, or so small that the low parts would lose bits, is divided by a power of two before the split, and its softmax
-// weights carry that power; blocks of keys without such a row (nearly all, for values around 1) run as if there were none.
+// Rebuilt values may lie outside f16 although the stored 16-bit components do not, or be so small that the low parts lose bits.  A
+// few sampled tokens tell the size of the call's values; one power of two brings it near 1 and goes back onto the outputs.  A row
+// (token, KV head) whose largest value still lies outside is divided by a power of its own, which its softmax weights carry; blocks of
+// keys without such a row (nearly all) run as if there were none.
 //
 // Cost per 128 x 128 tile of (query row, token): 2 + 3 tensor-core units of 2 x 128^3 flop; the softmax of one tile runs
 // beside the products of the other.
@@ -24,6 +25,7 @@
 
 #include "twkv_dev.h"
 #include "tc_util.cuh"
+#include "mma_util.cuh"
 #include "scan_util.cuh"
 #include "prefill.h"
 
@@ -116,8 +118,8 @@ __global__ void __launch_bounds__(1024) pf_scan_kernel(DevView v, PfCall a, int 
   if (tid == 0) *a.total = run;
 }
 
-// Segments past the last row have been launched as well (their set-up ran beside the kernel before).
-__device__ __forceinline__ bool pf_idle(const PfCall& a, int seg) { return seg > 0 && (long long)seg * a.seg_rows >= *a.total; }
+// Segments that only repeated positions could reach have been launched as well (their set-up ran beside the kernel before).
+__device__ __forceinline__ bool pf_idle(const PfCall& a, int seg) { return seg >= a.seg_rest && (long long)seg * a.seg_rows >= *a.total; }
 // Whether the attention kernel's result for a query is whole: one split of the only segment with rows.
 __device__ __forceinline__ bool pf_whole(const PfCall& a) { return a.n_splits == 1 && *a.total <= a.seg_rows; }
 
@@ -126,12 +128,56 @@ __device__ __forceinline__ int pf_rank(const PfCall& a, int off, int pos) {     
   return a.pref[w] + __popc(a.bits[w] & ((1u << (pos & 31)) - 1u));
 }
 
+// Size of the call's values: the largest of eight tokens' values, rebuilt from the first 16 components, in one KV head each (a fraction of
+// the real ones).  Values near 1 stay as they are; others are brought there by a power of two.  One chain of dependent reads, about as
+// long as the other CTAs'.
+constexpr int PF_SAMPLE = 16;
+template <bool BF16>
+__device__ __forceinline__ float pf_sample_value(const uint4* x, const unsigned short* u, int d_kv) {
+  unsigned short uj[PF_SAMPLE];
+#pragma unroll
+  for (int j = 0; j < PF_SAMPLE; ++j) uj[j] = u[(size_t)j * d_kv];
+  const uint4 x0 = x[0], x1 = x[1];
+  const unsigned w[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+  float sum = 0.f;
+#pragma unroll
+  for (int j = 0; j < PF_SAMPLE; ++j) sum += to_f32<BF16>((unsigned short)(w[j >> 1] >> (16 * (j & 1)))) * to_f32<BF16>(uj[j]);
+  return fabsf(sum);
+}
+__device__ void pf_value_scale(const DevView& v, const PfCall& a, int layer) {
+  __shared__ float s_max[32];
+  const int tid = threadIdx.x, k = tid >> 7;
+  const int seq = a.seqs[3 * (k * a.n_u / 8)], n = v.svc(layer)[seq];
+  float top = 0.f;
+  if (n > 0) {
+    const int4 d = v.desc(layer, 1)[v.svt(layer)[(size_t)seq * v.TPS + (2 * k + 1) * n / 16]];
+    const uint4* x = reinterpret_cast<const uint4*>(v.blocks + (size_t)d.w * BLOCK_BYTES + (d.z >> 1) * (PANEL * 2));
+    const unsigned short* u = a.uv + (k % v.Hkv) * HEAD_DIM + (tid & (HEAD_DIM - 1));
+    top = v.dtype == TWKV_BF16 ? pf_sample_value<true>(x, u, v.d_kv) : pf_sample_value<false>(x, u, v.d_kv);
+  }
+  for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+  if ((tid & 31) == 0) s_max[tid >> 5] = top;
+  __syncthreads();
+  if (tid >= 32) return;
+  top = s_max[tid];
+  for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+  if (tid > 0) return;
+  int e = 0;
+  if ((top > 1024.f && top < INFINITY) || (top < 0.0625f && top > 0.f)) e = max((int)(__float_as_uint(top) >> 23) - 127, PF_SCALE_MIN);
+  a.vscale[0] = __uint_as_float((unsigned)(127 - min(e, 126)) << 23);
+  a.vscale[1] = __uint_as_float((unsigned)(127 + min(e, 126)) << 23);
+}
+
 // Dense row of every K and V slot, position of every row, the segments a tile touches; per query and per block of queries
-// what it may see.  The last `qctas` CTAs take the queries.
+// what it may see.  The last CTA looks at the size of the values, the `qctas` before it take the queries.
 __global__ void __launch_bounds__(1024) pf_rows_kernel(DevView v, PfCall a, int layer, int qctas) {
   chain_start();
   chain_wait();
-  const int tctas = (int)gridDim.x - qctas;
+  const int tctas = (int)gridDim.x - 1 - qctas;
+  if ((int)blockIdx.x == tctas + qctas) {
+    pf_value_scale(v, a, layer);
+    return;
+  }
   if ((int)blockIdx.x >= tctas) {
     for (int b = ((int)blockIdx.x - tctas) * 32 + (threadIdx.x >> 5); b < a.n_blocks; b += qctas * 32) {       // a warp per block
       const int2 q = a.blocks[b];
@@ -199,11 +245,11 @@ constexpr int PR_ROPE_STRIDE = 33;                              // float4 per ro
 constexpr uint32_t PR_ROPE_BYTES = ROPE_LO * PR_ROPE_STRIDE * 16;
 constexpr uint32_t PR_SMEM = PR_STAGES * PR_STAGE_BYTES + 8 * PR_OUT_BYTES + PR_ROPE_BYTES + 8 * (2 * PR_STAGES + 4) + 16;
 static_assert(PR_SMEM > CHAIN_TMEM_SMEM, "no other CTA with tensor memory beside this one");
-// A row whose largest value lies outside these is scaled: a small one to [2^-3, 2^-2), a large one to [2^14, 2^15).  A part is exact
-// to 2^-25: values at the lower line keep 20 bits, scaled ones 22; scaled further up, their weights (which shrink by as much) would
-// lose bits beside those of rows that are not scaled.
-constexpr float PR_V_MIN = 0x1p-5f, PR_V_MAX = 65504.f;
-constexpr int PR_EXP_MIN = -90, PR_EXP_MAX = 113;               // 2^-e times a sum of weights stays an fp32 number
+// A row whose largest value (beside the call's scale) lies outside these is scaled by itself: a small one to [2^-3, 2^-2), a large one to
+// [2^14, 2^15).  A part is exact to 2^-25, 2^-22 of values of the usual size.  Scaled further up, a small row's weights (which shrink
+// by as much) would lose bits beside those of rows that are not scaled.
+constexpr float PR_V_MIN = 0x1p-8f, PR_V_MAX = 65504.f;
+constexpr int PR_EXP_MIN = -60, PR_EXP_MAX = 113;               // 2^-e times a sum of weights stays an fp32 number
 // Panels summed into one accumulator; the sums of several accumulators are added in fp32 registers.  The tensor core cuts its
 // fp32 sum after every instruction (K = 16), so the error grows with the length of a chain.  K: eight panels, the length of
 // decode attention's passes, so that both round alike.  V: two panels; decode attention sums values over tokens, not over
@@ -254,7 +300,7 @@ pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_con
   if (warp == 1) tmem_alloc(smem_addr(s_tmem_base), 512);
   chain_wait();
   const bool idle = pf_idle(a, seg);
-  for (int i = tid; i < ROPE_LO * 32 && !idle; i += PR_THREADS) sRope[(i >> 5) * PR_ROPE_STRIDE + (i & 31)] = v.rope_lo[i];
+  for (int i = tid; i < ROPE_LO * 32; i += PR_THREADS) sRope[(i >> 5) * PR_ROPE_STRIDE + (i & 31)] = v.rope_lo[i];
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
@@ -378,6 +424,7 @@ pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_con
     }
     uint32_t ac = 0;
     bool ok = true;
+    const float vscale = a.vscale[0];
     for (int i0 = blockIdx.x; i0 < n_items && ok; i0 += 32 * step) {
       for (unsigned m = lookup(i0); m; m &= m - 1) {
         const int i = i0 + (__ffs(m) - 1) * step;
@@ -511,7 +558,7 @@ pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_con
           float mx[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
           for (int k = 0; k < 128; k += 2) mx[(k >> 1) & 3] = max_abs3(mx[(k >> 1) & 3], x[k >> 6][k & 63], x[k >> 6][(k & 63) + 1]);
-          const float top = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+          const float top = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * vscale;
           int e = 0;                                             // (an infinite row is left as it is)
           if ((top > PR_V_MAX && top < INFINITY) || (top < PR_V_MIN && top > 0.f))
             e = max((int)(__float_as_uint(top) >> 23) - 127 + (top < 1.f ? 3 : -14), PR_EXP_MIN);
@@ -521,8 +568,8 @@ pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_con
             a.vexp[(size_t)g * a.seg_rows + local] = (signed char)e;
             if (e != 0) a.vflag[(local / TILE) * v.Hkv + g] = seg + 1;
           }
-          if (__any_sync(0xffffffffu, e != 0)) {
-            const float f = __uint_as_float((uint32_t)(127 - e) << 23);
+          if (__any_sync(0xffffffffu, e != 0 || vscale != 1.f)) {
+            const float f = __uint_as_float((uint32_t)(127 - e) << 23) * vscale;
 #pragma unroll
             for (int k = 0; k < 128; ++k) x[k >> 6][k & 63] = __float_as_uint(__uint_as_float(x[k >> 6][k & 63]) * f);
           }
@@ -931,7 +978,7 @@ pf_attn_kernel(const __grid_constant__ CUtensorMap map_seg, DevView v, PfCall a,
       if (whole) {
         // This is the whole result.  A thread writes its row's 64 columns itself (4096-token prompt in four
         // calls 783 -> 751 us, five short prompts 204 -> 189 against partial results and the combine kernel).
-        const float inv = l == 0.f ? 0.f : 1.f / l;              // 0: no token seen; a NaN stays one
+        const float inv = l == 0.f ? 0.f : a.vscale[1] / l;      // 0: no token seen; a NaN stays one
         const bool mine = ql < it.cnt;
         const size_t o0 = mine ? ((size_t)a.qrow[it.first + ql] * v.Hq + it.g * rep + row % rep) * HEAD_DIM + hf * 64 : 0;
 #pragma unroll 1
@@ -1025,7 +1072,7 @@ __global__ void __launch_bounds__(256) pf_combine_kernel(DevView v, PfCall a, vo
     for (int c = 0; c < 16; ++c) acc[c] = acc[c] * wo + x[c] * wk;
     m = mn;
   }
-  const float inv = l == 0.f ? 0.f : 1.f / l;
+  const float inv = l == 0.f ? 0.f : a.vscale[1] / l;
 #pragma unroll
   for (int c = 0; c < 16; ++c) s[row][cc + c] = acc[c] * inv;
   __syncthreads();
@@ -1059,7 +1106,7 @@ cudaError_t launch_pf_tables(const DevView& v, const PfCall& a, int layer, int s
   cudaError_t e = launch_chained(pf_init_kernel, dim3(zc < 1 ? 1 : (zc > sm_count ? sm_count : zc)), b, one, 0, st, v, a);
   if (e == cudaSuccess) e = launch_chained(pf_bits_kernel, dim3(sm_count), b, one, 0, st, v, a, layer);
   if (e == cudaSuccess) e = launch_chained(pf_scan_kernel, dim3(a.n_u), b, one, 0, st, v, a, layer);
-  if (e == cudaSuccess) e = launch_chained(pf_rows_kernel, dim3(sm_count + qc), b, one, 0, st, v, a, layer, qc);
+  if (e == cudaSuccess) e = launch_chained(pf_rows_kernel, dim3(sm_count + qc + 1), b, one, 0, st, v, a, layer, qc);
   if (e != cudaSuccess) return e;
   count_launch(4);
   return cudaGetLastError();
