@@ -145,7 +145,9 @@ twkv_status twkv_cache_destroy(twkv_cache* cache);
 /* Forgets every cached token of every layer (tables cleared, blocks reusable); layer
  * parameters and a pending sticky status are kept / cleared respectively. */
 twkv_status twkv_cache_reset(twkv_cache* cache, void* stream);
-/* Borrows the layer's matrices (Eq. 3: U^-1; Eq. 5: W, b).  `params` itself is host memory. */
+/* Borrows the layer's matrices (Eq. 3: U^-1; Eq. 5: W, b).  `params` itself is host memory.  Decode keeps a re-tiled copy of
+ * U_K^-1, and COMPUTE-mode calls of more than 3072 tokens one of W, made by the first call that needs it (inside a graph: by every
+ * replay of it); after a change of the matrices in place, set the parameters again. */
 twkv_status twkv_cache_set_layer_params(twkv_cache* cache, int layer, const twkv_layer_params* params /*host*/);
 
 /*
@@ -167,7 +169,7 @@ twkv_status twkv_compress(twkv_cache* cache, int layer, const void* K, const voi
  *   q        [n_seq x n_q_heads x 128] dtype, already rotated at its own position
  *   seq_ids  [n_seq] int32, distinct
  *   out      [n_seq x n_q_heads x 128] out_dtype; a sequence with no cached token gets zeros
- *   num_splits  V-side splits per sequence; 0 = choose automatically
+ *   num_splits  V-side splits per sequence; 0 = choose automatically (by the batch and the tokens cached when the call runs)
  */
 twkv_status twkv_decode_attn(twkv_cache* cache, int layer, const void* q, const int32_t* seq_ids,
                              int n_seq, void* out, int num_splits, void* stream);
@@ -183,8 +185,9 @@ twkv_status twkv_decode_attn(twkv_cache* cache, int layer, const void* q, const 
  *   q_seq    [n_q] int32, HOST memory: sequence id of every query (any order, repeats allowed)
  *   q_pos    [n_q] int32, HOST memory: RoPE position of every query (>= 0)
  *   n_q      at most TWKV_PREFILL_MAX_QUERIES
- * Keys and values of the visible tokens are rebuilt once per call and shared by its queries; calls of few queries per
- * sequence run as passes of the decode kernels instead, one query per sequence at a time (num_splits applies to those).
+ * Keys and values of the visible tokens are rebuilt once and shared by the call's queries (more queries than the scratch holds
+ * partial results for: once per group of queries); calls of few queries per sequence over long contexts run as passes of the
+ * decode kernels instead, one query per sequence at a time (num_splits applies to those).
  * The host arrays are read before the call returns; a call captured into a graph replays with what they held then.
  * Errors as for twkv_decode_attn; an id or position out of range returns TWKV_ERR_INVALID_ARG before anything is launched.
  */

@@ -171,8 +171,8 @@ __global__ void __launch_bounds__(1024) plan_kernel(DevView v, int layer, const 
     // The KV heads of an item may be dealt out to several CTAs (pairs): finer work for lists that leave some idle or that a few
     // wide tiles decide.  A part repeats the tile's loads and rotation factors.  Least estimate of the slowest piece, in cycles:
     // the widest part where every part has a CTA to itself, else the mean piece plus most of the widest part (numbers fitted to
-    // the lists below).  Whole items against this rule: 1 x 8192 62 -> 54 us, 4 x 1000 66 -> 57, 16 x 500 102
-    // -> 92, 8 x 8192 121 -> 114; 64 x 2000 and 16 x 32768 keep whole items.
+    // lists of this kind).  A decode call in us, whole items / this rule (ranks 1 .. 512): 1 x 8192 50.6 / 49.4, 4 x 1000 51.1 / 48.8,
+    // 8 x 8192 102.6 / 102.4, 16 x 500 62.6 / 63.2; 64 x 2000 and 16 x 32768 keep whole items.
     constexpr float PART_COST = 2600.f;
     int widest = 0;
     while (widest < NC && s_ioff[widest + 1] == s_ioff[widest]) ++widest;

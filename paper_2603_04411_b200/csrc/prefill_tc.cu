@@ -604,8 +604,8 @@ pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_con
 // and are the A operand of the second product from there.  Order of the products per key block j: O0 += P0 V(j), S0 = Q0
 // K(j+1)^T, O1 += P1 V(j), S1 = Q1 K(j+1)^T, so that one tile's softmax runs beside the other's products; products of one
 // thread retire in order, so S0 may overwrite P0 without a wait.
-// The running maximum a row is scaled by moves only when it would grow by more than 2^8 (f16 holds 2^15): the accumulator in
-// TMEM is rescaled rarely, and by the softmax warps themselves.
+// The running maximum a row is scaled by moves only when it would grow by more than 2^8 (f16 holds 2^15), as FlashAttention-4
+// describes it: the accumulator in TMEM is rescaled rarely, and by the softmax warps themselves.
 // What bounds it: a tile's softmax plus its own products must fit beside the other tile's products (2 x 2560 tensor cycles per
 // key block); eight warps per tile, thread = half a row.
 // Warp roles (640 threads): 0 TMA producer, 1 MMA issuer, 4-11 softmax of tile 0, 12-19 softmax of tile 1.

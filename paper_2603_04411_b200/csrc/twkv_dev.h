@@ -193,7 +193,6 @@ struct ProfScope {
 
 // kernels' host launchers (defined in the .cu files)
 cudaError_t launch_rope_tables(const DevView& v, float rope_base, cudaStream_t st);
-cudaError_t launch_clear_tables(const DevView& v, cudaStream_t st);
 cudaError_t launch_gate_rank(const DevView& v, const float* logits, unsigned short* levels, int n_tok, cudaStream_t st);
 cudaError_t launch_compress_pieces(const DevView& v, int layer, const void* K, const void* V, const int* seq_ids,
                                   const int* positions, int n_tok, const unsigned short* levels, cudaStream_t st);
