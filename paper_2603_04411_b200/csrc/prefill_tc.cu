@@ -118,8 +118,11 @@ __global__ void __launch_bounds__(1024) pf_scan_kernel(DevView v, PfCall a, int 
   if (tid == 0) *a.total = run;
 }
 
-// Segments that only repeated positions could reach have been launched as well (their set-up ran beside the kernel before).
-__device__ __forceinline__ bool pf_idle(const PfCall& a, int seg) { return seg >= a.seg_rest && (long long)seg * a.seg_rows >= *a.total; }
+// Segments that only repeated positions could reach have been launched as well (their set-up ran beside the kernel before).  Where the
+// first segment may be the whole result, a later one without rows must leave too: it would write its nothing over the outputs.
+__device__ __forceinline__ bool pf_idle(const PfCall& a, int seg) {
+  return seg > 0 && (seg >= a.seg_rest || a.n_splits == 1) && (long long)seg * a.seg_rows >= *a.total;
+}
 // Whether the attention kernel's result for a query is whole: one split of the only segment with rows.
 __device__ __forceinline__ bool pf_whole(const PfCall& a) { return a.n_splits == 1 && *a.total <= a.seg_rows; }
 

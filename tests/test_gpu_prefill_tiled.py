@@ -348,3 +348,22 @@ def test_prefill_of_few_queries_over_many_long_sequences_runs_in_passes(B):
     pick = np.arange(0, n_seq * n_q, 13)
     max_abs, rel_l2 = attn_errors(got[pick], _oracle_prefill(li, ranks, q[pick], q_seq[pick], q_pos[pick]))
     assert max_abs < MAX_ABS and rel_l2 < REL_L2, (max_abs, rel_l2)
+
+
+def test_tiled_prefill_where_fewer_rows_exist_than_positions_allow(B):
+    # 40 sequences are asked for, 15 hold tokens: planned for two segments by the positions, all rows lie in the first
+    n_seq, held, ctx, n_q = 40, 15, 100, 5
+    li = workloads.build_layer(869, n_seq=n_seq, ctx=ctx, n_q_heads=4, n_kv_heads=2, n_calib=512, dtype=torch.bfloat16, mode="forced", rank_recipe="any")
+    stay = li.seq_ids < held
+    for name in ["xt_k", "xt_v", "seq_ids", "positions", "ranks"]:
+        setattr(li, name, getattr(li, name)[stay].contiguous())
+    ranks = li.ranks.numpy().astype(np.int64)
+    q_seq, q_pos = np.repeat(np.arange(n_seq), n_q), np.tile(np.arange(ctx - n_q, ctx), n_seq)
+    q = torch.randn(n_seq * n_q, 4, 128, generator=torch.Generator().manual_seed(9)).to(torch.bfloat16)
+    gc = _filled(B, li, ranks, max_seqs=n_seq)
+    got = _prefill(B, gc, q, q_seq, q_pos)
+    gc.close()
+    some = q_seq < held
+    max_abs, rel_l2 = attn_errors(got[some], _oracle_prefill(li, ranks, q[some], q_seq[some], q_pos[some]))
+    assert max_abs < MAX_ABS and rel_l2 < REL_L2, (max_abs, rel_l2)
+    assert not got[~some].any()
