@@ -277,6 +277,11 @@ __device__ __forceinline__ void unpk2(uint64_t v, float& a, float& b) { asm("mov
 // half of a head's dims) rotate (K), split into two parts and hand the rows out through shared memory: a row's place in the
 // segment buffer is its token's dense row, so a warp stores four whole 128-byte pieces per instruction instead of 32
 // scattered 16-byte ones.
+// What bounds it: the epilogue's latencies, with two warps per scheduler, and the way of 128 KiB per item into L2 (about 5 TB/s over
+// all SMs: the same item takes 3.8 us with 128 live rows and 2.1 with twenty).  So the tables of the next item are read an item ahead,
+// a slab is read from tensor memory while the piece before it is rotated, and a part's rows are all read back before the first is
+// stored: a K item 7.3 -> 5 us, 512 queries behind 32768 tokens 880 -> 864 us, five ragged prompts 182 -> 178.  Storing 32 bytes per
+// thread straight from registers instead is as fast for tiles with few rows and 1.6 times slower for full ones.
 template <bool BF16>
 __global__ void __launch_bounds__(PR_THREADS, 1)
 pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_constant__ CUtensorMap map_uk,
@@ -428,31 +433,47 @@ pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_con
     uint32_t ac = 0;
     bool ok = true;
     const float vscale = a.vscale[0];
+    // what an item's rows need from the tables; fetched an item ahead, so that the reads do not add up at its start
+    int side = 0, t = 0, cls = 0, place = -1, pos = 0;
+    auto fetch = [&](int i) {
+      cls = entry(i, side, t).x & 0xff;
+      place = (side ? a.vrow : a.krow_out)[(size_t)t * TILE + row];                      // rows past the tile's last token hold -1
+      pos = side ? 0 : kpos[(size_t)t * TILE + row];
+    };
     for (int i0 = blockIdx.x; i0 < n_items && ok; i0 += 32 * step) {
-      for (unsigned m = lookup(i0); m; m &= m - 1) {
+      unsigned m = lookup(i0);
+      if (m) fetch(i0 + (__ffs(m) - 1) * step);
+      for (; m; m &= m - 1) {
         const int i = i0 + (__ffs(m) - 1) * step;
-        int side, t;
-        const int cls = entry(i, side, t).x & 0xff, chains = (cls + pr_chain(side) - 1) / pr_chain(side);
+        const int now_side = side, now_t = t, chains = (cls + pr_chain(side) - 1) / pr_chain(side), now_pos = pos;
         const int g0 = (i % n_slabs) * heads;
-        int local = (side ? a.vrow : a.krow_out)[(size_t)t * TILE + row] - seg0;         // rows past the tile's last token hold -1
-        if (local < 0 || local >= a.seg_rows) local = -1;
+        int local = place - seg0;
+        if (place < 0 || local < 0 || local >= a.seg_rows) local = -1;
+        if (const unsigned rest = m & (m - 1)) fetch(i0 + (__ffs(rest) - 1) * step);
         auto stage_piece = [&](int piece, const uint32_t* hi, const uint32_t* lo) {      // 16 bytes of this thread's row, both parts
           unsigned char* d = stage + lane * 128 + ((piece ^ (lane & 7)) << 4);
           *reinterpret_cast<uint4*>(d) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
           *reinterpret_cast<uint4*>(d + 4096) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
         };
-        auto rows_out = [&](int g, int half) {                   // the warp's 32 half rows: four whole 128-byte pieces per instruction
+        // The warp's 32 half rows: four whole 128-byte pieces per instruction.  All of a part's reads go out before its first store:
+        // with two warps per scheduler one read after the other cost the epilogue more than its arithmetic.
+        auto rows_out = [&](int g, int half) {
           __syncwarp();
-          unsigned char* dst = a.seg_buf + (g * 4 + side * 2) * plane + half * 128 + (lane & 7) * 16;
+          unsigned char* dst = a.seg_buf + (g * 4 + now_side * 2) * plane + half * 128 + (lane & 7) * 16;
+          int lr[8];
 #pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            const int r = 4 * k + (lane >> 3);
-            const int lr = __shfl_sync(0xffffffffu, local, r);
-            const unsigned char* s = stage + r * 128 + (((lane & 7) ^ (r & 7)) << 4);
-            if (lr >= 0) {
-              *reinterpret_cast<uint4*>(dst + (size_t)lr * 256) = *reinterpret_cast<const uint4*>(s);
-              *reinterpret_cast<uint4*>(dst + plane + (size_t)lr * 256) = *reinterpret_cast<const uint4*>(s + 4096);
+          for (int k = 0; k < 8; ++k) lr[k] = __shfl_sync(0xffffffffu, local, 4 * k + (lane >> 3));
+#pragma unroll
+          for (int part = 0; part < 2; ++part) {
+            uint4 w[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+              const int r = 4 * k + (lane >> 3);
+              w[k] = *reinterpret_cast<const uint4*>(stage + part * 4096 + r * 128 + (((lane & 7) ^ (r & 7)) << 4));
             }
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+              if (lr[k] >= 0) *reinterpret_cast<uint4*>(dst + part * plane + (size_t)lr[k] * 256) = w[k];
           }
           __syncwarp();
         };
@@ -466,24 +487,22 @@ pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_con
           __syncwarp();
           if (lane == 0) mbar_arrive(acc_empty + 8 * (n & 1u));
         };
-        if (!side) {
+        if (!now_side) {
           // K: this thread's half of the RoPE frequencies; dims 32 hf + 8 c .. + 7 and the eight 64 above them at a time.
           // cos / sin of (position, frequency pair) by the angle-addition formulas from the two table rows.
-          const int pos = local >= 0 ? kpos[(size_t)t * TILE + row] : 0;
-          const float4* __restrict__ th = v.rope_hi + (size_t)((pos >> 4) & (ROPE_HI - 1)) * 32 + hf * 16;
-          const float4* tl = sRope + (pos & 15) * PR_ROPE_STRIDE + hf * 16;
+          const float4* __restrict__ th = v.rope_hi + (size_t)((now_pos >> 4) & (ROPE_HI - 1)) * 32 + hf * 16;
+          const float4* tl = sRope + (now_pos & 15) * PR_ROPE_STRIDE + hf * 16;
           uint64_t cs[16], sn[16];
+          {
+            float4 h4[16];
 #pragma unroll
-          for (int b = 0; b < 16; b += 8) {
-            float4 h4[8];
+            for (int k = 0; k < 16; ++k) h4[k] = __ldg(th + k);
 #pragma unroll
-            for (int k = 0; k < 8; ++k) h4[k] = __ldg(th + b + k);
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-              const float4 l4 = tl[b + k];
+            for (int k = 0; k < 16; ++k) {
+              const float4 l4 = tl[k];
               const uint64_t ch = pk2(h4[k].x, h4[k].y), sh = pk2(h4[k].z, h4[k].w), cl = pk2(l4.x, l4.y), sl = pk2(l4.z, l4.w);
-              cs[b + k] = sub2(mul2(ch, cl), mul2(sh, sl));
-              sn[b + k] = fma2(sh, cl, mul2(ch, sl));
+              cs[k] = sub2(mul2(ch, cl), mul2(sh, sl));
+              sn[k] = fma2(sh, cl, mul2(ch, sl));
             }
           }
           ok = wait_chain(ac);
@@ -491,27 +510,34 @@ pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_con
           if (!ok) break;
           for (int hh = 0; hh < heads; ++hh) {
             const uint32_t src = lane_addr + (ac & 1u) * 256 + hh * 128 + hf * 32, src2 = lane_addr + ((ac + 1) & 1u) * 256 + hh * 128 + hf * 32;
-            uint32_t x[64];                                      // 32 dims, then the 32 dims 64 above
-            tmem_ld32(src, x);
-            tmem_ld32(src + 64, x + 32);
-            tmem_ld_wait();
-            if (chains == 2) {
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                uint32_t y[16];
-                tmem_ld16(src2 + 64 * (e >> 1) + 16 * (e & 1), y);
-                tmem_ld_wait();
-#pragma unroll
-                for (int k = 0; k < 16; ++k) x[16 * e + k] = __float_as_uint(__uint_as_float(x[16 * e + k]) + __uint_as_float(y[k]));
-              }
-            }
-            if (hh == heads - 1) { free_chain(ac); if (chains == 2) free_chain(ac + 1); }
+            uint32_t va[16], vb[16];                             // eight dims and the eight 64 above them; the next ones on their way
+            tmem_ld8(src, va);
+            tmem_ld8(src + 64, va + 8);
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
+              uint32_t* x = (c & 1) ? vb : va;
+              uint32_t* nx = (c & 1) ? va : vb;
+              if (chains == 2) {
+                uint32_t y[16];
+                tmem_ld8(src2 + 8 * c, y);
+                tmem_ld8(src2 + 64 + 8 * c, y + 8);
+                tmem_ld_wait();
+#pragma unroll
+                for (int k = 0; k < 16; ++k) x[k] = __float_as_uint(__uint_as_float(x[k]) + __uint_as_float(y[k]));
+              } else {
+                tmem_ld_wait();
+              }
+              if (c < 3) {
+                tmem_ld8(src + 8 * (c + 1), nx);
+                tmem_ld8(src + 64 + 8 * (c + 1), nx + 8);
+              } else if (hh == heads - 1) {
+                free_chain(ac);
+                if (chains == 2) free_chain(ac + 1);
+              }
               uint32_t hi[8], lo[8];
 #pragma unroll
               for (int k = 0; k < 4; ++k) {
-                const uint64_t L = pk2u(x[8 * c + 2 * k], x[8 * c + 2 * k + 1]), H = pk2u(x[32 + 8 * c + 2 * k], x[33 + 8 * c + 2 * k]);
+                const uint64_t L = pk2u(x[2 * k], x[2 * k + 1]), H = pk2u(x[8 + 2 * k], x[9 + 2 * k]);
                 const uint64_t rl = sub2(mul2(L, cs[4 * c + k]), mul2(H, sn[4 * c + k])), rh = fma2(L, sn[4 * c + k], mul2(H, cs[4 * c + k]));
                 split_pair_16<false>(rl, hi[k], lo[k]);
                 split_pair_16<false>(rh, hi[4 + k], lo[4 + k]);
@@ -566,7 +592,7 @@ pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_con
           if ((top > PR_V_MAX && top < INFINITY) || (top < PR_V_MIN && top > 0.f))
             e = max((int)(__float_as_uint(top) >> 23) - 127 + (top < 1.f ? 3 : -14), PR_EXP_MIN);
           const int g = heads == 2 ? g0 + hf : g0;
-          if (heads == 1 && (t & 1) != hf) local = -1;           // (leaving the branch here instead cost 12 % of the kernel in spills)
+          if (heads == 1 && (now_t & 1) != hf) local = -1;           // (leaving the branch here instead cost 12 % of the kernel in spills)
           if (local >= 0) {
             a.vexp[(size_t)g * a.seg_rows + local] = (signed char)e;
             if (e != 0) a.vflag[(local / TILE) * v.Hkv + g] = seg + 1;
@@ -579,11 +605,12 @@ pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_con
 #pragma unroll
           for (int p = 0; p < 2; ++p) {
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-              uint32_t hi[4], lo[4];
+            for (int c = 0; c < 4; ++c) {
+              uint32_t hi[8], lo[8];
 #pragma unroll
-              for (int k = 0; k < 4; ++k) split_pair_16<false, false>(pk2u(x[p][8 * c + 2 * k], x[p][8 * c + 2 * k + 1]), hi[k], lo[k]);
-              stage_piece(c, hi, lo);
+              for (int k = 0; k < 8; ++k) split_pair_16<false, false>(pk2u(x[p][16 * c + 2 * k], x[p][16 * c + 2 * k + 1]), hi[k], lo[k]);
+              stage_piece(2 * c, hi, lo);
+              stage_piece(2 * c + 1, hi + 4, lo + 4);
             }
             rows_out(g, p);
           }
