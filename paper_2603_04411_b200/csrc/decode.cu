@@ -234,32 +234,30 @@ __global__ void __launch_bounds__(1024) plan_kernel(DevView v, int layer, const 
 }
 
 // -------------------------------------------------------------- merge + V projection
-// A cluster of eight CTAs per (query slots, query heads of one KV head g): at most eight rows (slot, head).  CTA c takes
+// A cluster of eight CTAs per (query slots, query heads of one KV head g): ROWS rows (slot, head) at most.  CTA c takes
 // the spectral components [c d/8, (c+1) d/8): it sums their splits, normalises, and multiplies by its rows of
-// U_V^-1[:, g*128 .. g*128+127]; the eight partial [rows x 128] products meet through distributed shared memory, every CTA
-// adding and writing 16 of the columns.  What bounds it is latency: one CTA doing a group's whole sum and product went
-// through 256 KiB of U_V^-1 and every split by itself.  Cold caches: 29.9 -> 9.2 us for one sequence of 1024 tokens with 64
-// splits, 28 -> 19.3 us for one of 131072 tokens with 64 heads; 16 sequences of 32768 tokens stay at 22 us, their 19 MB of
-// partial sums coming from DRAM.  Empty splits are not read (the V pass does not write them).
+// U_V^-1[:, g*128 .. g*128+127]; every CTA hands each of the others its part of 16 columns through distributed shared memory and
+// adds the eight parts of its own.  What bounds it is latency: one CTA doing a group's whole sum and product went
+// through 256 KiB of U_V^-1 and every split by itself.  Empty splits are not read (the V pass does not write them).
+// A cluster takes 5 to 6 us whatever its rows, so all of them are to be resident at once (merge_fit(), below): 4 sequences of 1000
+// tokens ran as 512 CTAs in three rounds, 17 us; a whole call in us, before / now: 4 x 1000 57.0 / 51.0, 4 x 8192 73.6 / 67.4,
+// 2 x 2000 with 64 heads 53.5 / 48.3, 24 x 2000 with 16 heads on 4 54.1 / 50.3, 1 x 131072 with 64 heads 156.7 / 148.1.
 constexpr int MG_THREADS = 256;
 constexpr int MG_CL = 8;                             // CTAs of a cluster
-constexpr int MG_ROWS = 8;
 
-__device__ __forceinline__ float ld_cluster_f32(uint32_t addr) {
-  float x;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(addr));
-  return x;
-}
+constexpr size_t merge_smem(int rows) { return (size_t)(6 * rows * 128 + rows) * sizeof(float); }
 
-template <bool BF16>
-__global__ void __launch_bounds__(MG_THREADS)
+template <bool BF16, int ROWS>
+__global__ void __launch_bounds__(MG_THREADS, 2)
 merge_kernel(DevView v, const unsigned short* Uinv_v, int n_splits, int hp, int ns, int n_seq, void* out) {
-  __shared__ float4 s_part[MG_THREADS];              // split sums per (split group, row, four components)
-  __shared__ __align__(16) float s_acc[MG_ROWS * 128];    // [rows][d / 8] normalised
-  __shared__ float s_red[4][MG_ROWS][128];
-  __shared__ float s_out[MG_ROWS * 128];
-  __shared__ float s_invl[MG_ROWS];
+  extern __shared__ __align__(16) unsigned char mg_smem[];
+  float* s_red = reinterpret_cast<float*>(mg_smem);  // [4][ROWS][128]; before that the split sums per (split group, row, four components)
+  float4* s_part = reinterpret_cast<float4*>(mg_smem);
+  float* s_acc = s_red + 4 * ROWS * 128;             // [rows][d / 8] normalised
+  float* s_in = s_acc + ROWS * 128;                  // [CTA of the cluster][row][16 columns of this CTA]
+  float* s_invl = s_in + ROWS * 128;
   chain_start();
+  tc::cluster_arrive();                              // waited for before the first remote store: the partners run
   chain_wait();
   // blockIdx.y = KV head g and which hp of its query heads; blockIdx.x / 8 = ns query slots that share the reads of U_V^-1
   const int c = tc::cluster_cta_rank();
@@ -268,26 +266,24 @@ merge_kernel(DevView v, const unsigned short* Uinv_v, int n_splits, int hp, int 
   const int rows = min(ns, n_seq - qs0) * hp;
   const int head0 = g * v.rep + (blockIdx.y % parts) * hp;      // first query head of this CTA
   const int jn = d_kv / MG_CL, j0 = c * jn;                     // jn: a multiple of 16, at most 128
-  // this thread's rows of U_V^-1 do not depend on the sums: their reads go out first (pair of columns dp, a quarter of the rows)
+  // row sums over the splits: warp w takes rows w and w + 8, its lanes read the splits' parts together, lane 0 adds them in split
+  // order; the first reads go out before everything else
+  constexpr int LR = (ROWS + 7) / 8;
+  float l_first[LR];
+#pragma unroll
+  for (int k = 0; k < LR; ++k) {
+    const int r = (tid >> 5) + 8 * k;
+    l_first[k] = r < rows && lane < n_splits ? v.part_l[((size_t)(qs0 + r / hp) * n_splits + lane) * Hq + head0 + r % hp] : 0.f;
+  }
+  // this thread's rows of U_V^-1 (pair of columns dp, a quarter of the rows) do not depend on the sums: on their way meanwhile
   const int dp = tid & 63, jg = tid >> 6, jr = jn / 4;
   const unsigned* ucol = reinterpret_cast<const unsigned*>(Uinv_v + (size_t)(j0 + jg * jr) * d_kv + g * HEAD_DIM) + dp;
   unsigned u[32];
 #pragma unroll
   for (int t = 0; t < 32; ++t) u[t] = t < jr ? ucol[(size_t)t * (d_kv / 2)] : 0u;
-  // row sums over the splits: warp w takes row w, its lanes read the splits' parts together, lane 0 adds them in split order
-  if ((tid >> 5) < rows) {
-    const int r = tid >> 5, qs = qs0 + r / hp, head = head0 + r % hp;
-    float l = 0.f;
-    for (int s0 = 0; s0 < n_splits; s0 += 32) {
-      const float mine = s0 + lane < n_splits ? v.part_l[((size_t)qs * n_splits + s0 + lane) * Hq + head] : 0.f;
-      const int n = min(32, n_splits - s0);
-      for (int s = 0; s < n; ++s) l += __shfl_sync(0xffffffffu, mine, s);
-    }
-    if (lane == 0) s_invl[r] = l > 0.f ? 1.f / l : 0.f;
-  }
-  // split sums: a thread owns four components of one row and every sg_n-th split, with eight reads in flight
-  const int q4 = jn / 4, slots = rows * q4, sg_n = MG_THREADS / slots, sg = tid / slots, sl = tid - sg * slots;
-  if (sg < sg_n) {
+  // split sums: a thread owns four components of one row (two rows of sixteen) and every sg_n-th split, with eight reads in flight
+  const int q4 = jn / 4, slots = rows * q4, sg_n = slots < MG_THREADS ? MG_THREADS / slots : 1, sg = slots < MG_THREADS ? tid / slots : 0;
+  for (int sl = slots < MG_THREADS ? tid - sg * slots : tid; sl < slots && sg < sg_n; sl += MG_THREADS) {
     const int r = sl / q4, qs = qs0 + r / hp;
     const float4* p = reinterpret_cast<const float4*>(v.part_acc + (((size_t)qs * n_splits) * Hq + head0 + r % hp) * d_kv + j0) + (sl - r * q4);
     const size_t stride = (size_t)Hq * d_kv / 4;
@@ -305,20 +301,33 @@ merge_kernel(DevView v, const unsigned short* Uinv_v, int n_splits, int hp, int 
     }
     s_part[sg * slots + sl] = a;
   }
-  __syncthreads();
-  if (tid < slots) {
-    float4 a = s_part[tid];
-    for (int k = 1; k < sg_n; ++k) {                   // fixed order
-      const float4 b = s_part[k * slots + tid];
-      a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w;
+#pragma unroll
+  for (int k = 0; k < LR; ++k) {
+    const int r = (tid >> 5) + 8 * k;
+    if (r >= rows) break;
+    float l = 0.f;
+    for (int s0 = 0; s0 < n_splits; s0 += 32) {
+      const float mine = s0 == 0 ? l_first[k]
+                                 : s0 + lane < n_splits ? v.part_l[((size_t)(qs0 + r / hp) * n_splits + s0 + lane) * Hq + head0 + r % hp] : 0.f;
+      const int n = min(32, n_splits - s0);
+      for (int s = 0; s < n; ++s) l += __shfl_sync(0xffffffffu, mine, s);
     }
-    const float il = s_invl[tid / q4];
-    *reinterpret_cast<float4*>(s_acc + tid * 4) = make_float4(a.x * il, a.y * il, a.z * il, a.w * il);
+    if (lane == 0) s_invl[r] = l > 0.f ? 1.f / l : 0.f;
   }
   __syncthreads();
-  float o[MG_ROWS][2];
+  for (int sl = tid; sl < slots; sl += MG_THREADS) {
+    float4 a = s_part[sl];
+    for (int k = 1; k < sg_n; ++k) {                   // fixed order
+      const float4 b = s_part[k * slots + sl];
+      a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w;
+    }
+    const float il = s_invl[sl / q4];
+    *reinterpret_cast<float4*>(s_acc + sl * 4) = make_float4(a.x * il, a.y * il, a.z * il, a.w * il);
+  }
+  __syncthreads();
+  float o[ROWS][2];
 #pragma unroll
-  for (int h = 0; h < MG_ROWS; ++h) { o[h][0] = 0.f; o[h][1] = 0.f; }
+  for (int h = 0; h < ROWS; ++h) { o[h][0] = 0.f; o[h][1] = 0.f; }
 #pragma unroll
   for (int t = 0; t < 32; t += 4) {
     if (t >= jr) break;                                // jr is a multiple of 4
@@ -326,7 +335,7 @@ merge_kernel(DevView v, const unsigned short* Uinv_v, int n_splits, int hp, int 
 #pragma unroll
     for (int e = 0; e < 4; ++e) { u0[e] = to_f32<BF16>((unsigned short)(u[t + e] & 0xffffu)); u1[e] = to_f32<BF16>((unsigned short)(u[t + e] >> 16)); }
 #pragma unroll
-    for (int h = 0; h < MG_ROWS; ++h)
+    for (int h = 0; h < ROWS; ++h)
       if (h < rows) {
         const float4 a = *reinterpret_cast<const float4*>(s_acc + h * jn + jg * jr + t);
         o[h][0] += a.x * u0[0]; o[h][1] += a.x * u1[0];
@@ -336,26 +345,39 @@ merge_kernel(DevView v, const unsigned short* Uinv_v, int n_splits, int hp, int 
       }
   }
 #pragma unroll
-  for (int h = 0; h < MG_ROWS; ++h)
-    if (h < rows) *reinterpret_cast<float2*>(&s_red[jg][h][2 * dp]) = make_float2(o[h][0], o[h][1]);
+  for (int h = 0; h < ROWS; ++h)
+    if (h < rows) *reinterpret_cast<float2*>(s_red + (jg * ROWS + h) * 128 + 2 * dp) = make_float2(o[h][0], o[h][1]);
   __syncthreads();
-  for (int i = tid; i < rows * 128; i += MG_THREADS)
-    s_out[i] = ((s_red[0][i >> 7][i & 127] + s_red[1][i >> 7][i & 127]) + s_red[2][i >> 7][i & 127]) + s_red[3][i >> 7][i & 127];
-  tc::cluster_sync_all();
-  constexpr int CW = 128 / MG_CL;                      // columns this CTA writes
-  if (tid < rows * CW) {
-    const int h = tid / CW, dc = c * CW + tid % CW;
-    const uint32_t at = tc::smem_addr(s_out + h * 128 + dc);
+  constexpr int CW = 128 / MG_CL;                      // columns a CTA writes
+  tc::cluster_wait();
+  for (int i = tid; i < rows * 32; i += MG_THREADS) {  // four columns of a row, to the CTA that writes them
+    const int h = i >> 5, c4 = (i & 31) * 4;
+    float4 a = *reinterpret_cast<const float4*>(s_red + h * 128 + c4);
+#pragma unroll
+    for (int k = 1; k < 4; ++k) {
+      const float4 b = *reinterpret_cast<const float4*>(s_red + (k * ROWS + h) * 128 + c4);
+      a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w;
+    }
+    tc::st_cluster_f32x4(tc::cluster_map(tc::smem_addr(s_in + (c * ROWS + h) * CW + c4 % CW), c4 / CW), a);
+  }
+  tc::cluster_sync_all();                              // every part has arrived; nothing remote is touched from here on
+  for (int i = tid; i < rows * CW; i += MG_THREADS) {
+    const int h = i / CW, dc = c * CW + i % CW;
     float val = 0.f;
 #pragma unroll
-    for (int k = 0; k < MG_CL; ++k) val += ld_cluster_f32(tc::cluster_map(at, k));       // fixed order
+    for (int k = 0; k < MG_CL; ++k) val += s_in[(k * ROWS + h) * CW + i % CW];            // fixed order
     const int oslot = qs0 + h / hp;
     const size_t oi = ((size_t)(v.qmap ? v.qmap[oslot] : oslot) * Hq + head0 + h % hp) * HEAD_DIM + dc;
     if (v.out_dtype == TWKV_F32) reinterpret_cast<float*>(out)[oi] = val;
     else if (v.out_dtype == TWKV_BF16) reinterpret_cast<unsigned short*>(out)[oi] = from_f32<true>(val);
     else reinterpret_cast<unsigned short*>(out)[oi] = from_f32<false>(val);
   }
-  tc::cluster_sync_all();                              // the partners have read this CTA's part
+}
+
+__device__ __forceinline__ float ld_cluster_f32(uint32_t addr) {
+  float x;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(addr));
+  return x;
 }
 
 // The same for large batches: 32 rows per cluster share a CTA's slice of U_V^-1, staged in shared memory; thread = (pair of
@@ -460,6 +482,24 @@ cudaError_t launch_kscore_tc(const DevView& v, int layer, const CUtensorMap& map
 cudaError_t launch_vacc_tc(const DevView& v, int layer, const CUtensorMap& map_blocks, const CUtensorMap* map_scores, const int* seq_ids,
                            int n_seq, int n_splits, cudaStream_t st);
 
+// Clusters of the merge kernel that are resident at once on an empty device (those of sixteen rows, which need the most).
+template <bool BF16>
+static int merge_fit(int sm_count) {
+  static const int cached = [sm_count] {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = MG_CL; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(MG_CL); cfg.blockDim = dim3(MG_THREADS); cfg.dynamicSmemBytes = merge_smem(16);
+    cfg.attrs = &attr; cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaFuncSetAttribute(merge_kernel<BF16, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)merge_smem(16)) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, merge_kernel<BF16, 16>, &cfg) != cudaSuccess || n < 1) { cudaGetLastError(); n = sm_count / MG_CL; }
+    return n;
+  }();
+  return cached;
+}
+
 template <bool BF16>
 static cudaError_t launch_decode_t(const DevView& v, int layer, const LayerParams& lp, const void* q, const int* seq_ids,
                                    int n_seq, void* out, int n_splits, int min_splits, int sm_count, const TcMaps* maps, bool pairs,
@@ -496,13 +536,19 @@ static cudaError_t launch_decode_t(const DevView& v, int layer, const LayerParam
       e = cudaFuncSetAttribute(merge_wide_kernel<BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, MW_SMEM);
       if (e == cudaSuccess) e = launch_chained(merge_wide_kernel<BF16>, dim3(MG_CL * wide, v.Hkv), dim3(MG_THREADS), dim3(MG_CL), MW_SMEM, st, v, uv, n_splits, n_seq, out);
     } else {
-      // query heads per cluster: the whole group, fewer (a divisor) while there are less than two CTAs per SM; then query
-      // slots per cluster (they share the reads of U_V^-1) while there are more
-      int hp = v.rep, ns = 1;
-      while (hp % 2 == 0 && MG_CL * n_seq * v.Hkv * (v.rep / hp) < 2 * sm_count) hp /= 2;
-      while (2 * ns * hp <= MG_ROWS && MG_CL * (n_seq * v.Hkv * (v.rep / hp) / (2 * ns)) >= 2 * sm_count) ns *= 2;
-      e = launch_chained(merge_kernel<BF16>, dim3(MG_CL * ((n_seq + ns - 1) / ns), v.Hkv * (v.rep / hp)), dim3(MG_THREADS), dim3(MG_CL), 0, st, v, uv,
-                         n_splits, hp, ns, n_seq, out);
+      // Rows per cluster: as few as still leave all clusters resident at once (a cluster takes about as long whatever its rows, and a
+      // second round of clusters starts when the first has ended); query heads of one slot first, then slots.
+      const int fit = merge_fit<BF16>(sm_count);
+      int hp = 1, ns = 1;
+      auto clusters = [&] { return (n_seq + ns - 1) / ns * v.Hkv * (v.rep / hp); };
+      while (hp < v.rep && clusters() > fit) hp *= 2;
+      while (2 * hp * ns <= 16 && ns < n_seq && clusters() > fit) ns *= 2;
+      const dim3 grid(MG_CL * ((n_seq + ns - 1) / ns), v.Hkv * (v.rep / hp));
+      auto go = [&](auto kernel, int rows) {
+        cudaError_t r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)merge_smem(rows));
+        return r != cudaSuccess ? r : launch_chained(kernel, grid, dim3(MG_THREADS), dim3(MG_CL), merge_smem(rows), st, v, uv, n_splits, hp, ns, n_seq, out);
+      };
+      e = hp * ns <= 4 ? go(merge_kernel<BF16, 4>, 4) : hp * ns <= 8 ? go(merge_kernel<BF16, 8>, 8) : go(merge_kernel<BF16, 16>, 16);
     }
     if (e != cudaSuccess) return e;
   }

@@ -46,7 +46,18 @@ def test_decode_where_the_work_split_changes(hkv, rep, n_seq, ctx, recipe, pick)
     (1, 8, 33, 40),             # one KV head: wide from a few clusters on, one sequence in the last
     (1, 4, 35, 30),
     (4, 4, 47, 20),
-    (8, 4, 23, 30),             # just below: eight rows per cluster
+    (8, 4, 23, 30),             # four groups of eight sequences, the last of seven
 ])
 def test_merge_of_medium_batches(hkv, rep, n_seq, ctx):
+    test_decode_where_the_work_split_changes(hkv, rep, n_seq, ctx, "any", list(range(n_seq)))
+
+
+@pytest.mark.parametrize("hkv,rep,n_seq,ctx", [
+    (8, 4, 9, 60),              # sixteen rows per cluster: four sequences, the last cluster holds one
+    (8, 1, 10, 40),             # the same of one head each
+    (8, 8, 3, 60),              # eight rows: one sequence's group
+    (2, 8, 20, 30),             # sixteen rows of two groups, 32 spectral components per CTA
+    (1, 2, 3, 50),              # one row, 16 components
+])
+def test_merge_rows_per_cluster(hkv, rep, n_seq, ctx):
     test_decode_where_the_work_split_changes(hkv, rep, n_seq, ctx, "any", list(range(n_seq)))
