@@ -46,7 +46,7 @@ def test_decode_where_the_work_split_changes(hkv, rep, n_seq, ctx, recipe, pick)
     (1, 8, 33, 40),             # one KV head: wide from a few clusters on, one sequence in the last
     (1, 4, 35, 30),
     (4, 4, 47, 20),
-    (8, 4, 23, 30),             # four groups of eight sequences, the last of seven
+    (8, 4, 23, 30),             # just below: eight rows per cluster
 ])
 def test_merge_of_medium_batches(hkv, rep, n_seq, ctx):
     test_decode_where_the_work_split_changes(hkv, rep, n_seq, ctx, "any", list(range(n_seq)))
