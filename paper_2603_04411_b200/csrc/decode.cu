@@ -239,22 +239,29 @@ __global__ void __launch_bounds__(1024) plan_kernel(DevView v, int layer, const 
 // U_V^-1[:, g*128 .. g*128+127]; every CTA hands each of the others its part of 16 columns through distributed shared memory and
 // adds the eight parts of its own.  What bounds it is latency: one CTA doing a group's whole sum and product went
 // through 256 KiB of U_V^-1 and every split by itself.  Empty splits are not read (the V pass does not write them).
-// A cluster takes 5 to 6 us whatever its rows, so all of them are to be resident at once (merge_fit(), below): 4 sequences of 1000
-// tokens ran as 512 CTAs in three rounds, 17 us; a whole call in us, before / now: 4 x 1000 57.0 / 51.0, 4 x 8192 73.6 / 67.4,
-// 2 x 2000 with 64 heads 53.5 / 48.3, 24 x 2000 with 16 heads on 4 54.1 / 50.3, 1 x 131072 with 64 heads 156.7 / 148.1.
+// A cluster of four rows takes 6 us, one of sixteen 15 (its share of the splits, then the FMAs: 67 M of them for 512 rows), so all
+// of them are to be resident at once (merge_fit(), below), three CTAs per SM: U_V^-1 waits in shared memory, not in registers.
+// 4 sequences of 1000 tokens ran as 512 CTAs in three rounds, 17 us.  A whole call in us, two CTAs per SM / three: 1 x 300
+// 40.1 / 36.7, 4 x 1000 48.4 / 44.7, 4 x 8192 65.2 / 61.0, 8 x 5000 80.4 / 74.3, 16 x 500 91.2 / 82.7, 2 x 2000 with 64 heads
+// 45.9 / 42.1, 1 x 131072 with 64 heads 145.9 / 140.5; more CTAs than fit and as many rows as fit, two per SM: 4 x 1000 57.0 / 51.0.
 constexpr int MG_THREADS = 256;
 constexpr int MG_CL = 8;                             // CTAs of a cluster
 
-constexpr size_t merge_smem(int rows) { return (size_t)(6 * rows * 128 + rows) * sizeof(float); }
+// shared memory: slice of U_V^-1 [d / 8][128] and, once it has been used, the quarters' products [4][rows][128] | sums | parts | 1 / l
+constexpr size_t MG_U_BYTES = 128 * 128 * 2;
+__host__ __device__ constexpr size_t merge_acc_bytes(int rows) { return rows * 512 > MG_THREADS * 16 ? rows * 512 : MG_THREADS * 16; }
+constexpr size_t merge_smem(int rows) { return MG_U_BYTES + merge_acc_bytes(rows) + rows * 512 + rows * sizeof(float); }
 
 template <bool BF16, int ROWS>
-__global__ void __launch_bounds__(MG_THREADS, 2)
+__global__ void __launch_bounds__(MG_THREADS, 3)
 merge_kernel(DevView v, const unsigned short* Uinv_v, int n_splits, int hp, int ns, int n_seq, void* out) {
   extern __shared__ __align__(16) unsigned char mg_smem[];
-  float* s_red = reinterpret_cast<float*>(mg_smem);  // [4][ROWS][128]; before that the split sums per (split group, row, four components)
-  float4* s_part = reinterpret_cast<float4*>(mg_smem);
-  float* s_acc = s_red + 4 * ROWS * 128;             // [rows][d / 8] normalised
-  float* s_in = s_acc + ROWS * 128;                  // [CTA of the cluster][row][16 columns of this CTA]
+  static_assert(4 * ROWS * 512 <= (int)MG_U_BYTES, "the quarters' products fit where U_V^-1 was");
+  const unsigned* s_u = reinterpret_cast<const unsigned*>(mg_smem);                 // pairs of columns
+  float* s_red = reinterpret_cast<float*>(mg_smem);
+  float* s_acc = reinterpret_cast<float*>(mg_smem + MG_U_BYTES);                     // [rows][d / 8] normalised
+  float4* s_part = reinterpret_cast<float4*>(s_acc);                                 // before that: split sums per (split group, row, four components)
+  float* s_in = s_acc + merge_acc_bytes(ROWS) / sizeof(float);                       // [CTA of the cluster][row][16 columns of this CTA]
   float* s_invl = s_in + ROWS * 128;
   chain_start();
   tc::cluster_arrive();                              // waited for before the first remote store: the partners run
@@ -275,12 +282,10 @@ merge_kernel(DevView v, const unsigned short* Uinv_v, int n_splits, int hp, int 
     const int r = (tid >> 5) + 8 * k;
     l_first[k] = r < rows && lane < n_splits ? v.part_l[((size_t)(qs0 + r / hp) * n_splits + lane) * Hq + head0 + r % hp] : 0.f;
   }
-  // this thread's rows of U_V^-1 (pair of columns dp, a quarter of the rows) do not depend on the sums: on their way meanwhile
-  const int dp = tid & 63, jg = tid >> 6, jr = jn / 4;
-  const unsigned* ucol = reinterpret_cast<const unsigned*>(Uinv_v + (size_t)(j0 + jg * jr) * d_kv + g * HEAD_DIM) + dp;
-  unsigned u[32];
-#pragma unroll
-  for (int t = 0; t < 32; ++t) u[t] = t < jr ? ucol[(size_t)t * (d_kv / 2)] : 0u;
+  // this CTA's slice of U_V^-1 does not depend on the sums: on its way meanwhile
+  for (int i = tid; i < jn * 16; i += MG_THREADS)
+    cp_async16(tc::smem_addr(mg_smem) + i * 16, reinterpret_cast<const uint4*>(Uinv_v + (size_t)(j0 + (i >> 4)) * d_kv + g * HEAD_DIM) + (i & 15));
+  cp_async_commit();
   // split sums: a thread owns four components of one row (two rows of sixteen) and every sg_n-th split, with eight reads in flight
   const int q4 = jn / 4, slots = rows * q4, sg_n = slots < MG_THREADS ? MG_THREADS / slots : 1, sg = slots < MG_THREADS ? tid / slots : 0;
   for (int sl = slots < MG_THREADS ? tid - sg * slots : tid; sl < slots && sg < sg_n; sl += MG_THREADS) {
@@ -315,7 +320,7 @@ merge_kernel(DevView v, const unsigned short* Uinv_v, int n_splits, int hp, int 
     if (lane == 0) s_invl[r] = l > 0.f ? 1.f / l : 0.f;
   }
   __syncthreads();
-  for (int sl = tid; sl < slots; sl += MG_THREADS) {
+  for (int sl = tid; sl < slots; sl += MG_THREADS) {  // in place: nobody else reads or writes these entries
     float4 a = s_part[sl];
     for (int k = 1; k < sg_n; ++k) {                   // fixed order
       const float4 b = s_part[k * slots + sl];
@@ -324,16 +329,21 @@ merge_kernel(DevView v, const unsigned short* Uinv_v, int n_splits, int hp, int 
     const float il = s_invl[sl / q4];
     *reinterpret_cast<float4*>(s_acc + sl * 4) = make_float4(a.x * il, a.y * il, a.z * il, a.w * il);
   }
+  cp_async_wait<0>();
   __syncthreads();
+  // thread = a pair of columns, a quarter of the components
+  const int dp = tid & 63, jg = tid >> 6, jr = jn / 4;
   float o[ROWS][2];
 #pragma unroll
   for (int h = 0; h < ROWS; ++h) { o[h][0] = 0.f; o[h][1] = 0.f; }
-#pragma unroll
-  for (int t = 0; t < 32; t += 4) {
-    if (t >= jr) break;                                // jr is a multiple of 4
+#pragma unroll 2
+  for (int t = 0; t < jr; t += 4) {                    // jr is a multiple of 4
     float u0[4], u1[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) { u0[e] = to_f32<BF16>((unsigned short)(u[t + e] & 0xffffu)); u1[e] = to_f32<BF16>((unsigned short)(u[t + e] >> 16)); }
+    for (int e = 0; e < 4; ++e) {
+      const unsigned w = s_u[(jg * jr + t + e) * 64 + dp];
+      u0[e] = to_f32<BF16>((unsigned short)(w & 0xffffu)); u1[e] = to_f32<BF16>((unsigned short)(w >> 16));
+    }
 #pragma unroll
     for (int h = 0; h < ROWS; ++h)
       if (h < rows) {
@@ -344,6 +354,7 @@ merge_kernel(DevView v, const unsigned short* Uinv_v, int n_splits, int hp, int 
         o[h][0] += a.w * u0[3]; o[h][1] += a.w * u1[3];
       }
   }
+  __syncthreads();                                     // U_V^-1 has been used by everyone
 #pragma unroll
   for (int h = 0; h < ROWS; ++h)
     if (h < rows) *reinterpret_cast<float2*>(s_red + (jg * ROWS + h) * 128 + 2 * dp) = make_float2(o[h][0], o[h][1]);
@@ -495,7 +506,7 @@ static int merge_fit(int sm_count) {
     int n = 0;
     if (cudaFuncSetAttribute(merge_kernel<BF16, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)merge_smem(16)) != cudaSuccess ||
         cudaOccupancyMaxActiveClusters(&n, merge_kernel<BF16, 16>, &cfg) != cudaSuccess || n < 1) { cudaGetLastError(); n = sm_count / MG_CL; }
-    return n;
+    return n - n / 16;                                   // behind another kernel not quite as many find room together
   }();
   return cached;
 }
@@ -528,21 +539,17 @@ static cudaError_t launch_decode_t(const DevView& v, int layer, const LayerParam
     const unsigned short* uv = reinterpret_cast<const unsigned short*>(lp.Uinv_v);
     const int wide = (n_seq * v.rep + MW_ROWS - 1) / MW_ROWS;
     cudaError_t e;
-    if (4 * MG_CL * wide * v.Hkv >= sm_count * (v.Hkv < 4 ? v.Hkv : 4)) {
-      // 32 rows per cluster while that still makes a CTA per SM; with few KV heads a CTA's slice of U_V^-1 is small and it is the number
-      // of clusters that costs.  The merge in us, eight / 32 rows: 32 heads on 8 KV heads, 16 sequences 23.0 / 27.1, 32 sequences
-      // 35.7 / 24.7; 64 on 8, 8 sequences 23.0 / 25.3, 16 sequences 37.2 / 25.1; 16 on 4, 24 sequences a step of 44.4 / 47.9,
-      // 64 sequences 29.2 / 17.9; 8 on 1, 64 sequences 16.5 / 12.7; 4 on 1, 64 sequences 14.8 / 12.3.
+    // Rows per cluster: as few as still leave all clusters resident at once (a second round of clusters starts when the first has
+    // ended); query heads of one slot first, then slots; 32 rows where sixteen are not enough.
+    const int fit = merge_fit<BF16>(sm_count);
+    int hp = 1, ns = 1;
+    auto clusters = [&] { return (n_seq + ns - 1) / ns * v.Hkv * (v.rep / hp); };
+    while (hp < v.rep && clusters() > fit) hp *= 2;
+    while (2 * hp * ns <= 16 && ns < n_seq && clusters() > fit) ns *= 2;
+    if (clusters() > fit) {
       e = cudaFuncSetAttribute(merge_wide_kernel<BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, MW_SMEM);
       if (e == cudaSuccess) e = launch_chained(merge_wide_kernel<BF16>, dim3(MG_CL * wide, v.Hkv), dim3(MG_THREADS), dim3(MG_CL), MW_SMEM, st, v, uv, n_splits, n_seq, out);
     } else {
-      // Rows per cluster: as few as still leave all clusters resident at once (a cluster takes about as long whatever its rows, and a
-      // second round of clusters starts when the first has ended); query heads of one slot first, then slots.
-      const int fit = merge_fit<BF16>(sm_count);
-      int hp = 1, ns = 1;
-      auto clusters = [&] { return (n_seq + ns - 1) / ns * v.Hkv * (v.rep / hp); };
-      while (hp < v.rep && clusters() > fit) hp *= 2;
-      while (2 * hp * ns <= 16 && ns < n_seq && clusters() > fit) ns *= 2;
       const dim3 grid(MG_CL * ((n_seq + ns - 1) / ns), v.Hkv * (v.rep / hp));
       auto go = [&](auto kernel, int rows) {
         cudaError_t r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)merge_smem(rows));
