@@ -227,7 +227,7 @@ struct twkv_cache {
   int sm_count;
   std::vector<LayerParams> params;
   Prof prof;
-  CUtensorMap map_blocks;
+  CUtensorMap map_blocks, map_boxes;   // the blocks as rows of one panel, boxes of a tile's rows / of a joint tile's sixteen
   CUtensorMap map_scores;              // the score scratch as [V slot][Hq] fp32, boxes of one tile's rows x one V-pass CTA's heads
   bool scores_tma = false;             // the head count allows that map (rows must start on 16-byte boundaries)
   std::vector<CUtensorMap> map_uinvT;  // per layer, over the transposed copy of U_K^-1 inside the pool
@@ -396,7 +396,8 @@ twkv_status twkv_cache_create(const twkv_config* cfg, void* pool, size_t pool_by
   c->map_wT_half.resize(2 * (size_t)cfg->n_layers);
   c->prepared_w.assign(cfg->n_layers, 0);
   c->appended = std::vector<std::atomic<long long>>(cfg->n_layers);
-  if (!make_tmap_2d(&c->map_blocks, c->view.blocks, (uint64_t)c->view.n_blocks * TILE, PANEL, PANEL * 2, TILE)) { delete c; return TWKV_ERR_CUDA; }
+  if (!make_tmap_2d(&c->map_blocks, c->view.blocks, (uint64_t)c->view.n_blocks * TILE, PANEL, PANEL * 2, TILE) ||
+      !make_tmap_2d(&c->map_boxes, c->view.blocks, (uint64_t)c->view.n_blocks * TILE, PANEL, PANEL * 2, JOINT_ROWS)) { delete c; return TWKV_ERR_CUDA; }
   if (c->cfg.n_q_heads % 4 == 0) {
     const int hq = c->cfg.n_q_heads, nb = hq < 16 ? hq : (hq <= 16 ? 16 : 32);
     if (!make_tmap_2d_f32(&c->map_scores, c->view.scores, (uint64_t)c->dims.NT * TILE, (uint64_t)hq, TILE, (uint32_t)(nb < hq ? nb : hq))) { delete c; return TWKV_ERR_CUDA; }
@@ -579,6 +580,7 @@ static twkv_status decode_pass(twkv_cache* c, int layer, const void* q, const in
   }
   TcMaps maps;
   maps.blocks = c->map_blocks;
+  maps.boxes = c->map_boxes;
   maps.scores = c->scores_tma ? &c->map_scores : nullptr;
   maps.uinvT_k = c->map_uinvT[layer];
   maps.uinv_k = c->pool + c->off.prep_uinvT + (size_t)layer * c->dims.d_kv * c->dims.d_kv * 2;

@@ -10,6 +10,8 @@
 //
 // V is never reconstructed per token: by linearity of Eq. 3 the weighted sum is taken in
 // spectral space and projected once.
+#include <algorithm>
+
 #include "twkv_dev.h"
 #include "mma_util.cuh"
 #include "tc_util.cuh"
@@ -25,7 +27,8 @@ namespace twkv {
 // does not depend on thread timing.  CTA 0 also cuts the list into n_cta contiguous pieces of about equal estimated cost, so
 // that a CTA (pair) of the K-score kernel mostly stays inside one (class, sequence) run.  What bounds it is the chain of
 // dependent table reads: one CTA that walked the whole list took 17.5 us for 16 sequences of 32768 tokens (2200 tiles) and 17
-// for 64 of 8192; a CTA per class takes 8.6 and 9.5 (8.9 -> 8.4 for 8 tiles).
+// for 64 of 8192; a CTA per class took 8.6 and 9.5 (8.9 -> 8.4 for 8 tiles).  The tables of the joint tiles (below) have CTAs of
+// their own, and a class's first tiles are asked for before anything is counted.
 // cycles per tile of the K-score kernel by rank class: a least-squares fit, one coefficient per class, of every CTA's busy
 // time to its tile counts on the benchmark's mix of classes (8 KV heads, CTA pairs; residual 1.3 us rms of 330): a fixed
 // part (rotation factors, the per-slab epilogue and score products) plus a per-panel part, an odd panel count costing a
@@ -84,6 +87,76 @@ __device__ void vsplit_plan(const DevView& v, int layer, const int* seq_ids, int
   if (used + tid <= n_splits) cut[used + tid] = n;               // (the library's own choice is at most 64)
 }
 
+// Joint tiles.  A key (sequence, class) ends with a tile that is partly full, and sixteen of those cost a short sequence several times
+// its tokens: the K-score kernel pays for a tile, not for its rows.  The last tiles of a sequence are therefore laid together, from the
+// widest class to the narrowest, as long as their rows (rounded up to boxes of sixteen) fit one tile; it has the class of its first, and
+// the narrower ones' missing panels are zeros.  Every row is computed as in a tile of its own, so the scores are the same bit for bit.
+// A decode call in us, a tile per class / joint tiles: 16 x 500 82.7 / 60.5, 64 x 1000 216 / 146, 37 x 700 of any rank 140 / 105,
+// 32 x 2000 139 / 111, 4 x 1000 44.7 / 41.7, 8 x 5000 74.3 / 72.2; long sequences, whose tiles are nearly all full, pay for the tables:
+// 1 x 30000 62.4 / 64.6, 4 x 8192 61.0 / 62.7.
+// Returns the classes (bit class - 1) at which a joint tile starts, and << 16 the classes that lie in one.
+__device__ unsigned joint_masks(const DevView& v, int layer, int seq) {
+  const int* fill = v.fill_l(layer) + (size_t)seq * v.NC;
+  int boxes[TWKV_MAX_CLASSES];
+#pragma unroll
+  for (int k = 0; k < TWKV_MAX_CLASSES; ++k) boxes[k] = k < v.NC ? ((fill[k] & (TILE - 1)) + JOINT_ROWS - 1) / JOINT_ROWS : 0;
+  unsigned starts = 0u, joined = 0u, run = 0u, first = 0u;       // of the run being laid together: its classes, the widest
+  int used = 0;
+#pragma unroll
+  for (int k = TWKV_MAX_CLASSES - 1; k >= 0; --k) {
+    const int b = boxes[k];
+    if (b == 0 || b == TILE / JOINT_ROWS) continue;
+    if (used + b > TILE / JOINT_ROWS) {
+      if (run != first) { starts |= first; joined |= run; }
+      run = 0u; used = 0;
+    }
+    if (run == 0u) first = 1u << k;
+    run |= 1u << k;
+    used += b;
+  }
+  if (run != first) { starts |= first; joined |= run; }
+  return starts | (joined << 16);
+}
+
+// One warp writes the tables of the joint tile of sequence `seq` that starts at class index k0 (bit k0 of the masks).
+__device__ void joint_tile(const DevView& v, int layer, int seq, unsigned masks, int k0, int id) {
+  const int lane = threadIdx.x & 31;
+  const unsigned below = masks & ((1u << k0) - 1u);               // the next joint tile's first class, if any, ends this one
+  unsigned members = (masks >> 16) & ((2u << k0) - 1u);
+  if (below) members &= ~((2u << (31 - __clz(below))) - 1u);
+  const bool in = lane < TWKV_MAX_CLASSES && ((members >> lane) & 1u);
+  const int key = seq * v.NC + lane;
+  const int rest = in ? v.fill_l(layer)[key] & (TILE - 1) : 0, tile = in ? v.key_last_l(layer)[key] : 0;
+  const int block = in ? v.desc(layer, 0)[tile].w : 0, room = (rest + JOINT_ROWS - 1) / JOINT_ROWS * JOINT_ROWS;
+  int at = room;                                                  // wide classes first: the rooms of the lanes above
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_down_sync(0xffffffffu, at, o);
+    if (lane + o < 32) at += u;
+  }
+  at -= room;
+  int slot[4] = {-1, -1, -1, -1};
+  unsigned box = 0u;
+  for (unsigned m = members; m; m &= m - 1) {
+    const int k = __ffs(m) - 1;
+    const int a = __shfl_sync(0xffffffffu, at, k), n = __shfl_sync(0xffffffffu, rest, k), rm = __shfl_sync(0xffffffffu, room, k);
+    const int t = __shfl_sync(0xffffffffu, tile, k), b = __shfl_sync(0xffffffffu, block, k);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int r = 32 * j + lane - a;
+      if (r >= 0 && r < n) slot[j] = t * TILE + r;
+    }
+    const int r = JOINT_ROWS * lane - a;
+    if (r >= 0 && r < rm) box = (unsigned)((b * TILE + r) / JOINT_ROWS) << 5 | (unsigned)(k + 1);
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    v.joint_rows()[(size_t)id * TILE + 32 * j + lane] = slot[j];
+    v.joint_pos()[(size_t)id * TILE + 32 * j + lane] = slot[j] >= 0 ? v.aux(layer, 0)[slot[j]] : 0;
+  }
+  if (lane < TILE / JOINT_ROWS) v.joint_boxes()[(size_t)id * (TILE / JOINT_ROWS) + lane] = box;
+}
+
 // K slot -> V slot of every token of one sequence (the V slots carry the opposite link): the K-score kernel stores a
 // token's scores at its V slot, so that the V pass finds a tile's score rows next to each other.  CTA j of the vj CTAs of
 // a sequence takes the V tiles j * 8 .. j * 8 + 7, then vj * 8 further on, eight tiles (1024 slots) at a time.
@@ -113,93 +186,118 @@ __global__ void __launch_bounds__(1024) plan_kernel(DevView v, int layer, const 
   }
   chain_wait();
   const int NC = v.NC;
-  if ((int)blockIdx.x >= NC + n_seq) {                            // the last n_seq * vj CTAs: K slot -> V slot links
-    const int idx = (int)blockIdx.x - NC - n_seq;
+  if ((int)blockIdx.x >= NC + 2 * n_seq) {                        // the last n_seq * vj CTAs: K slot -> V slot links
+    const int idx = (int)blockIdx.x - NC - 2 * n_seq;
     vlink_plan(v, layer, seq_ids, idx / vj, idx % vj, vj);
     return;
   }
-  if ((int)blockIdx.x >= NC) {                                    // before them n_seq CTAs: the V pass's split plan, one sequence each
+  if ((int)blockIdx.x >= NC + n_seq) {                            // before them n_seq CTAs: the tables of a sequence's joint tiles, a warp each
+    const int i = (int)blockIdx.x - NC - n_seq, seq = seq_ids[i];
+    if (threadIdx.x >= TWKV_MAX_CLASSES / 2 * 32 || seq < 0 || seq >= v.S) return;
+    const unsigned masks = joint_masks(v, layer, seq);
+    unsigned starts = masks & 0xffffu;
+    for (int w = threadIdx.x >> 5; w > 0 && starts; --w) starts ^= 1u << (31 - __clz(starts));
+    if (starts) joint_tile(v, layer, seq, masks, 31 - __clz(starts), i * (NC / 2) + (threadIdx.x >> 5));
+    return;
+  }
+  if ((int)blockIdx.x >= NC) {                                    // before those n_seq CTAs: the V pass's split plan, one sequence each
     vsplit_plan(v, layer, seq_ids, (int)blockIdx.x - NC, n_splits, min_splits);
     return;
   }
-  extern __shared__ int s_slot[];                                 // sequence id -> query slot, -1
+  extern __shared__ int s_slot[];                                 // sequence id -> query slot, -1; behind it, per query slot, its joint tiles
+  unsigned* s_joint = reinterpret_cast<unsigned*>(s_slot + v.S);
   __shared__ int s_warp[32];
   __shared__ int s_keep[TWKV_MAX_CLASSES];                        // tiles of the listed sequences per class
+  __shared__ int s_any[TWKV_MAX_CLASSES];                         // whether joint tiles start at the class
   __shared__ int s_koff[TWKV_MAX_CLASSES + 1], s_ioff[TWKV_MAX_CLASSES + 1];    // start of run k (class NC - k) in the tile list / in the item list
   __shared__ unsigned long long s_coff[TWKV_MAX_CLASSES + 1];     // estimated cost of everything before run k
   __shared__ int s_hg;                                            // parts per item
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int run = blockIdx.x, cls = NC - run;
+  // the class's first 1024 tiles are asked for at once: they arrive while the joint tiles and the counts are worked out
   const int n_list = v.kcc(layer)[cls - 1];
+  const int4* desc = v.desc(layer, 0);
+  const int* list = v.kct(layer) + (size_t)(cls - 1) * v.NT;
+  const int t_first = tid < n_list ? list[tid] : 0;
+  const int4 d_first = tid < n_list ? desc[t_first] : make_int4(0, 0, 0, 0);
   for (int s = tid; s < v.S; s += 1024) s_slot[s] = -1;
-  if (tid < TWKV_MAX_CLASSES) s_keep[tid] = 0;
+  if (tid < TWKV_MAX_CLASSES) s_keep[tid] = s_any[tid] = 0;
   __syncthreads();
   for (int i = tid; i < n_seq; i += 1024) {
     const int s = seq_ids[i];
-    if (s >= 0 && s < v.S) s_slot[s] = i;
-    else if (run == 0) set_status(v, TWKV_ERR_INVALID_ARG);
+    unsigned joint = 0u;
+    if (s >= 0 && s < v.S) {
+      s_slot[s] = i;
+      joint = joint_masks(v, layer, s);
+    }
+    s_joint[i] = joint;
   }
   for (int i = run * 1024 + tid; i < n_seq * v.Hq; i += NC * 1024) v.seqmax[i] = 0u;
   __syncthreads();
-  if (run == 0)
-    for (int i = tid; i < n_seq; i += 1024) {
-      const int s = seq_ids[i];
-      if (s >= 0 && s < v.S && s_slot[s] != i) set_status(v, TWKV_ERR_INVALID_ARG);   // duplicate id
-    }
+  // (an id outside the cache, or listed again later, has no tiles here)
+  auto listed = [&](int i) -> int { const int s = seq_ids[i]; return s >= 0 && s < v.S && s_slot[s] == i ? s : -1; };
+  for (int i = tid; i < n_seq; i += 1024) {
+    if (listed(i) >= 0) continue;
+    s_joint[i] = 0u;
+    if (run == 0) set_status(v, TWKV_ERR_INVALID_ARG);                                 // also a duplicate id
+  }
+  __syncthreads();
   {
     // tiles per class: a warp per class (and part of the sequences), a lane per sequence
     const int parts = 32 / NC, k = warp % NC, part = warp / NC;
     int mine = 0;
     if (part < parts)
-      for (int s = part * 32 + lane; s < v.S; s += parts * 32)
-        if (s_slot[s] >= 0) mine += (v.fill_l(layer)[s * NC + k] + TILE - 1) / TILE;
+      for (int i = part * 32 + lane; i < n_seq; i += parts * 32) {
+        const int s = listed(i);
+        if (s < 0) continue;
+        const int f = v.fill_l(layer)[s * NC + k];
+        const unsigned j = s_joint[i];
+        const int joint = (int)((j >> k) & 1u);
+        mine += f / TILE + (f % TILE != 0 && !((j >> (16 + k)) & 1u) ? 1 : 0) + joint;
+        if (joint) s_any[k] = 1;
+      }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
     if (lane == 0 && mine) atomicAdd(&s_keep[k], mine);
   }
   __syncthreads();
-  if (tid == 0) {
-    int ko = 0, io = 0;
-    unsigned long long co = 0ull;
-    for (int k = 0; k < NC; ++k) {
-      s_koff[k] = ko; s_ioff[k] = io; s_coff[k] = co;
-      const int keep = s_keep[NC - k - 1], items = pairs ? (keep + 1) / 2 : keep;
-      ko += keep; io += items;
-      co += (unsigned long long)items * ktile_cost(NC - k);
+  if (warp == 0) {
+    // lane k = run k (class NC - k): where its tiles, items and costs start
+    const int keep = lane < NC ? s_keep[NC - lane - 1] : 0, items = pairs ? (keep + 1) / 2 : keep;
+    int ko = keep, io = items;
+    unsigned long long co = (unsigned long long)items * ktile_cost(NC - lane);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int a = __shfl_up_sync(0xffffffffu, ko, o), b = __shfl_up_sync(0xffffffffu, io, o);
+      const unsigned long long c = __shfl_up_sync(0xffffffffu, co, o);
+      if (lane >= o) { ko += a; io += b; co += c; }
     }
-    s_koff[NC] = ko; s_ioff[NC] = io; s_coff[NC] = co;
+    if (lane < NC) { s_koff[lane + 1] = ko; s_ioff[lane + 1] = io; s_coff[lane + 1] = co; }
+    if (lane == 0) { s_koff[0] = s_ioff[0] = 0; s_coff[0] = 0ull; }
+    io = __shfl_sync(0xffffffffu, io, 31); co = __shfl_sync(0xffffffffu, co, 31);
     // The KV heads of an item may be dealt out to several CTAs (pairs): finer work for lists that leave some idle or that a few
     // wide tiles decide.  A part repeats the tile's loads and rotation factors.  Least estimate of the slowest piece, in cycles:
     // the widest part where every part has a CTA to itself, else the mean piece plus most of the widest part (numbers fitted to
     // lists of this kind).  A decode call in us, whole items / this rule (ranks 1 .. 512): 1 x 8192 50.6 / 49.4, 4 x 1000 51.1 / 48.8,
     // 8 x 8192 102.6 / 102.4, 16 x 500 62.6 / 63.2; 64 x 2000 and 16 x 32768 keep whole items.
     constexpr float PART_COST = 2600.f;
-    int widest = 0;
-    while (widest < NC && s_ioff[widest + 1] == s_ioff[widest]) ++widest;
-    const float wide_cost = widest < NC ? (float)ktile_cost(NC - widest) : 0.f, per_cta = 1.f / (float)n_cta;
-    float best = 3.4e38f;
-    s_hg = 1;
-    float part = 1.f;
+    const unsigned used = __ballot_sync(0xffffffffu, items > 0);
+    const float wide_cost = used ? (float)ktile_cost(NC - (__ffs(used) - 1)) : 0.f, per_cta = 1.f / (float)n_cta;
+    float best = 3.4e38f, part = 1.f;
+    int parts = 1;
     for (int h = 1; v.Hkv % h == 0; h *= 2, part *= 0.5f) {
       const float est = io * h <= n_cta ? wide_cost * part
                                         : ((float)co + (float)io * (float)(h - 1) * PART_COST) * per_cta + 0.7f * wide_cost * part;
-      if (est < best) { best = est; s_hg = h; }
+      if (est < best) { best = est; parts = h; }
     }
+    if (lane == 0) s_hg = parts;
   }
   __syncthreads();
   // this class's entries; a run of odd length ends with a filler for the pair kernel: the same tile again, flagged so that its
   // scores are dropped
-  const int4* desc = v.desc(layer, 0);
-  const int* list = v.kct(layer) + (size_t)(cls - 1) * v.NT;
   const int n_keep = s_koff[run + 1] - s_koff[run];
   int base = 0;
-  for (int i0 = 0; i0 < n_list; i0 += 1024) {
-    int4 e = make_int4(0, 0, 0, -1);
-    if (i0 + tid < n_list) {
-      const int t = list[i0 + tid];
-      const int4 d = desc[t];
-      e = make_int4(t, d.y | (d.z << 8), d.w, s_slot[d.x]);
-    }
+  auto put = [&](const int4& e) {                                 // the next entries, of the threads that have one (.w >= 0), in thread order
     int total;
     const int at = base + block_scan_excl(e.w >= 0 ? 1 : 0, s_warp, &total);
     if (e.w >= 0 && at < n_keep) {
@@ -211,6 +309,23 @@ __global__ void __launch_bounds__(1024) plan_kernel(DevView v, int layer, const 
       }
     }
     base += total;
+  };
+  for (int i0 = 0; i0 < n_list; i0 += 1024) {
+    int4 e = make_int4(0, 0, 0, -1);
+    if (i0 + tid < n_list) {
+      const int t = i0 ? list[i0 + tid] : t_first;
+      const int4 d = i0 ? desc[t] : d_first;
+      int slot = s_slot[d.x];
+      if (slot >= 0 && d.z < TILE && ((s_joint[slot] >> (15 + cls)) & 1u)) slot = -1;     // lies in a joint tile
+      e = make_int4(t, d.y | (d.z << 8), d.w, slot);
+    }
+    put(e);
+  }
+  // the joint tiles that start at this class; their numbers count the sequence's from the widest on
+  for (int i0 = 0; i0 < n_seq && s_any[cls - 1]; i0 += 1024) {
+    const int i = i0 + tid;
+    const bool mine = i < n_seq && ((s_joint[i] >> (cls - 1)) & 1u);
+    put(mine ? make_int4(~(i * (NC / 2) + __popc((s_joint[i] & 0xffffu) >> cls)), cls | (TILE << 8), 0, i) : make_int4(0, 0, 0, -1));
   }
   if (run > 0) return;
   // (the parts the KV heads of an item are dealt out in: chosen above)
@@ -488,7 +603,7 @@ merge_wide_kernel(DevView v, const unsigned short* Uinv_v, int n_splits, int n_s
 }
 
 // ------------------------------------------------------------------------- host side
-cudaError_t launch_kscore_tc(const DevView& v, int layer, const CUtensorMap& map_blocks, const CUtensorMap& map_uinvT,
+cudaError_t launch_kscore_tc(const DevView& v, int layer, const CUtensorMap& map_blocks, const CUtensorMap& map_boxes, const CUtensorMap& map_uinvT,
                              const void* q, int n_pieces, bool pairs, cudaStream_t st);
 cudaError_t launch_vacc_tc(const DevView& v, int layer, const CUtensorMap& map_blocks, const CUtensorMap* map_scores, const int* seq_ids,
                            int n_seq, int n_splits, cudaStream_t st);
@@ -518,15 +633,15 @@ static cudaError_t launch_decode_t(const DevView& v, int layer, const LayerParam
   // the K-score kernel's work is cut into one piece per persistent CTA, or per CTA pair
   const int n_pieces = pairs ? kscore_max_pairs(sm_count) : sm_count;
   // CTAs per sequence that invert the V -> K links: enough of them that they finish inside the K work list's time
-  const int vj = n_seq >= 256 ? 1 : (256 / n_seq > 64 ? 64 : 256 / n_seq);
+  const int vj = n_seq >= 128 ? 1 : std::min(64, (256 - n_seq) / n_seq);
   {
     ProfScope ps(TWKV_K_PLAN, st);
-    cudaError_t e = launch_chained(plan_kernel, dim3(v.NC + n_seq + n_seq * vj), dim3(1024), dim3(1), (size_t)v.S * sizeof(int), st, v, layer, seq_ids,
+    cudaError_t e = launch_chained(plan_kernel, dim3(v.NC + n_seq * (2 + vj)), dim3(1024), dim3(1), (size_t)v.S * 2 * sizeof(int), st, v, layer, seq_ids,
                                    n_seq, n_pieces, pairs ? 1 : 0, n_splits, min_splits, vj, maps->uinv_k, lp.Uinv_v);
     if (e != cudaSuccess) return e;
   }
   {
-    cudaError_t e = launch_kscore_tc(v, layer, maps->blocks, maps->uinvT_k, q, n_pieces, pairs, st);
+    cudaError_t e = launch_kscore_tc(v, layer, maps->blocks, maps->boxes, maps->uinvT_k, q, n_pieces, pairs, st);
     if (e != cudaSuccess) return e;
   }
   {

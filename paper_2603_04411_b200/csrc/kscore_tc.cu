@@ -18,6 +18,8 @@
 // product and a tile has no tail: RoPE and the high / low split are the only per-element CUDA-core work.  Both products
 // are linear in X^_K, so a class wider than 8 panels runs as two passes over its panels; the second pass adds to the
 // scores the first one stored.
+// A tile may also be a joint one (plan_kernel): rows of several classes' partly full tiles of one sequence, sixteen-row boxes that the
+// producer brings together; where a class has no further panel its boxes are zeros.
 //
 // Tensor memory (512 columns): slabs 3 x 128 | score accumulators 4 x 16.
 // Warp roles (512 threads, one persistent CTA per SM working through a contiguous, cost-balanced piece of the tile list;
@@ -91,7 +93,7 @@ constexpr int KE_DISCARD = 0x80;                               // list entry, .y
 // DBG (caches created with TWKV_DEBUG=1): rotated keys that the f16 conversion clamps are reported.
 template <bool BF16, int REP, bool PAIR, bool DBG>
 __global__ void __launch_bounds__(KT_THREADS, 1)
-kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_constant__ CUtensorMap map_uinvT,
+kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_constant__ CUtensorMap map_boxes, const __grid_constant__ CUtensorMap map_uinvT,
                  DevView v, int layer, const unsigned short* q, int nb) {
   chain_start();
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -160,6 +162,12 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
   // (hg is a power of two; the single-thread roles pay for every instruction of theirs, so no divisions here)
   const int hs = __ffs(*v.kitem_parts) - 1, nh = Hkv >> hs;
   auto unit = [&](int w) -> int4 { return w < total ? klist[KSTEP * (w >> hs)] : kt_none; };
+  // K slot of a row of an entry, -1 where it holds no token
+  auto row_slot = [&](const int4& e, int row) -> int {
+    if (e.w < 0) return -1;
+    if (e.x < 0) return v.joint_rows()[(size_t)~e.x * TILE + row];
+    return row < (e.y >> 8) ? e.x * TILE + row : -1;
+  };
   // CTAs walk the KV heads in rotated order, so that at any moment they read different panels of U_K^-1 from L2
   const int g_rot = piece % nh;
   auto first_head = [&](int w) -> int { return (w & ((1 << hs) - 1)) * nh; };
@@ -176,18 +184,37 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
     // elect.sync issues the copy instruction directly; from lanes picked by their index each issue took hundreds of cycles.
     if (elect_one()) {
       tma_prefetch_desc(&map_blocks);
+      tma_prefetch_desc(&map_boxes);
       uint32_t ak = 0;                                          // panels so far; slot = ak % 8
       bool ok = true;
       int4 e = unit(w0);
       for (int w = w0; w < total && ok; ++w) {
         const int4 nxt = unit(w + 1);
         const int cls = e.y & 0x7f, blk = e.z;
+        const bool joint = e.x < 0;
+        unsigned box[TILE / JOINT_ROWS];
+        if (joint) {
+          const uint4* b4 = reinterpret_cast<const uint4*>(v.joint_boxes() + (size_t)~e.x * (TILE / JOINT_ROWS));
+          const uint4 lo = b4[0], hi = b4[1];
+          box[0] = lo.x; box[1] = lo.y; box[2] = lo.z; box[3] = lo.w; box[4] = hi.x; box[5] = hi.y; box[6] = hi.z; box[7] = hi.w;
+        }
         for (int j = 0; j < cls; ++j, ++ak) {
           const uint32_t slot = ak % KT_A_SLOTS, ph = (ak / KT_A_SLOTS) & 1u;
           if (!(ok = mbar_wait_thin(a_empty + 8 * slot, ph ^ 1u, abort_flag))) break;
           if (crank == 0) mbar_expect_tx(a_full + 8 * slot, CG * PANEL_BYTES);          // this CTA's copy and the partner's
-          if constexpr (PAIR) tma_load_2d_pair(sA + slot * PANEL_BYTES, &map_blocks, a_full_own + 8 * slot, 0, (blk + j) * TILE);
-          else tma_load_2d(sA + slot * PANEL_BYTES, &map_blocks, a_full + 8 * slot, 0, (blk + j) * TILE);
+          if (!joint) {
+            if constexpr (PAIR) tma_load_2d_pair(sA + slot * PANEL_BYTES, &map_blocks, a_full_own + 8 * slot, 0, (blk + j) * TILE);
+            else tma_load_2d(sA + slot * PANEL_BYTES, &map_blocks, a_full + 8 * slot, 0, (blk + j) * TILE);
+          } else {
+            // sixteen rows at a time; a box of a narrower class lies behind the last block from its class on and reads zeros there
+#pragma unroll
+            for (int b = 0; b < TILE / JOINT_ROWS; ++b) {
+              const int y = j < (int)(box[b] & 31u) ? (int)(box[b] >> 5) * JOINT_ROWS + j * TILE : v.n_blocks * TILE;
+              const uint32_t dst = sA + slot * PANEL_BYTES + b * (JOINT_ROWS * PANEL * 2);
+              if constexpr (PAIR) tma_load_2d_pair(dst, &map_boxes, a_full_own + 8 * slot, 0, y);
+              else tma_load_2d(dst, &map_boxes, a_full + 8 * slot, 0, y);
+            }
+          }
         }
         e = nxt;
       }
@@ -388,14 +415,16 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
     };
     uint32_t last_slot = 0, last_slph = 0;                          // score accumulator of the slab rotated last, and its phase
     int4 e = unit(w0);
-    int pos_cur = w0 < total ? kpos[(size_t)e.x * TILE + row] : 0;              // this row's position in the current tile
+    auto row_pos = [&](const int4& e) -> int { return e.w < 0 ? 0 : e.x < 0 ? v.joint_pos()[(size_t)~e.x * TILE + row] : kpos[(size_t)e.x * TILE + row]; };
+    int pos_cur = row_pos(e);                                                    // this row's position in the current tile
     if (w0 < total) { write_q(e.w); rope_setup(pos_cur); }
     for (int w = w0; w < total && ok; ++w) {
       const int4 nxt = unit(w + 1);
       const int cls = e.y & 0x7f, qs = e.w;
-      [[maybe_unused]] const int n_valid = e.y >> 8;
+      [[maybe_unused]] bool has_row = true;
+      if constexpr (DBG) has_row = row_slot(e, row) >= 0;
       const int passes = (cls + KT_A_SLOTS - 1) / KT_A_SLOTS;
-      const int pos_next = nxt.w >= 0 ? kpos[(size_t)nxt.x * TILE + row] : 0;      // fetched now, used after the tile's slabs
+      const int pos_next = row_pos(nxt);                                          // fetched now, used after the tile's slabs
       for (int ps = 0; ps < passes && ok; ++ps) {
         for (int sli = 0; sli < nh; ++sli) {
           if (!(ok = __all_sync(0xffffffffu, mbar_wait(slab_full + 8 * sbuf, sph, abort_flag)))) break;
@@ -434,7 +463,7 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
               bool sat = false;
 #pragma unroll
               for (int u = 0; u < 8; ++u) sat |= (oh[u] & 0x7fffu) == 0x7bffu || ((oh[u] >> 16) & 0x7fffu) == 0x7bffu;
-              if (sat && row < n_valid) set_status(v, TWKV_ERR_DEVICE_CHECK);
+              if (sat && has_row) set_status(v, TWKV_ERR_DEVICE_CHECK);
             }
             tmem_st8(sl_addr + 8 * c, oh);                                    // high parts: columns 0 .. 63 of the slab
             tmem_st8(sl_addr + 64 + 8 * c, ol);                               // low parts: columns 64 .. 127
@@ -480,22 +509,24 @@ kscore_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_co
     uint32_t slot = 0, slph = 0;
     bool ok = true;
     int4 e = unit(w0);
-    int pos_cur = w0 < total ? kpos[(size_t)e.x * TILE + row] : 0;
+    int kslot = row_slot(e, row);
+    int pos_cur = kslot >= 0 ? kpos[kslot] : 0;
     // the row of the score scratch this token's scores go to: its V slot (rows past the tile's last token have none)
-    int vrow_cur = w0 < total && row < (e.y >> 8) ? v.kv_link[(size_t)e.x * TILE + row] : 0;
+    int vrow_cur = kslot >= 0 ? v.kv_link[kslot] : 0;
     for (int w = w0; w < total && ok; ++w) {
       const int4 nxt = unit(w + 1);
-      const int cls = e.y & 0x7f, n_valid = e.y >> 8, qs = e.w;
+      const int cls = e.y & 0x7f, qs = e.w;
       const int g0 = first_head(w);
+      const bool has_row = kslot >= 0;
       const bool discard = (e.y & KE_DISCARD) != 0;
       const int passes = (cls + KT_A_SLOTS - 1) / KT_A_SLOTS;
-      const int pos_next = nxt.w >= 0 ? kpos[(size_t)nxt.x * TILE + row] : 0;
-      const int vrow_next = nxt.w >= 0 && row < (nxt.y >> 8) ? v.kv_link[(size_t)nxt.x * TILE + row] : 0;
-      const bool has_row = row < n_valid;
+      kslot = row_slot(nxt, row);
+      const int pos_next = kslot >= 0 ? kpos[kslot] : 0;
+      const int vrow_next = kslot >= 0 ? v.kv_link[kslot] : 0;
       float* const out_row = v.scores + (size_t)vrow_cur * Hq;
       // a row counts if it holds a token and, for a causal (prefill) query, the token is not after the query
       const int pos_limit = v.qpos ? v.qpos[qs] : 0x7fffffff;
-      const bool live = row < n_valid && pos_cur <= pos_limit;
+      const bool live = has_row && pos_cur <= pos_limit;
       for (int ps = 0; ps < passes && ok; ++ps) {
         const uint32_t mode = discard ? KP_DISCARD : passes == 1 ? KP_STORE_FINAL : (ps == 0 ? KP_STORE_PART : KP_ADD_FINAL);
         for (int sli = 0; sli < nh; ++sli) {
@@ -641,7 +672,7 @@ int kscore_max_pairs(int sm_count) {
 }
 
 template <bool BF16, bool PAIR, bool DBG>
-static cudaError_t launch_kscore_tc_t(const DevView& v, int layer, const CUtensorMap& map_blocks, const CUtensorMap& map_uinvT,
+static cudaError_t launch_kscore_tc_t(const DevView& v, int layer, const CUtensorMap& map_blocks, const CUtensorMap& map_boxes, const CUtensorMap& map_uinvT,
                                       const void* q, int n_pieces, cudaStream_t st) {
   const int nb = PAIR ? KT_NB_PAIR : KT_NB_SINGLE;
   const size_t smem = kscore_tc_smem_bytes(nb, PAIR ? PANEL_BYTES : 2 * PANEL_BYTES);
@@ -653,7 +684,7 @@ static cudaError_t launch_kscore_tc_t(const DevView& v, int layer, const CUtenso
     e = cudaFuncSetAttribute(kscore_tc_kernel<BF16, REP, PAIR, DBG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
     if (e != cudaSuccess) return e;                                                                                   \
     e = launch_chained(kscore_tc_kernel<BF16, REP, PAIR, DBG>, dim3(PAIR ? 2 * n_pieces : n_pieces), dim3(KT_THREADS),   \
-                       dim3(PAIR ? 2 : 1), smem, st, map_blocks, map_uinvT, v, layer, qq, nb);                         \
+                       dim3(PAIR ? 2 : 1), smem, st, map_blocks, map_boxes, map_uinvT, v, layer, qq, nb);                         \
   }
   switch (v.rep) {
     case 1: TWKV_KT(1) break;
@@ -667,11 +698,11 @@ static cudaError_t launch_kscore_tc_t(const DevView& v, int layer, const CUtenso
 }
 
 // `pairs`: run on CTA pairs (n_pieces pairs, map_uinvT with 64-row boxes) instead of single CTAs (128-row boxes).
-cudaError_t launch_kscore_tc(const DevView& v, int layer, const CUtensorMap& map_blocks, const CUtensorMap& map_uinvT,
+cudaError_t launch_kscore_tc(const DevView& v, int layer, const CUtensorMap& map_blocks, const CUtensorMap& map_boxes, const CUtensorMap& map_uinvT,
                              const void* q, int n_pieces, bool pairs, cudaStream_t st) {
 #define TWKV_KS_LAUNCH(BF, PR)                                                                                  \
-  (v.debug ? launch_kscore_tc_t<BF, PR, true>(v, layer, map_blocks, map_uinvT, q, n_pieces, st)                 \
-           : launch_kscore_tc_t<BF, PR, false>(v, layer, map_blocks, map_uinvT, q, n_pieces, st))
+  (v.debug ? launch_kscore_tc_t<BF, PR, true>(v, layer, map_blocks, map_boxes, map_uinvT, q, n_pieces, st)                 \
+           : launch_kscore_tc_t<BF, PR, false>(v, layer, map_blocks, map_boxes, map_uinvT, q, n_pieces, st))
   if (pairs) return v.dtype == TWKV_BF16 ? TWKV_KS_LAUNCH(true, true) : TWKV_KS_LAUNCH(false, true);
   return v.dtype == TWKV_BF16 ? TWKV_KS_LAUNCH(true, false) : TWKV_KS_LAUNCH(false, false);
 #undef TWKV_KS_LAUNCH

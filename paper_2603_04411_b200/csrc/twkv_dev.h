@@ -18,6 +18,7 @@ constexpr int ROPE_LO = 16;                 // pos = hi * 16 + lo
 constexpr int ROPE_HI = 32768;              // positions up to 16 * 32768 - 1
 constexpr int MAX_PARTIALS_EXTRA = 320;     // V-side partial slots beyond max_seqs
 constexpr int MAX_PLAN_CTAS = 1024;         // upper bound on the K-score kernel's grid
+constexpr int JOINT_ROWS = 16;              // rows of a box of a joint tile
 constexpr int DECODE_SPLIT_TOKENS = 512;    // tokens a V split is worth where the library chooses the number of splits
 constexpr unsigned long long TWKV_GUARD_WORD = 0x7477b2006b765f67ull;   // written behind every region of the pool
 
@@ -66,7 +67,8 @@ struct DevView {
   int* evict_fill;           // [2][NC]  survivors per key
   int* wave_buf;             // [3 * TWKV_PREFILL_MAX_QUERIES]  the host's tables of a prefill call; in waves: sequence, row and position of
                              // the queries, wave by wave
-  int4* klist;               // [NT]  K tiles of the current decode call, widest class first: (tile, class | n_valid << 8, base block, query slot)
+  int4* klist;               // [NT]  K tiles of the current decode call, widest class first: (tile, class | n_valid << 8, base block, query slot);
+                             //       a joint tile: (~ its number, class | 128 << 8, 0, query slot)
   int4* kpairs;              // [NT + 64]  the same list as items of two tiles of one class (entries 2 i, 2 i + 1) for the CTA-pair kernel;
                              //            a class with an odd number of tiles ends with a filler entry (.y bit 7 set)
   int* kitem_parts;          // [1]  parts the KV heads of a list item are dealt out in
@@ -78,6 +80,12 @@ struct DevView {
   int4* gate_fix;            // rows the fused gate kernel hands to its fix-up kernel
   float* gate_scratch;       // COMPUTE mode logits: [GATE_PIECE][2][d_kv] (small calls) or one [128][d_kv] block per CTA (fused kernel)
 
+  // Joint tiles of a decode pass, in the eviction's scratch (a decode pass does not use it otherwise): per tile the K slot of each of
+  // its rows (-1: none) and their positions, and its eight boxes of sixteen rows (first row among all blocks' rows / 16 << 5 | class).
+  // At most NC / 2 per sequence, a fraction of the regions' room of TPS > NC tiles.
+  __host__ __device__ int* joint_rows() const { return evict_map; }
+  __host__ __device__ int* joint_pos() const { return evict_map + (size_t)NT * TILE; }
+  __host__ __device__ unsigned* joint_boxes() const { return reinterpret_cast<unsigned*>(joint_pos() + (size_t)S * (NC / 2) * TILE); }
   __host__ __device__ int4* desc(int l, int side) const { return tile_desc + ((size_t)l * 2 + side) * NT; }
   __host__ __device__ int* aux(int l, int side) const { return tile_aux + ((size_t)l * 2 + side) * NT * TILE; }
   __host__ __device__ unsigned short* rank(int l, int side) const { return tile_rank + ((size_t)l * 2 + side) * NT * TILE; }

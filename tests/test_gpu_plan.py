@@ -61,3 +61,62 @@ def test_merge_of_medium_batches(hkv, rep, n_seq, ctx):
 ])
 def test_merge_rows_per_cluster(hkv, rep, n_seq, ctx):
     test_decode_where_the_work_split_changes(hkv, rep, n_seq, ctx, "any", list(range(n_seq)))
+
+
+@pytest.mark.parametrize("hkv,single,counts", [
+    (8, False, {16: 1, 15: 16, 14: 17, 13: 64, 9: 3}),             # 16 + 16 + 32 + 64 rows fill a tile; class 9 stays by itself
+    (8, False, {16: 16, 8: 112, 7: 113, 5: 127, 3: 128, 2: 1, 1: 15}),    # rests that fit exactly, that fit nothing, and a full tile between
+    (8, True, {12: 200, 10: 33, 9: 130, 1: 129}),                  # single CTAs; full tiles beside the joint one
+    (1, False, {2: 5, 1: 140}),                                    # two classes
+    (4, False, {k: 40 for k in range(1, 9)}),                      # every class: three joint tiles
+])
+def test_joint_tiles_of_partly_full_classes(hkv, single, counts, monkeypatch):
+    """Three sequences with these tokens per class (K; V in reverse), one a token longer, one holding the widest class alone; decoded
+    in two orders, again after an append, and after an eviction."""
+    from paper_2603_04411_b200 import binding as B
+    if single:
+        monkeypatch.setenv("TWKV_KSCORE_SINGLE", "1")
+    d, hq = hkv * 128, hkv * 4
+    rng = np.random.default_rng(31 * hkv + len(counts))
+    per_class = np.concatenate([rng.integers(64 * c - 63, 64 * c + 1, n) for c, n in counts.items()])
+    rk = [rng.permutation(per_class), rng.permutation(np.append(per_class, 64 * max(counts))), np.full(7, 64 * max(counts))]
+    n = [len(r) for r in rk]
+    room = max(n) + 1
+    li = workloads.build_layer(77 + hkv, n_seq=3, ctx=room, n_q_heads=hq, n_kv_heads=hkv, n_calib=2 * d, outlier="none", mode="forced",
+                               rank_recipe="any")
+    ranks = np.zeros((3, room, 2), dtype=np.int64)
+    for s in range(3):
+        ranks[s, :n[s], 0], ranks[s, :n[s], 1] = rk[s], rk[s][::-1]
+        ranks[s, n[s]] = 1                                          # the token appended later
+    ranks = ranks.reshape(-1, 2)
+    seq, pos = li.seq_ids.numpy(), li.positions.numpy()
+    assert np.array_equal(pos.reshape(3, room), np.tile(np.arange(room), (3, 1)))
+    first, then = pos < np.array(n)[seq], pos == np.array(n)[seq]
+    gc = GpuCache(B, n_layers=1, n_q_heads=hq, n_kv_heads=hkv, dtype=torch.float16, out_dtype=torch.float32, max_seqs=3, max_tokens_per_seq=room,
+                  payload_bytes=room * 12 * d)
+    B.twkv_cache_set_layer_params(gc.h, 0, li.Uinv_k.cuda(), li.Uinv_v.cuda())
+
+    def compress(rows):
+        t = torch.from_numpy(np.nonzero(rows)[0])
+        B.twkv_compress(gc.h, 0, li.xt_k[t].cuda(), li.xt_v[t].cuda(), li.seq_ids[t].cuda(), li.positions[t].cuda(), None,
+                        torch.from_numpy(ranks[rows].astype(np.int16)).cuda(), B.TWKV_GATE_FORCED)
+
+    def check(rows, order):
+        out = torch.full((len(order), hq, 128), float("nan"), device="cuda")
+        B.twkv_decode_attn(gc.h, 0, li.q[order].cuda(), torch.tensor(order, dtype=torch.int32, device="cuda"), out)
+        assert B.twkv_cache_status(gc.h) == B.TWKV_OK
+        t = torch.from_numpy(np.nonzero(rows)[0])
+        part = workloads.LayerInputs(**{**vars(li), "xt_k": li.xt_k[t], "xt_v": li.xt_v[t], "seq_ids": li.seq_ids[t], "positions": li.positions[t],
+                                        "q": li.q[order]})
+        max_abs, rel_l2 = attn_errors(out.cpu().numpy(), oracle_decode(part, ranks[rows], order))
+        assert max_abs < 2e-3 and rel_l2 < 1e-3, (max_abs, rel_l2)  # the bars of every decode test
+
+    compress(first)
+    check(first, [0, 1, 2])
+    check(first, [2, 0])
+    compress(then)
+    check(first | then, [1, 2, 0])
+    keep = np.sort(rng.permutation(n[0])[:n[0] // 2])
+    B.twkv_evict(gc.h, 0, 0, torch.from_numpy(keep.astype(np.int32)).cuda())
+    check(((first | then) & (seq > 0)) | ((seq == 0) & np.isin(pos, keep)), [0, 1])
+    gc.close()
