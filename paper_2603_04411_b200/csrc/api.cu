@@ -338,7 +338,7 @@ static void fill_view(twkv_cache* c) {
   v.gate_fix = (int4*)(p + o.gate_fix);
   v.wave_buf = (int*)(p + o.wave_buf);
   v.evict_bitmap = (unsigned*)(p + o.evict_bitmap); v.evict_map = (int*)(p + o.evict_map); v.evict_fill = (int*)(p + o.evict_fill);
-  v.qmap = nullptr; v.qpos = nullptr;
+  v.qmap = nullptr; v.qpos = nullptr; v.vmeta = nullptr;
 }
 
 twkv_status twkv_cache_reset(twkv_cache* c, void* stream) {
@@ -586,6 +586,7 @@ static twkv_status decode_pass(twkv_cache* c, int layer, const void* q, const in
   maps.uinv_k = c->pool + c->off.prep_uinvT + (size_t)layer * c->dims.d_kv * c->dims.d_kv * 2;
   DevView v = c->view;
   v.qmap = qmap; v.qpos = qpos;
+  v.vmeta = c->kscore_pairs ? v.klist : v.kpairs;
   if (launch_decode(v, layer, c->params[layer], q, seq_ids, n_seq, out, num_splits, min_splits, c->sm_count, &maps, c->kscore_pairs,
                     (cudaStream_t)stream) != cudaSuccess) return TWKV_ERR_CUDA;
   return TWKV_OK;

@@ -54,8 +54,16 @@ __device__ void vsplit_plan(const DevView& v, int layer, const int* seq_ids, int
   const int4* desc = v.desc(layer, 1);
   int* cut = v.vcut + (size_t)qs * (n_splits + 1);
   const int stride = vtile_stride(n);
-  // cost of the i-th tile in stride order (its sum over a list stays below 2^31: 32 * 16 + 64 units, at most 2^13 tiles)
-  auto cost = [&](int i) -> int { return i < n ? 32 * desc[list[vtile_at(i, stride, n)]].y + v.Hq : 0; };
+  int4* meta = v.vmeta + (size_t)(n > 0 ? seq : 0) * v.TPS;
+  // cost of the i-th tile in stride order (its sum over a list stays below 2^31: 32 * 16 + 64 units, at most 2^13 tiles), whose
+  // description the V pass finds in that order
+  auto cost = [&](int i) -> int {
+    if (i >= n) return 0;
+    const int t = list[vtile_at(i, stride, n)];
+    const int4 d = desc[t];
+    meta[i] = make_int4(t, d.y, d.z, d.w);
+    return 32 * d.y + v.Hq;
+  };
   // a list of up to 1024 tiles is read once; a longer one first for its total
   const int first = cost(tid);
   int total = 0, w = first, off = 0;
@@ -605,7 +613,7 @@ merge_wide_kernel(DevView v, const unsigned short* Uinv_v, int n_splits, int n_s
 // ------------------------------------------------------------------------- host side
 cudaError_t launch_kscore_tc(const DevView& v, int layer, const CUtensorMap& map_blocks, const CUtensorMap& map_boxes, const CUtensorMap& map_uinvT,
                              const void* q, int n_pieces, bool pairs, cudaStream_t st);
-cudaError_t launch_vacc_tc(const DevView& v, int layer, const CUtensorMap& map_blocks, const CUtensorMap* map_scores, const int* seq_ids,
+cudaError_t launch_vacc_tc(const DevView& v, const CUtensorMap& map_blocks, const CUtensorMap* map_scores, const int* seq_ids,
                            int n_seq, int n_splits, cudaStream_t st);
 
 // Clusters of the merge kernel that are resident at once on an empty device (those of sixteen rows, which need the most).
@@ -646,7 +654,7 @@ static cudaError_t launch_decode_t(const DevView& v, int layer, const LayerParam
   }
   {
     ProfScope ps(TWKV_K_VACC, st);
-    cudaError_t e = launch_vacc_tc(v, layer, maps->blocks, maps->scores, seq_ids, n_seq, n_splits, st);
+    cudaError_t e = launch_vacc_tc(v, maps->blocks, maps->scores, seq_ids, n_seq, n_splits, st);
     if (e != cudaSuccess) return e;
   }
   {

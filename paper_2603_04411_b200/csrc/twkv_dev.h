@@ -71,6 +71,8 @@ struct DevView {
                              //       a joint tile: (~ its number, class | 128 << 8, 0, query slot)
   int4* kpairs;              // [NT + 64]  the same list as items of two tiles of one class (entries 2 i, 2 i + 1) for the CTA-pair kernel;
                              //            a class with an odd number of tiles ends with a filler entry (.y bit 7 set)
+  int4* vmeta;               // [NT]  V tiles of the current decode call, a sequence's from seq * TPS on in stride order: (tile, class, tokens, first block)
+                             //       (the region of the two above that the call's K list does not use)
   int* kitem_parts;          // [1]  parts the KV heads of a list item are dealt out in
   int* cta_start;            // [MAX_PLAN_CTAS + 1]  first item part of every K-score CTA (pair)
   int* kv_link;              // [NT * 128]  K slot -> V slot of the same token, for the sequences of the current decode pass (rebuilt by every pass)

@@ -71,7 +71,7 @@ __host__ __device__ constexpr uint32_t vt_idesc(int fmt, int n) { return idesc_f
 
 template <bool BF16, int N, bool TS>
 __global__ void __launch_bounds__(VT_THREADS, 1)
-vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_constant__ CUtensorMap map_scores, DevView v, int layer,
+vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_constant__ CUtensorMap map_scores, DevView v,
                const int* seq_ids, int n_splits) {
   chain_start();
   using C = VtCfg<BF16, N>;
@@ -125,14 +125,12 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
   chain_wait();
   const int seq = seq_ids[qs];
   const bool seq_ok = seq >= 0 && seq < v.S;
-  // this split's range of the sequence's V tile list in stride order, cut by plan_kernel to equal cost; an id outside
-  // the cache has no tiles and contributes nothing: zero partials
+  // this split's range of the sequence's V tiles in stride order, laid out and cut to equal cost by plan_kernel; an id outside
+  // the cache has no tiles and contributes nothing: zero partials.  (Walking the cache's own list here took two more dependent reads and
+  // the search for the stride: 2 us at the start of every CTA, 4 with 270 tiles per sequence, instead of 1.)
   const int* cut = v.vcut + (size_t)qs * (n_splits + 1) + split;
   const int t_first = cut[0], n_mine = seq_ok ? cut[1] - t_first : 0;
-  const int n_tiles = seq_ok ? v.svc(layer)[seq] : 0;
-  const int t_stride = vtile_stride(n_tiles);
-  const int* list = v.svt(layer) + (size_t)(seq_ok ? seq : 0) * v.TPS;
-  const int4* desc = v.desc(layer, 1);
+  const int4* meta = v.vmeta + (size_t)(seq_ok ? seq : 0) * v.TPS + t_first;
 
   // role state that survives the descriptor chunks
   uint32_t st = 0, st_ph = 0;                                   // producer / issuer: ring stage and its phase
@@ -158,11 +156,7 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
   for (int c0 = 0; c0 < n_mine; c0 += VT_META) {
     const int cn = min(VT_META, n_mine - c0);
     // descriptors of this chunk of the split's tiles
-    for (int i = tid; i < cn; i += VT_THREADS) {
-      const int t = list[vtile_at(t_first + c0 + i, t_stride, n_tiles)];
-      const int4 d = desc[t];
-      s_meta[i] = make_int4(t, d.y, d.z, d.w);
-    }
+    for (int i = tid; i < cn; i += VT_THREADS) s_meta[i] = meta[c0 + i];
     __syncthreads();
 
     if (warp == 0) {
@@ -408,7 +402,7 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
 }
 
 template <bool BF16, int N, bool TS>
-static cudaError_t launch_vacc_tc_n(const DevView& v, int layer, const CUtensorMap& map_blocks, const CUtensorMap& map_scores,
+static cudaError_t launch_vacc_tc_n(const DevView& v, const CUtensorMap& map_blocks, const CUtensorMap& map_scores,
                                     const int* seq_ids, int n_seq, int n_splits, cudaStream_t st) {
   using C = VtCfg<BF16, N>;
   static_assert(C::STAGES >= 3, "the ring needs a few stages");
@@ -417,18 +411,18 @@ static cudaError_t launch_vacc_tc_n(const DevView& v, int layer, const CUtensorM
   cudaError_t e = cudaFuncSetAttribute(vacc_tc_kernel<BF16, N, TS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM_BYTES);
   if (e != cudaSuccess) return e;
   const dim3 grid(n_seq * n_splits, (v.Hq + N - 1) / N);
-  e = launch_chained(vacc_tc_kernel<BF16, N, TS>, grid, dim3(VT_THREADS), dim3(1), C::SMEM_BYTES, st, map_blocks, map_scores, v, layer, seq_ids, n_splits);
+  e = launch_chained(vacc_tc_kernel<BF16, N, TS>, grid, dim3(VT_THREADS), dim3(1), C::SMEM_BYTES, st, map_blocks, map_scores, v, seq_ids, n_splits);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // map_scores: the score scratch as a tensor map (boxes of 128 rows x min(N, Hq) heads), or null: rows copied with cp.async.
-cudaError_t launch_vacc_tc(const DevView& v, int layer, const CUtensorMap& map_blocks, const CUtensorMap* map_scores, const int* seq_ids,
+cudaError_t launch_vacc_tc(const DevView& v, const CUtensorMap& map_blocks, const CUtensorMap* map_scores, const int* seq_ids,
                            int n_seq, int n_splits, cudaStream_t st) {
   const bool bf16 = v.dtype == TWKV_BF16;
   // up to 32 heads per CTA; more heads run as further CTAs that read the same panels (through L2)
 #define TWKV_VT(BF, NN)                                                                                                   \
-  (map_scores ? launch_vacc_tc_n<BF, NN, true>(v, layer, map_blocks, *map_scores, seq_ids, n_seq, n_splits, st)           \
-              : launch_vacc_tc_n<BF, NN, false>(v, layer, map_blocks, map_blocks, seq_ids, n_seq, n_splits, st))
+  (map_scores ? launch_vacc_tc_n<BF, NN, true>(v, map_blocks, *map_scores, seq_ids, n_seq, n_splits, st)           \
+              : launch_vacc_tc_n<BF, NN, false>(v, map_blocks, map_blocks, seq_ids, n_seq, n_splits, st))
   if (v.Hq <= 16) return bf16 ? TWKV_VT(true, 16) : TWKV_VT(false, 16);
   return bf16 ? TWKV_VT(true, 32) : TWKV_VT(false, 32);
 #undef TWKV_VT
