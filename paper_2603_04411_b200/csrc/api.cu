@@ -228,7 +228,7 @@ struct twkv_cache {
   std::vector<LayerParams> params;
   Prof prof;
   CUtensorMap map_blocks, map_boxes;   // the blocks as rows of one panel, boxes of a tile's rows / of a joint tile's sixteen
-  CUtensorMap map_scores;              // the score scratch as [V slot][Hq] fp32, boxes of one tile's rows x one V-pass CTA's heads
+  CUtensorMap map_scores, map_score_boxes;   // the score scratch as [V slot][Hq] fp32, boxes of one tile's rows (of sixteen) x one V-pass CTA's heads
   bool scores_tma = false;             // the head count allows that map (rows must start on 16-byte boundaries)
   std::vector<CUtensorMap> map_uinvT;  // per layer, over the transposed copy of U_K^-1 inside the pool
   std::vector<char> prepared;          // per layer: transposed copy and its map are current
@@ -400,7 +400,9 @@ twkv_status twkv_cache_create(const twkv_config* cfg, void* pool, size_t pool_by
       !make_tmap_2d(&c->map_boxes, c->view.blocks, (uint64_t)c->view.n_blocks * TILE, PANEL, PANEL * 2, JOINT_ROWS)) { delete c; return TWKV_ERR_CUDA; }
   if (c->cfg.n_q_heads % 4 == 0) {
     const int hq = c->cfg.n_q_heads, nb = hq < 16 ? hq : (hq <= 16 ? 16 : 32);
-    if (!make_tmap_2d_f32(&c->map_scores, c->view.scores, (uint64_t)c->dims.NT * TILE, (uint64_t)hq, TILE, (uint32_t)(nb < hq ? nb : hq))) { delete c; return TWKV_ERR_CUDA; }
+    const uint32_t cols = (uint32_t)(nb < hq ? nb : hq);
+    if (!make_tmap_2d_f32(&c->map_scores, c->view.scores, (uint64_t)c->dims.NT * TILE, (uint64_t)hq, TILE, cols) ||
+        !make_tmap_2d_f32(&c->map_score_boxes, c->view.scores, (uint64_t)c->dims.NT * TILE, (uint64_t)hq, JOINT_ROWS, cols)) { delete c; return TWKV_ERR_CUDA; }
     c->scores_tma = true;
   }
   {
@@ -582,6 +584,7 @@ static twkv_status decode_pass(twkv_cache* c, int layer, const void* q, const in
   maps.blocks = c->map_blocks;
   maps.boxes = c->map_boxes;
   maps.scores = c->scores_tma ? &c->map_scores : nullptr;
+  maps.score_boxes = c->scores_tma ? &c->map_score_boxes : nullptr;
   maps.uinvT_k = c->map_uinvT[layer];
   maps.uinv_k = c->pool + c->off.prep_uinvT + (size_t)layer * c->dims.d_kv * c->dims.d_kv * 2;
   DevView v = c->view;

@@ -38,7 +38,7 @@ __constant__ unsigned kTileCost[TWKV_MAX_CLASSES] = {14300u, 16600u, 18600u, 195
 __device__ __forceinline__ unsigned ktile_cost(int cls) { return kTileCost[min(max(cls, 1), TWKV_MAX_CLASSES) - 1]; }
 
 // Cut points of one sequence's V tile list into n_splits contiguous ranges of about equal cost (a tile costs its
-// panels plus its score rows, counted in 512-byte units): the V pass is bound by the bytes a CTA reads, and tiles of
+// panels' rows that hold tokens plus its score rows, counted in 512-byte units): the V pass is bound by the bytes a CTA reads, and tiles of
 // classes 1 to 16 dealt out by count alone left the slowest CTA with half as much again as the mean.
 // The list is taken in the stride order of vtile_stride(); cut[s] = number of tiles (in that order) whose inclusive cost
 // prefix is <= s / n_splits of the total; split s takes positions cut[s] .. cut[s + 1] - 1 of that order.
@@ -62,7 +62,7 @@ __device__ void vsplit_plan(const DevView& v, int layer, const int* seq_ids, int
     const int t = list[vtile_at(i, stride, n)];
     const int4 d = desc[t];
     meta[i] = make_int4(t, d.y, d.z, d.w);
-    return 32 * d.y + v.Hq;
+    return TILE / 32 * vtile_boxes(d.z) * d.y + v.Hq;
   };
   // a list of up to 1024 tiles is read once; a longer one first for its total
   const int first = cost(tid);
@@ -613,7 +613,7 @@ merge_wide_kernel(DevView v, const unsigned short* Uinv_v, int n_splits, int n_s
 // ------------------------------------------------------------------------- host side
 cudaError_t launch_kscore_tc(const DevView& v, int layer, const CUtensorMap& map_blocks, const CUtensorMap& map_boxes, const CUtensorMap& map_uinvT,
                              const void* q, int n_pieces, bool pairs, cudaStream_t st);
-cudaError_t launch_vacc_tc(const DevView& v, const CUtensorMap& map_blocks, const CUtensorMap* map_scores, const int* seq_ids,
+cudaError_t launch_vacc_tc(const DevView& v, const TcMaps& maps, const int* seq_ids,
                            int n_seq, int n_splits, cudaStream_t st);
 
 // Clusters of the merge kernel that are resident at once on an empty device (those of sixteen rows, which need the most).
@@ -654,7 +654,7 @@ static cudaError_t launch_decode_t(const DevView& v, int layer, const LayerParam
   }
   {
     ProfScope ps(TWKV_K_VACC, st);
-    cudaError_t e = launch_vacc_tc(v, maps->blocks, maps->scores, seq_ids, n_seq, n_splits, st);
+    cudaError_t e = launch_vacc_tc(v, *maps, seq_ids, n_seq, n_splits, st);
     if (e != cudaSuccess) return e;
   }
   {

@@ -19,6 +19,8 @@
 // reads as many bytes of scores as of values, and with one tile in flight their latency bound the kernel.  Where the
 // head count is not a multiple of four (rows not 16-byte aligned: no tensor map) each warp copies the rows of its own
 // token groups with cp.async instead (TS = false).
+// Of a tile that is less than half full (each class of a sequence ends with a partly full one) only the boxes of sixteen rows that hold
+// tokens are read, and the products run over as many tokens: a batch of short sequences is bound by the bytes of such tiles.
 // Weights go in as two parts of the cache type (see below): 2 N rows of one B operand, so that a panel is read once for both;
 // the two halves of the accumulator are added at the end.
 //
@@ -71,7 +73,8 @@ __host__ __device__ constexpr uint32_t vt_idesc(int fmt, int n) { return idesc_f
 
 template <bool BF16, int N, bool TS>
 __global__ void __launch_bounds__(VT_THREADS, 1)
-vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_constant__ CUtensorMap map_scores, DevView v,
+vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_constant__ CUtensorMap map_boxes,
+               const __grid_constant__ CUtensorMap map_scores, const __grid_constant__ CUtensorMap map_score_boxes, DevView v,
                const int* seq_ids, int n_splits) {
   chain_start();
   using C = VtCfg<BF16, N>;
@@ -167,8 +170,12 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
         auto score_box = [&](int i) -> bool {
           const uint32_t k = (uint32_t)(c0 + i), stg = k % VT_SC;
           if (!mbar_wait_thin(sc_empty + 8 * stg, ((k / VT_SC) & 1u) ^ 1u, abort_flag)) return false;
-          mbar_expect_tx(sc_full + 8 * stg, (uint32_t)(TILE * NB * 4));
-          tma_load_2d(sS + stg * C::SC_STAGE_BYTES, &map_scores, sc_full + 8 * stg, h0, s_meta[i].x * TILE);
+          const int nb = vtile_boxes(s_meta[i].z), row = s_meta[i].x * TILE;
+          mbar_expect_tx(sc_full + 8 * stg, (uint32_t)(nb * JOINT_ROWS * NB * 4));
+          if (nb == TILE / JOINT_ROWS) tma_load_2d(sS + stg * C::SC_STAGE_BYTES, &map_scores, sc_full + 8 * stg, h0, row);
+          else
+            for (int b = 0; b < nb; ++b)
+              tma_load_2d(sS + stg * C::SC_STAGE_BYTES + b * JOINT_ROWS * NB * 4, &map_score_boxes, sc_full + 8 * stg, h0, row + b * JOINT_ROWS);
           n_boxes = k + 1;
           return true;
         };
@@ -177,15 +184,25 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
         }
         for (int i = 0; i < cn && ok; ++i) {
           const int4 m = s_meta[i];
+          const int nb = vtile_boxes(m.z);
           if constexpr (TS) {
             if (i + 2 < cn && !(ok = score_box(i + 2))) break;
           }
           for (int j = 0; j < m.y; j += 2) {
             if (!(ok = mbar_wait_thin(empty + 8 * st, st_ph ^ 1u, abort_flag))) break;
             const bool two = j + 1 < m.y;
-            mbar_expect_tx(full + 8 * st, two ? VT_STAGE_BYTES : VT_PANEL_BYTES);
-            tma_load_2d(sRing + st * VT_STAGE_BYTES, &map_blocks, full + 8 * st, 0, (m.w + j) * TILE);
-            if (two) tma_load_2d(sRing + st * VT_STAGE_BYTES + VT_PANEL_BYTES, &map_blocks, full + 8 * st, 0, (m.w + j + 1) * TILE);
+            if (nb == TILE / JOINT_ROWS) {
+              mbar_expect_tx(full + 8 * st, two ? VT_STAGE_BYTES : VT_PANEL_BYTES);
+              tma_load_2d(sRing + st * VT_STAGE_BYTES, &map_blocks, full + 8 * st, 0, (m.w + j) * TILE);
+              if (two) tma_load_2d(sRing + st * VT_STAGE_BYTES + VT_PANEL_BYTES, &map_blocks, full + 8 * st, 0, (m.w + j + 1) * TILE);
+            } else {                                            // only the rows that hold tokens: the products go no further either
+              mbar_expect_tx(full + 8 * st, (uint32_t)((two ? 2 : 1) * nb * JOINT_ROWS * PANEL * 2));
+              for (int b = 0; b < nb; ++b) {
+                const uint32_t dst = sRing + st * VT_STAGE_BYTES + b * (JOINT_ROWS * PANEL * 2);
+                tma_load_2d(dst, &map_boxes, full + 8 * st, 0, (m.w + j) * TILE + b * JOINT_ROWS);
+                if (two) tma_load_2d(dst + VT_PANEL_BYTES, &map_boxes, full + 8 * st, 0, (m.w + j + 1) * TILE + b * JOINT_ROWS);
+              }
+            }
             ++n_loaded;
             if (++st == (uint32_t)S) { st = 0; st_ph ^= 1u; }
           }
@@ -208,7 +225,7 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
         constexpr uint32_t idesc = vt_idesc(BF16 ? 1 : 0, C::NB);
         for (int i = 0; i < cn && ok; ++i) {
           const int k = c0 + i;
-          const int cls = s_meta[i].y;
+          const int cls = s_meta[i].y, nb = vtile_boxes(s_meta[i].z);
           const uint32_t buf = (uint32_t)k & 1u;
           if (!(ok = mbar_wait_thin(p_full + 8 * buf, ((uint32_t)k >> 1) & 1u, abort_flag))) break;
           const uint32_t pb = sP + buf * C::P_BUF_BYTES;
@@ -219,8 +236,7 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
             const bool two = j + 1 < cls;
             const uint32_t pair = (uint32_t)j >> 1, d_tmem = tmem_base + pair * C::NB;
             uint32_t acc = (touched >> pair) & 1u;
-#pragma unroll
-            for (int ks = 0; ks < 8; ++ks) {
+            auto step = [&](int ks) {
               const uint32_t a_addr = a0 + ks * 2048u;                                     // 16 token rows per instruction
               const uint32_t lbo = two ? VT_PANEL_BYTES : sZero - a_addr;                 // where the second 64 columns are
               const uint32_t a_lo = ((a_addr >> 4) & 0x3fffu) | ((lbo >> 4) << 16);
@@ -228,6 +244,13 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
               const uint64_t ad = ((uint64_t)KMAJOR_SW128_DESC_HI << 32) | a_lo, bd = ((uint64_t)KMAJOR_SW128_DESC_HI << 32) | b_lo;
               mma_f16_ss(d_tmem, ad, bd, idesc, acc);
               acc = 1u;
+            };
+            if (nb == TILE / JOINT_ROWS) {                      // (a loop of its own: the checks would cost this thread its pace)
+#pragma unroll
+              for (int ks = 0; ks < 8; ++ks) step(ks);
+            } else {
+#pragma unroll 1
+              for (int ks = 0; ks < nb; ++ks) step(ks);
             }
             touched |= 1u << pair;
             mma_commit(empty + 8 * st);
@@ -305,6 +328,7 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
 #pragma unroll
         for (int it = 0; it < ITEMS; ++it) {
           const int tg = (it * VT_PTHREADS + pt) / N;
+          if (tg * 8 >= vtile_boxes(n_valid_i) * JOINT_ROWS) break;      // the products leave these rows out
           // Two weights at a time, packed: exp2 of one fused multiply-add, then the nearest value of the type and the rest.  bf16 keeps 8 bits of a weight, f16 11: with few tokens per sequence that rounding alone reaches 1e-3
           // and 1e-4 of the output, so the remainder goes into a second operand (16 and 22 bits in all).
           // Measured with both parts in one B operand: 64 heads bf16 over 131072 tokens 33.4 us (41.3 with two chains of products and
@@ -402,8 +426,7 @@ vacc_tc_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_cons
 }
 
 template <bool BF16, int N, bool TS>
-static cudaError_t launch_vacc_tc_n(const DevView& v, const CUtensorMap& map_blocks, const CUtensorMap& map_scores,
-                                    const int* seq_ids, int n_seq, int n_splits, cudaStream_t st) {
+static cudaError_t launch_vacc_tc_n(const DevView& v, const TcMaps& maps, const int* seq_ids, int n_seq, int n_splits, cudaStream_t st) {
   using C = VtCfg<BF16, N>;
   static_assert(C::STAGES >= 3, "the ring needs a few stages");
   static_assert(C::STAGES * VT_STAGE_BYTES >= (uint32_t)N * TWKV_MAX_CLASSES * PANEL * 4, "the partial sums leave through the ring's memory");
@@ -411,18 +434,17 @@ static cudaError_t launch_vacc_tc_n(const DevView& v, const CUtensorMap& map_blo
   cudaError_t e = cudaFuncSetAttribute(vacc_tc_kernel<BF16, N, TS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM_BYTES);
   if (e != cudaSuccess) return e;
   const dim3 grid(n_seq * n_splits, (v.Hq + N - 1) / N);
-  e = launch_chained(vacc_tc_kernel<BF16, N, TS>, grid, dim3(VT_THREADS), dim3(1), C::SMEM_BYTES, st, map_blocks, map_scores, v, seq_ids, n_splits);
+  e = launch_chained(vacc_tc_kernel<BF16, N, TS>, grid, dim3(VT_THREADS), dim3(1), C::SMEM_BYTES, st, maps.blocks, maps.boxes, TS ? *maps.scores : maps.blocks,
+                     TS ? *maps.score_boxes : maps.boxes, v, seq_ids, n_splits);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-// map_scores: the score scratch as a tensor map (boxes of 128 rows x min(N, Hq) heads), or null: rows copied with cp.async.
-cudaError_t launch_vacc_tc(const DevView& v, const CUtensorMap& map_blocks, const CUtensorMap* map_scores, const int* seq_ids,
-                           int n_seq, int n_splits, cudaStream_t st) {
+// maps.scores: the score scratch as a tensor map (boxes of 128 rows x min(N, Hq) heads), or null: rows copied with cp.async.
+cudaError_t launch_vacc_tc(const DevView& v, const TcMaps& maps, const int* seq_ids, int n_seq, int n_splits, cudaStream_t st) {
   const bool bf16 = v.dtype == TWKV_BF16;
   // up to 32 heads per CTA; more heads run as further CTAs that read the same panels (through L2)
 #define TWKV_VT(BF, NN)                                                                                                   \
-  (map_scores ? launch_vacc_tc_n<BF, NN, true>(v, map_blocks, *map_scores, seq_ids, n_seq, n_splits, st)           \
-              : launch_vacc_tc_n<BF, NN, false>(v, map_blocks, map_blocks, seq_ids, n_seq, n_splits, st))
+  (maps.scores ? launch_vacc_tc_n<BF, NN, true>(v, maps, seq_ids, n_seq, n_splits, st) : launch_vacc_tc_n<BF, NN, false>(v, maps, seq_ids, n_seq, n_splits, st))
   if (v.Hq <= 16) return bf16 ? TWKV_VT(true, 16) : TWKV_VT(false, 16);
   return bf16 ? TWKV_VT(true, 32) : TWKV_VT(false, 32);
 #undef TWKV_VT
