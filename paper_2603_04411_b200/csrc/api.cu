@@ -507,7 +507,10 @@ twkv_status twkv_compress(twkv_cache* c, int layer, const void* K, const void* V
   const size_t row = (size_t)v.d_kv * 2;
   if (is_capturing(st)) c->append_captured.store(true, std::memory_order_relaxed);
   c->appended[layer].fetch_add(n_tok, std::memory_order_relaxed);
-  if (mode == TWKV_GATE_LOGITS) {
+  const float* to_rank = nullptr;                          // logits of a call that is ranked where it is placed
+  if (mode == TWKV_GATE_LOGITS && n_tok <= CHUNK_TOKENS) {
+    to_rank = scores;
+  } else if (mode == TWKV_GATE_LOGITS) {
     if (launch_gate_rank(v, scores, levels, n_tok, st) != cudaSuccess) return TWKV_ERR_CUDA;
   } else if (mode == TWKV_GATE_COMPUTE && n_tok > GATE_LOGITS_TC_MAX && c->sm_count <= 160) {
     // fused tcgen05 kernel: logits and ranks in one launch, the logits never leave the CTA's staging block
@@ -538,14 +541,15 @@ twkv_status twkv_compress(twkv_cache* c, int layer, const void* K, const void* V
       const int n = n_tok - lo < GATE_PIECE ? n_tok - lo : GATE_PIECE;
       const twkv_status s = gate_logits(c, layer, (const unsigned char*)K + lo * row, (const unsigned char*)V + lo * row, n, st);
       if (s != TWKV_OK) return s;
-      if (launch_gate_rank(v, v.gate_scratch, levels + 2 * (size_t)lo, n, st) != cudaSuccess) return TWKV_ERR_CUDA;
+      if (n_tok <= CHUNK_TOKENS) to_rank = v.gate_scratch;
+      else if (launch_gate_rank(v, v.gate_scratch, levels + 2 * (size_t)lo, n, st) != cudaSuccess) return TWKV_ERR_CUDA;
     }
   }
   const int group = TWKV_PIECE_TOKENS * c->dims.batch;     // tokens whose pieces are handled by one set of launches
   for (int lo = 0; lo < n_tok; lo += group) {
     const int n = n_tok - lo < group ? n_tok - lo : group;
     if (launch_compress_pieces(v, layer, (const unsigned char*)K + lo * row, (const unsigned char*)V + lo * row, seq_ids + lo,
-                               positions + lo, n, levels + 2 * (size_t)lo, st) != cudaSuccess) return TWKV_ERR_CUDA;
+                               positions + lo, n, levels + 2 * (size_t)lo, to_rank, st) != cudaSuccess) return TWKV_ERR_CUDA;
   }
   return TWKV_OK;
 }

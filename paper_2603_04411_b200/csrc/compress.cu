@@ -7,6 +7,7 @@
 // packed bytes and tables are reproducible.
 #include "twkv_dev.h"
 #include "scan_util.cuh"
+#include "tc_util.cuh"
 
 namespace twkv {
 
@@ -17,15 +18,11 @@ namespace twkv {
 //   r = #{i : m_i > tau} = d - #{n : c_n <= tau} (Eq. 8).
 // The comparison c_n <= tau is done as S_n <= tau * S_d on the unnormalised sums.
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) gate_rank_kernel(const float* logits, unsigned short* levels, int n_rows, int d, float tau,
-                                                        int* status) {
-  chain_start();
-  chain_wait();
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+// Rank of one row of logits, by one warp (all lanes return it).
+__device__ __forceinline__ int gate_rank_row(const float* row, int d, float tau, int* status) {
   const int lane = threadIdx.x & 31;
-  if (warp >= n_rows) return;
   const int per = d >> 5;                       // 4 .. 32, multiple of 4
-  const float* z = logits + (size_t)warp * d + lane * per;
+  const float* z = row + lane * per;
   float v[32];
   float mx = -INFINITY;
 #pragma unroll
@@ -61,11 +58,19 @@ __global__ void __launch_bounds__(256) gate_rank_kernel(const float* logits, uns
   for (int o = 16; o > 0; o >>= 1) below += __shfl_xor_sync(0xffffffffu, below, o);
   int r = d - below;
   if (r < 1) r = 1;                             // only reachable with tau >= 1 or NaN logits
-  if (lane == 0) {
-    levels[warp] = (unsigned short)r;
-    // a row with a NaN or an infinite logit has no softmax: the rank above is a placeholder, the call reports it
-    if (status && !(total > 0.f && total < INFINITY)) atomicCAS(status, 0, TWKV_ERR_DEVICE_CHECK);
-  }
+  // a row with a NaN or an infinite logit has no softmax: the rank above is a placeholder, the call reports it
+  if (lane == 0 && status && !(total > 0.f && total < INFINITY)) atomicCAS(status, 0, TWKV_ERR_DEVICE_CHECK);
+  return r;
+}
+
+__global__ void __launch_bounds__(256) gate_rank_kernel(const float* logits, unsigned short* levels, int n_rows, int d, float tau,
+                                                        int* status) {
+  chain_start();
+  chain_wait();
+  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (warp >= n_rows) return;
+  const int r = gate_rank_row(logits + (size_t)warp * d, d, tau, status);
+  if ((threadIdx.x & 31) == 0) levels[warp] = (unsigned short)r;
 }
 
 cudaError_t launch_gate_rank(const DevView& v, const float* logits, unsigned short* levels, int n_tok, cudaStream_t st) {
@@ -143,167 +148,145 @@ __global__ void __launch_bounds__(256) scan_kernel(DevView v0, int n_pieces, int
 
 __device__ __forceinline__ int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
-// One CTA of 1024 threads, the pieces of the launch group one after the other.  Per piece: checks capacity and, if
-// the whole piece fits, creates the new tiles in ascending key order; a piece that does not fit (or holds an invalid
-// token) is refused whole and the later pieces carry on from the unchanged tables.
-// A call of at most one chunk (the decode-time append) skips the histogram and scan launches: `count_tok` > 0 makes
-// this kernel count the call's tokens per key itself (one piece, one chunk, so every per-chunk base is 0).
-__global__ void __launch_bounds__(1024) alloc_kernel(DevView v0, int layer, int n_pieces, const int* seq_ids, const int* positions,
-                                                     const unsigned short* levels, int count_tok) {
-  chain_start();
-  chain_wait();
+// Places one piece; one CTA of 1024 threads.  Checks capacity and, if the whole piece fits, creates the new tiles in ascending key
+// order; a piece that does not fit (or holds an invalid token) is refused whole and the tables stay as they are.
+__device__ void alloc_piece(const DevView& v, int layer) {
   __shared__ int s_warp[32];
   __shared__ int s_fail;
-  const int tid = threadIdx.x;
-  const int NK = v0.NK;
-  int* fill = v0.fill_l(layer);
-  int* key_last = v0.key_last_l(layer);
-  const int KPT = ceil_div(NK, 1024);
-  const int k0 = tid * KPT, k1 = min(NK, k0 + KPT);
-  const int half = v0.S * v0.NC;                      // keys per side
-  int* ntiles = v0.ntiles(layer);
-  int* stok = v0.stok(layer);
-  const int warp = tid >> 5, lane = tid & 31;
-  if (count_tok > 0) {
-    for (int k = k0; k < k1; ++k) v0.key_cnt[k] = 0;
-    if (tid < 2) v0.pflags[tid] = 0;
-    __syncthreads();
-    if (tid < count_tok) {
-      const int seq = seq_ids[tid], rk = levels[2 * tid], rv = levels[2 * tid + 1], pos = positions[tid];
-      if (seq < 0 || seq >= v0.S || rk < 1 || rk > v0.d_kv || rv < 1 || rv > v0.d_kv || pos < 0 || pos >= ROPE_LO * ROPE_HI) {
-        atomicOr(&v0.pflags[1], 1);
-      } else {
-        const int kk = key_of(v0, 0, seq, (rk + PANEL - 1) / PANEL), kv = key_of(v0, 1, seq, (rv + PANEL - 1) / PANEL);
-        atomicAdd(&v0.key_cnt[kk], 1);
-        atomicAdd(&v0.key_cnt[kv], 1);
-        v0.hist[(size_t)kk * PIECE_CHUNKS] = 0;                // the chunk's base inside the piece
-        v0.hist[(size_t)kv * PIECE_CHUNKS] = 0;
-      }
-    }
-    // the barrier at the top of the piece loop publishes the counts
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  int* fill = v.fill_l(layer);
+  int* key_last = v.key_last_l(layer);
+  const int KPT = ceil_div(v.NK, 1024);
+  const int k0 = tid * KPT, k1 = min(v.NK, k0 + KPT);
+  const int half = v.S * v.NC;                      // keys per side
+  int* ntiles = v.ntiles(layer);
+  int* stok = v.stok(layer);
+  if (tid == 0) s_fail = 0;
+  __syncthreads();                                   // also: the previous piece's table updates are visible
+  // (per-key counts and per-chunk bases come from scan_kernel)  new tiles / blocks per key, scanned in key order
+  int sum_tk = 0, sum_tv = 0, sum_b = 0;
+  for (int k = k0; k < k1; ++k) {
+    const int cnt = v.key_cnt[k], old = fill[k];
+    v.key_old_fill[k] = old;
+    const int nnew = ceil_div(old + cnt, TILE) - ceil_div(old, TILE);
+    if (k < half) sum_tk += nnew; else sum_tv += nnew;
+    sum_b += nnew * (k % v.NC + 1);
   }
-  for (int piece = 0; piece < n_pieces; ++piece) {
-    const DevView v = piece_view(v0, piece);
-    if (tid == 0) s_fail = 0;
-    __syncthreads();                                   // also: the previous piece's table updates are visible
-    // (per-key counts and per-chunk bases come from scan_kernel)  new tiles / blocks per key, scanned in key order
-    int sum_tk = 0, sum_tv = 0, sum_b = 0;
-    for (int k = k0; k < k1; ++k) {
-      const int cnt = v.key_cnt[k], old = fill[k];
-      v.key_old_fill[k] = old;
-      const int nnew = ceil_div(old + cnt, TILE) - ceil_div(old, TILE);
-      if (k < half) sum_tk += nnew; else sum_tv += nnew;
-      sum_b += nnew * (k % v.NC + 1);
-    }
-    int tot_tk, tot_tv, tot_b;
-    int off_tk = block_scan_excl(sum_tk, s_warp, &tot_tk), off_tv = block_scan_excl(sum_tv, s_warp, &tot_tv), off_b = block_scan_excl(sum_b, s_warp, &tot_b);
-    const int next_block = v.status[1];
-    const int ntk = ntiles[0], ntv = ntiles[1];
-    // capacity: tokens per sequence
-    for (int s = tid; s < v.S; s += 1024) {
-      int add = 0;
-      for (int c = 0; c < v.NC; ++c) add += v.key_cnt[s * v.NC + c];
-      if (stok[s] + add > v.tmax) atomicOr(&s_fail, 1);
-    }
+  int tot_tk, tot_tv, tot_b;
+  int off_tk = block_scan_excl(sum_tk, s_warp, &tot_tk), off_tv = block_scan_excl(sum_tv, s_warp, &tot_tv), off_b = block_scan_excl(sum_b, s_warp, &tot_b);
+  const int next_block = v.status[1];
+  const int ntk = ntiles[0], ntv = ntiles[1];
+  // capacity: tokens per sequence
+  for (int s = tid; s < v.S; s += 1024) {
+    int add = 0;
+    for (int c = 0; c < v.NC; ++c) add += v.key_cnt[s * v.NC + c];
+    if (stok[s] + add > v.tmax) atomicOr(&s_fail, 1);
+  }
+  if (tid == 0) {
+    if (next_block + tot_b > v.n_blocks || ntk + tot_tk > v.NT || ntv + tot_tv > v.NT) atomicOr(&s_fail, 1);
+    if (v.pflags[1]) atomicOr(&s_fail, 2);
+  }
+  __syncthreads();
+  if (s_fail) {
     if (tid == 0) {
-      if (next_block + tot_b > v.n_blocks || ntk + tot_tk > v.NT || ntv + tot_tv > v.NT) atomicOr(&s_fail, 1);
-      if (v.pflags[1]) atomicOr(&s_fail, 2);
+      v.pflags[0] = 0;
+      set_status(v, (s_fail & 2) ? TWKV_ERR_INVALID_ARG : TWKV_ERR_CAPACITY);
     }
-    __syncthreads();
-    if (s_fail) {
-      if (tid == 0) {
-        v.pflags[0] = 0;
-        set_status(v, (s_fail & 2) ? TWKV_ERR_INVALID_ARG : TWKV_ERR_CAPACITY);
-      }
-      __syncthreads();                                 // s_fail is reset at the top of the next round
-      continue;
+    __syncthreads();                                 // s_fail is reset for the next piece
+    return;
+  }
+  // commit
+  for (int k = k0; k < k1; ++k) {
+    const int cnt = v.key_cnt[k], old = v.key_old_fill[k];
+    const int side = k >= half ? 1 : 0;
+    const int cls = k % v.NC + 1;
+    const int seq = (k / v.NC) % v.S;
+    const int old_tiles = ceil_div(old, TILE);
+    const int nnew = ceil_div(old + cnt, TILE) - old_tiles;
+    const int first_id = (side ? ntv + off_tv : ntk + off_tk);
+    const int first_base = next_block + off_b;
+    v.key_first_id[k] = first_id;
+    v.key_first_base[k] = first_base;
+    v.key_old_last[k] = key_last[k];
+    if (cnt > 0) {
+      const int nf = old + cnt;
+      int4* desc = v.desc(layer, side);
+      if (old % TILE != 0) desc[key_last[k]].z = min(TILE, nf - (old_tiles - 1) * TILE);
+      for (int j = 0; j < nnew; ++j)
+        desc[first_id + j] = make_int4(seq, cls, min(TILE, nf - (old_tiles + j) * TILE), first_base + j * cls);
+      if (nnew > 0) key_last[k] = first_id + nnew - 1;
+      fill[k] = nf;
     }
-    // commit
-    for (int k = k0; k < k1; ++k) {
-      const int cnt = v.key_cnt[k], old = v.key_old_fill[k];
-      const int side = k >= half ? 1 : 0;
-      const int cls = k % v.NC + 1;
-      const int seq = (k / v.NC) % v.S;
-      const int old_tiles = ceil_div(old, TILE);
-      const int nnew = ceil_div(old + cnt, TILE) - old_tiles;
-      const int first_id = (side ? ntv + off_tv : ntk + off_tk);
-      const int first_base = next_block + off_b;
-      v.key_first_id[k] = first_id;
-      v.key_first_base[k] = first_base;
-      v.key_old_last[k] = key_last[k];
-      if (cnt > 0) {
-        const int nf = old + cnt;
-        int4* desc = v.desc(layer, side);
-        if (old % TILE != 0) desc[key_last[k]].z = min(TILE, nf - (old_tiles - 1) * TILE);
-        for (int j = 0; j < nnew; ++j)
-          desc[first_id + j] = make_int4(seq, cls, min(TILE, nf - (old_tiles + j) * TILE), first_base + j * cls);
-        if (nnew > 0) key_last[k] = first_id + nnew - 1;
-        fill[k] = nf;
-      }
-      if (side) off_tv += nnew; else off_tk += nnew;
-      off_b += nnew * cls;
-    }
-    __syncthreads();
-    // tile lists: K per class (ascending sequence), V per sequence (ascending class); one warp per list, one lane per
-    // key of the list: the lanes read their keys' tables together, a warp scan places their runs of tile ids
-    if (warp < v.NC) {
-      int* cnt = v.kcc(layer);
-      int* list = v.kct(layer) + (size_t)warp * v.NT;
-      int run = cnt[warp];
-      for (int s0 = 0; s0 < v.S; s0 += 32) {
-        const int s = s0 + lane;
-        int nnew = 0, first = 0;
-        if (s < v.S) {
-          const int k = s * v.NC + warp;
-          const int c = v.key_cnt[k], old = v.key_old_fill[k];
-          nnew = ceil_div(old + c, TILE) - ceil_div(old, TILE);
-          first = v.key_first_id[k];
-        }
-        int incl = nnew;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int u = __shfl_up_sync(0xffffffffu, incl, o);
-          if (lane >= o) incl += u;
-        }
-        int* dst = list + run + incl - nnew;
-        for (int j = 0; j < nnew; ++j) dst[j] = first + j;
-        run += __shfl_sync(0xffffffffu, incl, 31);
-      }
-      if (lane == 0) cnt[warp] = run;
-    }
-    for (int s = warp; s < v.S; s += 32) {
-      int* list = v.svt(layer) + (size_t)s * v.TPS;
-      const int run0 = v.svc(layer)[s];
-      int nnew = 0, first = 0, add = 0;
-      if (lane < v.NC) {
-        const int k = half + s * v.NC + lane;
-        const int cn = v.key_cnt[k], old = v.key_old_fill[k];
-        nnew = ceil_div(old + cn, TILE) - ceil_div(old, TILE);
+    if (side) off_tv += nnew; else off_tk += nnew;
+    off_b += nnew * cls;
+  }
+  __syncthreads();
+  // tile lists: K per class (ascending sequence), V per sequence (ascending class); one warp per list, one lane per
+  // key of the list: the lanes read their keys' tables together, a warp scan places their runs of tile ids
+  if (warp < v.NC) {
+    int* cnt = v.kcc(layer);
+    int* list = v.kct(layer) + (size_t)warp * v.NT;
+    int run = cnt[warp];
+    for (int s0 = 0; s0 < v.S; s0 += 32) {
+      const int s = s0 + lane;
+      int nnew = 0, first = 0;
+      if (s < v.S) {
+        const int k = s * v.NC + warp;
+        const int c = v.key_cnt[k], old = v.key_old_fill[k];
+        nnew = ceil_div(old + c, TILE) - ceil_div(old, TILE);
         first = v.key_first_id[k];
-        add = v.key_cnt[s * v.NC + lane];
       }
       int incl = nnew;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const int u = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += u;
-        add += __shfl_xor_sync(0xffffffffu, add, o);              // butterfly: every lane ends with the total
       }
-      int* dst = list + run0 + incl - nnew;
+      int* dst = list + run + incl - nnew;
       for (int j = 0; j < nnew; ++j) dst[j] = first + j;
-      if (lane == 31) {
-        v.svc(layer)[s] = run0 + incl;
-        stok[s] += add;
-      }
+      run += __shfl_sync(0xffffffffu, incl, 31);
     }
-    if (tid == 0) {
-      v.status[1] = next_block + tot_b;
-      ntiles[0] = ntk + tot_tk;
-      ntiles[1] = ntv + tot_tv;
-      v.pflags[0] = 1;
-    }
-    __syncthreads();
+    if (lane == 0) cnt[warp] = run;
   }
+  for (int s = warp; s < v.S; s += 32) {
+    int* list = v.svt(layer) + (size_t)s * v.TPS;
+    const int run0 = v.svc(layer)[s];
+    int nnew = 0, first = 0, add = 0;
+    if (lane < v.NC) {
+      const int k = half + s * v.NC + lane;
+      const int cn = v.key_cnt[k], old = v.key_old_fill[k];
+      nnew = ceil_div(old + cn, TILE) - ceil_div(old, TILE);
+      first = v.key_first_id[k];
+      add = v.key_cnt[s * v.NC + lane];
+    }
+    int incl = nnew;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
+      add += __shfl_xor_sync(0xffffffffu, add, o);              // butterfly: every lane ends with the total
+    }
+    int* dst = list + run0 + incl - nnew;
+    for (int j = 0; j < nnew; ++j) dst[j] = first + j;
+    if (lane == 31) {
+      v.svc(layer)[s] = run0 + incl;
+      stok[s] += add;
+    }
+  }
+  if (tid == 0) {
+    v.status[1] = next_block + tot_b;
+    ntiles[0] = ntk + tot_tk;
+    ntiles[1] = ntv + tot_tv;
+    v.pflags[0] = 1;
+  }
+  __syncthreads();
+}
+
+// One CTA, the pieces of the launch group one after the other (a refused one leaves the later ones to carry on).
+__global__ void __launch_bounds__(1024) alloc_kernel(DevView v, int layer, int n_pieces) {
+  chain_start();
+  chain_wait();
+  for (int piece = 0; piece < n_pieces; ++piece) alloc_piece(piece_view(v, piece), layer);
 }
 
 struct Place { int base, slot_cls_r; };   // slot | cls << 8 | r << 16
@@ -486,10 +469,150 @@ __global__ void __launch_bounds__(CHUNK_TOKENS, 7) pack_kernel(DevView v0, int l
   }
 }
 
+// A call of at most one chunk (the append of a decode step) in one kernel, a cluster of eight CTAs: ranks, a warp per row (logits
+// given), counts and allocation by one of the CTAs, then the rows' way into their slots by all.  What bounds such a call is the chain
+// of dependent reads and of kernel boundaries around them: rank, allocation and pack as kernels of their own took 5, 8 and 9 us.
+constexpr int AP_CL = 8;
+__global__ void __launch_bounds__(1024) append_kernel(DevView v, int layer, const void* K, const void* V, const int* seq_ids, const int* positions,
+                                                      unsigned short* levels, int n_tok, const float* logits) {
+  chain_start();
+  chain_wait();
+  const int part = tc::cluster_cta_rank(), tid = threadIdx.x;
+  if (logits) {
+    const int row = part * 32 + (tid >> 5);                // at most 256 rows
+    if (row < 2 * n_tok) {
+      const int r = gate_rank_row(logits + (size_t)row * v.d_kv, v.d_kv, v.tau, v.status);
+      if ((tid & 31) == 0) levels[row] = (unsigned short)r;
+    }
+    tc::cluster_sync_all();
+  }
+  int seq = 0, r[2] = {1, 1}, pos = 0;
+  const bool valid = tid < n_tok;
+  if (valid) { seq = seq_ids[tid]; r[0] = levels[2 * tid]; r[1] = levels[2 * tid + 1]; pos = positions[tid]; }
+  if (part == 0) {
+    for (int k = tid; k < v.NK; k += 1024) v.key_cnt[k] = 0;
+    if (tid < 2) v.pflags[tid] = 0;
+    __syncthreads();
+    if (valid) {
+      if (seq < 0 || seq >= v.S || r[0] < 1 || r[0] > v.d_kv || r[1] < 1 || r[1] > v.d_kv || pos < 0 || pos >= ROPE_LO * ROPE_HI) {
+        atomicOr(&v.pflags[1], 1);
+      } else {
+        for (int side = 0; side < 2; ++side) atomicAdd(&v.key_cnt[key_of(v, side, seq, (r[side] + PANEL - 1) / PANEL)], 1);
+      }
+    }
+    alloc_piece(v, layer);                                 // (its first barrier publishes the counts)
+  }
+  tc::cluster_sync_all();
+  if (v.pflags[0] == 0) return;                            // refused
+  __shared__ __align__(16) int s_key[2][CHUNK_TOKENS];
+  __shared__ Place s_place[2][CHUNK_TOKENS];
+  __shared__ int2 s_tail[2 * CHUNK_TOKENS];                // (first block, class | first slot to zero << 8) of tiles that end here
+  __shared__ unsigned short s_oct[2 * CHUNK_TOKENS * TWKV_MAX_CLASSES];        // (row << 4) | panel, as in pack_kernel
+  __shared__ int s_wtot[CHUNK_TOKENS / 32], s_total, s_tails;
+  __shared__ unsigned long long s_sum[2];
+  int key[2];
+  if (tid < CHUNK_TOKENS) {
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+      key[side] = valid ? key_of(v, side, seq, (r[side] + PANEL - 1) / PANEL) : -1 - side;
+      s_key[side][tid] = key[side];
+    }
+    if (tid < 2) s_sum[tid] = 0ull;
+    if (tid == 0) s_tails = 0;
+  }
+  __syncthreads();
+  int octs = 0, incl = 0;
+  if (tid < CHUNK_TOKENS) {
+    // tokens of the same key before this one: in earlier warps by four keys a read, in this warp by a match
+    int before[2] = {0, 0};
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+      for (int j = 0; j < (tid & ~31); j += 4) {
+        const int4 k = *reinterpret_cast<const int4*>(&s_key[side][j]);
+        before[side] += (k.x == key[side] ? 1 : 0) + (k.y == key[side] ? 1 : 0) + (k.z == key[side] ? 1 : 0) + (k.w == key[side] ? 1 : 0);
+      }
+      before[side] += __popc(__match_any_sync(0xffffffffu, key[side]) & ((1u << (tid & 31)) - 1u));
+    }
+    if (valid) {
+      int kslot = 0;
+#pragma unroll
+      for (int side = 0; side < 2; ++side) {
+        const int k = key[side], cls = k % v.NC + 1, old = v.key_old_fill[k], g = old + before[side];
+        const int ord = g / TILE, slot = g % TILE, old_tiles = ceil_div(old, TILE);
+        int tile, base;
+        if (ord >= old_tiles) {
+          tile = v.key_first_id[k] + (ord - old_tiles);
+          base = v.key_first_base[k] + (ord - old_tiles) * cls;
+          // the key's last token, in a tile of this call: the slots behind it are zeroed (decode reads whole tiles)
+          if (before[side] + 1 == v.key_cnt[k] && slot + 1 < TILE) s_tail[atomicAdd(&s_tails, 1)] = make_int2(base, cls | ((slot + 1) << 8));
+        } else {
+          tile = v.key_old_last[k];
+          base = v.desc(layer, side)[tile].w;
+        }
+        s_place[side][tid].base = base;
+        s_place[side][tid].slot_cls_r = slot | (cls << 8) | (r[side] << 16);
+        octs += cls;
+        if (part == 0) {
+          v.rank(layer, side)[(size_t)tile * TILE + slot] = (unsigned short)r[side];
+          v.aux(layer, side)[(size_t)tile * TILE + slot] = side == 0 ? pos : kslot;
+          atomicAdd(&s_sum[side], (unsigned long long)r[side]);
+        }
+        if (side == 0) kslot = tile * TILE + slot;
+      }
+    }
+    incl = octs;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int n = __shfl_up_sync(0xffffffffu, incl, o);
+      if ((tid & 31) >= o) incl += n;
+    }
+    if ((tid & 31) == 31) s_wtot[tid >> 5] = incl;
+  }
+  __syncthreads();
+  if (tid < CHUNK_TOKENS) {
+    for (int w = 0; w < (tid >> 5); ++w) incl += s_wtot[w];
+    int at = incl - octs;
+    if (valid)
+      for (int side = 0; side < 2; ++side)
+        for (int p = 0; p < ((s_place[side][tid].slot_cls_r >> 8) & 0xff); ++p) s_oct[at++] = (unsigned short)(((2 * tid + side) << 4) | p);
+    if (tid == CHUNK_TOKENS - 1) s_total = incl * 8;
+    if (part == 0 && tid < 2) atomicAdd(&v.rank_sums[layer * 2 + tid], s_sum[tid]);
+  }
+  __syncthreads();
+  // the rows as one list of 16-byte pieces over all threads of the cluster
+  const size_t row_bytes = (size_t)v.d_kv * 2;
+  for (int c = part * 1024 + tid; c < s_total; c += AP_CL * 1024) {
+    const int info = s_oct[c >> 3], t = info >> 5, side = (info >> 4) & 1, j = (info & 15) * 8 + (c & 7);
+    const Place p = s_place[side][t];
+    const int keep = (p.slot_cls_r >> 16) - j * 8;         // elements kept in this piece
+    uint4 o = make_uint4(0u, 0u, 0u, 0u);
+    if (keep > 0) o = reinterpret_cast<const uint4*>(reinterpret_cast<const unsigned char*>(side ? V : K) + (size_t)t * row_bytes)[j];
+    if (keep < 8) {
+      unsigned* w = reinterpret_cast<unsigned*>(&o);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int left = keep - 2 * q;
+        if (left <= 0) w[q] = 0u;
+        else if (left == 1) w[q] &= 0x0000ffffu;
+      }
+    }
+    *reinterpret_cast<uint4*>(v.blocks + (size_t)(p.base + (j >> 3)) * BLOCK_BYTES + (p.slot_cls_r & 0xff) * (PANEL * 2) + (j & 7) * 16) = o;
+  }
+  for (int e = 0; e < s_tails; ++e) {
+    const int2 tail = s_tail[e];
+    const int cls = tail.y & 0xff, first = tail.y >> 8, n16 = (TILE - first) * 8;
+    for (int i = part * 1024 + tid; i < n16 * cls; i += AP_CL * 1024) {
+      const int panel = i / n16;
+      reinterpret_cast<uint4*>(v.blocks + (size_t)(tail.x + panel) * BLOCK_BYTES + first * (PANEL * 2))[i - panel * n16] = make_uint4(0u, 0u, 0u, 0u);
+    }
+  }
+}
+
 // The pieces of up to v.batch * TWKV_PIECE_TOKENS tokens: one launch each of the histogram, the per-key scan, the
-// allocator (which takes the pieces in order) and the packer.
+// allocator (which takes the pieces in order) and the packer; calls of at most one chunk take append_kernel, which ranks the
+// tokens itself where `logits` are given (larger calls have been ranked).
 cudaError_t launch_compress_pieces(const DevView& v, int layer, const void* K, const void* V, const int* seq_ids,
-                                   const int* positions, int n_tok, const unsigned short* levels, cudaStream_t st) {
+                                   const int* positions, int n_tok, unsigned short* levels, const float* logits, cudaStream_t st) {
   if (n_tok <= 0) return cudaSuccess;
   const int n_chunks = (n_tok + CHUNK_TOKENS - 1) / CHUNK_TOKENS;
   const int n_pieces = (n_chunks + PIECE_CHUNKS - 1) / PIECE_CHUNKS;
@@ -504,15 +627,10 @@ cudaError_t launch_compress_pieces(const DevView& v, int layer, const void* K, c
   }
   // scan_kernel reads the counts four at a time; a launch group of several pieces clears its tables whole
   if (n_chunks == 1) {
-    // decode-time append: the allocator counts the tokens itself, two launches in all
-    { ProfScope ps(TWKV_K_ALLOC, st); e = launch_chained(alloc_kernel, dim3(1), dim3(1024), dim3(1), 0, st, v, layer, 1, seq_ids, positions, levels, n_tok); }
+    // decode-time append
+    { ProfScope ps(TWKV_K_PACK, st); e = launch_chained(append_kernel, dim3(AP_CL), dim3(1024), dim3(AP_CL), 0, st, v, layer, K, V, seq_ids, positions, levels, n_tok, logits); }
     if (e != cudaSuccess) return e;
-    {
-      ProfScope ps(TWKV_K_PACK, st);
-      e = launch_chained(pack_kernel, dim3(parts + v.NK), dim3(CHUNK_TOKENS), dim3(1), 0, st, v, layer, K, V, seq_ids, positions, levels, n_tok, parts);
-    }
-    if (e != cudaSuccess) return e;
-    count_launch(2);
+    count_launch();
     return cudaGetLastError();
   }
   const int n_cols = n_pieces > 1 ? PIECE_CHUNKS : (n_chunks + 3) & ~3;
@@ -525,8 +643,7 @@ cudaError_t launch_compress_pieces(const DevView& v, int layer, const void* K, c
     ProfScope ps(TWKV_K_ALLOC, st);
     e = launch_chained(scan_kernel, dim3((v.NK * n_pieces + 7) / 8), dim3(256), dim3(1), 0, st, v, n_pieces, n_chunks);
     if (e == cudaSuccess)
-      e = launch_chained(alloc_kernel, dim3(1), dim3(1024), dim3(1), 0, st, v, layer, n_pieces, (const int*)nullptr, (const int*)nullptr,
-                         (const unsigned short*)nullptr, 0);
+      e = launch_chained(alloc_kernel, dim3(1), dim3(1024), dim3(1), 0, st, v, layer, n_pieces);
     if (e != cudaSuccess) return e;
   }
   {

@@ -212,7 +212,7 @@ struct ProfScope {
 cudaError_t launch_rope_tables(const DevView& v, float rope_base, cudaStream_t st);
 cudaError_t launch_gate_rank(const DevView& v, const float* logits, unsigned short* levels, int n_tok, cudaStream_t st);
 cudaError_t launch_compress_pieces(const DevView& v, int layer, const void* K, const void* V, const int* seq_ids,
-                                  const int* positions, int n_tok, const unsigned short* levels, cudaStream_t st);
+                                  const int* positions, int n_tok, unsigned short* levels, const float* logits, cudaStream_t st);
 struct TcMaps;   // tensor maps of the K-score kernel (api.cu)
 cudaError_t launch_decode(const DevView& v, int layer, const LayerParams& lp, const void* q, const int* seq_ids,
                           int n_seq, void* out, int num_splits, int min_splits, int sm_count, const TcMaps* maps, bool pairs, cudaStream_t st);
