@@ -470,16 +470,17 @@ __global__ void __launch_bounds__(CHUNK_TOKENS, 7) pack_kernel(DevView v0, int l
 }
 
 // A call of at most one chunk (the append of a decode step) in one kernel, a cluster of eight CTAs: ranks, a warp per row (logits
-// given), counts and allocation by one of the CTAs, then the rows' way into their slots by all.  What bounds such a call is the chain
+// given), counts and allocation by one of the CTAs, then (`rows`) the rows' way into their slots by all.  What bounds such a call is the chain
 // of dependent reads and of kernel boundaries around them: rank, allocation and pack as kernels of their own took 5, 8 and 9 us.
 constexpr int AP_CL = 8;
+constexpr int APPEND_ROWS = 8;
 __global__ void __launch_bounds__(1024) append_kernel(DevView v, int layer, const void* K, const void* V, const int* seq_ids, const int* positions,
-                                                      unsigned short* levels, int n_tok, const float* logits) {
+                                                      unsigned short* levels, int n_tok, const float* logits, bool rows) {
   chain_start();
   chain_wait();
   const int part = tc::cluster_cta_rank(), tid = threadIdx.x;
   if (logits) {
-    const int row = part * 32 + (tid >> 5);                // at most 256 rows
+    const int row = (tid >> 5) * AP_CL + part;             // at most 256 rows, dealt out
     if (row < 2 * n_tok) {
       const int r = gate_rank_row(logits + (size_t)row * v.d_kv, v.d_kv, v.tau, v.status);
       if ((tid & 31) == 0) levels[row] = (unsigned short)r;
@@ -497,11 +498,16 @@ __global__ void __launch_bounds__(1024) append_kernel(DevView v, int layer, cons
       if (seq < 0 || seq >= v.S || r[0] < 1 || r[0] > v.d_kv || r[1] < 1 || r[1] > v.d_kv || pos < 0 || pos >= ROPE_LO * ROPE_HI) {
         atomicOr(&v.pflags[1], 1);
       } else {
-        for (int side = 0; side < 2; ++side) atomicAdd(&v.key_cnt[key_of(v, side, seq, (r[side] + PANEL - 1) / PANEL)], 1);
+        for (int side = 0; side < 2; ++side) {
+          const int k = key_of(v, side, seq, (r[side] + PANEL - 1) / PANEL);
+          atomicAdd(&v.key_cnt[k], 1);
+          v.hist[(size_t)k * PIECE_CHUNKS] = 0;            // the only chunk's base, for pack_kernel
+        }
       }
     }
     alloc_piece(v, layer);                                 // (its first barrier publishes the counts)
   }
+  if (!rows) return;
   tc::cluster_sync_all();
   if (v.pflags[0] == 0) return;                            // refused
   __shared__ __align__(16) int s_key[2][CHUNK_TOKENS];
@@ -627,10 +633,15 @@ cudaError_t launch_compress_pieces(const DevView& v, int layer, const void* K, c
   }
   // scan_kernel reads the counts four at a time; a launch group of several pieces clears its tables whole
   if (n_chunks == 1) {
-    // decode-time append
-    { ProfScope ps(TWKV_K_PACK, st); e = launch_chained(append_kernel, dim3(AP_CL), dim3(1024), dim3(AP_CL), 0, st, v, layer, K, V, seq_ids, positions, levels, n_tok, logits); }
+    // decode-time append; more rows than these are moved by more CTAs, and new tiles cleared by theirs
+    const bool rows = n_tok <= APPEND_ROWS;
+    { ProfScope ps(TWKV_K_ALLOC, st); e = launch_chained(append_kernel, dim3(AP_CL), dim3(1024), dim3(AP_CL), 0, st, v, layer, K, V, seq_ids, positions, levels, n_tok, logits, rows); }
+    if (e == cudaSuccess && !rows) {
+      ProfScope ps(TWKV_K_PACK, st);
+      e = launch_chained(pack_kernel, dim3(parts + v.NK), dim3(CHUNK_TOKENS), dim3(1), 0, st, v, layer, K, V, seq_ids, positions, levels, n_tok, parts);
+    }
     if (e != cudaSuccess) return e;
-    count_launch();
+    count_launch(rows ? 1 : 2);
     return cudaGetLastError();
   }
   const int n_cols = n_pieces > 1 ? PIECE_CHUNKS : (n_chunks + 3) & ~3;
