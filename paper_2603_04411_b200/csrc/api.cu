@@ -508,7 +508,7 @@ twkv_status twkv_compress(twkv_cache* c, int layer, const void* K, const void* V
   if (is_capturing(st)) c->append_captured.store(true, std::memory_order_relaxed);
   c->appended[layer].fetch_add(n_tok, std::memory_order_relaxed);
   const float* to_rank = nullptr;                          // logits of a call that is ranked where it is placed
-  if (mode == TWKV_GATE_LOGITS && n_tok <= CHUNK_TOKENS) {
+  if (mode == TWKV_GATE_LOGITS && n_tok <= APPEND_TOKENS) {
     to_rank = scores;
   } else if (mode == TWKV_GATE_LOGITS) {
     if (launch_gate_rank(v, scores, levels, n_tok, st) != cudaSuccess) return TWKV_ERR_CUDA;
@@ -541,7 +541,7 @@ twkv_status twkv_compress(twkv_cache* c, int layer, const void* K, const void* V
       const int n = n_tok - lo < GATE_PIECE ? n_tok - lo : GATE_PIECE;
       const twkv_status s = gate_logits(c, layer, (const unsigned char*)K + lo * row, (const unsigned char*)V + lo * row, n, st);
       if (s != TWKV_OK) return s;
-      if (n_tok <= CHUNK_TOKENS) to_rank = v.gate_scratch;
+      if (n_tok <= APPEND_TOKENS) to_rank = v.gate_scratch;
       else if (launch_gate_rank(v, v.gate_scratch, levels + 2 * (size_t)lo, n, st) != cudaSuccess) return TWKV_ERR_CUDA;
     }
   }

@@ -1,8 +1,9 @@
 // Compress step: gate -> rank (Eq. 5, 6, 8), slot allocation, truncate + pack (Eq. 2).
 //
-// A compress piece (<= TWKV_PIECE_TOKENS = 131072 tokens) runs as: hist (per-chunk key counts) -> alloc (one CTA:
-// exclusive scans, capacity check, tile and block allocation in ascending key order) -> pack
-// (warp per token: 128-bit loads / stores of the retained prefix, +0 fill to the class width).
+// A compress piece (<= TWKV_PIECE_TOKENS = 131072 tokens) runs as: hist (per-chunk key counts) -> scan (a warp per key: the counts
+// become bases) -> alloc (one CTA: exclusive scans, capacity check, tile and block allocation in ascending key order) -> pack
+// (128-bit loads / stores of the retained prefixes, +0 fill to the class width).  A call of at most one chunk (128 tokens) has no
+// histogram, the allocating CTA counts; one of at most 32 tokens is a single kernel behind the logits (append_kernel).
 // Slot assignment is a function of the token order only (no atomics decide placement), so the
 // packed bytes and tables are reproducible.
 #include "twkv_dev.h"
@@ -163,7 +164,7 @@ __device__ void alloc_piece(const DevView& v, int layer) {
   int* stok = v.stok(layer);
   if (tid == 0) s_fail = 0;
   __syncthreads();                                   // also: the previous piece's table updates are visible
-  // (per-key counts and per-chunk bases come from scan_kernel)  new tiles / blocks per key, scanned in key order
+  // (per-key counts and per-chunk bases come from scan_kernel, of a call of one chunk from count_token)  new tiles / blocks per key, scanned in key order
   int sum_tk = 0, sum_tv = 0, sum_b = 0;
   for (int k = k0; k < k1; ++k) {
     const int cnt = v.key_cnt[k], old = fill[k];
@@ -282,10 +283,35 @@ __device__ void alloc_piece(const DevView& v, int layer) {
   __syncthreads();
 }
 
-// One CTA, the pieces of the launch group one after the other (a refused one leaves the later ones to carry on).
-__global__ void __launch_bounds__(1024) alloc_kernel(DevView v, int layer, int n_pieces) {
+// The counts of a call of at most one chunk, which has no histogram, by the CTA that allocates (1024 threads, token tid of the call in
+// thread tid); alloc_piece's first barrier publishes them.
+__device__ __forceinline__ void clear_counts(const DevView& v) {
+  for (int k = threadIdx.x; k < v.NK; k += 1024) v.key_cnt[k] = 0;
+  if (threadIdx.x < 2) v.pflags[threadIdx.x] = 0;
+  __syncthreads();
+}
+__device__ __forceinline__ void count_token(const DevView& v, int seq, int rk, int rv, int pos, bool bases) {
+  if (seq < 0 || seq >= v.S || rk < 1 || rk > v.d_kv || rv < 1 || rv > v.d_kv || pos < 0 || pos >= ROPE_LO * ROPE_HI) {
+    atomicOr(&v.pflags[1], 1);
+    return;
+  }
+  const int kk = key_of(v, 0, seq, (rk + PANEL - 1) / PANEL), kv = key_of(v, 1, seq, (rv + PANEL - 1) / PANEL);
+  atomicAdd(&v.key_cnt[kk], 1);
+  atomicAdd(&v.key_cnt[kv], 1);
+  if (bases) v.hist[(size_t)kk * PIECE_CHUNKS] = v.hist[(size_t)kv * PIECE_CHUNKS] = 0;      // the only chunk's, for pack_kernel
+}
+
+// One CTA, the pieces of the launch group one after the other (a refused one leaves the later ones to carry on).  count_tok > 0: a call
+// of so many tokens that has had no histogram.
+__global__ void __launch_bounds__(1024) alloc_kernel(DevView v, int layer, int n_pieces, const int* seq_ids, const int* positions,
+                                                     const unsigned short* levels, int count_tok) {
   chain_start();
   chain_wait();
+  const int tid = threadIdx.x;
+  if (count_tok > 0) {
+    clear_counts(v);
+    if (tid < count_tok) count_token(v, seq_ids[tid], levels[2 * tid], levels[2 * tid + 1], positions[tid], true);
+  }
   for (int piece = 0; piece < n_pieces; ++piece) alloc_piece(piece_view(v, piece), layer);
 }
 
@@ -469,18 +495,24 @@ __global__ void __launch_bounds__(CHUNK_TOKENS, 7) pack_kernel(DevView v0, int l
   }
 }
 
-// A call of at most one chunk (the append of a decode step) in one kernel, a cluster of eight CTAs: ranks, a warp per row (logits
-// given), counts and allocation by one of the CTAs, then (`rows`) the rows' way into their slots by all.  What bounds such a call is the chain
-// of dependent reads and of kernel boundaries around them: rank, allocation and pack as kernels of their own took 5, 8 and 9 us.
+// A call of at most APPEND_TOKENS tokens (the append of a decode step) in one kernel, a cluster of eight CTAs: ranks, a warp per row
+// (where logits are given), counts and allocation by one of the CTAs, then the rows' way into their slots and the clearing of new
+// tiles' rests by all.  What bounds such a call is the chain of dependent reads and of kernel boundaries around them; with more
+// tokens the bytes that eight SMs can move do.  A compress call of n tokens with d_kv 1024 in us, separate kernels / this one (64 and
+// 128 in an eight-CTA form for 128 tokens):
+//   logits given  1 12.9/11.2  8 13.9/11.7  16 14.6/12.5  24 17.3/13.4  32 18.1/14.3  64 18.9/24.1  128 25.1/34.3
+//   ranks given   1 10.2/8.7   8 10.8/9.25  16 11.1/9.8   24 12.2/10.5  32 12.4/11.2  64 15.4/20.2  128 22.0/30.5
+// The slots and the zero fill follow pack_kernel's rules; sharing its code cost pack_kernel 0.1 us of 12 (its reads were ordered anew).
 constexpr int AP_CL = 8;
-constexpr int APPEND_ROWS = 8;
+static_assert(2 * APPEND_TOKENS <= AP_CL * 32, "a warp per row of logits");
+static_assert(APPEND_TOKENS <= 32, "one warp places the tokens");
 __global__ void __launch_bounds__(1024) append_kernel(DevView v, int layer, const void* K, const void* V, const int* seq_ids, const int* positions,
-                                                      unsigned short* levels, int n_tok, const float* logits, bool rows) {
+                                                      unsigned short* levels, int n_tok, const float* logits) {
   chain_start();
   chain_wait();
   const int part = tc::cluster_cta_rank(), tid = threadIdx.x;
   if (logits) {
-    const int row = (tid >> 5) * AP_CL + part;             // at most 256 rows, dealt out
+    const int row = (tid >> 5) * AP_CL + part;
     if (row < 2 * n_tok) {
       const int r = gate_rank_row(logits + (size_t)row * v.d_kv, v.d_kv, v.tau, v.status);
       if ((tid & 31) == 0) levels[row] = (unsigned short)r;
@@ -491,66 +523,33 @@ __global__ void __launch_bounds__(1024) append_kernel(DevView v, int layer, cons
   const bool valid = tid < n_tok;
   if (valid) { seq = seq_ids[tid]; r[0] = levels[2 * tid]; r[1] = levels[2 * tid + 1]; pos = positions[tid]; }
   if (part == 0) {
-    for (int k = tid; k < v.NK; k += 1024) v.key_cnt[k] = 0;
-    if (tid < 2) v.pflags[tid] = 0;
-    __syncthreads();
-    if (valid) {
-      if (seq < 0 || seq >= v.S || r[0] < 1 || r[0] > v.d_kv || r[1] < 1 || r[1] > v.d_kv || pos < 0 || pos >= ROPE_LO * ROPE_HI) {
-        atomicOr(&v.pflags[1], 1);
-      } else {
-        for (int side = 0; side < 2; ++side) {
-          const int k = key_of(v, side, seq, (r[side] + PANEL - 1) / PANEL);
-          atomicAdd(&v.key_cnt[k], 1);
-          v.hist[(size_t)k * PIECE_CHUNKS] = 0;            // the only chunk's base, for pack_kernel
-        }
-      }
-    }
-    alloc_piece(v, layer);                                 // (its first barrier publishes the counts)
+    clear_counts(v);
+    if (valid) count_token(v, seq, r[0], r[1], pos, false);
+    alloc_piece(v, layer);
   }
-  if (!rows) return;
   tc::cluster_sync_all();
   if (v.pflags[0] == 0) return;                            // refused
-  __shared__ __align__(16) int s_key[2][CHUNK_TOKENS];
-  __shared__ Place s_place[2][CHUNK_TOKENS];
-  __shared__ int2 s_tail[2 * CHUNK_TOKENS];                // (first block, class | first slot to zero << 8) of tiles that end here
-  __shared__ unsigned short s_oct[2 * CHUNK_TOKENS * TWKV_MAX_CLASSES];        // (row << 4) | panel, as in pack_kernel
-  __shared__ int s_wtot[CHUNK_TOKENS / 32], s_total, s_tails;
-  __shared__ unsigned long long s_sum[2];
-  int key[2];
-  if (tid < CHUNK_TOKENS) {
-#pragma unroll
-    for (int side = 0; side < 2; ++side) {
-      key[side] = valid ? key_of(v, side, seq, (r[side] + PANEL - 1) / PANEL) : -1 - side;
-      s_key[side][tid] = key[side];
-    }
-    if (tid < 2) s_sum[tid] = 0ull;
+  __shared__ Place s_place[2][APPEND_TOKENS];
+  __shared__ int2 s_tail[2 * APPEND_TOKENS];               // (first block, class | first slot to zero << 8) of tiles that end here
+  __shared__ unsigned short s_oct[2 * APPEND_TOKENS * TWKV_MAX_CLASSES];       // (row << 4) | panel, as in pack_kernel
+  __shared__ int s_octs, s_tails;                          // of the call: panel rows (eight pieces of 16 bytes each), tails
+  if (tid < 32) {
     if (tid == 0) s_tails = 0;
-  }
-  __syncthreads();
-  int octs = 0, incl = 0;
-  if (tid < CHUNK_TOKENS) {
-    // tokens of the same key before this one: in earlier warps by four keys a read, in this warp by a match
-    int before[2] = {0, 0};
+    __syncwarp();
+    int octs = 0, kslot = 0;
 #pragma unroll
     for (int side = 0; side < 2; ++side) {
-      for (int j = 0; j < (tid & ~31); j += 4) {
-        const int4 k = *reinterpret_cast<const int4*>(&s_key[side][j]);
-        before[side] += (k.x == key[side] ? 1 : 0) + (k.y == key[side] ? 1 : 0) + (k.z == key[side] ? 1 : 0) + (k.w == key[side] ? 1 : 0);
-      }
-      before[side] += __popc(__match_any_sync(0xffffffffu, key[side]) & ((1u << (tid & 31)) - 1u));
-    }
-    if (valid) {
-      int kslot = 0;
-#pragma unroll
-      for (int side = 0; side < 2; ++side) {
-        const int k = key[side], cls = k % v.NC + 1, old = v.key_old_fill[k], g = old + before[side];
+      const int k = valid ? key_of(v, side, seq, (r[side] + PANEL - 1) / PANEL) : -1;
+      const int before = __popc(__match_any_sync(0xffffffffu, k) & ((1u << tid) - 1u));     // tokens of the same key before this one
+      if (valid) {
+        const int cls = k % v.NC + 1, old = v.key_old_fill[k], g = old + before;
         const int ord = g / TILE, slot = g % TILE, old_tiles = ceil_div(old, TILE);
         int tile, base;
         if (ord >= old_tiles) {
           tile = v.key_first_id[k] + (ord - old_tiles);
           base = v.key_first_base[k] + (ord - old_tiles) * cls;
           // the key's last token, in a tile of this call: the slots behind it are zeroed (decode reads whole tiles)
-          if (before[side] + 1 == v.key_cnt[k] && slot + 1 < TILE) s_tail[atomicAdd(&s_tails, 1)] = make_int2(base, cls | ((slot + 1) << 8));
+          if (before + 1 == v.key_cnt[k] && slot + 1 < TILE) s_tail[atomicAdd(&s_tails, 1)] = make_int2(base, cls | ((slot + 1) << 8));
         } else {
           tile = v.key_old_last[k];
           base = v.desc(layer, side)[tile].w;
@@ -561,33 +560,28 @@ __global__ void __launch_bounds__(1024) append_kernel(DevView v, int layer, cons
         if (part == 0) {
           v.rank(layer, side)[(size_t)tile * TILE + slot] = (unsigned short)r[side];
           v.aux(layer, side)[(size_t)tile * TILE + slot] = side == 0 ? pos : kslot;
-          atomicAdd(&s_sum[side], (unsigned long long)r[side]);
         }
         if (side == 0) kslot = tile * TILE + slot;
       }
     }
-    incl = octs;
+    int incl = octs, sum_k = valid ? r[0] : 0, sum_v = valid ? r[1] : 0;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int n = __shfl_up_sync(0xffffffffu, incl, o);
-      if ((tid & 31) >= o) incl += n;
+      if (tid >= o) incl += n;
+      sum_k += __shfl_xor_sync(0xffffffffu, sum_k, o); sum_v += __shfl_xor_sync(0xffffffffu, sum_v, o);
     }
-    if ((tid & 31) == 31) s_wtot[tid >> 5] = incl;
-  }
-  __syncthreads();
-  if (tid < CHUNK_TOKENS) {
-    for (int w = 0; w < (tid >> 5); ++w) incl += s_wtot[w];
     int at = incl - octs;
     if (valid)
       for (int side = 0; side < 2; ++side)
         for (int p = 0; p < ((s_place[side][tid].slot_cls_r >> 8) & 0xff); ++p) s_oct[at++] = (unsigned short)(((2 * tid + side) << 4) | p);
-    if (tid == CHUNK_TOKENS - 1) s_total = incl * 8;
-    if (part == 0 && tid < 2) atomicAdd(&v.rank_sums[layer * 2 + tid], s_sum[tid]);
+    if (tid == 31) s_octs = incl;
+    if (part == 0 && tid < 2) atomicAdd(&v.rank_sums[layer * 2 + tid], (unsigned long long)(tid ? sum_v : sum_k));
   }
   __syncthreads();
   // the rows as one list of 16-byte pieces over all threads of the cluster
   const size_t row_bytes = (size_t)v.d_kv * 2;
-  for (int c = part * 1024 + tid; c < s_total; c += AP_CL * 1024) {
+  for (int c = part * 1024 + tid; c < 8 * s_octs; c += AP_CL * 1024) {
     const int info = s_oct[c >> 3], t = info >> 5, side = (info >> 4) & 1, j = (info & 15) * 8 + (c & 7);
     const Place p = s_place[side][t];
     const int keep = (p.slot_cls_r >> 16) - j * 8;         // elements kept in this piece
@@ -615,8 +609,8 @@ __global__ void __launch_bounds__(1024) append_kernel(DevView v, int layer, cons
 }
 
 // The pieces of up to v.batch * TWKV_PIECE_TOKENS tokens: one launch each of the histogram, the per-key scan, the
-// allocator (which takes the pieces in order) and the packer; calls of at most one chunk take append_kernel, which ranks the
-// tokens itself where `logits` are given (larger calls have been ranked).
+// allocator (which takes the pieces in order) and the packer, of a call of at most one chunk the last two.  Calls of at most
+// APPEND_TOKENS tokens take append_kernel, which ranks the tokens itself where `logits` are given (larger calls have been ranked).
 cudaError_t launch_compress_pieces(const DevView& v, int layer, const void* K, const void* V, const int* seq_ids,
                                    const int* positions, int n_tok, unsigned short* levels, const float* logits, cudaStream_t st) {
   if (n_tok <= 0) return cudaSuccess;
@@ -632,16 +626,22 @@ cudaError_t launch_compress_pieces(const DevView& v, int layer, const void* K, c
     while (2 * parts * n_chunks <= 7 * sms && 2 * parts <= rounds && parts < 32) parts *= 2;
   }
   // scan_kernel reads the counts four at a time; a launch group of several pieces clears its tables whole
+  if (n_tok <= APPEND_TOKENS) {
+    ProfScope ps(TWKV_K_ALLOC, st);
+    e = launch_chained(append_kernel, dim3(AP_CL), dim3(1024), dim3(AP_CL), 0, st, v, layer, K, V, seq_ids, positions, levels, n_tok, logits);
+    if (e != cudaSuccess) return e;
+    count_launch();
+    return cudaGetLastError();
+  }
   if (n_chunks == 1) {
-    // decode-time append; more rows than these are moved by more CTAs, and new tiles cleared by theirs
-    const bool rows = n_tok <= APPEND_ROWS;
-    { ProfScope ps(TWKV_K_ALLOC, st); e = launch_chained(append_kernel, dim3(AP_CL), dim3(1024), dim3(AP_CL), 0, st, v, layer, K, V, seq_ids, positions, levels, n_tok, logits, rows); }
-    if (e == cudaSuccess && !rows) {
+    { ProfScope ps(TWKV_K_ALLOC, st); e = launch_chained(alloc_kernel, dim3(1), dim3(1024), dim3(1), 0, st, v, layer, 1, seq_ids, positions, (const unsigned short*)levels, n_tok); }
+    if (e != cudaSuccess) return e;
+    {
       ProfScope ps(TWKV_K_PACK, st);
       e = launch_chained(pack_kernel, dim3(parts + v.NK), dim3(CHUNK_TOKENS), dim3(1), 0, st, v, layer, K, V, seq_ids, positions, levels, n_tok, parts);
     }
     if (e != cudaSuccess) return e;
-    count_launch(rows ? 1 : 2);
+    count_launch(2);
     return cudaGetLastError();
   }
   const int n_cols = n_pieces > 1 ? PIECE_CHUNKS : (n_chunks + 3) & ~3;
@@ -654,7 +654,8 @@ cudaError_t launch_compress_pieces(const DevView& v, int layer, const void* K, c
     ProfScope ps(TWKV_K_ALLOC, st);
     e = launch_chained(scan_kernel, dim3((v.NK * n_pieces + 7) / 8), dim3(256), dim3(1), 0, st, v, n_pieces, n_chunks);
     if (e == cudaSuccess)
-      e = launch_chained(alloc_kernel, dim3(1), dim3(1024), dim3(1), 0, st, v, layer, n_pieces);
+      e = launch_chained(alloc_kernel, dim3(1), dim3(1024), dim3(1), 0, st, v, layer, n_pieces, (const int*)nullptr, (const int*)nullptr,
+                         (const unsigned short*)nullptr, 0);
     if (e != cudaSuccess) return e;
   }
   {

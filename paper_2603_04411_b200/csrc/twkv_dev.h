@@ -19,6 +19,7 @@ constexpr int ROPE_HI = 32768;              // positions up to 16 * 32768 - 1
 constexpr int MAX_PARTIALS_EXTRA = 320;     // V-side partial slots beyond max_seqs
 constexpr int MAX_PLAN_CTAS = 1024;         // upper bound on the K-score kernel's grid
 constexpr int JOINT_ROWS = 16;              // rows of a box of a joint K tile, or of a partly full V tile
+constexpr int APPEND_TOKENS = 32;           // a compress call of at most this many tokens is one kernel behind its logits
 constexpr int DECODE_SPLIT_TOKENS = 512;    // tokens a V split is worth where the library chooses the number of splits
 constexpr unsigned long long TWKV_GUARD_WORD = 0x7477b2006b765f67ull;   // written behind every region of the pool
 
