@@ -225,6 +225,7 @@ struct twkv_cache {
   size_t pool_bytes;
   int device;
   int sm_count;
+  int merge_fit;                       // clusters of the decode merge that are resident at once on the device
   std::vector<LayerParams> params;
   Prof prof;
   CUtensorMap map_blocks, map_boxes;   // the blocks as rows of one panel, boxes of a tile's rows / of a joint tile's sixteen
@@ -378,6 +379,7 @@ twkv_status twkv_cache_create(const twkv_config* cfg, void* pool, size_t pool_by
   if (!g.ok) { delete c; return TWKV_ERR_CUDA; }
   if (cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) { delete c; return TWKV_ERR_CUDA; }
   if (c->sm_count > MAX_PLAN_CTAS) c->sm_count = MAX_PLAN_CTAS;
+  c->merge_fit = merge_clusters(cfg->dtype == TWKV_BF16, c->sm_count);
   {
     // TWKV_KSCORE_SINGLE=1 keeps the K-score kernel on single CTAs (the fallback where CTA pairs cannot be scheduled)
     const char* single = getenv("TWKV_KSCORE_SINGLE");
@@ -594,7 +596,7 @@ static twkv_status decode_pass(twkv_cache* c, int layer, const void* q, const in
   DevView v = c->view;
   v.qmap = qmap; v.qpos = qpos;
   v.vmeta = c->kscore_pairs ? v.klist : v.kpairs;
-  if (launch_decode(v, layer, c->params[layer], q, seq_ids, n_seq, out, num_splits, min_splits, c->sm_count, &maps, c->kscore_pairs,
+  if (launch_decode(v, layer, c->params[layer], q, seq_ids, n_seq, out, num_splits, min_splits, c->sm_count, c->merge_fit, &maps, c->kscore_pairs,
                     (cudaStream_t)stream) != cudaSuccess) return TWKV_ERR_CUDA;
   return TWKV_OK;
 }

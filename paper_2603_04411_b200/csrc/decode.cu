@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(1024) plan_kernel(DevView v, int layer, const 
 // adds the eight parts of its own.  What bounds it is latency: one CTA doing a group's whole sum and product went
 // through 256 KiB of U_V^-1 and every split by itself.  Empty splits are not read (the V pass does not write them).
 // A cluster of four rows takes 6 us, one of sixteen 15 (its share of the splits, then the FMAs: 67 M of them for 512 rows), so all
-// of them are to be resident at once (merge_fit(), below), three CTAs per SM: U_V^-1 waits in shared memory, not in registers.
+// of them are to be resident at once (merge_rows(), below), three CTAs per SM: U_V^-1 waits in shared memory, not in registers.
 // 4 sequences of 1000 tokens ran as 512 CTAs in three rounds, 17 us.  A whole call in us, two CTAs per SM / three: 1 x 300
 // 40.1 / 36.7, 4 x 1000 48.4 / 44.7, 4 x 8192 65.2 / 61.0, 8 x 5000 80.4 / 74.3, 16 x 500 91.2 / 82.7, 2 x 2000 with 64 heads
 // 45.9 / 42.1, 1 x 131072 with 64 heads 145.9 / 140.5; more CTAs than fit and as many rows as fit, two per SM: 4 x 1000 57.0 / 51.0.
@@ -616,28 +616,37 @@ cudaError_t launch_kscore_tc(const DevView& v, int layer, const CUtensorMap& map
 cudaError_t launch_vacc_tc(const DevView& v, const TcMaps& maps, const int* seq_ids,
                            int n_seq, int n_splits, cudaStream_t st);
 
-// Clusters of the merge kernel that are resident at once on an empty device (those of sixteen rows, which need the most).
+// Clusters of the merge kernel that are resident at once on the current device, empty (those of sixteen rows, which need the most).
 template <bool BF16>
-static int merge_fit(int sm_count) {
-  static const int cached = [sm_count] {
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = MG_CL; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(MG_CL); cfg.blockDim = dim3(MG_THREADS); cfg.dynamicSmemBytes = merge_smem(16);
-    cfg.attrs = &attr; cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaFuncSetAttribute(merge_kernel<BF16, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)merge_smem(16)) != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&n, merge_kernel<BF16, 16>, &cfg) != cudaSuccess || n < 1) { cudaGetLastError(); n = sm_count / MG_CL; }
-    return n - n / 16;                                   // behind another kernel not quite as many find room together
-  }();
-  return cached;
+static int merge_clusters_t(int sm_count) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = MG_CL; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(MG_CL); cfg.blockDim = dim3(MG_THREADS); cfg.dynamicSmemBytes = merge_smem(16);
+  cfg.attrs = &attr; cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaFuncSetAttribute(merge_kernel<BF16, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)merge_smem(16)) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, merge_kernel<BF16, 16>, &cfg) != cudaSuccess || n < 1) { cudaGetLastError(); n = sm_count / MG_CL; }
+  return n - n / 16;                                     // behind another kernel not quite as many find room together
+}
+int merge_clusters(bool bf16, int sm_count) { return bf16 ? merge_clusters_t<true>(sm_count) : merge_clusters_t<false>(sm_count); }
+
+// Rows (query slot, query head of a KV head) per cluster of the merge, hp heads of ns slots: as few as still leave all clusters
+// resident at once (a second round of clusters starts when the first has ended); query heads of one slot first, then slots.  False
+// where sixteen rows are not enough: rows of 32 (merge_wide_kernel).
+bool merge_rows(int n_seq, int n_kv_heads, int rep, int fit, int* hp, int* ns) {
+  *hp = *ns = 1;
+  auto clusters = [&] { return (n_seq + *ns - 1) / *ns * n_kv_heads * (rep / *hp); };
+  while (*hp < rep && clusters() > fit) *hp *= 2;
+  while (2 * *hp * *ns <= 16 && *ns < n_seq && clusters() > fit) *ns *= 2;
+  return clusters() <= fit;
 }
 
 template <bool BF16>
 static cudaError_t launch_decode_t(const DevView& v, int layer, const LayerParams& lp, const void* q, const int* seq_ids,
-                                   int n_seq, void* out, int n_splits, int min_splits, int sm_count, const TcMaps* maps, bool pairs,
-                                   cudaStream_t st) {
+                                   int n_seq, void* out, int n_splits, int min_splits, int sm_count, int merge_fit, const TcMaps* maps,
+                                   bool pairs, cudaStream_t st) {
   // the K-score kernel's work is cut into one piece per persistent CTA, or per CTA pair
   const int n_pieces = pairs ? kscore_max_pairs(sm_count) : sm_count;
   // CTAs per sequence that invert the V -> K links: enough of them that they finish inside the K work list's time
@@ -662,14 +671,8 @@ static cudaError_t launch_decode_t(const DevView& v, int layer, const LayerParam
     const unsigned short* uv = reinterpret_cast<const unsigned short*>(lp.Uinv_v);
     const int wide = (n_seq * v.rep + MW_ROWS - 1) / MW_ROWS;
     cudaError_t e;
-    // Rows per cluster: as few as still leave all clusters resident at once (a second round of clusters starts when the first has
-    // ended); query heads of one slot first, then slots; 32 rows where sixteen are not enough.
-    const int fit = merge_fit<BF16>(sm_count);
-    int hp = 1, ns = 1;
-    auto clusters = [&] { return (n_seq + ns - 1) / ns * v.Hkv * (v.rep / hp); };
-    while (hp < v.rep && clusters() > fit) hp *= 2;
-    while (2 * hp * ns <= 16 && ns < n_seq && clusters() > fit) ns *= 2;
-    if (clusters() > fit) {
+    int hp, ns;
+    if (!merge_rows(n_seq, v.Hkv, v.rep, merge_fit, &hp, &ns)) {
       e = cudaFuncSetAttribute(merge_wide_kernel<BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, MW_SMEM);
       if (e == cudaSuccess) e = launch_chained(merge_wide_kernel<BF16>, dim3(MG_CL * wide, v.Hkv), dim3(MG_THREADS), dim3(MG_CL), MW_SMEM, st, v, uv, n_splits, n_seq, out);
     } else {
@@ -687,10 +690,10 @@ static cudaError_t launch_decode_t(const DevView& v, int layer, const LayerParam
 }
 
 cudaError_t launch_decode(const DevView& v, int layer, const LayerParams& lp, const void* q, const int* seq_ids,
-                          int n_seq, void* out, int num_splits, int min_splits, int sm_count, const TcMaps* maps, bool pairs, cudaStream_t st) {
+                          int n_seq, void* out, int num_splits, int min_splits, int sm_count, int merge_fit, const TcMaps* maps, bool pairs, cudaStream_t st) {
   if (n_seq <= 0) return cudaSuccess;
-  return v.dtype == TWKV_BF16 ? launch_decode_t<true>(v, layer, lp, q, seq_ids, n_seq, out, num_splits, min_splits, sm_count, maps, pairs, st)
-                              : launch_decode_t<false>(v, layer, lp, q, seq_ids, n_seq, out, num_splits, min_splits, sm_count, maps, pairs, st);
+  return v.dtype == TWKV_BF16 ? launch_decode_t<true>(v, layer, lp, q, seq_ids, n_seq, out, num_splits, min_splits, sm_count, merge_fit, maps, pairs, st)
+                              : launch_decode_t<false>(v, layer, lp, q, seq_ids, n_seq, out, num_splits, min_splits, sm_count, merge_fit, maps, pairs, st);
 }
 
 }  // namespace twkv

@@ -216,7 +216,8 @@ cudaError_t launch_compress_pieces(const DevView& v, int layer, const void* K, c
                                   const int* positions, int n_tok, unsigned short* levels, const float* logits, cudaStream_t st);
 struct TcMaps;   // tensor maps of the K-score kernel (api.cu)
 cudaError_t launch_decode(const DevView& v, int layer, const LayerParams& lp, const void* q, const int* seq_ids,
-                          int n_seq, void* out, int num_splits, int min_splits, int sm_count, const TcMaps* maps, bool pairs, cudaStream_t st);
+                          int n_seq, void* out, int num_splits, int min_splits, int sm_count, int merge_fit, const TcMaps* maps, bool pairs, cudaStream_t st);
+int merge_clusters(bool bf16, int sm_count);
 struct GateMaps;   // tensor maps of the fused gate kernel (api.cu)
 cudaError_t launch_gate_ranks_tc(const DevView& v, const GateMaps& maps, const LayerParams& lp, int n_tok, unsigned short* levels,
                                  int sm_count, bool pairs, cudaStream_t st);

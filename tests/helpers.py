@@ -1,5 +1,7 @@
 """Shared machinery of the GPU parity tests: run libtwkv through its C ABI, read its tables
 back, and compare with the CPU oracle on the same buffers."""
+import ctypes
+
 import numpy as np
 import torch
 
@@ -143,3 +145,11 @@ def attn_errors(got, want):
     max_abs = float(np.max(np.abs(got - want)))
     rel_l2 = float(np.linalg.norm(got - want) / max(np.linalg.norm(want), 1e-300))
     return max_abs, rel_l2
+
+
+def merge_variant(B, n_seq, n_kv_heads, rep, fit):
+    """Rows per cluster that the decode merge takes where `fit` of its clusters are resident at once (32: the wide kernel)."""
+    hp, ns = ctypes.c_int(), ctypes.c_int()
+    rule = B.lib._ZN4twkv10merge_rowsEiiiiPiS0_                     # twkv::merge_rows, inside the library
+    rule.restype, rule.argtypes = ctypes.c_bool, [ctypes.c_int] * 4 + [ctypes.POINTER(ctypes.c_int)] * 2
+    return hp.value * ns.value if rule(n_seq, n_kv_heads, rep, fit, ctypes.byref(hp), ctypes.byref(ns)) else 32

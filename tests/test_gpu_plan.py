@@ -5,7 +5,7 @@ import pytest
 import torch
 
 from paper_2603_04411_b200 import workloads
-from tests.helpers import GpuCache, attn_errors, oracle_decode
+from tests.helpers import GpuCache, attn_errors, merge_variant, oracle_decode
 
 pytestmark = pytest.mark.gpu
 
@@ -42,24 +42,38 @@ def test_decode_where_the_work_split_changes(hkv, rep, n_seq, ctx, recipe, pick)
 
 
 @pytest.mark.parametrize("hkv,rep,n_seq,ctx", [
-    (8, 8, 13, 40),             # 64 query heads: the last cluster of the wide merge holds two sequences of four
-    (1, 8, 33, 40),             # one KV head: wide from a few clusters on, one sequence in the last
-    (1, 4, 35, 30),
-    (4, 4, 47, 20),
-    (8, 4, 23, 30),             # just below: eight rows per cluster
+    (8, 8, 13, 40), (1, 8, 33, 40), (1, 4, 35, 30), (4, 4, 47, 20), (8, 4, 23, 30),
 ])
 def test_merge_of_medium_batches(hkv, rep, n_seq, ctx):
     test_decode_where_the_work_split_changes(hkv, rep, n_seq, ctx, "any", list(range(n_seq)))
 
 
-@pytest.mark.parametrize("hkv,rep,n_seq,ctx", [
-    (8, 4, 9, 60),              # sixteen rows per cluster: four sequences, the last cluster holds one
-    (8, 1, 10, 40),             # the same of one head each
-    (8, 8, 3, 60),              # eight rows: one sequence's group
-    (2, 8, 20, 30),             # sixteen rows of two groups, 32 spectral components per CTA
-    (1, 2, 3, 50),              # one row, 16 components
-])
+@pytest.mark.parametrize("hkv,rep,n_seq,ctx", [(8, 4, 9, 60), (8, 1, 10, 40), (8, 8, 3, 60), (2, 8, 20, 30), (1, 2, 3, 50)])
 def test_merge_rows_per_cluster(hkv, rep, n_seq, ctx):
+    test_decode_where_the_work_split_changes(hkv, rep, n_seq, ctx, "any", list(range(n_seq)))
+
+
+@pytest.mark.parametrize("rows,hkv,rep,n_seq,ctx", [
+    (1, 1, 2, 3, 50),           # 16 spectral components per CTA
+    (2, 8, 1, 10, 40),          # two slots
+    (4, 8, 4, 5, 60),           # the heads of one slot
+    (8, 8, 8, 4, 60),           # eight of them
+    (8, 8, 4, 9, 60),           # two slots, one in the last cluster
+    (16, 8, 4, 15, 30),         # four slots, three in the last cluster
+    (16, 2, 8, 37, 30),         # two slots, one in the last cluster; 32 spectral components
+    (16, 8, 1, 70, 20),         # sixteen slots, six in the last cluster
+    (32, 8, 8, 15, 40),         # wide: four slots, three in the last cluster
+    (32, 4, 4, 59, 20),         # eight slots, three in the last; 64 spectral components
+    (32, 1, 8, 117, 20),        # one KV head, 16 spectral components
+    (32, 1, 4, 227, 12),
+])
+def test_every_form_of_the_merge(rows, hkv, rep, n_seq, ctx):
+    """The sizes are well inside their form on a device of 148 SMs; the form itself is asked of the library's rule."""
+    from paper_2603_04411_b200 import build
+    build.build()
+    from paper_2603_04411_b200 import binding as B
+    fit = B.lib._ZN4twkv14merge_clustersEbi(False, torch.cuda.get_device_properties(0).multi_processor_count)    # twkv::merge_clusters
+    assert merge_variant(B, n_seq, hkv, rep, fit) == rows, fit
     test_decode_where_the_work_split_changes(hkv, rep, n_seq, ctx, "any", list(range(n_seq)))
 
 
