@@ -134,3 +134,55 @@ def test_joint_tiles_of_partly_full_classes(hkv, single, counts, monkeypatch):
     B.twkv_evict(gc.h, 0, 0, torch.from_numpy(keep.astype(np.int32)).cuda())
     check(((first | then) & (seq > 0)) | ((seq == 0) & np.isin(pos, keep)), [0, 1])
     gc.close()
+
+
+@pytest.mark.parametrize("counts,single", [
+    ({16: 16, 8: 64, 3: 32}, False),         # a pass of its own for the panels above the eighth
+    ({8: 30, 2: 17, 1: 33}, False),
+    ({12: 1, 11: 15, 9: 16, 4: 70}, True),
+])
+def test_joint_rows_score_as_in_tiles_of_their_own(counts, single, monkeypatch):
+    """The same tokens decoded twice, their K rows in one joint tile and in a full tile per class: the tokens that fill the tiles up score
+    so low that their weights are zero, and all weight lies in one V tile, so that the outputs are equal bit for bit if the scores are."""
+    from paper_2603_04411_b200 import build
+    build.build()
+    from paper_2603_04411_b200 import binding as B
+    if single:
+        monkeypatch.setenv("TWKV_KSCORE_SINGLE", "1")
+    heads, d, pos_fill = 8, 1024, 1000
+    g = torch.Generator().manual_seed(sum(counts))
+    n = sum(counts.values())
+    assert sum(-(-c // 16) for c in counts.values()) <= 8
+    uinv = torch.linalg.qr(torch.randn(d, d, generator=g))[0].half().contiguous()
+    q = torch.randn(heads, 128, generator=g).half()
+    classes = torch.tensor([c for c, m in counts.items() for _ in range(m)])[torch.randperm(n, generator=g)]
+    x = torch.randn(2, n, d, generator=g).half()
+    # a filler of rank r: minus the query, rotated back from the filler's position, projected on the r leading axes
+    theta = pos_fill * 500000.0 ** (-torch.arange(64, dtype=torch.float64) / 64)
+    lo, hi = q[:, :64].double(), q[:, 64:].double()
+    back = torch.cat([lo * theta.cos() + hi * theta.sin(), hi * theta.cos() - lo * theta.sin()], 1)
+    fill_x = (-600.0 * (uinv.double() @ back.reshape(d))).half()
+    fill_classes = torch.tensor([c for c, m in counts.items() for _ in range(128 - m)])
+    for c in counts:
+        k = (fill_x[:64 * c].double() @ uinv[:64 * c].double()).reshape(heads, 128)
+        assert ((k * back).sum(1) * 128 ** -0.5).max() < -150         # 87 below a sequence's maximum and a weight is less than 2^-126: zero
+
+    def decode(filled):
+        m = len(fill_classes) if filled else 0
+        xk, xv = torch.cat([x[0], fill_x.expand(m, d)]), torch.cat([x[1], torch.zeros(m, d).half()])
+        rk = torch.cat([classes, fill_classes[:m]]) * 64
+        rv = torch.cat([torch.full((n,), 320), torch.full((m,), 64)])             # the tokens in a V tile of class 5, the fillers in others
+        gc = GpuCache(B, n_layers=1, n_q_heads=heads, n_kv_heads=heads, dtype=torch.float16, out_dtype=torch.float32, max_seqs=1,
+                      max_tokens_per_seq=2048, payload_bytes=(n + m) * 4 * d)
+        u = uinv.cuda()
+        B.twkv_cache_set_layer_params(gc.h, 0, u, u)
+        pos = torch.cat([torch.arange(n), torch.full((m,), pos_fill)]).to(torch.int32).cuda()
+        B.twkv_compress(gc.h, 0, xk.cuda(), xv.cuda(), torch.zeros(n + m, dtype=torch.int32).cuda(), pos, None,
+                        torch.stack([rk, rv], 1).to(torch.int16).cuda(), B.TWKV_GATE_FORCED)
+        out = torch.full((1, heads, 128), float("nan"), device="cuda")
+        B.twkv_decode_attn(gc.h, 0, q[None].cuda(), torch.zeros(1, dtype=torch.int32, device="cuda"), out, 1)
+        assert B.twkv_cache_status(gc.h) == B.TWKV_OK
+        gc.close()
+        return out.cpu()
+
+    assert torch.equal(decode(False), decode(True))
