@@ -301,7 +301,9 @@ twkv_status twkv_projector_status(twkv_projector* projector, void* stream);
  * bracketed by CUDA events on the launching stream (events are host-side resources; no device memory
  * is allocated).  twkv_profile_read synchronises `stream`, adds the elapsed times of the launches
  * recorded since the last read to ms[kind] / launches[kind] (host arrays of TWKV_N_KERNELS entries,
- * overwritten) and forgets them.  At most 8192 launches are kept between reads; later ones are not timed. */
+ * overwritten) and forgets them.  At most 8192 launches are kept between reads; later ones are not timed.
+ * A compress call of at most 32 tokens ranks, allocates and moves its rows in one kernel, which counts as
+ * TWKV_K_ALLOC: TWKV_K_GATE_RANK and TWKV_K_PACK have nothing then. */
 typedef enum {
   TWKV_K_GATE_GEMM = 0, TWKV_K_GATE_RANK = 1, TWKV_K_HIST = 2, TWKV_K_ALLOC = 3, TWKV_K_PACK = 4,
   TWKV_K_PLAN = 5, TWKV_K_KSCORE = 6, TWKV_K_VACC = 7, TWKV_K_MERGE = 8, TWKV_K_OTHER = 9, TWKV_N_KERNELS = 10

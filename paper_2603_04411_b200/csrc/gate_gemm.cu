@@ -43,9 +43,9 @@ gate_gemm_kernel(const unsigned short* Xk, const unsigned short* Xv, const unsig
       for (int i = 0; i < 4; ++i) {
         const int c = tid + i * GG_THREADS, row = c >> 3, ch = c & 7;
         const int grow = min(m0 + row, n_tok - 1);            // rows past the end repeat the last row (never stored)
-        if (m0 + (row & ~15) < n_tok) cp_async16(             // (sixteen-row groups without a token are not read at all)
-dA + row * 128 + ((ch ^ (row & 7)) << 4),
-                   reinterpret_cast<const unsigned char*>(X) + ((size_t)grow * d + (k0 + it) * 64) * 2 + ch * 16);
+        if (m0 + (row & ~15) < n_tok)                         // sixteen-row groups without a token are not read at all
+          cp_async16(dA + row * 128 + ((ch ^ (row & 7)) << 4),
+                     reinterpret_cast<const unsigned char*>(X) + ((size_t)grow * d + (k0 + it) * 64) * 2 + ch * 16);
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i) {

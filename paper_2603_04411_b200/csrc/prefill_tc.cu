@@ -280,8 +280,8 @@ __device__ __forceinline__ void unpk2(uint64_t v, float& a, float& b) { asm("mov
 // What bounds it: the epilogue's latencies, with two warps per scheduler, and the way of 128 KiB per item into L2 (about 5 TB/s over
 // all SMs: the same item takes 3.8 us with 128 live rows and 2.1 with twenty).  So the tables of the next item are read an item ahead,
 // a slab is read from tensor memory while the piece before it is rotated, and a part's rows are all read back before the first is
-// stored: a K item 7.3 -> 5 us, 512 queries behind 32768 tokens 880 -> 864 us, five ragged prompts 182 -> 178.  Storing 32 bytes per
-// thread straight from registers instead is as fast for tiles with few rows and 1.6 times slower for full ones.
+// stored: the segments of 32768 tokens 243 -> 227 us by themselves, five ragged prompts 49 -> 45 (the calls 880 -> 864 and 182 -> 178).
+// Storing 32 bytes per thread straight from registers instead is as fast for tiles with few rows and 1.6 times slower for full ones.
 template <bool BF16>
 __global__ void __launch_bounds__(PR_THREADS, 1)
 pf_recon_kernel(const __grid_constant__ CUtensorMap map_blocks, const __grid_constant__ CUtensorMap map_uk,

@@ -19,7 +19,7 @@
 // reads as many bytes of scores as of values, and with one tile in flight their latency bound the kernel.  Where the
 // head count is not a multiple of four (rows not 16-byte aligned: no tensor map) each warp copies the rows of its own
 // token groups with cp.async instead (TS = false).
-// Of a tile that is less than half full (each class of a sequence ends with a partly full one) only the boxes of sixteen rows that hold
+// Of a tile that is at most half full (each class of a sequence ends with a partly full one) only the boxes of sixteen rows that hold
 // tokens are read, and the products run over as many tokens: a batch of short sequences is bound by the bytes of such tiles.
 // Weights go in as two parts of the cache type (see below): 2 N rows of one B operand, so that a panel is read once for both;
 // the two halves of the accumulator are added at the end.
