@@ -500,7 +500,7 @@ __global__ void __launch_bounds__(CHUNK_TOKENS, 7) pack_kernel(DevView v0, int l
 // tiles' rests by all.  What bounds such a call is the chain of dependent reads and of kernel boundaries around them; with more
 // tokens the bytes that eight SMs can move do.  A compress call of n tokens with d_kv 1024 in us, separate kernels / this one (64 and
 // 128 in an eight-CTA form for 128 tokens):
-//   logits given  1 12.9/11.2  8 13.9/11.7  16 14.6/12.5  24 17.3/13.4  32 18.1/14.3  64 18.9/24.1  128 25.1/34.3
+//   logits given  1 12.9/11.2  8 13.9/11.7  16 14.6/12.5  24 17.3/13.4  32 18.1/14.3  64 18.9/24.8  128 25.1/38.1
 //   ranks given   1 10.2/8.7   8 10.8/9.25  16 11.1/9.8   24 12.2/10.5  32 12.4/11.2  64 15.4/20.2  128 22.0/30.5
 // The slots and the zero fill follow pack_kernel's rules; sharing its code cost pack_kernel 0.1 us of 12 (its reads were ordered anew).
 constexpr int AP_CL = 8;
